@@ -12,7 +12,7 @@ CHECKED_LIB_PATH = os.path.join(_HERE, "libkimad_checked.so")  # -DKIMAD_CHECKED
 SOURCES = [os.path.join(_HERE, "csrc", "kimad_api.cu")]
 HEADERS = [os.path.join(_HERE, "csrc", "kimad_kernels.cuh"), os.path.join(_HERE, "csrc", "kimad_select.cuh"),
            os.path.join(_HERE, "csrc", "kimad_curve.cuh"), os.path.join(_HERE, "csrc", "kimad_common.h"),
-           os.path.join(_HERE, "csrc", "kimad_receiver.cuh"),
+           os.path.join(_HERE, "csrc", "kimad_receiver.cuh"), os.path.join(_HERE, "csrc", "kimad_dp.cuh"),
            os.path.join(_ROOT, "include", "kimad.h")]
 
 

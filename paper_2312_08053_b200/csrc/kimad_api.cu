@@ -8,6 +8,7 @@
 #include <new>
 #include <vector>
 
+#include "kimad_dp.cuh"
 #include "kimad_select.cuh"
 #include "kimad_receiver.cuh"
 
@@ -22,12 +23,12 @@ inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Layout {
     // static tables
-    size_t dbuf, chunks, layers, ktab, ktab_dyn, reg_layers, tiny_layers, reg_index, runs;
+    size_t dbuf, chunks, layers, ktab, costs, ktab_dyn, reg_layers, tiny_layers, reg_index, runs;
     // zeroed at set_workspace and kept clean by the kernels
     size_t zero_from, h1_cnt, h1_ss, h23_cnt, h23_ss, bh_cnt, bh_sum, low_hist, recount, recount_bytes, fb, r2, flags;
     // scratch without initial-state requirements
     size_t cell_tab, cell_win, bin_lo, meta, cands, slots, err, tau, keep_eq, shift, sel, chunk_cnt, jobs, csel,
-        fb_chunks, fb_layers, r2_chunks, r2_layers, rf, rf_chunks, rf_layers, pd, total;
+        fb_chunks, fb_layers, r2_chunks, r2_layers, rf, rf_chunks, rf_layers, pd, rows, total;
 };
 
 } // namespace
@@ -50,8 +51,13 @@ struct kimad_ctx {
     size_t sample_smem = 0, pass_a_smem = 0, tiny_smem = 0;
     Layout lay{};
     unsigned char* ws = nullptr;
-    DpPlan dp_plan{};
-    size_t dp_smem = 0;
+    DpPlan dp_plan{};          // policy 0: the knapsack over the budget axis
+    uint32_t dp_cells = 0, dp_threads = 0; // most cells a row can have; threads of a CTA
+    uint32_t hist_row = 0;     // words of a row of the knapsack kept for the backtracking ...
+    bool rows_in_bins = false; // ... in the memory of the bin tables where those are large enough
+    PickPlan pick_plan{};      // the other policies, and given candidates
+    size_t pick_smem = 0;
+    uint32_t pd_stride = 0;    // policy 2: bytes of a row of back-pointers kept in the workspace (0: none are)
     uint64_t launches = 0;
     kimad_packed last_out{};
     bool have_last = false;
@@ -94,6 +100,7 @@ void plan_layout(kimad_ctx* c) {
     y.chunks = take(nch * sizeof(Chunk));
     y.layers = take(c->layers.size() * sizeof(LayerDesc));
     y.ktab = take(c->ktab.size() * sizeof(uint64_t));
+    y.costs = take(c->policy == 0 ? c->ktab.size() * sizeof(double) : 0);
     y.ktab_dyn = take(c->policy == 3 ? (size_t)c->W * c->L * sizeof(uint64_t) : 0); // per-worker rows of the fitted ratio
     y.reg_layers = take(c->reg_layers.size() * sizeof(uint32_t));
     y.tiny_layers = take(c->tiny_layers.size() * sizeof(uint32_t));
@@ -134,7 +141,8 @@ void plan_layout(kimad_ctx* c) {
     y.rf = take(WLK * sizeof(RefineCand));
     y.rf_chunks = take(kGroups * align_up((size_t)c->W * nch * sizeof(uint2)));
     y.rf_layers = take(kGroups * align_up(WL * sizeof(uint2)));
-    y.pd = take(c->dp_plan.pd_in_smem ? 0 : (size_t)c->W * c->L * c->dp_plan.pd_row_bytes);
+    y.pd = take((size_t)c->W * c->L * c->pd_stride);
+    y.rows = take(c->policy == 0 && !c->rows_in_bins ? WL * c->hist_row * sizeof(float) + 16 : 0);
     y.total = o;
 }
 
@@ -143,7 +151,7 @@ void plan_layout(kimad_ctx* c) {
         if ((x) != cudaSuccess) return KIMAD_ERR_CUDA; \
     } while (0)
 
-constexpr size_t kDpSmemMax = 225 * 1024; // dynamic shared memory the DP kernel may ask for
+constexpr size_t kDpSmemMax = 225 * 1024; // dynamic shared memory k_dp and k_pick may ask for
 constexpr uint64_t kSweepRunElems = 4ull << 20; // elements a CTA of the sweep takes at most (as long as four waves suffice)
 constexpr uint64_t kPipelineMinElems = 1ull << 25; // W N from which a step is run as two groups of workers
 
@@ -156,7 +164,7 @@ static int preload_kernels() {
     KIMAD_PRELOAD(k_refine_hist); KIMAD_PRELOAD(k_refine_resolve);
     KIMAD_PRELOAD(k_tiny_exact); KIMAD_PRELOAD(k_fb_hist1); KIMAD_PRELOAD(k_fb_hist23<2>); KIMAD_PRELOAD(k_fb_hist23<3>);
     KIMAD_PRELOAD(k_resolve1); KIMAD_PRELOAD(k_resolve23<2>); KIMAD_PRELOAD(k_resolve23<3>); KIMAD_PRELOAD(k_rebuild_slots);
-    KIMAD_PRELOAD(k_dp); KIMAD_PRELOAD(k_fit_ratio); KIMAD_PRELOAD(k_sel_count); KIMAD_PRELOAD(k_sel_count_r2); KIMAD_PRELOAD(k_sel_resolve);
+    KIMAD_PRELOAD(k_dp<2>); KIMAD_PRELOAD(k_dp<4>); KIMAD_PRELOAD(k_dp<8>); KIMAD_PRELOAD(k_pick); KIMAD_PRELOAD(k_fit_ratio); KIMAD_PRELOAD(k_sel_count); KIMAD_PRELOAD(k_sel_count_r2); KIMAD_PRELOAD(k_sel_resolve);
     KIMAD_PRELOAD(k_sel_resolve_r2); KIMAD_PRELOAD(k_sel_recount); KIMAD_PRELOAD(k_sel_slices); KIMAD_PRELOAD(k_sel_scan);
     KIMAD_PRELOAD((k_sel_write<false, false>)); KIMAD_PRELOAD((k_sel_write<false, true>));
     KIMAD_PRELOAD((k_sel_write<true, false>)); KIMAD_PRELOAD((k_sel_write<true, true>));
@@ -218,6 +226,49 @@ static int ensure_side_stream(kimad_ctx* c) {
     return KIMAD_OK;
 }
 
+// Cells of a row per thread of k_dp.  More cells per thread share the reads of a layer's record (a 1996-cell axis with 1995
+// layers: 2.57 ms with two, 1.87 with four, 1.94 with eight); with fewer, more warps overlap the latencies that bound short rows, and
+// with two all cells of a layer's candidates are requested together (707 cells, 148 layers: 69 us with two, 72 with four).
+static uint32_t dp_cells_per_thread(uint32_t cells) { return cells <= 1024 ? 2 : cells <= 2048 ? 4 : 8; }
+
+// Shared-memory plans of the kernels that choose the candidates; false when the context's policy cannot be run.
+static bool plan_choice(kimad_ctx* c) {
+    const size_t Kp = (c->K + 3) & ~(size_t)3;
+    // k_pick: two rows with their margins and the choice; the error axis (policy 2) also keeps the candidates' tables there
+    PickPlan& q = c->pick_plan;
+    q.pd_nibble = c->K <= 16 ? 1u : 0u;
+    q.pd_row_bytes = q.pd_nibble ? (c->D + 2) / 2 : (c->D + 1);
+    size_t used = ((size_t)2 * (2 * c->D + 3) + c->L) * 4;
+    if (c->policy == 2) {
+        used += (size_t)c->L * Kp * 8;
+        if (used > kDpSmemMax) return false;
+        const size_t pd_bytes = (size_t)c->L * q.pd_row_bytes;
+        q.pd_in_smem = used + pd_bytes <= kDpSmemMax ? 1u : 0u;
+        if (q.pd_in_smem) used += pd_bytes;
+        else c->pd_stride = q.pd_row_bytes;
+    }
+    if (used > kDpSmemMax) return false;
+    c->pick_smem = used;
+    if (c->policy != 0) return true;
+    // k_dp.  Every layer takes at least one cell, so a row has at most D - L + 1 cells.
+    DpPlan& p = c->dp_plan;
+    c->dp_cells = c->D - c->L + 1;
+    const uint32_t per = dp_cells_per_thread(c->dp_cells);
+    c->dp_threads = std::max<uint32_t>(512, ((c->dp_cells + per - 1) / per + 31) & ~31u);
+    c->hist_row = (c->dp_cells + 3 + 4) & ~3u;
+    c->rows_in_bins = c->reg_layers.size() * (size_t)(kMaxBins + 1) >= (size_t)c->L * c->hist_row + 4; // (rows start on a 16-byte boundary)
+    p.kr = (c->K + 7) & ~7u;
+    p.rw = 2 * p.kr + 4;
+    p.chunk_layers = std::min<uint32_t>(std::min(kDpMaxChunkLayers, c->L), 32768 / (p.rw * 4));
+    const size_t tab = (size_t)2 * p.chunk_layers * p.rw * 4, slot = (size_t)(2 * c->dp_cells + 8) * 4, tail = (7 * c->L + 15) & ~15u;
+    const size_t beyond = 32 * 8 * 4; // the last warp reads past the row's last cell, at most so far
+    const size_t most = (kDpSmemMax - tail - beyond) & ~(size_t)15;
+    if (tab + 2 * slot > most) return false;
+    p.work_bytes = (uint32_t)std::min(most, (std::max<size_t>(tab + kDpMaxRing * slot, 96 * 1024) + 15) & ~(size_t)15);
+    p.smem = (uint32_t)(p.work_bytes + tail + beyond);
+    return 8 * (size_t)c->L <= p.work_bytes;
+}
+
 // Once per device and process: shared-memory limits of the kernels (a property of the function, shared by all
 // contexts: the limits do not depend on the context) and the kernel preload.  Per context: its side stream.
 static int prepare_device(kimad_ctx* c) {
@@ -226,7 +277,10 @@ static int prepare_device(kimad_ctx* c) {
     CUDA_TRY(cudaGetDevice(&dev));
     if (dev < 0 || dev >= KIMAD_BUILTIN_MAX_DEVICES) return KIMAD_ERR_INVALID_ARG;
     if (!ready[dev]) {
-        CUDA_TRY(cudaFuncSetAttribute(k_dp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDpSmemMax));
+        CUDA_TRY(cudaFuncSetAttribute(k_dp<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDpSmemMax));
+        CUDA_TRY(cudaFuncSetAttribute(k_dp<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDpSmemMax));
+        CUDA_TRY(cudaFuncSetAttribute(k_dp<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDpSmemMax));
+        CUDA_TRY(cudaFuncSetAttribute(k_pick, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDpSmemMax));
         CUDA_TRY(cudaFuncSetAttribute(k_sample, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->sample_smem));
         CUDA_TRY(cudaFuncSetAttribute(k_pass_a<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->pass_a_smem));
         CUDA_TRY(cudaFuncSetAttribute(k_pass_a<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->pass_a_smem));
@@ -298,6 +352,7 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
     const uint32_t R = (uint32_t)c->reg_layers.size(), T = (uint32_t)c->tiny_layers.size();
     const dim3 blk(kThreads);
     const uint32_t list_cap = W * nch; // entries of every chunk list (twice that for the recount list)
+    const CodeSpace codes{reg_index, meta, cell_tab, cell_win, R};
     int stage = 0;
     auto mark = [&](cudaStream_t st) { if (c->timing) cudaEventRecord(c->ev[stage++], st); };
     auto budgets_of = [&](uint32_t w0, uint32_t nw) {
@@ -387,7 +442,7 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
         mark(big);
         CUDA_TRY(hand_over(big, small));
         if (R) {
-            CUDA_TRY(launch_pdl(k_resolve_a, dim3(R, nw), kBigThreads, 0, small, layers, reg_layers, R, L, ktab, K, meta, binlo, bhc, bhs,
+            CUDA_TRY(launch_pdl(k_resolve_a, dim3(R, nw), kBigThreads, 0, small, layers, reg_layers, R, L, ktab, K, meta, cell_win, binlo, bhc, bhs,
                                 err, tau, keq, shf, flags, fb, fb_chunks, fb_layers, rf, rf_chunks, rf_layers, list_cap, w0));
             c->launches += 1;
         }
@@ -397,11 +452,30 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
         auto launch_dp = [&](cudaStream_t st, uint32_t when) -> int {
             for (uint32_t wa = w0; wa < w0 + nw; wa += kDpWorkersPerLaunch) {
                 const uint32_t nwa = std::min<uint32_t>(kDpWorkersPerLaunch, w0 + nw - wa);
-                const int dp_mode = mode == kGivenJ ? 1 : (c->policy == 1 ? 2 : (c->policy == 2 ? 3 : (c->policy == 3 ? 4 : 0)));
-                CUDA_TRY(launch_pdl(k_dp, nwa, kDpThreads, c->dp_smem, st, budgets_of(wa, nwa), wa, W, L, K, c->D, c->bpe, c->full_bytes,
-                                    c->cap, c->check_finite, dp_mode, c->cost_model, c->dp_plan, layers,
-                                    ktab, mode == kInjectErr ? err_dev : err, tau, keq, shf, j_dev, flags, pd, sel, out->k, out->j,
-                                    out->offs, out->stats, out->dense, CodeSpace{reg_index, meta, cell_tab, cell_win, R}, when, fb));
+                const ChooseArgs ca{W, L, K, c->D, c->bpe, c->check_finite, c->cost_model, c->full_bytes, c->cap, layers, ktab,
+                                    mode == kInjectErr ? err_dev : err, tau, keq, shf, flags, sel, out->k, out->j, out->offs,
+                                    out->stats, out->dense, fb, when};
+                if (mode != kGivenJ && c->policy == 0) {
+                    const DpPlan& p = c->dp_plan;
+                    // A worker's candidate records lie where the exact path keeps its slots (for long grids its candidates): the
+                    // DP only goes ahead when that path has nothing to do for the worker's group or is done.  The rows kept
+                    // for the backtracking lie where the sample kernel left the bins' lower keys, which nobody reads after
+                    // the curves.
+                    const bool in_slots = 2 * p.rw * 4 <= sizeof(SlotTab);
+                    uint32_t* tab = in_slots ? reinterpret_cast<uint32_t*>(slots) : reinterpret_cast<uint32_t*>(cands);
+                    const size_t tab_stride = (in_slots ? L * sizeof(SlotTab) : (size_t)L * K * sizeof(Cand)) / 16 * 4;
+                    float* rows = c->rows_in_bins ? reinterpret_cast<float*>(binlo) : c->at<float>(y.rows);
+                    const size_t row_stride = c->rows_in_bins ? (size_t)R * (kMaxBins + 1) : (size_t)L * c->hist_row;
+                    auto launch = [&](auto kern) {
+                        return launch_named("k_dp", kern, nwa, c->dp_threads, p.smem, st, budgets_of(wa, nwa), wa, ca, p, c->at<double>(y.costs), tab, tab_stride,
+                                            rows, row_stride, c->hist_row);
+                    };
+                    const uint32_t per = dp_cells_per_thread(c->dp_cells);
+                    CUDA_TRY(per == 2 ? launch(k_dp<2>) : (per == 4 ? launch(k_dp<4>) : launch(k_dp<8>)));
+                } else {
+                    const int pick = mode == kGivenJ ? 1 : (c->policy == 1 ? 2 : (c->policy == 2 ? 3 : 4));
+                    CUDA_TRY(launch_pdl(k_pick, nwa, kPickThreads, c->pick_smem, st, budgets_of(wa, nwa), wa, ca, pick, c->pick_plan, j_dev, pd));
+                }
                 c->launches += 1;
             }
             return KIMAD_OK;
@@ -413,17 +487,16 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
             const uint32_t gfb = 4 * 148, glay = std::min<uint32_t>(nw * R, 32u);
             const dim3 gslot(glay, 1, K);
             // candidates with a loose bound first (they may still end on the exact path's lists)
-            CUDA_TRY(launch_pdl(k_refine_hist, 6 * 148, blk, 0, st, dbuf, chunks, c->dstride, L, K, fb, rf_chunks, rf,
-                                CodeSpace{reg_index, meta, cell_tab, cell_win, R}, h23c, h23s));
+            CUDA_TRY(launch_pdl(k_refine_hist, 6 * 148, blk, 0, st, dbuf, chunks, c->dstride, L, K, fb, rf_chunks, rf, codes, h23c, h23s));
             CUDA_TRY(launch_pdl(k_refine_resolve, glay, blk, 0, st, layers, L, K, fb, rf_layers, rf, h23c, h23s, err, tau, keq, shf,
-                                fb_chunks, fb_layers, list_cap));
+                                codes, fb_chunks, fb_layers, list_cap));
             CUDA_TRY(launch_pdl(k_fb_hist1, gfb, blk, 0, st, dbuf, chunks, c->dstride, L, fb, fb_chunks, h1c, h1s, flags));
             CUDA_TRY(launch_pdl(k_resolve1, glay, blk, 0, st, fb, fb_layers, h1c, h1s, ktab, L, K, cands, slots));
             CUDA_TRY(launch_pdl(k_fb_hist23<2>, gfb, blk, 0, st, dbuf, chunks, c->dstride, L, K, fb, fb_chunks, slots, h23c, h23s));
-            CUDA_TRY(launch_pdl(k_resolve23<2>, gslot, blk, 0, st, fb, fb_layers, h23c, h23s, L, K, cands, slots, err, tau, keq, shf));
+            CUDA_TRY(launch_pdl(k_resolve23<2>, gslot, blk, 0, st, fb, fb_layers, h23c, h23s, L, K, cands, slots, err, tau, keq, shf, codes));
             CUDA_TRY(launch_pdl(k_rebuild_slots, (nw * R + kThreads - 1) / kThreads, blk, 0, st, fb, fb_layers, L, K, cands, slots));
             CUDA_TRY(launch_pdl(k_fb_hist23<3>, gfb, blk, 0, st, dbuf, chunks, c->dstride, L, K, fb, fb_chunks, slots, h23c, h23s));
-            CUDA_TRY(launch_pdl(k_resolve23<3>, gslot, blk, 0, st, fb, fb_layers, h23c, h23s, L, K, cands, slots, err, tau, keq, shf));
+            CUDA_TRY(launch_pdl(k_resolve23<3>, gslot, blk, 0, st, fb, fb_layers, h23c, h23s, L, K, cands, slots, err, tau, keq, shf, codes));
             c->launches += 9;
             return KIMAD_OK;
         };
@@ -510,6 +583,8 @@ int kimad_create(kimad_ctx** out, const uint64_t* layer_sizes, uint32_t n_layers
         c->L = n_layers; c->W = n_workers; c->K = n_ratios; c->D = o.D;
         c->value_dtype = o.value_dtype; c->check_finite = o.check_finite;
         c->bpe = o.value_dtype == 0 ? 8 : 6;
+        c->policy = o.policy;
+        c->cost_model = o.cost_model;
         c->layer_sizes.assign(layer_sizes, layer_sizes + n_layers);
         c->grid.assign(ratio_grid, ratio_grid + n_ratios);
         c->ktab.resize((size_t)n_layers * n_ratios);
@@ -547,23 +622,8 @@ int kimad_create(kimad_ctx** out, const uint64_t* layer_sizes, uint32_t n_layers
         c->cap = o.max_packed_elems ? o.max_packed_elems : N;
         if (c->stride < N || c->chunks.size() > 0x7fffffffull) { delete c; return KIMAD_ERR_INVALID_ARG; }
         c->dstride = (N + 15) / 16 * 16; // every worker's code plane starts on a 16-byte boundary
-        // shared-memory plan of the DP kernel
-        const size_t Kp = (c->K + 3) & ~(size_t)3;
-        const size_t dp_base = ((size_t)2 * (2 * c->D + 3) + c->L) * 4 + 16; // + alignment slack of the candidate tables
-        const size_t tab_all = (size_t)c->L * (Kp * 8 + 4), tab_one = Kp * 8 + 4;
-        c->dp_plan.pd_nibble = c->K <= 16 ? 1u : 0u;
-        c->dp_plan.pd_row_bytes = c->dp_plan.pd_nibble ? (c->D + 2) / 2 : (c->D + 1);
-        const size_t pd_bytes = (size_t)c->L * c->dp_plan.pd_row_bytes;
-        if (dp_base + tab_one > kDpSmemMax) { delete c; return KIMAD_ERR_INVALID_ARG; }
-        c->dp_plan.tab_in_smem = dp_base + tab_all <= kDpSmemMax ? 1u : 0u;
-        size_t used = dp_base + (c->dp_plan.tab_in_smem ? tab_all : tab_one);
-        c->dp_plan.pd_in_smem = used + pd_bytes <= kDpSmemMax ? 1u : 0u;
-        if (c->dp_plan.pd_in_smem) used += pd_bytes;
-        c->dp_smem = used;
+        if (!plan_choice(c)) { delete c; return KIMAD_ERR_INVALID_ARG; }
         c->curve_mode = o.curve_mode;
-        c->policy = o.policy;
-        c->cost_model = o.cost_model;
-        if (c->policy == 2 && !c->dp_plan.tab_in_smem) { delete c; return KIMAD_ERR_INVALID_ARG; }
         c->sample_smem = (size_t)(2 * (1024 + 32) + 32768 + 1024 + 2 * kMaxGaps + 32 + 3 * 128) * 4;
         c->pass_a_smem = (size_t)(2 * kMaxBins + kCellTab) * 4;
         { // the sweep's runs, one CTA each: every worker's chunk list is cut into pieces of about equal element counts.
@@ -593,6 +653,11 @@ int kimad_create(kimad_ctx** out, const uint64_t* layer_sizes, uint32_t n_layers
             std::memcpy(im + y.chunks, c->chunks.data(), c->chunks.size() * sizeof(Chunk));
             std::memcpy(im + y.layers, c->layers.data(), c->layers.size() * sizeof(LayerDesc));
             std::memcpy(im + y.ktab, c->ktab.data(), c->ktab.size() * sizeof(uint64_t));
+            if (c->policy == 0) {
+                double* costs = reinterpret_cast<double*>(im + y.costs);
+                for (size_t i = 0; i < c->ktab.size(); ++i)
+                    costs[i] = candidate_cost(c->layer_sizes[i / c->K], c->ktab[i], c->bpe, c->cost_model, c->D);
+            }
             if (!c->reg_layers.empty()) std::memcpy(im + y.reg_layers, c->reg_layers.data(), c->reg_layers.size() * 4);
             if (!c->tiny_layers.empty()) std::memcpy(im + y.tiny_layers, c->tiny_layers.data(), c->tiny_layers.size() * 4);
             std::memcpy(im + y.reg_index, c->reg_index.data(), c->reg_index.size() * 4);
@@ -806,7 +871,10 @@ int kimad_debug_get_curve(kimad_ctx* c, float* host_err, uint32_t* host_tau, uin
     if (host_err) CUDA_TRY(cudaMemcpy(host_err, c->ws + c->lay.err, n * 4, cudaMemcpyDeviceToHost));
     if (host_tau) CUDA_TRY(cudaMemcpy(host_tau, c->ws + c->lay.tau, n * 4, cudaMemcpyDeviceToHost));
     if (host_keep_eq) CUDA_TRY(cudaMemcpy(host_keep_eq, c->ws + c->lay.keep_eq, n * 4, cudaMemcpyDeviceToHost));
-    if (host_shift) CUDA_TRY(cudaMemcpy(host_shift, c->ws + c->lay.shift, n * 4, cudaMemcpyDeviceToHost));
+    if (host_shift) {
+        CUDA_TRY(cudaMemcpy(host_shift, c->ws + c->lay.shift, n * 4, cudaMemcpyDeviceToHost));
+        for (size_t i = 0; i < n; ++i) host_shift[i] &= 255u; // the code of the interval's keys lies above
+    }
     return KIMAD_OK;
 }
 

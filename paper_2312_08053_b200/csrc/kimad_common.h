@@ -95,4 +95,12 @@ KIMAD_HD uint64_t candidate_bytes(uint64_t n, uint64_t k, uint32_t bpe, uint32_t
 // the byte constraint of Eq. 3 can never be exceeded).  c > 0.
 KIMAD_HD uint64_t budget_cells(uint64_t bytes, uint32_t D, uint64_t c) { return (bytes * (uint64_t)D + c - 1) / c; }
 
+// The numerator's share of that for a candidate, bytes * D, as the knapsack kernel reads it (binary64, exact: below 2^48);
+// negative where the layer is sent densely.
+inline double candidate_cost(uint64_t n, uint64_t k, uint32_t bpe, uint32_t cost_model, uint32_t D) {
+    bool dense;
+    const double x = (double)(candidate_bytes(n, k, bpe, cost_model, &dense) * (uint64_t)D);
+    return dense ? -x : x;
+}
+
 } // namespace kimad

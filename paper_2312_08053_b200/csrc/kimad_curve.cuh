@@ -610,7 +610,7 @@ k_pass_a(const float* __restrict__ grads, const float* __restrict__ state, uint8
 // ------------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(kBigThreads)
 k_resolve_a(const LayerDesc* __restrict__ layers, const uint32_t* __restrict__ reg_layers, uint32_t R, uint32_t L,
-            const KTab ktab, uint32_t K, const BandMeta* __restrict__ meta,
+            const KTab ktab, uint32_t K, const BandMeta* __restrict__ meta, const int4* __restrict__ cell_win,
             const uint32_t* __restrict__ bin_lo, uint32_t* __restrict__ bh_cnt, unsigned long long* __restrict__ bh_sum,
             float* __restrict__ err_out, uint32_t* __restrict__ tau_out, uint32_t* __restrict__ rank_out,
             uint32_t* __restrict__ shift_out, uint32_t* __restrict__ flags, FbList* __restrict__ fb,
@@ -639,6 +639,7 @@ k_resolve_a(const LayerDesc* __restrict__ layers, const uint32_t* __restrict__ r
     if (!mt.flagged) {
         const uint32_t nb = mt.n_bins, ngrp = (nb + 31u) >> 5; // groups of 32 consecutive bins (ascending keys)
         const uint32_t* blo = bin_lo + wr * (kMaxBins + 1);
+        const uint32_t ls = (uint32_t)cell_win[wr].w & 31u;
         uint32_t* gc = bh_cnt + wr * kMaxBins;
         unsigned long long* gs = bh_sum + wr * kMaxBins;
         const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -727,7 +728,7 @@ k_resolve_a(const LayerDesc* __restrict__ layers, const uint32_t* __restrict__ r
             err_out[o] = (float)e;
             tau_out[o] = klo;
             rank_out[o] = cb - drop;
-            shift_out[o] = 31 - __clz(width);
+            shift_out[o] = (31 - __clz(width)) | (bin >> ls) << 8; // with the code of the bin's entries
         }
         __syncthreads();
         for (uint32_t bb = threadIdx.x; bb < nb; bb += kBigThreads) // clean for the next step
@@ -853,7 +854,7 @@ __global__ void __launch_bounds__(kThreads)
 k_refine_resolve(const LayerDesc* __restrict__ layers, uint32_t L, uint32_t K, FbList* __restrict__ fb,
                  const uint2* __restrict__ rf_layers, RefineCand* __restrict__ rf, uint32_t* __restrict__ g_cnt,
                  unsigned long long* __restrict__ g_ss, float* __restrict__ err_out, uint32_t* __restrict__ tau_out,
-                 uint32_t* __restrict__ rank_out, uint32_t* __restrict__ shift_out, uint2* __restrict__ fb_chunks,
+                 uint32_t* __restrict__ rank_out, uint32_t* __restrict__ shift_out, const CodeSpace codes, uint2* __restrict__ fb_chunks,
                  uint2* __restrict__ fb_layers, uint32_t list_cap) {
     pdl_wait();
     __shared__ uint32_t s_w32[8];
@@ -907,7 +908,8 @@ k_refine_resolve(const LayerDesc* __restrict__ layers, uint32_t L, uint32_t K, F
                     if (slack > e * 5e-6) {
                         s_bad = 1;
                     } else {
-                        err_out[o] = (float)e; tau_out[o] = klo; rank_out[o] = c[i] - d2; shift_out[o] = sub;
+                        err_out[o] = (float)e; tau_out[o] = klo; rank_out[o] = c[i] - d2;
+                        shift_out[o] = sub | codes.code(w, l, klo) << 8;
                     }
                 }
                 before += c[i];
@@ -1097,7 +1099,7 @@ k_tiny_exact(const float* __restrict__ grads, const float* __restrict__ state, u
         err_out[o] = k < n ? (float)s_suf[k] : 0.f;
         tau_out[o] = t;
         rank_out[o] = k - (uint32_t)lo;
-        shift_out[o] = 0;
+        shift_out[o] = code_of_key(t) << 8;
     }
 }
 

@@ -1,0 +1,815 @@
+// Stage (c): the knapsack dynamic program over the budget axis (Eq. 2, Eq. 3, Section 3.2, Algorithm 3), one CTA per
+// worker, and what every way of choosing the candidates ends with (offsets, statistics, the select records).
+//
+// The recursion cur[b] = min_j fl(prev[b - u_j] + e_j) is serial in the layers and its binary32 sums must be taken left
+// to right (the value decides ties), so the only parallelism is over the cells of a row.
+//
+//   * The row is cut to the cells that can matter.  Every layer takes at least its smallest candidate's cells, so the
+//     row is kept relative to the sum of those: width = D - sum_l u_{l,0} + 1, candidates shifted by u_{l,0}.
+//   * Where all candidates of a layer take the same number of cells (small tensors under a coarse cell) the shifted
+//     layer reads its own cell only: such layers are applied in registers.  Between other layers the row is exchanged
+//     through shared memory.
+//   * A candidate only reads cells at or below its own, so an exchange needs no barrier: a warp owns consecutive cells and
+//     waits for the warps below it only, by a progress counter per warp; rows live in a ring of a few slots, so lower
+//     warps run ahead and the latencies of the warps' chains overlap.
+//   * The recursion carries values only, and of several candidates with the same cells only the smallest error.  The
+//     exchanged rows go to the workspace, and the winning candidates -- the first that attains the minimum -- are found on
+//     the chosen path alone, last layer first, by repeating the one cell's sums.
+//
+// Bound by instruction issue and shared-memory reads of one SM on wide axes (a record's uniform 128-bit reads cost about as
+// much as the cells they address), by the chain of latencies per exchange on short ones, and by the cold start of the
+// records and of the backtracking's rows.  Against one CTA with a barrier per layer, every candidate's index carried along
+// and back-pointers for every cell: GPT-2 small's 148 layers, 16 candidates, D = 1000: 163 -> 69 us; 1995 blocks of it,
+// D = 3990: 12.4 -> 1.87 ms; ResNet-18's 62 layers, 7 candidates: 60 -> 32 us.
+//
+// Waits are on warps of the same CTA and are bounded: a wait that runs out marks the worker's result KIMAD_ERR_TIMEOUT and
+// the remaining waits are skipped.
+#pragma once
+#include <type_traits>
+
+#include "kimad_kernels.cuh"
+
+namespace kimad {
+
+constexpr int kDpMaxThreads = 1024;
+constexpr int kDpMaxRing = 8;                  // rows in flight at most
+constexpr uint32_t kDpMaxChunkLayers = 256;    // layers whose records are staged at a time (two buffers)
+constexpr long long kDpWaitClocks = 1ll << 31; // about a second; an exchange takes about a microsecond
+constexpr uint32_t kDpSameBit = 0x10000u;      // head: all usable candidates of the layer take the same number of cells
+
+// Plan of a launch (host).  A layer has two records of rw = 2 kr + 4 words (kr = K rounded up to 8): {byte offsets of the
+// cells read, i.e. -4 (u_j - u_0), [kr] | errors [kr] | head}.  The first holds the distinct cells with their smallest
+// error (head: their number | kDpSameBit, smallest error of all), the second all usable candidates (head: their number,
+// the smallest error, the largest u_j - u_0); entries that cannot be used repeat candidate 0.
+// Shared memory: work_bytes (two chunks of first records | ring of rows; the backtracking's rows and records lie over
+// them), then a value, the exchange's layer and the choice per layer (7 bytes).
+struct DpPlan {
+    uint32_t kr, rw;
+    uint32_t chunk_layers;
+    uint32_t work_bytes;
+    uint32_t smem; // dynamic shared memory in all
+};
+
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void cp_async_16(uint32_t dst, const void* src) { asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory"); }
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+template <int OFF>
+__device__ __forceinline__ float lds_f32(uint32_t addr) { float x; asm volatile("ld.shared.f32 %0, [%1+%2];" : "=f"(x) : "r"(addr), "n"(OFF)); return x; }
+// x[q][k] = word 32 q of the row at addr, q < CPT
+template <int CPT, int N, int Q = 0>
+__device__ __forceinline__ void lds_cells(float (&x)[CPT][N], int k, uint32_t addr) {
+    if constexpr (Q < CPT) {
+        x[Q][k] = lds_f32<128 * Q>(addr);
+        lds_cells<CPT, N, Q + 1>(x, k, addr);
+    }
+}
+__device__ __forceinline__ float min3(float a, float b, float c) { float m; asm("min.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(a), "f"(b), "f"(c)); return m; }
+// orders the accesses before it and after it for the threads of the CTA (the progress counters need no more than this;
+// __threadfence_block is the sequentially consistent fence and costs several times as much here)
+__device__ __forceinline__ void fence_cta() { asm volatile("fence.acq_rel.cta;" ::: "memory"); }
+// bounded wait of a warp: until every lane's counter has reached the lane's target
+__device__ __forceinline__ void progress_wait(const volatile uint32_t* counter, int target, volatile uint32_t* failed) {
+    if (!__all_sync(0xffffffffu, (int)*counter >= target)) {
+        const long long start = clock64();
+        while (!__all_sync(0xffffffffu, (int)*counter >= target)) {
+            if (clock64() - start > kDpWaitClocks) *failed = 1u;
+            if (__any_sync(0xffffffffu, *failed != 0u)) break;
+        }
+    }
+    fence_cta();
+    __syncwarp();
+}
+
+// ------------------------------------------------------------------------------------------------
+// What follows the choice of a candidate per layer, by one CTA: totals, capacity check, output offsets, statistics and
+// the records of the select stage.
+// ------------------------------------------------------------------------------------------------
+struct DpBudgets { uint64_t c[kDpWorkersPerLaunch]; };
+
+struct ChooseArgs {
+    uint32_t W, L, K, D, bpe, check_finite, cost_model;
+    uint64_t full_bytes, cap;
+    const LayerDesc* layers;
+    KTab ktab;
+    const float* err;          // [W][L][K]
+    const uint32_t *tau, *keep_eq, *shift; // shift: log2 of the interval's width | code of its keys << 8
+    uint32_t* flags;
+    Sel* sel;
+    uint32_t *out_k, *out_j;
+    uint64_t* out_offs;
+    kimad_stats* out_stats;
+    uint32_t* out_dense;       // may be null
+    const FbList* lists;
+    uint32_t when; // 0: always; 1: only if no layer is listed for refinement or the exact path; 2: only if one is
+};
+
+// a layer listed for refinement may move on to the exact path's list while a launch with when = 1 runs, but then the
+// refinement's list alone decides
+__device__ __forceinline__ bool choose_applies(const ChooseArgs& a) {
+    return a.when == 0u || ((a.lists->rf_layers != 0u || a.lists->n_layers != 0u) == (a.when == 2u));
+}
+
+// s_j[L]: the chosen candidates (read when status >= 0); s_k[L], s_e[L]: scratch.  `fitted`: the candidates come from the
+// ratio sized to the budget, feasibility is decided here.  The total error is added left to right in binary32, over the
+// layers in order, unless the caller already has that sum (`total`: the knapsack's own value of the chosen cell).
+template <typename J>
+__device__ __forceinline__ void choose_finish(const ChooseArgs& a, uint32_t w, uint64_t c, int status, bool fitted,
+                                              const float* total, const J* s_j, uint32_t* s_k, float* s_e) {
+    __shared__ unsigned long long s_nsel, s_used, s_part[kDpMaxThreads / 32];
+    __shared__ int s_final;
+    const uint32_t L = a.L, K = a.K, lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const float* e_w = a.err + (size_t)w * L * K;
+    if (threadIdx.x == 0) { s_nsel = 0; s_used = 0; }
+    __syncthreads();
+    auto record = [&](uint32_t l) { // everything of the select record that does not depend on the totals
+        const size_t o = ((size_t)w * L + l) * K + s_j[l];
+        Sel s;
+        s.tau = a.tau[o];
+        s.keep_eq = a.keep_eq[o];
+        s.shift = a.shift[o];
+        s.tau_low = 0;
+        s.code = s.shift >> 8; // (kept beside the interval's width)
+        s.shift &= 255u;
+        s.k = 0;
+        s.base = 0;
+        return s;
+    };
+    if (status >= 0) {
+        unsigned long long my_n = 0, my_b = 0;
+        for (uint32_t l = threadIdx.x; l < L; l += blockDim.x) {
+            const uint64_t n = a.layers[l].n, k = a.ktab.at(w, (size_t)l * K + s_j[l]);
+            bool dense;
+            my_b += candidate_bytes(n, k, a.bpe, a.cost_model, &dense);
+            const uint32_t k_eff = (uint32_t)(dense ? n : k);
+            my_n += k_eff;
+            s_k[l] = k_eff;
+            if (!total) s_e[l] = dense ? 0.f : e_w[(size_t)l * K + s_j[l]];
+            if (a.out_dense) a.out_dense[(size_t)w * L + l] = dense ? 1u : 0u;
+        }
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+            my_n += __shfl_xor_sync(0xffffffffu, my_n, o);
+            my_b += __shfl_xor_sync(0xffffffffu, my_b, o);
+        }
+        if (lane == 0) { atomicAdd(&s_nsel, my_n); atomicAdd(&s_used, my_b); }
+    } else if (a.out_dense) {
+        for (uint32_t l = threadIdx.x; l < L; l += blockDim.x) a.out_dense[(size_t)w * L + l] = 0u;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const uint64_t nsel = s_nsel;
+        float tot = 0.f;
+        if (status >= 0) {
+            if (total) tot = *total;
+            else
+                for (uint32_t l = 0; l < L; ++l) tot = __fadd_rn(tot, s_e[l]);
+        }
+        if (status == KIMAD_OK && fitted && s_used > c) status = KIMAD_STATUS_INFEASIBLE; // not even one entry per layer fits
+        if (status >= 0 && nsel > a.cap) status = KIMAD_ERR_CAPACITY;
+        kimad_stats s;
+        s.budget_bytes = c;
+        s.n_selected = status >= 0 ? nsel : 0;
+        s.used_bytes = status >= 0 ? s_used : 0;
+        s.total_err = status >= 0 ? tot : 0.f;
+        s.status = status;
+        a.out_stats[w] = s;
+        s_final = status;
+        a.flags[w] = 0; // consumed
+    }
+    __syncthreads();
+    status = s_final;
+    unsigned long long run = 0; // entries kept in the layers before this pass
+    for (uint32_t l0 = 0; l0 < L; l0 += blockDim.x) {
+        const uint32_t l = l0 + threadIdx.x;
+        const unsigned long long k = l < L && status >= 0 ? s_k[l] : 0u;
+        unsigned long long incl = k;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= (uint32_t)o) incl += y;
+        }
+        __syncthreads(); // s_part may still be read from the previous pass
+        if (lane == 31) s_part[wid] = incl;
+        __syncthreads();
+        unsigned long long before = run, all = 0;
+        for (uint32_t i = 0; i < nw; ++i) {
+            const unsigned long long t = s_part[i];
+            if (i < wid) before += t;
+            all += t;
+        }
+        if (l < L) {
+            const size_t wl = (size_t)w * L + l;
+            const unsigned long long base = before + incl - k;
+            a.out_offs[(size_t)w * (L + 1) + l] = base;
+            Sel s{};
+            uint32_t j = 0;
+            if (status >= 0) {
+                j = s_j[l];
+                s = record(l);
+                s.k = (uint32_t)k;
+                s.base = base;
+            }
+            a.out_k[wl] = s.k;
+            a.out_j[wl] = j;
+            a.sel[wl] = s;
+        }
+        run += all;
+    }
+    if (threadIdx.x == 0) a.out_offs[(size_t)w * (L + 1) + L] = run;
+}
+
+// ------------------------------------------------------------------------------------------------
+// k_dp: one CTA per worker; a thread owns CPT cells of a row (32 apart: a warp owns 32 CPT consecutive cells)
+// ------------------------------------------------------------------------------------------------
+template <int CPT>
+__global__ void __launch_bounds__(CPT <= 4 ? 512 : kDpMaxThreads, 1)
+k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double* __restrict__ cost /* [L][K], see kimad_common.h */,
+     uint32_t* __restrict__ tab_all /* [W] at tab_stride words, [L][2][rw] each */, size_t tab_stride,
+     float* __restrict__ hist_all /* [W] at hist_stride words, [exchanges][hist_row] each */, size_t hist_stride, uint32_t hist_row) {
+    pdl_wait();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ uint32_t s_prog[32], s_failed, s_reach, s_cell, s_left;
+    __shared__ unsigned long long s_sum;
+    __shared__ float s_redv[kDpMaxThreads / 32], s_total;
+    __shared__ uint32_t s_redb[kDpMaxThreads / 32];
+
+    const uint32_t w = w_base + blockIdx.x;
+    if (!choose_applies(a)) return;
+    const uint32_t L = a.L, K = a.K, D = a.D, T = blockDim.x;
+    const uint32_t t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    const uint64_t c = budgets.c[blockIdx.x];
+    const float kInf = __int_as_float(0x7f800000);
+    const uint32_t kr = plan.kr, rw = plan.rw, rec16 = rw / 4u, CL = plan.chunk_layers;
+    uint32_t* s_tab = reinterpret_cast<uint32_t*>(smem_raw);           // [2][CL * rw]
+    float* ring = reinterpret_cast<float*>(s_tab + 2u * CL * rw);
+    float* s_p = reinterpret_cast<float*>(smem_raw + plan.work_bytes); // [L] smallest error, later the value before the layer
+    uint16_t* s_ex = reinterpret_cast<uint16_t*>(s_p + L);             // [L] layer of every exchange
+    uint8_t* s_j = reinterpret_cast<uint8_t*>(s_ex + L);               // [L]
+    uint32_t* s_k = reinterpret_cast<uint32_t*>(smem_raw);             // [L], [L]: scratch of the end (work_bytes >= 8 L)
+    float* s_e = reinterpret_cast<float*>(s_k + L);
+    uint32_t* tab = tab_all + w * tab_stride;
+    float* hist = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(hist_all + w * hist_stride) + 15u) & ~(uintptr_t)15u);
+
+    int status = KIMAD_OK;
+    if (a.check_finite && (a.flags[w] & 1u)) status = KIMAD_ERR_NONFINITE;
+    else if (c >= a.full_bytes) status = KIMAD_STATUS_PLATEAU;
+    else if (c == 0) status = KIMAD_STATUS_INFEASIBLE;
+    if (t == 0) { s_failed = 0; s_sum = 0; s_reach = 0; }
+    __syncthreads(); // (and the flags are read before the end of the choice resets them)
+
+    // ---- the layers' records; 8, 16 or 32 lanes per layer, the loads of the next layers ahead of the current ones' work
+    const uint32_t G = kr <= 8u ? 8u : (kr <= 16u ? 16u : 32u), per = 32u / G; // lanes per layer, layers per warp
+    const uint32_t sub = lane / G, jj = lane % G, stride = (T >> 5) * per;
+    if (status == KIMAD_OK) {
+        const uint32_t gmask = G == 32u ? 0xffffffffu : (((1u << G) - 1u) << (sub * G));
+        constexpr int AHEAD = 4; // layers per group of lanes whose inputs are requested together (they come from DRAM on most steps)
+        const uint32_t rounds = (kr + G - 1u) / G; // above 1: more than 32 candidates
+        unsigned long long sum = 0;
+        uint32_t reach = 0;
+        // budget_cells = (bytes D + c - 1) / c in binary64: everything is an integer below 2^50 (bytes < 2^35, D < 2^13, c below
+        // the sum of the layers' sizes), the quotient from the reciprocal is off by one at most and the remainder is exact
+        const double cd = (double)c, inv_c = 1.0 / cd, c_1 = cd - 1.0, most = (double)(D + 1u);
+        for (uint32_t l4 = wid * per; l4 < L; l4 += AHEAD * stride) {
+            double x_[AHEAD];
+            float e_[AHEAD];
+            auto fetch = [&](uint32_t l, uint32_t j, double& x, float& e) {
+                x = 0.0; e = 0.f;
+                if (l < L && j < K) { x = cost[(size_t)l * K + j]; e = a.err[((size_t)w * L + l) * K + j]; }
+            };
+#pragma unroll
+            for (int i = 0; i < AHEAD; ++i) fetch(l4 + i * stride + sub, jj, x_[i], e_[i]);
+#pragma unroll
+            for (int i = 0; i < AHEAD; ++i) {
+                if (l4 + i * stride >= L) break;
+                const uint32_t l = l4 + i * stride + sub;
+                const bool have = l < L;
+                uint32_t* rec = tab + (size_t)l * 2u * rw; // (written where `have`)
+                uint32_t u0 = 0, nu = 0, nd = 0, far = 0;
+                float e0 = 0.f, emin = kInf;
+                bool same = true;
+                for (uint32_t r = 0; r < rounds; ++r) {
+                    const uint32_t j = r * G + jj;
+                    if (r) fetch(l, j, x_[i], e_[i]);
+                    const double num = fabs(x_[i]) + c_1;
+                    uint32_t u = (uint32_t)fmin(num * inv_c, most);
+                    const double rest = fma(-(double)u, cd, num);
+                    u = min(rest < 0.0 ? u - 1u : (rest >= cd ? u + 1u : u), D + 1u);
+                    const bool in = have && j < K, ok = in && u <= D; // sizes ascend with j: the usable candidates come first
+                    const float e = x_[i] < 0.0 ? 0.f : e_[i];        // a layer sent densely (negative cost) loses nothing
+                    if (r == 0) { u0 = __shfl_sync(0xffffffffu, u, sub * G); e0 = __shfl_sync(0xffffffffu, e, sub * G); }
+                    const uint32_t du = min(u - u0, D - L + 1u); // (a row has at most D - L + 1 cells: that far is out of it from anywhere)
+                    const uint32_t oks = __ballot_sync(0xffffffffu, ok) & gmask;
+                    same &= (__ballot_sync(0xffffffffu, ok && u != u0) & gmask) == 0u;
+                    if (oks) far = __shfl_sync(gmask, du, 31 - __clz(oks));
+                    nu += __popc(oks);
+                    emin = fminf(emin, ok ? e : kInf);
+                    // of two neighbours with the same cells the first is left out unless its error is the smaller one
+                    const float e_right = __shfl_down_sync(0xffffffffu, e, 1);
+                    const uint32_t u_right = __shfl_down_sync(0xffffffffu, u, 1);
+                    const bool keep = ok && !(jj + 1u < G && ((oks >> lane) & 2u) && u_right == u && e_right <= e);
+                    const uint32_t kept = __ballot_sync(0xffffffffu, keep) & gmask;
+                    if (keep) {
+                        const uint32_t at = nd + __popc(kept & ((1u << lane) - 1u));
+                        rec[at] = 0u - 4u * du;
+                        rec[kr + at] = __float_as_uint(e);
+                    }
+                    nd += __popc(kept);
+                    if (have && j < kr) {
+                        rec[rw + j] = ok ? 0u - 4u * (u - u0) : 0u;
+                        rec[rw + kr + j] = __float_as_uint(ok ? e : e0);
+                    }
+                }
+                for (uint32_t o = G >> 1; o; o >>= 1) emin = fminf(emin, __shfl_xor_sync(0xffffffffu, emin, o));
+                if (have) {
+                    for (uint32_t x = nd + jj; x < ((nd + 7u) & ~7u); x += G) { // the last batch repeats candidate 0
+                        rec[x] = 0u;
+                        rec[kr + x] = __float_as_uint(e0);
+                    }
+                    if (jj == 0) {
+                        *reinterpret_cast<uint4*>(rec + 2u * kr) = make_uint4(nd | (same ? kDpSameBit : 0u), __float_as_uint(emin), far, 0u);
+                        *reinterpret_cast<uint4*>(rec + rw + 2u * kr) = make_uint4(nu, __float_as_uint(emin), far, 0u);
+                        sum += nu ? u0 : D + 1u; // not even the smallest candidate fits
+                        reach = max(reach, far);
+                    }
+                }
+            }
+        }
+        if (jj == 0 && sum) { atomicAdd(&s_sum, sum); atomicMax(&s_reach, reach); }
+    }
+    __syncthreads();
+    const uint64_t least = s_sum;
+    if (status == KIMAD_OK && least > D) status = KIMAD_STATUS_INFEASIBLE;
+    if (status != KIMAD_OK) { // nothing to search
+        for (uint32_t l = t; l < L; l += T) s_j[l] = (uint8_t)(status == KIMAD_STATUS_PLATEAU ? K - 1 : 0u);
+        __syncthreads();
+        choose_finish(a, w, c, status, false, nullptr, s_j, s_k, s_e);
+        return;
+    }
+    const uint32_t width = D - (uint32_t)least + 1u; // cells 0 .. width - 1 above the smallest total
+    const uint32_t reach = s_reach;                  // cells that a candidate reads below its own at most
+    // a row has +inf in front of it, for the cells below its start
+    const uint32_t margin = (reach + 3u) & ~3u, slot_words = margin + ((width + 3u) & ~3u);
+    const uint32_t n_ring = min((uint32_t)kDpMaxRing, (plan.work_bytes - 8u * CL * rw) / (4u * slot_words)); // (at least 2)
+    for (uint32_t i = t; i < n_ring * margin; i += T) ring[(i / margin) * slot_words + i % margin] = kInf;
+
+
+    // ---- the recursion
+    const uint32_t wcell = wid * (32u * CPT), cell0 = wcell + lane; // the thread's cells: cell0 + 32 q
+    const bool busy = wcell < width;
+    // Progress: a warp publishes s + 1 when its part of row s is written; it is then done with reading row s - 1.
+    if (t < 32u) s_prog[t] = t < T / 32u && t * (32u * CPT) < width ? 0u : 0x7fffffffu; // no work: never holds anybody up
+    volatile uint32_t* prog = s_prog;
+    volatile uint32_t* failed = &s_failed;
+    const uint32_t n_chunks = (L + CL - 1) / CL;
+    auto stage_tab = [&](uint32_t ch) { // the first records of a chunk of layers
+        const uint32_t l0 = ch * CL, n16 = min(CL, L - l0) * rec16;
+        const uint4* src = reinterpret_cast<const uint4*>(tab + (size_t)l0 * 2u * rw);
+        const uint32_t dst = smem_u32(s_tab + (ch & 1u) * CL * rw);
+        for (uint32_t i = t; i < n16; i += T) cp_async_16(dst + 16u * i, src + (i / rec16) * 2u * rec16 + i % rec16);
+    };
+    float v[CPT];
+#pragma unroll
+    for (int q = 0; q < CPT; ++q) v[q] = cell0 + 32u * q == 0u ? 0.f : kInf;
+    __syncthreads(); // the records are final
+    stage_tab(0);
+    uint32_t seq = 0, slot = 0; // exchanges so far; slot of the next one
+    float* hist_at = hist + cell0;
+    for (uint32_t ch = 0; ch < n_chunks; ++ch) {
+        cp_async_wait();
+        __syncthreads(); // this chunk's records are there, nobody reads the other buffer any more
+        if (ch + 1 < n_chunks) stage_tab(ch + 1);
+        if (!busy) continue;
+        const uint32_t* rec = s_tab + (ch & 1u) * CL * rw;
+        const uint32_t l0 = ch * CL, nl = min(CL, L - l0);
+        uint2 head = *reinterpret_cast<const uint2*>(rec + 2u * kr);
+        for (uint32_t i = 0; i < nl; ++i, rec += rw) {
+            const uint2 h = head;
+            if (i + 1 < nl) head = *reinterpret_cast<const uint2*>(rec + rw + 2u * kr);
+            if (h.x & kDpSameBit) { // own cell only: the smallest error decides the value
+#pragma unroll
+                for (int q = 0; q < CPT; ++q) v[q] = __fadd_rn(v[q], __uint_as_float(h.y));
+                if (t == 0) s_p[l0 + i] = __uint_as_float(h.y);
+                continue;
+            }
+            const uint32_t nd = h.x;
+            float* row = ring + slot * slot_words + margin;
+#pragma unroll
+            for (int q = 0; q < CPT; ++q)
+                if (cell0 + 32u * q < width) row[cell0 + 32u * q] = v[q];
+            if (t == 0) s_ex[seq] = (uint16_t)(l0 + i);
+            __syncwarp();
+            if (lane == 0) { fence_cta(); prog[wid] = seq + 1u; }
+            const uint32_t* er = rec + kr;
+            uint4 u4 = *reinterpret_cast<const uint4*>(rec), e4 = *reinterpret_cast<const uint4*>(er);
+            // Two cells per thread (short rows: bound by the chain of latencies per layer): up to sixteen candidates' records
+            // are read ahead of the wait and all their cells requested together.
+            const bool wide = CPT == 2 && nd <= 16u;
+            uint32_t u[16];
+            float e[16];
+            if (wide) {
+                auto take = [&](int i, uint4 a, uint4 b) {
+                    u[i] = a.x; u[i + 1] = a.y; u[i + 2] = a.z; u[i + 3] = a.w;
+                    e[i] = __uint_as_float(b.x); e[i + 1] = __uint_as_float(b.y); e[i + 2] = __uint_as_float(b.z); e[i + 3] = __uint_as_float(b.w);
+                };
+                take(0, u4, e4);
+                take(4, *reinterpret_cast<const uint4*>(rec + 4), *reinterpret_cast<const uint4*>(er + 4));
+                if (nd > 8u) {
+                    take(8, *reinterpret_cast<const uint4*>(rec + 8), *reinterpret_cast<const uint4*>(er + 8));
+                    take(12, *reinterpret_cast<const uint4*>(rec + 12), *reinterpret_cast<const uint4*>(er + 12));
+                }
+            }
+            // the warps below have written their part of this row; the others are done with the slot of the next one
+            progress_wait(prog + lane, lane < wid ? (int)seq + 1 : (lane == wid ? 0 : (int)seq + 3 - (int)n_ring), failed);
+            const uint32_t addr = smem_u32(row + cell0);
+            const int top = -4 * (int)(wcell + 32u * CPT - 1u); // offset from the warp's last cell to the row's start
+#pragma unroll
+            for (int q = 0; q < CPT; ++q) {
+                if (cell0 + 32u * q < width) hist_at[32u * q] = v[q];
+                v[q] = kInf;
+            }
+            hist_at += hist_row;
+            auto gather = [&](auto count) { // the first `count` candidates
+                constexpr int N = decltype(count)::value;
+                float x[CPT][N];
+#pragma unroll
+                for (int k = 0; k < N; ++k) lds_cells<CPT, N>(x, k, addr + u[k]);
+#pragma unroll
+                for (int q = 0; q < CPT; ++q) {
+#pragma unroll
+                    for (int k = 0; k < N; ++k) x[q][k] = __fadd_rn(x[q][k], e[k]);
+#pragma unroll
+                    for (int k = 0; k < N; k += 4) v[q] = min3(min3(x[q][k], x[q][k + 1], x[q][k + 2]), x[q][k + 3], v[q]);
+                }
+            };
+            if (wide) {
+                if (nd <= 8u || (int)u[8] < top) gather(std::integral_constant<int, 8>{}); // (the rest: out of reach for the warp's cells)
+                else gather(std::integral_constant<int, 16>{});
+            } else
+            for (uint32_t j0 = 4;; j0 += 4u) { // the offsets' sizes ascend with the entry
+                const uint32_t u[4] = {u4.x, u4.y, u4.z, u4.w};
+                const float e[4] = {__uint_as_float(e4.x), __uint_as_float(e4.y), __uint_as_float(e4.z), __uint_as_float(e4.w)};
+                float x[CPT][4]; // cells beyond the row (last warp) read what lies behind it and are never stored
+#pragma unroll
+                for (int k = 0; k < 4; ++k) lds_cells<CPT, 4>(x, k, addr + u[k]);
+                bool more = j0 < nd;
+                if (more) {
+                    u4 = *reinterpret_cast<const uint4*>(rec + j0);
+                    e4 = *reinterpret_cast<const uint4*>(er + j0);
+                    more = (int)u4.x >= top; // else out of reach for all of the warp's cells, and so are the rest
+                }
+#pragma unroll
+                for (int q = 0; q < CPT; ++q)
+                    v[q] = min3(min3(__fadd_rn(x[q][0], e[0]), __fadd_rn(x[q][1], e[1]), __fadd_rn(x[q][2], e[2])), __fadd_rn(x[q][3], e[3]), v[q]);
+                if (!more) break;
+            }
+            ++seq;
+            if (++slot == n_ring) slot = 0;
+        }
+    }
+
+    // ---- lowest cell attaining the minimum: lexicographic (value, cell)
+    float bv = kInf;
+    uint32_t bb = 0xffffffffu;
+#pragma unroll
+    for (int q = 0; q < CPT; ++q) {
+        const uint32_t b = cell0 + 32u * q;
+        if (b < width && v[q] < bv) { bv = v[q]; bb = b; } // q ascending: cells ascend
+    }
+    auto lower = [](float ov, uint32_t ob, float v, uint32_t b) { return ov < v || (ov == v && ob < b); };
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
+        const uint32_t ob = __shfl_xor_sync(0xffffffffu, bb, o);
+        if (lower(ov, ob, bv, bb)) { bv = ov; bb = ob; }
+    }
+    if (lane == 0) { s_redv[wid] = bv; s_redb[wid] = bb; }
+    if (t == 0) s_left = seq; // (warp 0 owns the lowest cells: always busy)
+    __syncthreads();          // the recursion is over for all warps, its rows are in the workspace
+    const uint32_t n_ex = s_left;
+    bv = s_redv[0]; bb = s_redb[0];
+    for (uint32_t i = 1; i < T / 32; ++i)
+        if (lower(s_redv[i], s_redb[i], bv, bb)) { bv = s_redv[i]; bb = s_redb[i]; }
+    if (*failed) {
+        status = KIMAD_ERR_TIMEOUT;
+    } else if (!(bv < kInf)) {
+        status = KIMAD_STATUS_INFEASIBLE;
+        for (uint32_t l = t; l < L; l += T) s_j[l] = 0;
+    } else {
+        // Backtracking over the exchanged rows, last to first.  The whole CTA stages the rows of some exchanges (a window of
+        // cells below the current one) and their layers' second records, then one warp walks them, a lane per candidate:
+        // the first candidate that attains the minimum, and the cell it came from.
+        __syncthreads(); // everybody has read the number of exchanges
+        if (t == 0) s_cell = bb;
+        __syncthreads();
+        for (uint32_t left = n_ex; left;) {
+            const uint32_t b0 = s_cell, lo = (b0 - min(b0, reach + 256u)) & ~3u;
+            const uint32_t row16 = (b0 - lo) / 4u + 1u, per16 = rec16 + row16;
+            const uint32_t nx = min(left, plan.work_bytes / (16u * per16));
+            uint4* buf = reinterpret_cast<uint4*>(smem_raw);
+            for (uint32_t i = wid; i < nx; i += T / 32) { // a warp per exchange
+                const uint4* r16 = reinterpret_cast<const uint4*>(tab + (size_t)s_ex[left - 1u - i] * 2u * rw + rw);
+                const uint4* h16 = reinterpret_cast<const uint4*>(hist + (size_t)(left - 1u - i) * hist_row + lo);
+                const uint32_t dst = smem_u32(buf + i * per16);
+                for (uint32_t x = lane; x < per16; x += 32u) cp_async_16(dst + 16u * x, x < rec16 ? r16 + x : h16 + (x - rec16));
+            }
+            cp_async_wait();
+            __syncthreads();
+            if (wid == 0) {
+                uint32_t b = b0, i = 0;
+                const uint32_t* rec = reinterpret_cast<const uint32_t*>(buf);
+                if (kr <= 32u) { // the next exchange's record is read ahead; lane i mod 32 keeps the result of exchange i
+                    const float* row = reinterpret_cast<const float*>(rec + rw) - lo;
+                    uint32_t my_j = 0;
+                    float my_best = 0.f;
+                    auto keep = [&](uint32_t n, uint32_t upto) { // results of the n exchanges before `upto`
+                        if (lane < n) {
+                            const uint32_t l = s_ex[left - 1u - (upto - n + lane)];
+                            s_j[l] = (uint8_t)my_j;
+                            s_p[l] = my_best;
+                        }
+                    };
+                    const uint32_t lane_j = min(lane, kr - 1u);
+                    uint32_t nu = rec[2u * kr], far = rec[2u * kr + 2u], off = (0u - rec[lane_j]) >> 2;
+                    float e = __uint_as_float(rec[kr + lane_j]);
+                    while (i < nx) {
+                        if (lo && b - lo < far) break; // left the window: staged anew from here (never on the first exchange)
+                        const bool fits = lane < nu && off <= b;
+                        const float sum = fits ? __fadd_rn(row[b - off], e) : kInf;
+                        const uint32_t mine = lane << 16 | off;
+                        row += 4u * per16; rec += 4u * per16; // (the last ones read lie inside the buffer: work_bytes is below its end)
+                        nu = rec[2u * kr]; far = rec[2u * kr + 2u]; off = (0u - rec[lane_j]) >> 2;
+                        e = __uint_as_float(rec[kr + lane_j]);
+                        const float best = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(sum))); // (sums of squares: not negative)
+                        const uint32_t win = __reduce_min_sync(0xffffffffu, fits && sum == best ? mine : 0xffffffffu); // the first of them
+                        if (lane == (i & 31u)) { my_j = win >> 16; my_best = best; }
+                        b -= win & 0xffffu;
+                        if ((++i & 31u) == 0) keep(32u, i);
+                    }
+                    keep(i & 31u, i);
+                } else {
+                    for (; i < nx; ++i, rec += 4u * per16) {
+                        const float* row = reinterpret_cast<const float*>(rec + rw) - lo;
+                        const uint32_t nu = rec[2u * kr], far = rec[2u * kr + 2u];
+                        if (lo && b - lo < far) break;
+                        uint32_t off[4], step = 0, j = 0;
+                        float sum[4], best = kInf;
+#pragma unroll
+                        for (int h = 0; h < 4; ++h) {
+                            const uint32_t x = 32u * h + lane;
+                            off[h] = 0;
+                            sum[h] = kInf;
+                            if (x < nu) {
+                                off[h] = (0u - rec[x]) >> 2;
+                                if (off[h] <= b) sum[h] = __fadd_rn(row[b - off[h]], __uint_as_float(rec[kr + x]));
+                            }
+                            best = fminf(best, sum[h]);
+                        }
+                        best = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(best)));
+#pragma unroll
+                        for (int h = 3; h >= 0; --h) {
+                            const uint32_t eq = __ballot_sync(0xffffffffu, sum[h] == best);
+                            const uint32_t from = __shfl_sync(0xffffffffu, off[h], eq ? __ffs(eq) - 1 : 0);
+                            if (eq) { j = 32u * h + __ffs(eq) - 1u; step = from; }
+                        }
+                        if (lane == 0) {
+                            const uint32_t l = s_ex[left - 1u - i];
+                            s_j[l] = (uint8_t)j;
+                            s_p[l] = best;
+                        }
+                        b -= step;
+                    }
+                }
+                if (lane == 0) { s_cell = b; s_left = left - i; }
+            }
+            __syncthreads();
+            left = s_left;
+        }
+        // The layers in between: the value before each of them (a thread per run of such layers), then the first candidate
+        // that attains the layer's smallest sum.
+        for (uint32_t x = t; x <= n_ex; x += T) { // run x follows exchange x - 1
+            const uint32_t l0 = x ? s_ex[x - 1] + 1u : 0u, l1 = x < n_ex ? s_ex[x] : L;
+            float p = x ? s_p[l0 - 1] : 0.f;
+            for (uint32_t l = l0; l < l1; ++l) {
+                const float q = __fadd_rn(p, s_p[l]);
+                s_p[l] = p;
+                s_j[l] = 0xffu;
+                p = q;
+            }
+        }
+        __syncthreads();
+        for (uint32_t l = t; l < L; l += T) {
+            if (s_j[l] != 0xffu) continue;
+            const uint32_t* rec = tab + (size_t)l * 2u * rw + rw;
+            const uint4 head = __ldcg(reinterpret_cast<const uint4*>(rec + 2u * kr));
+            const float p = s_p[l], least_sum = __fadd_rn(p, __uint_as_float(head.y));
+            uint32_t j = 0;
+            for (uint32_t j0 = (head.x - 1u) & ~7u;; j0 -= 8u) {
+                const float4 ea = __ldcg(reinterpret_cast<const float4*>(rec + kr + j0)), eb = __ldcg(reinterpret_cast<const float4*>(rec + kr + j0 + 4));
+                const float e[8] = {ea.x, ea.y, ea.z, ea.w, eb.x, eb.y, eb.z, eb.w};
+#pragma unroll
+                for (int i = 7; i >= 0; --i) j = __fadd_rn(p, e[i]) == least_sum ? j0 + i : j;
+                if (j0 == 0) break;
+            }
+            s_j[l] = (uint8_t)j;
+        }
+    }
+    if (t == 0) s_total = bv;
+    __syncthreads();
+    choose_finish(a, w, c, status, false, status == KIMAD_OK ? &s_total : nullptr, s_j, s_k, s_e);
+}
+
+// ------------------------------------------------------------------------------------------------
+// k_pick: the other ways to choose a candidate per layer, one CTA per worker.
+// mode 1: candidates given (j_in); mode 2: one candidate index for all layers, the largest whose total size fits the
+// budget (Kimad on the grid, Section 3.1); mode 3: Algorithm 3 read with the discretised error as the axis and the size
+// as the value; mode 4: the table holds, per worker, the single candidate of the ratio fitted to the budget
+// (k_fit_ratio): nothing to search.
+// Shared memory (the host computes the same sizes): two rows of (D + 2) "none" followed by D + 1 values | j[L] | mode 3:
+// cells[L Kp], sizes[L Kp], Kp = K rounded up to 4 | back-pointers, where they fit.  The margin in front of each row lets
+// prev[b - u] be read without a bounds test.  Back-pointers: a nibble when K <= 16, else a byte.
+// ------------------------------------------------------------------------------------------------
+constexpr int kPickThreads = 512;
+constexpr int kPickCells = 2; // budget cells per thread (mode 3)
+struct PickPlan {
+    uint32_t pd_in_smem; // else in the caller's workspace
+    uint32_t pd_nibble;
+    uint32_t pd_row_bytes;
+};
+
+__global__ void __launch_bounds__(kPickThreads)
+k_pick(DpBudgets budgets, uint32_t w_base, ChooseArgs a, int mode, PickPlan plan, const uint32_t* __restrict__ j_in,
+       uint8_t* __restrict__ pd_global) {
+    pdl_wait();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const uint32_t w = w_base + blockIdx.x, L = a.L, K = a.K, D = a.D;
+    if (!choose_applies(a)) return;
+    const uint64_t c = budgets.c[blockIdx.x];
+    const uint32_t row = D + 1, pad = D + 2, rowp = row + pad, Kp = (K + 3) & ~3u;
+    uint32_t* prow = reinterpret_cast<uint32_t*>(smem_raw);
+    uint32_t* s_j = prow + 2 * rowp; // [L]
+    __shared__ int s_status;
+    const LayerDesc* layers = a.layers;
+    const KTab ktab = a.ktab;
+
+    int status = KIMAD_OK;
+    if (a.check_finite && (a.flags[w] & 1u)) status = KIMAD_ERR_NONFINITE;
+    __syncthreads(); // the flags are read before the end of the choice resets them
+    if (status == KIMAD_OK) {
+        if (mode == 1) {
+            for (uint32_t l = threadIdx.x; l < L; l += blockDim.x) s_j[l] = min(j_in[(size_t)w * L + l], K - 1);
+        } else if (c >= a.full_bytes) {
+            status = KIMAD_STATUS_PLATEAU;
+            for (uint32_t l = threadIdx.x; l < L; l += blockDim.x) s_j[l] = K - 1;
+        } else if (c == 0) {
+            status = KIMAD_STATUS_INFEASIBLE;
+            for (uint32_t l = threadIdx.x; l < L; l += blockDim.x) s_j[l] = 0;
+        } else if (mode == 2) {
+            // total size of candidate j over the layers; sizes ascend with j.  A warp per j, layers dealt out to its lanes
+            __shared__ uint32_t s_fit; // number of candidates that fit
+            if (threadIdx.x == 0) s_fit = 0;
+            __syncthreads();
+            for (uint32_t j = threadIdx.x >> 5; j < K; j += blockDim.x >> 5) {
+                unsigned long long bytes = 0;
+                for (uint32_t l = threadIdx.x & 31u; l < L; l += 32u)
+                    bytes += candidate_bytes(layers[l].n, ktab.at(w, (size_t)l * K + j), a.bpe, a.cost_model, nullptr);
+#pragma unroll
+                for (int o = 16; o; o >>= 1) bytes += __shfl_xor_sync(0xffffffffu, bytes, o);
+                if ((threadIdx.x & 31u) == 0 && bytes <= c) atomicMax(&s_fit, j + 1);
+            }
+            __syncthreads();
+            const uint32_t fit = s_fit;
+            if (fit == 0) status = KIMAD_STATUS_INFEASIBLE;
+            for (uint32_t l = threadIdx.x; l < L; l += blockDim.x) s_j[l] = fit ? fit - 1 : 0;
+        } else if (mode == 4) {
+            for (uint32_t l = threadIdx.x; l < L; l += blockDim.x) s_j[l] = 0; // feasibility is decided on the totals
+        } else {
+            // Error axis: E_max = sum_l err_{l,0} (binary64, layers in order), cells e_{l,j} = floor(err D / E_max),
+            // value = fewest kept entries for a total of exactly e cells; answer = lowest e whose value fits c.
+            __shared__ double s_emax;
+            __shared__ uint32_t s_best;
+            uint32_t* pv = prow + pad;
+            uint32_t* cu = prow + rowp + pad;
+            const float* e_w = a.err + (size_t)w * L * K;
+            uint32_t* s_units = s_j + L;       // [L * Kp]
+            uint32_t* s_kk = s_units + L * Kp; // [L * Kp]
+            uint8_t* pd = plan.pd_in_smem ? reinterpret_cast<uint8_t*>(s_kk + L * Kp) : pd_global + (size_t)w * L * plan.pd_row_bytes;
+            const uint32_t kNone = 0xffffffffu;
+            if (threadIdx.x == 0) {
+                double e = 0.0;
+                for (uint32_t l = 0; l < L; ++l) e = __dadd_rn(e, (double)e_w[(size_t)l * K]);
+                s_emax = e;
+                s_best = kNone;
+            }
+            __syncthreads();
+            const double emax = s_emax;
+            for (uint32_t i = threadIdx.x; i < L * Kp; i += blockDim.x) {
+                const uint32_t l = i / Kp, j = i % Kp;
+                uint32_t u = D + 1, kk = 0; // padding reads the margin
+                if (j < K) {
+                    const double q = emax > 0.0 ? floor(__ddiv_rn(__dmul_rn((double)e_w[(size_t)l * K + j], (double)D), emax)) : 0.0;
+                    u = q > (double)D ? D : (uint32_t)q;
+                    kk = (uint32_t)ktab.at(w, (size_t)l * K + j);
+                }
+                s_units[i] = u;
+                s_kk[i] = kk;
+            }
+            for (uint32_t i = threadIdx.x; i < 2 * rowp; i += blockDim.x) prow[i] = kNone;
+            __syncthreads();
+            if (threadIdx.x == 0) pv[0] = 0;
+            for (uint32_t l = 0; l < L; ++l) {
+                __syncthreads();
+                const uint32_t* un = s_units + l * Kp;
+                const uint32_t* kk = s_kk + l * Kp;
+                uint8_t* pdl = pd + (size_t)l * plan.pd_row_bytes;
+                for (uint32_t bb = 0; bb < row; bb += kPickCells * blockDim.x) {
+#pragma unroll
+                    for (int q = 0; q < kPickCells; ++q) {
+                        const uint32_t b = bb + threadIdx.x + q * blockDim.x;
+                        const uint32_t bc = min(b, row - 1);
+                        uint32_t best = kNone, bj = 0;
+                        for (uint32_t j = 0; j < K; ++j) {
+                            const uint32_t p = pv[(int)bc - (int)un[j]];
+                            const uint32_t t = p > kNone - kk[j] ? kNone : p + kk[j];
+                            if (t < best) { best = t; bj = j; }
+                        }
+                        if (b < row) cu[b] = best;
+                        if (plan.pd_nibble) {
+                            const uint32_t nb = __shfl_down_sync(0xffffffffu, bj, 1);
+                            if (!(threadIdx.x & 1) && b < row) pdl[b >> 1] = (uint8_t)(bj | (nb << 4));
+                        } else if (b < row) {
+                            pdl[b] = (uint8_t)bj;
+                        }
+                    }
+                }
+                uint32_t* sw = pv; pv = cu; cu = sw;
+            }
+            __syncthreads();
+            const uint64_t cap_k = c / a.bpe;
+            for (uint32_t b = threadIdx.x; b < row; b += blockDim.x)
+                if (pv[b] != kNone && (uint64_t)pv[b] <= cap_k) atomicMin(&s_best, b);
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                if (s_best == kNone) {
+                    s_status = KIMAD_STATUS_INFEASIBLE;
+                } else {
+                    s_status = KIMAD_OK;
+                    uint32_t b = s_best;
+                    for (uint32_t l = L; l-- > 0;) {
+                        const uint8_t* pdl = pd + (size_t)l * plan.pd_row_bytes;
+                        const uint32_t j = plan.pd_nibble ? ((pdl[b >> 1] >> (4 * (b & 1))) & 15u) : pdl[b];
+                        s_j[l] = j;
+                        b -= s_units[l * Kp + j];
+                    }
+                }
+            }
+            __syncthreads();
+            status = s_status;
+            if (status == KIMAD_STATUS_INFEASIBLE)
+                for (uint32_t l = threadIdx.x; l < L; l += blockDim.x) s_j[l] = 0;
+        }
+    }
+    __syncthreads();
+    // (the rows are free now; L <= D < the rows' size)
+    choose_finish(a, w, c, status, mode == 4, nullptr, s_j, prow, reinterpret_cast<float*>(prow) + rowp);
+}
+
+// The ratio of Section 3.1 sized to the budget: r = q / 2^32 with the largest q whose entries
+// sum_l min(n_l, max(1, floor(q n_l / 2^32))) fit floor(c / (4 + vb)); the worker's table row gets those k_l.
+// One CTA per worker; the sum is an order-free integer reduction, q is found by bisection (33 steps).
+__global__ void __launch_bounds__(kThreads)
+k_fit_ratio(DpBudgets budgets, uint32_t w_base, uint32_t W, uint32_t L, uint32_t bpe, uint64_t N,
+            const LayerDesc* __restrict__ layers, uint64_t* __restrict__ ktab_w /* [W][L] */) {
+    pdl_wait();
+    const uint32_t w = w_base + blockIdx.x;
+    if (w >= W) return;
+    __shared__ unsigned long long s_sum;
+    const uint64_t entries = budgets.c[blockIdx.x] / bpe;
+    auto k_of = [&](uint64_t q, uint64_t n) {
+        uint64_t k = q >= 4294967296ull ? n : (q * n) >> 32;
+        k = k < 1 ? 1 : k;
+        return k > n ? n : k;
+    };
+    uint64_t q;
+    if (entries < (uint64_t)L) q = 0;
+    else if (entries >= N) q = 4294967296ull;
+    else {
+        uint64_t lo = 0, hi = 4294967296ull; // sum(lo) <= entries < sum(hi)
+        while (hi - lo > 1) {
+            const uint64_t mid = lo + (hi - lo) / 2;
+            if (threadIdx.x == 0) s_sum = 0;
+            __syncthreads();
+            unsigned long long mine = 0;
+            for (uint32_t l = threadIdx.x; l < L; l += kThreads) mine += k_of(mid, layers[l].n);
+#pragma unroll
+            for (int o = 16; o; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
+            if ((threadIdx.x & 31) == 0) atomicAdd(&s_sum, mine);
+            __syncthreads();
+            if (s_sum <= entries) lo = mid; else hi = mid;
+            __syncthreads();
+        }
+        q = lo;
+    }
+    for (uint32_t l = threadIdx.x; l < L; l += kThreads) ktab_w[(size_t)w * L + l] = k_of(q, layers[l].n);
+}
+
+} // namespace kimad
