@@ -25,10 +25,10 @@ struct Layout {
     // static tables
     size_t dbuf, chunks, layers, ktab, costs, ktab_dyn, reg_layers, tiny_layers, reg_index, runs;
     // zeroed at set_workspace and kept clean by the kernels
-    size_t zero_from, h1_cnt, h1_ss, h23_cnt, h23_ss, bh_cnt, bh_sum, low_hist, recount, recount_bytes, fb, r2, flags;
+    size_t zero_from, h1_cnt, h1_ss, h23_cnt, h23_ss, bh_cnt, bh_sum, in_n, fb, rc, flags;
     // scratch without initial-state requirements
-    size_t cell_tab, cell_win, bin_lo, meta, cands, slots, err, tau, keep_eq, shift, sel, chunk_cnt, jobs, csel,
-        fb_chunks, fb_layers, r2_chunks, r2_layers, rf, rf_chunks, rf_layers, pd, rows, total;
+    size_t cell_tab, cell_win, bin_lo, meta, cands, slots, err, tau, keep_eq, shift, sel, jobs, csel,
+        fb_chunks, fb_layers, rc_chunks, rf, rf_chunks, rf_layers, pd, rows, total;
 };
 
 } // namespace
@@ -46,6 +46,7 @@ struct kimad_ctx {
     std::vector<SweepRun> runs;                               // the sweep's CTAs: static runs of chunks, balanced by elements
     std::vector<unsigned char> static_image;                  // the static tables as they lie in the workspace, one block
     std::vector<size_t> guards;                               // checked build: offsets of the canary words between regions
+    uint32_t most_chunks = 0; // of a layer
     uint32_t curve_mode = 0;
     uint32_t policy = 0, cost_model = 0;
     size_t sample_smem = 0, pass_a_smem = 0, tiny_smem = 0;
@@ -107,18 +108,16 @@ void plan_layout(kimad_ctx* c) {
     y.reg_index = take(c->reg_index.size() * sizeof(uint32_t));
     y.runs = take(c->runs.size() * sizeof(SweepRun));
     y.zero_from = o;
-    y.h1_cnt = take(WL * kL1Bins * sizeof(uint32_t));
-    y.h1_ss = take(WL * kL1Bins * sizeof(uint64_t));
-    y.h23_cnt = take(WLK * kL23Bins * sizeof(uint32_t));
-    y.h23_ss = take(WLK * kL23Bins * sizeof(uint64_t));
+    y.h1_cnt = take(WR * kL1Bins * sizeof(uint32_t));
+    y.h1_ss = take(WR * kL1Bins * sizeof(uint64_t));
+    y.h23_cnt = take(WR * c->K * kL23Bins * sizeof(uint32_t));
+    y.h23_ss = take(WR * c->K * kL23Bins * sizeof(uint64_t));
     y.bh_cnt = take(WR * kMaxBins * sizeof(uint32_t));
     y.bh_sum = take(WR * kMaxBins * sizeof(uint64_t));
-    y.low_hist = take(WL * kLowBins * sizeof(uint32_t));
+    y.in_n = take(WL * sizeof(uint32_t));
     // work lists, one set per group of workers
-    y.recount_bytes = align_up(256 + (size_t)2 * c->W * nch * sizeof(uint2));
-    y.recount = take(kGroups * y.recount_bytes);
     y.fb = take(kGroups * align_up(sizeof(FbList)));
-    y.r2 = take(kGroups * align_up(sizeof(Round2)));
+    y.rc = take(kGroups * align_up(sizeof(Recount)));
     y.flags = take((size_t)c->W * sizeof(uint32_t));
     y.cell_tab = take(WR * kCellTab * sizeof(uint32_t));
     y.cell_win = take(WR * sizeof(int4));
@@ -131,13 +130,11 @@ void plan_layout(kimad_ctx* c) {
     y.keep_eq = take(WLK * sizeof(uint32_t));
     y.shift = take(WLK * sizeof(uint32_t));
     y.sel = take(WL * sizeof(Sel));
-    y.chunk_cnt = take((size_t)c->W * nch * sizeof(uint2));
     y.jobs = take((size_t)c->W * nch * sizeof(ChunkJob));
     y.csel = take((size_t)c->W * nch * sizeof(ChunkSel));
     y.fb_chunks = take(kGroups * align_up((size_t)c->W * nch * sizeof(uint2)));
     y.fb_layers = take(kGroups * align_up(WL * sizeof(uint2)));
-    y.r2_chunks = take(kGroups * align_up((size_t)c->W * nch * sizeof(uint2)));
-    y.r2_layers = take(kGroups * align_up(WL * sizeof(uint2)));
+    y.rc_chunks = take(kGroups * align_up((size_t)c->W * nch * sizeof(uint2)));
     y.rf = take(WLK * sizeof(RefineCand));
     y.rf_chunks = take(kGroups * align_up((size_t)c->W * nch * sizeof(uint2)));
     y.rf_layers = take(kGroups * align_up(WL * sizeof(uint2)));
@@ -164,8 +161,8 @@ static int preload_kernels() {
     KIMAD_PRELOAD(k_refine_hist); KIMAD_PRELOAD(k_refine_resolve);
     KIMAD_PRELOAD(k_tiny_exact); KIMAD_PRELOAD(k_fb_hist1); KIMAD_PRELOAD(k_fb_hist23<2>); KIMAD_PRELOAD(k_fb_hist23<3>);
     KIMAD_PRELOAD(k_resolve1); KIMAD_PRELOAD(k_resolve23<2>); KIMAD_PRELOAD(k_resolve23<3>); KIMAD_PRELOAD(k_rebuild_slots);
-    KIMAD_PRELOAD(k_dp<2>); KIMAD_PRELOAD(k_dp<4>); KIMAD_PRELOAD(k_dp<8>); KIMAD_PRELOAD(k_pick); KIMAD_PRELOAD(k_fit_ratio); KIMAD_PRELOAD(k_sel_count); KIMAD_PRELOAD(k_sel_count_r2); KIMAD_PRELOAD(k_sel_resolve);
-    KIMAD_PRELOAD(k_sel_resolve_r2); KIMAD_PRELOAD(k_sel_recount); KIMAD_PRELOAD(k_sel_slices); KIMAD_PRELOAD(k_sel_scan);
+    KIMAD_PRELOAD(k_dp<2>); KIMAD_PRELOAD(k_dp<4>); KIMAD_PRELOAD(k_dp<8>); KIMAD_PRELOAD(k_pick); KIMAD_PRELOAD(k_fit_ratio); KIMAD_PRELOAD(k_sel_count);
+    KIMAD_PRELOAD(k_sel_offsets<128>); KIMAD_PRELOAD(k_sel_offsets<512>); KIMAD_PRELOAD(k_sel_recount);
     KIMAD_PRELOAD((k_sel_write<false, false>)); KIMAD_PRELOAD((k_sel_write<false, true>));
     KIMAD_PRELOAD((k_sel_write<true, false>)); KIMAD_PRELOAD((k_sel_write<true, true>));
     KIMAD_PRELOAD(k_apply_packed<false>); KIMAD_PRELOAD(k_apply_packed<true>);
@@ -341,17 +338,15 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
     uint32_t* keq = c->at<uint32_t>(y.keep_eq);
     uint32_t* shf = c->at<uint32_t>(y.shift);
     Sel* sel = c->at<Sel>(y.sel);
-    uint2* ccnt = c->at<uint2>(y.chunk_cnt);
     ChunkJob* jobs = c->at<ChunkJob>(y.jobs);
     ChunkSel* csel = c->at<ChunkSel>(y.csel);
-    uint32_t* lowh = c->at<uint32_t>(y.low_hist);
     uint32_t* flags = c->at<uint32_t>(y.flags);
     uint8_t* pd = c->at<uint8_t>(y.pd);
     const SweepRun* runs = c->at<SweepRun>(y.runs);
 
     const uint32_t R = (uint32_t)c->reg_layers.size(), T = (uint32_t)c->tiny_layers.size();
     const dim3 blk(kThreads);
-    const uint32_t list_cap = W * nch; // entries of every chunk list (twice that for the recount list)
+    const uint32_t list_cap = W * nch; // entries of every chunk list
     const CodeSpace codes{reg_index, meta, cell_tab, cell_win, R};
     int stage = 0;
     auto mark = [&](cudaStream_t st) { if (c->timing) cudaEventRecord(c->ev[stage++], st); };
@@ -414,17 +409,15 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
             ++hand;
             return e;
         };
-        uint32_t* recount_n = c->at<uint32_t>(y.recount + g * y.recount_bytes);
-        uint2* recount_list = c->at<uint2>(y.recount + g * y.recount_bytes + 256);
         FbList* fb = c->at<FbList>(y.fb + g * align_up(sizeof(FbList)));
-        Round2* r2 = c->at<Round2>(y.r2 + g * align_up(sizeof(Round2)));
+        Recount* rc = c->at<Recount>(y.rc + g * align_up(sizeof(Recount)));
+        const Interval in{c->at<uint32_t>(y.in_n), binlo, bhc, bhs, reg_index, R};
         uint2* fb_chunks = c->at<uint2>(y.fb_chunks + g * align_up((size_t)W * nch * sizeof(uint2)));
-        uint2* r2_chunks = c->at<uint2>(y.r2_chunks + g * align_up((size_t)W * nch * sizeof(uint2)));
+        uint2* rc_chunks = c->at<uint2>(y.rc_chunks + g * align_up((size_t)W * nch * sizeof(uint2)));
         uint2* fb_layers = c->at<uint2>(y.fb_layers + g * align_up((size_t)W * L * sizeof(uint2)));
         RefineCand* rf = c->at<RefineCand>(y.rf);
         uint2* rf_chunks = c->at<uint2>(y.rf_chunks + g * align_up((size_t)W * nch * sizeof(uint2)));
         uint2* rf_layers = c->at<uint2>(y.rf_layers + g * align_up((size_t)W * L * sizeof(uint2)));
-        uint2* r2_layers = c->at<uint2>(y.r2_layers + g * align_up((size_t)W * L * sizeof(uint2)));
         const dim3 gch(nch, nw), glw(L, nw);
         // the group's runs of the sweep: the run table is sorted by worker
         uint32_t run0 = 0, run1 = 0;
@@ -490,12 +483,12 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
             CUDA_TRY(launch_pdl(k_refine_hist, 6 * 148, blk, 0, st, dbuf, chunks, c->dstride, L, K, fb, rf_chunks, rf, codes, h23c, h23s));
             CUDA_TRY(launch_pdl(k_refine_resolve, glay, blk, 0, st, layers, L, K, fb, rf_layers, rf, h23c, h23s, err, tau, keq, shf,
                                 codes, fb_chunks, fb_layers, list_cap));
-            CUDA_TRY(launch_pdl(k_fb_hist1, gfb, blk, 0, st, dbuf, chunks, c->dstride, L, fb, fb_chunks, h1c, h1s, flags));
-            CUDA_TRY(launch_pdl(k_resolve1, glay, blk, 0, st, fb, fb_layers, h1c, h1s, ktab, L, K, cands, slots));
-            CUDA_TRY(launch_pdl(k_fb_hist23<2>, gfb, blk, 0, st, dbuf, chunks, c->dstride, L, K, fb, fb_chunks, slots, h23c, h23s));
+            CUDA_TRY(launch_pdl(k_fb_hist1, gfb, blk, 0, st, dbuf, chunks, c->dstride, fb, fb_chunks, h1c, h1s, flags, codes));
+            CUDA_TRY(launch_pdl(k_resolve1, glay, blk, 0, st, fb, fb_layers, h1c, h1s, ktab, L, K, cands, slots, codes));
+            CUDA_TRY(launch_pdl(k_fb_hist23<2>, gfb, blk, 0, st, dbuf, chunks, c->dstride, L, K, fb, fb_chunks, slots, h23c, h23s, codes));
             CUDA_TRY(launch_pdl(k_resolve23<2>, gslot, blk, 0, st, fb, fb_layers, h23c, h23s, L, K, cands, slots, err, tau, keq, shf, codes));
             CUDA_TRY(launch_pdl(k_rebuild_slots, (nw * R + kThreads - 1) / kThreads, blk, 0, st, fb, fb_layers, L, K, cands, slots));
-            CUDA_TRY(launch_pdl(k_fb_hist23<3>, gfb, blk, 0, st, dbuf, chunks, c->dstride, L, K, fb, fb_chunks, slots, h23c, h23s));
+            CUDA_TRY(launch_pdl(k_fb_hist23<3>, gfb, blk, 0, st, dbuf, chunks, c->dstride, L, K, fb, fb_chunks, slots, h23c, h23s, codes));
             CUDA_TRY(launch_pdl(k_resolve23<3>, gslot, blk, 0, st, fb, fb_layers, h23c, h23s, L, K, cands, slots, err, tau, keq, shf, codes));
             c->launches += 9;
             return KIMAD_OK;
@@ -520,18 +513,17 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
         mark(small);
         CUDA_TRY(hand_over(small, big));
         // (d), (e), (f)
-        CUDA_TRY(launch_pdl(k_sel_count, gch, blk, 0, big, dbuf, chunks, nch, c->dstride, L, sel, layers, csel, lowh, recount_n,
-                            recount_list, 2 * list_cap, w0));
+        CUDA_TRY(launch_pdl(k_sel_count, gch, blk, 0, big, dbuf, chunks, nch, c->dstride, L, sel, layers, csel, in, rc, w0));
         mark(big);
         CUDA_TRY(hand_over(big, small));
-        CUDA_TRY(launch_pdl(k_sel_resolve, glw, blk, 0, small, L, layers, nch, csel, lowh, sel, r2, r2_layers, r2_chunks, w0));
-        CUDA_TRY(launch_pdl(k_sel_count_r2, 148, blk, 0, small, dbuf, chunks, nch, c->dstride, L, sel, layers, csel, lowh, recount_n,
-                            recount_list, 2 * list_cap, r2, r2_chunks));
-        CUDA_TRY(launch_pdl(k_sel_resolve_r2, std::min<uint32_t>(nw * L, 32u), blk, 0, small, L, layers, nch, csel, lowh, sel, r2,
-                            r2_layers, r2_chunks));
-        CUDA_TRY(launch_pdl(k_sel_recount, 148, blk, 0, small, dbuf, chunks, nch, c->dstride, L, sel, recount_n, recount_list, csel));
-        CUDA_TRY(launch_pdl(k_sel_slices, (uint32_t)(((uint64_t)nw * nch + 7) / 8), blk, 0, small, chunks, nch, w0, nw, L, sel, csel, ccnt));
-        CUDA_TRY(launch_pdl(k_sel_scan, glw, blk, 0, small, layers, chunks, nch, L, sel, ccnt, jobs, recount_n, fb, r2, w0));
+        {
+            auto launch = [&](auto kern, uint32_t threads) {
+                return launch_named("k_sel_offsets", kern, glw, threads, 0, small, layers, chunks, nch, L, sel, csel, jobs, in, fb, rc,
+                                    rc_chunks, list_cap, w0);
+            };
+            CUDA_TRY(c->most_chunks > 256 ? launch(k_sel_offsets<512>, 512) : launch(k_sel_offsets<128>, 128));
+        }
+        CUDA_TRY(launch_pdl(k_sel_recount, 148, blk, 0, small, dbuf, layers, chunks, nch, c->dstride, L, sel, csel, jobs, in, rc, rc_chunks));
         mark(small);
         CUDA_TRY(hand_over(small, big));
         {
@@ -543,7 +535,7 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
             else CUDA_TRY(dense_write ? launch(k_sel_write<false, true>) : launch(k_sel_write<false, false>));
         }
         mark(big);
-        c->launches += 8;
+        c->launches += 4;
         if (two) CUDA_TRY(cudaEventRecord(c->ev_done[g], big));
     }
     if (two)
@@ -608,6 +600,7 @@ int kimad_create(kimad_ctx** out, const uint64_t* layer_sizes, uint32_t n_layers
             }
             ld.n_chunks = (uint32_t)c->chunks.size() - ld.first_chunk;
             c->layers.push_back(ld);
+            c->most_chunks = std::max(c->most_chunks, ld.n_chunks);
             if (n <= (uint64_t)kTinyMax) {
                 c->reg_index.push_back(0xffffffffu);
                 c->tiny_layers.push_back(l);

@@ -13,7 +13,7 @@
 // Checked build (-DKIMAD_CHECKED): indices into the workspace and the output buffers are tested before use; a failed
 // test sets its bit in a status word that the host reads (kimad_debug_check) and the access is skipped -- nothing
 // traps.  Bits: 0 sweep: bin outside the layer's histogram; 1 counting sweep: bin outside the in-interval histogram;
-// 2 a work list (exact path, second select round, recount) appended beyond its capacity; 3 write sweep: packed
+// 2 a work list (exact path, recount) appended beyond its capacity; 3 write sweep: packed
 // position beyond the capacity; 4 write sweep: element index outside its layer; 5 DP: cell or back-pointer outside
 // its row; 6 curve: bin outside the layer's histogram; 7 curve: the pieces of a refined bin do not add up to the bin.
 // In the ordinary build KIMAD_CHECK(cond, bit) is `true`.
@@ -60,7 +60,7 @@ struct SlotTab {
 };
 
 // What the select kernels need to know about one (worker, layer) after the DP.  The threshold lies in
-// the key interval [tau, tau + 2^shift) and is the keep_eq-th largest key inside it; k_sel_resolve
+// the key interval [tau, tau + 2^shift) and is the keep_eq-th largest key inside it; k_sel_offsets
 // narrows that to the exact threshold (shift = 0) and to the number of ties kept.
 struct Sel {
     uint32_t tau;     // lower key of the interval, then the exact threshold key

@@ -777,7 +777,7 @@ k_refine_hist(DSource dbuf, const Chunk* __restrict__ chunks, uint64_t dstride, 
     for (uint32_t it = blockIdx.x; it < n; it += gridDim.x) {
         const uint2 e = rf_chunks[it];
         const Chunk ch = chunks[e.y];
-        const size_t wl = (size_t)e.x * L + ch.layer;
+        const size_t wl = (size_t)e.x * L + ch.layer, wr = codes.slot(e.x, ch.layer);
         __syncthreads();
         if (threadIdx.x < 4) s_mask[threadIdx.x] = 0;
         if (threadIdx.x == 0) s_n = 0;
@@ -807,7 +807,7 @@ k_refine_hist(DSource dbuf, const Chunk* __restrict__ chunks, uint64_t dstride, 
             for (uint32_t p = 0; p < nc; ++p) {
                 const uint32_t d1 = key - s_klo[p], sh = s_shift[p];
                 if (d1 < (1u << sh)) {
-                    const size_t at = (wl * K + s_j[p]) * kL23Bins + (d1 >> (sh > 10u ? sh - 10u : 0u));
+                    const size_t at = (wr * K + s_j[p]) * kL23Bins + (d1 >> (sh > 10u ? sh - 10u : 0u));
                     atomicAdd(&g_cnt[at], 1u);
                     atomicAdd(&g_ss[at], (unsigned long long)sq_fixed(key));
                     break; // bins are disjoint; candidates that share a bin share a piece histogram (see k_refine_resolve)
@@ -864,7 +864,7 @@ k_refine_resolve(const LayerDesc* __restrict__ layers, uint32_t L, uint32_t K, F
     const uint32_t n = fb->rf_layers;
     for (uint32_t it = blockIdx.x; it < n; it += gridDim.x) {
         const uint32_t w = rf_layers[it].x, l = rf_layers[it].y;
-        const size_t wl = (size_t)w * L + l;
+        const size_t wl = (size_t)w * L + l, wr = codes.slot(w, l);
         __syncthreads();
         if (threadIdx.x == 0) s_bad = 0;
         __syncthreads();
@@ -877,8 +877,8 @@ k_refine_resolve(const LayerDesc* __restrict__ layers, uint32_t L, uint32_t K, F
                 if (o.shift != kNoRefine && o.klo == rc.klo) { owner = i; break; }
             }
             const uint32_t sub = rc.shift > 10u ? rc.shift - 10u : 0u, nsub = 1u << (rc.shift - sub);
-            const uint32_t* gc = g_cnt + (wl * K + owner) * kL23Bins;
-            const unsigned long long* gs = g_ss + (wl * K + owner) * kL23Bins;
+            const uint32_t* gc = g_cnt + (wr * K + owner) * kL23Bins;
+            const unsigned long long* gs = g_ss + (wr * K + owner) * kL23Bins;
             const double scale = sq_scale(rc.klo >> 23);
             // four consecutive pieces per thread, ascending keys
             uint32_t c[4], csum = 0;
@@ -921,8 +921,8 @@ k_refine_resolve(const LayerDesc* __restrict__ layers, uint32_t L, uint32_t K, F
         for (uint32_t j = 0; j < K; ++j) {
             if (rf[wl * K + j].shift == kNoRefine) continue;
             for (uint32_t b = threadIdx.x; b < (uint32_t)kL23Bins; b += kThreads) {
-                g_cnt[(wl * K + j) * kL23Bins + b] = 0;
-                g_ss[(wl * K + j) * kL23Bins + b] = 0ull;
+                g_cnt[(wr * K + j) * kL23Bins + b] = 0;
+                g_ss[(wr * K + j) * kL23Bins + b] = 0ull;
             }
         }
         __syncthreads();
@@ -1112,9 +1112,9 @@ k_tiny_exact(const float* __restrict__ grads, const float* __restrict__ state, u
 constexpr int kFbAhead = 4; // elements per thread whose loads are issued together
 
 __global__ void __launch_bounds__(kThreads)
-k_fb_hist1(DSource dbuf, const Chunk* __restrict__ chunks, uint64_t dstride, uint32_t L,
+k_fb_hist1(DSource dbuf, const Chunk* __restrict__ chunks, uint64_t dstride,
            const FbList* __restrict__ fb, const uint2* __restrict__ fb_chunks, uint32_t* __restrict__ g_cnt,
-           unsigned long long* __restrict__ g_ss, uint32_t* __restrict__ flags) {
+           unsigned long long* __restrict__ g_ss, uint32_t* __restrict__ flags, const CodeSpace codes) {
     pdl_wait();
     __shared__ uint32_t s_cnt[kL1Bins], s_hi[kL1Bins], s_lo[kL1Bins];
     const uint32_t n = fb->n_chunks;
@@ -1148,8 +1148,9 @@ k_fb_hist1(DSource dbuf, const Chunk* __restrict__ chunks, uint64_t dstride, uin
         flush();
         if (nonfinite) atomicOr(&flags[e.x], 1u);
         __syncthreads();
-        uint32_t* gc = g_cnt + ((size_t)e.x * L + ch.layer) * kL1Bins;
-        unsigned long long* gs = g_ss + ((size_t)e.x * L + ch.layer) * kL1Bins;
+        const size_t wr = codes.slot(e.x, ch.layer);
+        uint32_t* gc = g_cnt + wr * kL1Bins;
+        unsigned long long* gs = g_ss + wr * kL1Bins;
         for (int b = threadIdx.x; b < kL1Bins; b += kThreads)
             if (s_cnt[b]) {
                 atomicAdd(&gc[b], s_cnt[b]);
@@ -1163,7 +1164,7 @@ template <int LEVEL>
 __global__ void __launch_bounds__(kThreads)
 k_fb_hist23(DSource dbuf, const Chunk* __restrict__ chunks, uint64_t dstride, uint32_t L, uint32_t K,
             const FbList* __restrict__ fb, const uint2* __restrict__ fb_chunks, const SlotTab* __restrict__ slots,
-            uint32_t* __restrict__ g_cnt, unsigned long long* __restrict__ g_ss) {
+            uint32_t* __restrict__ g_cnt, unsigned long long* __restrict__ g_ss, const CodeSpace codes) {
     pdl_wait();
     __shared__ uint8_t s_first[kL1Bins]; // level-1 bin -> first slot whose prefix starts with it (0xff: none)
     __shared__ uint8_t s_num[kL1Bins];   // ... and how many consecutive slots share that bin (level 3)
@@ -1187,8 +1188,9 @@ k_fb_hist23(DSource dbuf, const Chunk* __restrict__ chunks, uint64_t dstride, ui
         __syncthreads();
         const ChunkView cv(ch);
         const DView dd(dbuf, e.x, dstride, cv.a0);
-        uint32_t* gc = g_cnt + wl * K * kL23Bins;
-        unsigned long long* gs = g_ss + wl * K * kL23Bins;
+        const size_t wr = codes.slot(e.x, ch.layer);
+        uint32_t* gc = g_cnt + wr * K * kL23Bins;
+        unsigned long long* gs = g_ss + wr * K * kL23Bins;
         uint32_t cur = 0xffffffffu, cn = 0; // (slot, bin) of the thread's current run, its entries and squares
         unsigned long long csq = 0;
         auto flush = [&]() {

@@ -17,7 +17,7 @@
 //                                                                          [kimad_curve.cuh, this file]
 //   k_dp            (c) Algorithm 3 on the budget axis (Eq. 2, Eq. 3, Section 3.2), one CTA per worker [kimad_dp.cuh]
 //   k_pick          (c) the uniform-ratio policies and the error-axis reading                     [kimad_dp.cuh]
-//   k_sel_count, k_sel_resolve(_r2), k_sel_count_r2, k_sel_recount, k_sel_slices, k_sel_scan
+//   k_sel_count, k_sel_offsets, k_sel_recount
 //                   (d) exact threshold and per-slice output offsets at the chosen k             [kimad_select.cuh]
 //   k_sel_write     (e)+(f) ordered (index, value) pack and g += C(d) (Algorithm 1, Eq. 6)       [kimad_select.cuh]
 //   k_apply_packed, k_aggregate   receiving side and model step (Algorithm 1, server lines)      [kimad_receiver.cuh]
@@ -234,6 +234,8 @@ struct CodeSpace { // how the sweep coded the elements of one (worker, layer)
     const uint32_t* cell_tab;  // [W][R][kCellTab]
     const int4* cell_win;      // [W][R]
     uint32_t R;
+    // index of a (worker, regular layer) in the per-layer arrays of the curve stage
+    __device__ __forceinline__ size_t slot(uint32_t w, uint32_t l) const { return (size_t)w * R + reg_index[l]; }
     // code of a key of layer l of worker w, as the sweep wrote it for every element of that layer
     __device__ __forceinline__ uint32_t code(uint32_t w, uint32_t l, uint32_t key) const {
         const uint32_t r = reg_index[l];
@@ -249,7 +251,7 @@ struct CodeSpace { // how the sweep coded the elements of one (worker, layer)
 __global__ void __launch_bounds__(kThreads)
 k_resolve1(const FbList* __restrict__ fb, const uint2* __restrict__ fb_layers, uint32_t* __restrict__ g_cnt,
            unsigned long long* __restrict__ g_ss, const KTab ktab, uint32_t L, uint32_t K,
-           Cand* __restrict__ cands, SlotTab* __restrict__ slots) {
+           Cand* __restrict__ cands, SlotTab* __restrict__ slots, const CodeSpace codes) {
     pdl_wait();
     __shared__ __align__(16) uint32_t s_incl[kL1Bins];
     __shared__ __align__(16) double s_below[kL1Bins];
@@ -258,8 +260,9 @@ k_resolve1(const FbList* __restrict__ fb, const uint2* __restrict__ fb_layers, u
   for (uint32_t it = blockIdx.x; it < fb->n_layers; it += gridDim.x) {
     const uint32_t l = fb_layers[it].y, w = fb_layers[it].x;
     const size_t wl = (size_t)w * L + l;
-    uint32_t* gc = g_cnt + wl * kL1Bins;
-    unsigned long long* gs = g_ss + wl * kL1Bins;
+    const size_t wr = codes.slot(w, l);
+    uint32_t* gc = g_cnt + wr * kL1Bins;
+    unsigned long long* gs = g_ss + wr * kL1Bins;
     {
         constexpr int PER = kL1Bins / kThreads;
         uint32_t c[PER];
@@ -323,8 +326,9 @@ k_resolve23(const FbList* __restrict__ fb, const uint2* __restrict__ fb_layers, 
     const SlotTab& stab = slots[wl];
     if (s >= stab.n) continue;
     Cand* cd = cands + wl * K;
-    uint32_t* gc = g_cnt + (wl * K + s) * kL23Bins;
-    unsigned long long* gs = g_ss + (wl * K + s) * kL23Bins;
+    const size_t wr = codes.slot(w, l);
+    uint32_t* gc = g_cnt + (wr * K + s) * kL23Bins;
+    unsigned long long* gs = g_ss + (wr * K + s) * kL23Bins;
     const uint32_t prefix = stab.prefix[s];
     {
         constexpr int PER = kL23Bins / kThreads;

@@ -2,39 +2,34 @@
 //
 // After the DP every (worker, layer) knows a key interval [lo, lo + 2^shift) that contains its
 // threshold and the rank of the threshold inside that interval (shift = 0 when the curve stage already
-// resolved all 31 bits).  One sweep over the byte codes the curve stage left (k_sel_count) counts, per 2048-element slice,
-// the entries above the interval, remembers the few entries inside it and marks the 32-element groups that
-// can hold a kept entry; k_sel_resolve turns the remembered entries (or their per-layer histogram) into the
-// exact threshold; k_sel_slices and k_sel_scan derive every slice's and chunk's output offset and leave one
-// job record per chunk; k_sel_write compacts in index order and updates the estimator, reading only the
-// marked groups of sparse slices.  No kernel waits on another: offsets come from stored counts.
+// resolved all 31 bits).  k_sel_count, one sweep over the byte codes the curve stage left, counts, per 2048-element
+// slice, the entries above the interval, lists the few entries inside it per layer and marks the 32-element groups that
+// can hold a kept entry; k_sel_offsets (a CTA per layer) takes the exact threshold from the listed entries and leaves one
+// job record per chunk with the chunk's output offset; k_sel_write compacts in index order and updates the estimator,
+// reading only the marked groups of sparse slices.  A layer with more entries in its interval than its list holds counts
+// the rest in a histogram of single keys; its chunks are counted once more against the exact threshold (k_sel_recount,
+// usually nothing to do).  No kernel waits on another: offsets come from stored counts.
 #pragma once
 #include "kimad_curve.cuh"
 
 namespace kimad {
-
-constexpr int kListCap = 32;                    // in-interval entries remembered per chunk
-constexpr uint32_t kListOverflow = 0xffffffffu; // more than that: the chunk is recounted exactly
-constexpr int kLowBins = 1024;                  // bins of the in-interval histogram
 
 // A chunk (at most 32768 elements from its 16-byte aligned start) is cut into 16 slices of 2048 elements; in
 // the sweeps of this stage a warp works on a slice by itself, so no sweep needs a block-wide barrier.
 constexpr int kSliceElems = 2048;
 constexpr int kSlices = 16;
 constexpr int kSparseGroups = 32; // the write sweep reads a slice group by group when at most this many are marked
+constexpr int kListCap = 4096;    // entries inside the interval listed per layer
+constexpr int kStageCap = 128;    // ... of which a CTA of the counting sweep gathers as many before it appends them
 
 struct ChunkSel { // per (worker, chunk)
-    uint32_t n_in;             // entries inside the interval, or kListOverflow
-    uint16_t above[kSlices];   // per slice: entries whose key lies above the interval; after k_sel_scan: entries kept
-                               // before the slice inside the chunk
-    uint16_t eq[kSlices];      // after k_sel_recount / k_sel_scan: entries equal to tau per slice, then before the slice
-    uint32_t low[kListCap];    // the entries inside the interval: slice << 16 | (key - lo), any order
-    uint32_t _pad;
+    uint16_t above[kSlices];   // per slice: entries whose key lies above the interval, after k_sel_offsets above the threshold
+    uint16_t eq[kSlices];      // per slice: entries equal to the threshold
     uint64_t mask[kSlices];    // per slice: bit g set when the 32-element group g may hold a kept entry (key >= the
                                // interval's lower end); a superset of the groups the write sweep has to read
 };
 
-// Everything the write sweep needs to know about a (worker, chunk) besides the data, gathered by k_sel_scan so
+// Everything the write sweep needs to know about a (worker, chunk) besides the data, gathered by k_sel_offsets so
 // that the write sweep starts from loads whose addresses depend on the block index only.
 struct ChunkJob {
     uint32_t mode;      // 0: nothing of this chunk is kept; 1: threshold tau; 2: the whole layer is kept
@@ -42,51 +37,74 @@ struct ChunkJob {
     uint32_t keep_eq;   // entries equal to tau that are kept, over the layer (lowest indices first)
     uint32_t gt_before; // entries above tau in the layer's earlier chunks
     uint32_t eq_before; // entries equal to tau in the layer's earlier chunks
-    uint32_t cnt_gt;    // entries above tau / equal to tau in this chunk
-    uint32_t cnt_eq;
     uint32_t idx0;      // layer-local index of the chunk's aligned start (may wrap; added back by the sweep)
     uint64_t base;      // first output position of the layer in the worker's packed buffers
 };
 
-// Second round of the select stage: layers whose interval was wider than 2^10 keys and whose entries
-// inside it could not be collected (a chunk list overflowed, or more than kSortCap entries) get their
-// interval narrowed by the coarse histogram and are counted once more over their own chunks.
-struct Round2 {
-    uint32_t n_chunks;
-    uint32_t n_layers;
-    uint32_t _pad[2];
+// Entries inside the intervals.  Only layers swept with a histogram have an interval wider than one key; their bin tables
+// and bin histograms are free after the DP, and hold the layer's list (kListCap records {chunk of the layer, slice << 16 |
+// key - lo}) and, beyond that many entries, the count of every key of the interval (clean before and after).
+struct Interval {
+    uint32_t* n;        // [W][L] entries inside the interval; zero between steps
+    uint32_t* bin_lo;   // [W][R][kMaxBins + 1]
+    uint32_t* bh_cnt;   // [W][R][kMaxBins]
+    unsigned long long* bh_sum;
+    const uint32_t* reg_index;
+    uint32_t R;
+    __device__ __forceinline__ size_t slot(uint32_t w, uint32_t l) const { return (size_t)w * R + reg_index[l]; }
+    __device__ __forceinline__ uint2* list(size_t wr) const {
+        return reinterpret_cast<uint2*>((reinterpret_cast<uintptr_t>(bin_lo + wr * (kMaxBins + 1)) + 7u) & ~(uintptr_t)7u);
+    }
+    __device__ __forceinline__ uint32_t* key_count(size_t wr, uint32_t d) const {
+        return d < (uint32_t)kMaxBins ? bh_cnt + wr * kMaxBins + d : reinterpret_cast<uint32_t*>(bh_sum + wr * kMaxBins) + (d - kMaxBins);
+    }
 };
-constexpr int kSortCap = 4096;
+static_assert(kListCap * 8 + 8 <= (kMaxBins + 1) * 4 && 3 * kMaxBins >= (1 << kMaxShift), "list and key counts fit the bin arrays");
+
+// chunks of layers whose interval held more entries than the list
+struct Recount {
+    uint32_t n_chunks;
+    uint32_t _pad[3];
+};
 
 // ------------------------------------------------------------------------------------------------
-// Counting sweep of one chunk: warp w takes the slices w and w + 8.
-__device__ __forceinline__ void sel_count_chunk(const DSource& dbuf, const Chunk& ch, uint32_t w,
-                                                uint32_t chunk_id, uint32_t n_chunks, uint64_t dstride, uint32_t L,
-                                                const Sel* __restrict__ sel, const LayerDesc* __restrict__ layers,
-                                                ChunkSel* __restrict__ csel, uint32_t* __restrict__ low_hist,
-                                                uint32_t* __restrict__ recount_n, uint2* __restrict__ recount_list,
-                                                uint32_t list_cap, uint32_t* s_n, uint32_t* s_low) {
+// Counting sweep: a CTA per chunk, warp w takes the slices w and w + 8.
+// ------------------------------------------------------------------------------------------------
+__global__ void __launch_bounds__(kThreads, 6)
+k_sel_count(DSource dbuf, const Chunk* __restrict__ chunks, uint32_t n_chunks, uint64_t dstride, uint32_t L,
+            const Sel* __restrict__ sel, const LayerDesc* __restrict__ layers, ChunkSel* __restrict__ csel, const Interval in,
+            Recount* __restrict__ rc, uint32_t w_base) {
+    pdl_wait();
+    __shared__ uint32_t s_n, s_at;
+    __shared__ uint32_t s_low[kStageCap];
+    const Chunk ch = chunks[blockIdx.x];
+    const uint32_t w = w_base + blockIdx.y;
     const size_t wl = (size_t)w * L + ch.layer;
     const Sel s = sel[wl];
-    ChunkSel* out = csel + (size_t)w * n_chunks + chunk_id;
+    const LayerDesc ld = layers[ch.layer];
+    ChunkSel* out = csel + (size_t)w * n_chunks + blockIdx.x;
     const ChunkView cv(ch);
     const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (s.k == 0 || (uint64_t)s.k == layers[ch.layer].n) { // nothing / everything kept: no need to look at the data
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) rc->n_chunks = 0; // consumed by the step before
+    if (s.k == 0 || (uint64_t)s.k == ld.n) { // nothing / everything kept: no need to look at the data
         if (threadIdx.x < kSlices) {
             const uint32_t lo = max(cv.first, threadIdx.x * kSliceElems), hi = min(cv.len, (threadIdx.x + 1) * kSliceElems);
             out->above[threadIdx.x] = (uint16_t)((s.k && hi > lo) ? hi - lo : 0u);
             out->eq[threadIdx.x] = 0;
         }
-        if (threadIdx.x == 0) out->n_in = 0;
         return;
     }
     const uint32_t lo = s.tau, width = 1u << s.shift;
-    const uint32_t hshift = s.shift > 10 ? s.shift - 10 : 0; // the histogram has at most kLowBins bins
     const bool exact = s.shift == 0;
-    if (threadIdx.x == 0) *s_n = 0;
-    uint32_t* gh = low_hist + wl * kLowBins; // the layer's in-interval histogram: few entries, counted in place
+    const uint32_t rel = blockIdx.x - ld.first_chunk;
+    if (threadIdx.x == 0) s_n = 0;
     __syncthreads();
     const DView dd(dbuf, w, dstride, cv.a0);
+    auto append = [&](uint32_t at, uint32_t rec) { // one entry of the layer's interval, the at-th
+        const size_t wr = in.slot(w, ch.layer);
+        if (at < (uint32_t)kListCap) in.list(wr)[at] = make_uint2(rel, rec);
+        else if (KIMAD_CHECK((rec & 0xffffu) < width, 1)) atomicAdd(in.key_count(wr, rec & 0xffffu), 1u);
+    };
     // Codes first: an entry whose code (the byte the sweep left for it) is larger than the code of the interval's
     // keys lies above the interval, one with a smaller code below; only entries with the interval's own code are
     // completed from the inputs.  Codes are 7-bit numbers, so "x >= t" for the four bytes of a word is bit 7 of
@@ -98,14 +116,14 @@ __device__ __forceinline__ void sel_count_chunk(const DSource& dbuf, const Chunk
         auto visit = [&](uint32_t key) -> bool { // true: the key is not below the interval
             const uint32_t d1 = key - lo; // wraps to >= 2^31 for keys below the interval
             if (d1 < width) {
-                // an exact threshold needs no list and no histogram, only the slice's number of equal entries (there
-                // may be millions of them: the exact zeros of a sparse gradient)
+                // an exact threshold needs no list, only the slice's number of equal entries (there may be millions of
+                // them: the exact zeros of a sparse gradient)
                 if (exact) {
                     above += 0x10000u;
                 } else {
-                    if (KIMAD_CHECK((d1 >> hshift) < (uint32_t)kLowBins, 1)) atomicAdd(&gh[d1 >> hshift], 1u);
-                    const uint32_t p = atomicAdd(s_n, 1u);
-                    if (p < (uint32_t)kListCap) s_low[p] = (sl << 16) | d1;
+                    const uint32_t p = atomicAdd(&s_n, 1u);
+                    if (p < (uint32_t)kStageCap) s_low[p] = (sl << 16) | d1;
+                    else append(atomicAdd(in.n + wl, 1u), (sl << 16) | d1);
                 }
             } else {
                 above += d1 < 0x80000000u;
@@ -170,97 +188,91 @@ __device__ __forceinline__ void sel_count_chunk(const DSource& dbuf, const Chunk
         if (lane == 0) { out->above[sl] = (uint16_t)above; out->eq[sl] = (uint16_t)(above >> 16); out->mask[sl] = mask; }
     }
     __syncthreads();
-    const uint32_t n_in = *s_n;
-    if (threadIdx.x < min(n_in, (uint32_t)kListCap)) out->low[threadIdx.x] = s_low[threadIdx.x];
-    if (threadIdx.x == 0) {
-        if (n_in <= (uint32_t)kListCap) {
-            out->n_in = n_in;
-        } else {
-            out->n_in = kListOverflow;
-            const uint32_t at = atomicAdd(recount_n, 1u);
-            // capacity: a chunk can be listed once per select round
-            if (KIMAD_CHECK(at < list_cap, 2)) recount_list[at] = make_uint2(w, chunk_id);
+    const uint32_t n_in = min(s_n, (uint32_t)kStageCap);
+    if (n_in) {
+        if (threadIdx.x == 0) s_at = atomicAdd(in.n + wl, n_in);
+        __syncthreads();
+        if (threadIdx.x < n_in) append(s_at + threadIdx.x, s_low[threadIdx.x]);
+    }
+}
+
+// Job records of a layer's chunks: exclusive prefix of the chunk totals over the layer's earlier chunks, stored with the
+// layer's threshold.  The whole CTA works on it.
+template <int NT>
+__device__ __forceinline__ void sel_scan_layer(const LayerDesc& ld, const Sel& s, const Chunk* __restrict__ chunks,
+                                               const ChunkSel* cs /* the layer's */, ChunkJob* __restrict__ jb, uint32_t* s_w) {
+    const bool all = (uint64_t)s.k == ld.n;
+    uint32_t run_g = 0, run_e = 0;
+    for (uint32_t base = 0; base < ld.n_chunks; base += NT) {
+        const uint32_t i = base + threadIdx.x;
+        uint32_t g = 0, q = 0;
+        if (i < ld.n_chunks) { // sixteen 16-bit counts each
+            const uint4* p = reinterpret_cast<const uint4*>(cs + i);
+            const uint4 a = __ldcg(p), b = __ldcg(p + 1), c = __ldcg(p + 2), d = __ldcg(p + 3);
+            auto sum = [](const uint4& x, const uint4& y) {
+                const uint32_t t = (x.x & 0xffffu) + (x.y & 0xffffu) + (x.z & 0xffffu) + (x.w & 0xffffu) + (y.x & 0xffffu) +
+                                   (y.y & 0xffffu) + (y.z & 0xffffu) + (y.w & 0xffffu);
+                return t + (x.x >> 16) + (x.y >> 16) + (x.z >> 16) + (x.w >> 16) + (y.x >> 16) + (y.y >> 16) + (y.z >> 16) + (y.w >> 16);
+            };
+            g = sum(a, b);
+            q = sum(c, d);
         }
-    }
-    __syncthreads();
-}
-
-__global__ void __launch_bounds__(kThreads, 6)
-k_sel_count(DSource dbuf, const Chunk* __restrict__ chunks, uint32_t n_chunks, uint64_t dstride,
-            uint32_t L, const Sel* __restrict__ sel, const LayerDesc* __restrict__ layers, ChunkSel* __restrict__ csel,
-            uint32_t* __restrict__ low_hist, uint32_t* __restrict__ recount_n, uint2* __restrict__ recount_list,
-            uint32_t list_cap, uint32_t w_base) {
-    pdl_wait();
-    __shared__ uint32_t s_n;
-    __shared__ uint32_t s_low[kListCap];
-    sel_count_chunk(dbuf, chunks[blockIdx.x], w_base + blockIdx.y, blockIdx.x, n_chunks, dstride, L, sel, layers, csel, low_hist,
-                    recount_n, recount_list, list_cap, &s_n, s_low);
-}
-
-// second round: only the chunks of the layers listed in r2
-__global__ void __launch_bounds__(kThreads)
-k_sel_count_r2(DSource dbuf, const Chunk* __restrict__ chunks, uint32_t n_chunks, uint64_t dstride,
-               uint32_t L, const Sel* __restrict__ sel, const LayerDesc* __restrict__ layers,
-               ChunkSel* __restrict__ csel, uint32_t* __restrict__ low_hist, uint32_t* __restrict__ recount_n,
-               uint2* __restrict__ recount_list, uint32_t list_cap, const Round2* __restrict__ r2,
-               const uint2* __restrict__ r2_chunks) {
-    pdl_wait();
-    __shared__ uint32_t s_n;
-    __shared__ uint32_t s_low[kListCap];
-    const uint32_t n = r2->n_chunks;
-    for (uint32_t it = blockIdx.x; it < n; it += gridDim.x) {
-        const uint2 e = r2_chunks[it];
-        sel_count_chunk(dbuf, chunks[e.y], e.x, e.y, n_chunks, dstride, L, sel, layers, csel, low_hist, recount_n,
-                        recount_list, list_cap, &s_n, s_low);
+        uint32_t tg, te;
+        const uint32_t eg = block_excl_scan<uint32_t, NT>(g, s_w, &tg);
+        const uint32_t ee = block_excl_scan<uint32_t, NT>(q, s_w, &te);
+        if (i < ld.n_chunks) {
+            const ChunkView cv(chunks[ld.first_chunk + i]);
+            ChunkJob j;
+            j.tau = s.tau;
+            j.keep_eq = s.keep_eq;
+            j.gt_before = run_g + eg;
+            j.eq_before = run_e + ee;
+            j.idx0 = (uint32_t)(cv.a0 - ld.begin);
+            j.base = s.base;
+            const bool none = s.k == 0 || (!all && g == 0 && (q == 0 || j.eq_before >= s.keep_eq));
+            j.mode = none ? 0u : (all ? 2u : 1u);
+            jb[i] = j;
+        }
+        run_g += tg;
+        run_e += te;
     }
 }
 
-// Exact threshold of one (worker, layer) from what the counting sweep left behind.  The whole CTA works on it.
-// first round: may narrow the interval and list the layer for the second round; second round: the interval is at
-// most 32 keys wide and the histogram is exact.
-__device__ __forceinline__ void sel_resolve_layer(uint32_t l, uint32_t w, uint32_t L, const LayerDesc* __restrict__ layers,
-                                                  uint32_t n_chunks, const ChunkSel* __restrict__ csel,
-                                                  uint32_t* __restrict__ low_hist, Sel* __restrict__ sel, bool round1,
-                                                  Round2* __restrict__ r2, uint2* __restrict__ r2_layers,
-                                                  uint2* __restrict__ r2_chunks, uint32_t* s_key /* [kSortCap] */,
-                                                  uint32_t* s_w32, uint32_t* s_n, uint32_t* s_over) {
+// Exact threshold and job records, one CTA per (layer, worker).  The listed entries (16-bit distances from the interval's
+// lower key) are ranked by two 8-bit digits; each then joins its slice's counts.  Bound by the latency of a few dependent
+// rounds per layer: NT = 512 where a layer has thousands of chunks, 128 where none has more than 256 (1995 layers of two
+// chunks: 40 us with 512 threads, which need two waves of CTAs).
+template <int NT>
+__global__ void __launch_bounds__(NT)
+k_sel_offsets(const LayerDesc* __restrict__ layers, const Chunk* __restrict__ chunks, uint32_t n_chunks, uint32_t L,
+              Sel* __restrict__ sel, ChunkSel* __restrict__ csel, ChunkJob* __restrict__ jobs, const Interval in, FbList* __restrict__ fb,
+              Recount* __restrict__ rc, uint2* __restrict__ rc_chunks, uint32_t list_cap, uint32_t w_base) {
+    pdl_wait();
+    __shared__ uint32_t s_w[NT / 32], s_h[256], s_digit, s_gt, s_at;
+    __shared__ uint16_t s_key[kListCap];
+    const uint32_t l = blockIdx.x, w = w_base + blockIdx.y;
     const size_t wl = (size_t)w * L + l;
     const LayerDesc ld = layers[l];
     Sel s = sel[wl];
-    if (s.k == 0 || (uint64_t)s.k == ld.n) return;
-    uint32_t* gh = low_hist + wl * kLowBins;
-    const uint32_t hshift = s.shift > 10 ? s.shift - 10 : 0;
-    if (s.shift == 0) { // already exact: bin 0 holds the number of entries equal to tau
-        if (threadIdx.x == 0) gh[0] = 0;
-        return;
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) { // the curve stage's lists (of these workers) have been consumed
+        fb->n_chunks = 0;
+        fb->n_layers = 0;
+        fb->rf_chunks = 0;
+        fb->rf_layers = 0;
     }
-    bool sorted = false;
-    if (round1) { // collect the entries inside the interval from the chunk lists and sort them
-        if (threadIdx.x == 0) { *s_n = 0; *s_over = 0; }
-        __syncthreads();
-        const ChunkSel* cs = csel + (size_t)w * n_chunks + ld.first_chunk;
-        for (uint32_t i = threadIdx.x; i < ld.n_chunks; i += kThreads) {
-            const uint32_t n_in = cs[i].n_in;
-            if (n_in == kListOverflow) { *s_over = 1; continue; }
-            if (!n_in) continue;
-            const uint32_t at = atomicAdd(s_n, n_in);
-            if (at + n_in > (uint32_t)kSortCap) { *s_over = 1; continue; }
-            for (uint32_t e = 0; e < n_in; ++e) s_key[at + e] = cs[i].low[e] & 0xffffu;
-        }
-        __syncthreads();
-        sorted = !*s_over;
-        if (sorted) {
-            // the rank-th largest of the collected entries (16-bit numbers) by two 8-bit digits: a histogram of the
-            // upper digit, then one of the lower digit among the entries that share the upper digit found
-            const uint32_t cnt = *s_n;
-            static_assert(kThreads == 256, "one thread per digit");
-            __shared__ uint32_t s_h[256];
-            __shared__ uint32_t s_digit, s_gt;
+    ChunkSel* cs = csel + (size_t)w * n_chunks + ld.first_chunk;
+    if (s.k != 0 && (uint64_t)s.k != ld.n && s.shift != 0) {
+        const size_t wr = in.slot(w, l);
+        const uint2* list = in.list(wr);
+        const uint32_t total = in.n[wl], cnt = min(total, (uint32_t)kListCap);
+        const bool over = total > (uint32_t)kListCap;
+        if (!over) {
+            for (uint32_t i = threadIdx.x; i < cnt; i += NT) s_key[i] = (uint16_t)(list[i].y & 0xffffu);
             uint32_t rank = s.keep_eq, hi_digit = 0, greater = 0; // rank <= cnt by construction
             for (int pass = 0; pass < 2; ++pass) {
-                s_h[threadIdx.x] = 0; // kThreads == 256
+                for (uint32_t i = threadIdx.x; i < 256; i += NT) s_h[i] = 0;
                 __syncthreads();
-                for (uint32_t i = threadIdx.x; i < cnt; i += kThreads) {
+                for (uint32_t i = threadIdx.x; i < cnt; i += NT) {
                     const uint32_t k = s_key[i];
                     if (pass == 0) atomicAdd(&s_h[k >> 8], 1u);
                     else if ((k >> 8) == hi_digit) atomicAdd(&s_h[k & 255u], 1u);
@@ -289,85 +301,70 @@ __device__ __forceinline__ void sel_resolve_layer(uint32_t l, uint32_t w, uint32
                 if (pass == 0) { hi_digit = s_digit; greater = s_gt; rank -= s_gt; }
                 else { greater += s_gt; }
             }
-            if (threadIdx.x == 0) {
-                const uint32_t t = (hi_digit << 8) | s_digit;
-                s.tau_low = t;
-                s.tau += t;
-                s.keep_eq = s.keep_eq - greater; // rank among the entries equal to t: those above t come first
-                s.shift = 0;
-                sel[wl] = s;
+            s.tau_low = (hi_digit << 8) | s_digit;
+            s.keep_eq -= greater; // rank among the entries equal to the threshold: those above it come first
+            for (uint32_t i = threadIdx.x; i < cnt; i += NT) {
+                const uint2 e = list[i];
+                const uint32_t k = e.y & 0xffffu, sl = e.y >> 16;
+                if (k < s.tau_low) continue;
+                uint32_t* c = reinterpret_cast<uint32_t*>(k > s.tau_low ? cs[e.x].above : cs[e.x].eq) + (sl >> 1);
+                atomicAdd(c, 1u << (16u * (sl & 1u)));
             }
-        }
-    }
-    __syncthreads();
-    if (!sorted) { // histogram of the interval: exact when it has at most kLowBins keys, else it narrows the interval
-        uint32_t* s_incl = s_key; // [kLowBins], reuse
-        for (int b = threadIdx.x; b < kLowBins; b += kThreads) s_incl[kLowBins - 1 - b] = gh[b];
-        __syncthreads();
-        scan_bins<kLowBins>(s_incl, nullptr, s_w32, nullptr);
-        if (threadIdx.x == 0) {
-            const int p = find_pos<kLowBins>(s_incl, s.keep_eq); // keep_eq holds the rank inside the interval
-            const uint32_t above = p ? s_incl[p - 1] : 0u;
-            const uint32_t bin = (uint32_t)(kLowBins - 1 - p);
-            s.keep_eq -= above;
-            s.tau += bin << hshift;
-            s.tau_low = hshift ? 0u : bin;
-            s.shift = hshift;
-            sel[wl] = s;
-        }
-        if (hshift) { // not exact yet: the layer and its chunks go to the second round
-            __shared__ uint32_t s_at;
-            if (threadIdx.x == 0) {
-                s_at = atomicAdd(&r2->n_chunks, ld.n_chunks);
-                r2_layers[atomicAdd(&r2->n_layers, 1u)] = make_uint2(w, l);
+            __threadfence(); // the counts are read back below by other threads of this CTA
+        } else { // every key of the interval was counted, but for the listed entries
+            for (uint32_t i = threadIdx.x; i < cnt; i += NT) atomicAdd(in.key_count(wr, list[i].y & 0xffffu), 1u);
+            __threadfence();
+            __syncthreads();
+            // thread t takes the keys [k0, k1), descending with t
+            const uint32_t width = 1u << s.shift, per = (width + NT - 1) / NT;
+            const uint32_t k1 = threadIdx.x * per < width ? width - threadIdx.x * per : 0u, k0 = k1 > per ? k1 - per : 0u;
+            uint32_t mine = 0;
+            for (uint32_t k = k0; k < k1; ++k) mine += __ldcg(in.key_count(wr, k));
+            uint32_t before = block_excl_scan<uint32_t, NT>(mine, s_w, nullptr);
+            if (before < s.keep_eq && before + mine >= s.keep_eq) {
+                uint32_t k = k1 - 1;
+                for (;; --k) {
+                    const uint32_t c = __ldcg(in.key_count(wr, k));
+                    if (before + c >= s.keep_eq) break;
+                    before += c;
+                }
+                s_digit = k;
+                s_gt = before;
             }
             __syncthreads();
-            for (uint32_t i = threadIdx.x; i < ld.n_chunks; i += kThreads) r2_chunks[s_at + i] = make_uint2(w, ld.first_chunk + i);
+            s.tau_low = s_digit;
+            s.keep_eq -= s_gt;
+            for (uint32_t k = k0; k < k1; ++k) *in.key_count(wr, k) = 0; // clean for the next use
+            if (threadIdx.x == 0) s_at = atomicAdd(&rc->n_chunks, ld.n_chunks);
+        }
+        s.tau += s.tau_low;
+        s.shift = 0;
+        __syncthreads();
+        if (threadIdx.x == 0) { sel[wl] = s; in.n[wl] = 0; }
+        if (over) { // its chunks are counted again
+            for (uint32_t i = threadIdx.x; i < ld.n_chunks; i += NT)
+                if (KIMAD_CHECK(s_at + i < list_cap, 2)) rc_chunks[s_at + i] = make_uint2(w, ld.first_chunk + i);
+            return;
         }
     }
-    __syncthreads();
-    for (int b = threadIdx.x; b < kLowBins; b += kThreads) gh[b] = 0; // clean for the next use
-    __syncthreads();
+    sel_scan_layer<NT>(ld, s, chunks, cs, jobs + (size_t)w * n_chunks + ld.first_chunk, s_w);
 }
 
+// Exact per-slice (gt, eq) of the listed chunks: warp w recounts the slices w and w + 8.  The CTA that finishes the last
+// chunk of a layer makes the layer's job records (Interval::n counts the finished ones).
 __global__ void __launch_bounds__(kThreads)
-k_sel_resolve(uint32_t L, const LayerDesc* __restrict__ layers, uint32_t n_chunks, const ChunkSel* __restrict__ csel,
-              uint32_t* __restrict__ low_hist, Sel* __restrict__ sel, Round2* __restrict__ r2,
-              uint2* __restrict__ r2_layers, uint2* __restrict__ r2_chunks, uint32_t w_base) {
+k_sel_recount(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* __restrict__ chunks, uint32_t n_chunks, uint64_t dstride,
+              uint32_t L, const Sel* __restrict__ sel, ChunkSel* __restrict__ csel, ChunkJob* __restrict__ jobs, const Interval in,
+              const Recount* __restrict__ rc, const uint2* __restrict__ rc_chunks) {
     pdl_wait();
-    __shared__ __align__(16) uint32_t s_key[kSortCap];
-    __shared__ uint32_t s_w32[8];
-    __shared__ uint32_t s_n, s_over;
-    sel_resolve_layer(blockIdx.x, w_base + blockIdx.y, L, layers, n_chunks, csel, low_hist, sel, true, r2, r2_layers, r2_chunks, s_key,
-                      s_w32, &s_n, &s_over);
-}
-
-__global__ void __launch_bounds__(kThreads)
-k_sel_resolve_r2(uint32_t L, const LayerDesc* __restrict__ layers, uint32_t n_chunks, const ChunkSel* __restrict__ csel,
-                 uint32_t* __restrict__ low_hist, Sel* __restrict__ sel, Round2* __restrict__ r2,
-                 uint2* __restrict__ r2_layers, uint2* __restrict__ r2_chunks) {
-    pdl_wait();
-    __shared__ __align__(16) uint32_t s_key[kSortCap];
-    __shared__ uint32_t s_w32[8];
-    __shared__ uint32_t s_n, s_over;
-    const uint32_t n = r2->n_layers;
-    for (uint32_t it = blockIdx.x; it < n; it += gridDim.x)
-        sel_resolve_layer(r2_layers[it].y, r2_layers[it].x, L, layers, n_chunks, csel, low_hist, sel, false, r2, r2_layers,
-                          r2_chunks, s_key, s_w32, &s_n, &s_over);
-}
-
-// Exact per-slice (gt, eq) of the chunks whose list overflowed: warp w recounts the slices w and w + 8.
-__global__ void __launch_bounds__(kThreads)
-k_sel_recount(DSource dbuf, const Chunk* __restrict__ chunks, uint32_t n_chunks, uint64_t dstride,
-              uint32_t L, const Sel* __restrict__ sel, const uint32_t* __restrict__ recount_n,
-              const uint2* __restrict__ recount_list, ChunkSel* __restrict__ csel) {
-    pdl_wait();
-    const uint32_t n = *recount_n;
+    __shared__ uint32_t s_w[kThreads / 32], s_last;
+    const uint32_t n = rc->n_chunks;
     const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (uint32_t it = blockIdx.x; it < n; it += gridDim.x) {
-        const uint2 e = recount_list[it];
+        const uint2 e = rc_chunks[it];
         const Chunk ch = chunks[e.y];
-        const Sel s = sel[(size_t)e.x * L + ch.layer];
+        const size_t wl = (size_t)e.x * L + ch.layer;
+        const Sel s = sel[wl];
         const ChunkView cv(ch);
         const DView dd(dbuf, e.x, dstride, cv.a0);
         ChunkSel* out = csel + (size_t)e.x * n_chunks + e.y;
@@ -386,94 +383,18 @@ k_sel_recount(DSource dbuf, const Chunk* __restrict__ chunks, uint32_t n_chunks,
             }
             if (lane == 0) { out->above[sl] = (uint16_t)gt; out->eq[sl] = (uint16_t)eq; }
         }
-        // The recount is authoritative.  A chunk listed in the first round may have been counted again in the
-        // second (narrowed interval) and then own a fresh in-interval list; k_sel_slices must not add that list
-        // on top of the exact counts written here.
-        if (threadIdx.x == 0) out->n_in = kListOverflow;
-    }
-}
-
-// Per chunk (one warp each, lane = slice): entries above tau and equal to tau in every slice (from the lists, or
-// already recounted), turned into prefixes inside the chunk; chunk_cnt = the chunk's totals.
-__global__ void __launch_bounds__(kThreads)
-k_sel_slices(const Chunk* __restrict__ chunks, uint32_t n_chunks, uint32_t w_base, uint32_t n_workers, uint32_t L,
-             const Sel* __restrict__ sel, ChunkSel* __restrict__ csel, uint2* __restrict__ chunk_cnt) {
-    pdl_wait();
-    const uint32_t lane = threadIdx.x & 31;
-    uint64_t it = (uint64_t)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
-    if (it >= (uint64_t)n_workers * n_chunks) return;
-    it += (uint64_t)w_base * n_chunks; // workers w_base .. w_base + n_workers - 1
-    const uint32_t w = (uint32_t)(it / n_chunks), ci = (uint32_t)(it % n_chunks);
-    const Sel s = sel[(size_t)w * L + chunks[ci].layer];
-    ChunkSel& c = csel[it];
-    uint32_t g = 0, q = 0;
-    if (lane < (uint32_t)kSlices) { g = c.above[lane]; q = c.eq[lane]; }
-    const uint32_t n_in = c.n_in;
-    if (n_in != kListOverflow)
-        for (uint32_t e = 0; e < n_in; ++e) { // entries inside the interval join their slice's counts
-            const uint32_t en = c.low[e];
-            if ((en >> 16) == lane) {
-                g += (en & 0xffffu) > s.tau_low;
-                q += (en & 0xffffu) == s.tau_low;
-            }
+        const LayerDesc ld = layers[ch.layer];
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) s_last = atomicAdd(in.n + wl, 1u) + 1u == ld.n_chunks;
+        __syncthreads();
+        if (s_last) {
+            __threadfence();
+            sel_scan_layer<kThreads>(ld, s, chunks, csel + (size_t)e.x * n_chunks + ld.first_chunk,
+                                     jobs + (size_t)e.x * n_chunks + ld.first_chunk, s_w);
+            if (threadIdx.x == 0) in.n[wl] = 0;
         }
-    uint32_t ig = g, iq = q;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t yg = __shfl_up_sync(0xffffffffu, ig, o), yq = __shfl_up_sync(0xffffffffu, iq, o);
-        if (lane >= (uint32_t)o) { ig += yg; iq += yq; }
-    }
-    if (lane < (uint32_t)kSlices) { c.above[lane] = (uint16_t)(ig - g); c.eq[lane] = (uint16_t)(iq - q); }
-    if (lane == 31) chunk_cnt[it] = make_uint2(ig, iq);
-}
-
-// Exclusive prefix of the chunk totals over the layer's earlier chunks, stored with the layer's threshold as the
-// write sweep's job record of every chunk.
-__global__ void __launch_bounds__(kThreads)
-k_sel_scan(const LayerDesc* __restrict__ layers, const Chunk* __restrict__ chunks, uint32_t n_chunks, uint32_t L,
-           const Sel* __restrict__ sel, const uint2* __restrict__ chunk_cnt, ChunkJob* __restrict__ jobs,
-           uint32_t* __restrict__ recount_n, FbList* __restrict__ fb, Round2* __restrict__ r2, uint32_t w_base) {
-    pdl_wait();
-    __shared__ uint32_t s_w[8];
-    const LayerDesc ld = layers[blockIdx.x];
-    const uint32_t w = w_base + blockIdx.y;
-    const Sel s = sel[(size_t)w * L + blockIdx.x];
-    const uint2* cc = chunk_cnt + (size_t)w * n_chunks + ld.first_chunk;
-    ChunkJob* jb = jobs + (size_t)w * n_chunks + ld.first_chunk;
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) { // all work lists (of these workers) have been consumed by now
-        *recount_n = 0;
-        fb->n_chunks = 0;
-        fb->n_layers = 0;
-        fb->rf_chunks = 0;
-        fb->rf_layers = 0;
-        r2->n_chunks = 0;
-        r2->n_layers = 0;
-    }
-    const bool all = (uint64_t)s.k == ld.n;
-    uint32_t run_g = 0, run_e = 0;
-    for (uint32_t base = 0; base < ld.n_chunks; base += kThreads) {
-        const uint32_t i = base + threadIdx.x;
-        const uint2 v = i < ld.n_chunks ? cc[i] : make_uint2(0, 0);
-        uint32_t tg, te;
-        const uint32_t eg = block_excl_scan<uint32_t>(v.x, s_w, &tg);
-        const uint32_t ee = block_excl_scan<uint32_t>(v.y, s_w, &te);
-        if (i < ld.n_chunks) {
-            const ChunkView cv(chunks[ld.first_chunk + i]);
-            ChunkJob j;
-            j.tau = s.tau;
-            j.keep_eq = s.keep_eq;
-            j.gt_before = run_g + eg;
-            j.eq_before = run_e + ee;
-            j.cnt_gt = v.x;
-            j.cnt_eq = v.y;
-            j.idx0 = (uint32_t)(cv.a0 - ld.begin);
-            j.base = s.base;
-            const bool none = s.k == 0 || (!all && v.x == 0 && (v.y == 0 || j.eq_before >= s.keep_eq));
-            j.mode = none ? 0u : (all ? 2u : 1u);
-            jb[i] = j;
-        }
-        run_g += tg;
-        run_e += te;
+        __syncthreads();
     }
 }
 
@@ -496,7 +417,6 @@ k_sel_write(const float* __restrict__ grads, float* __restrict__ state, const Ch
     const Chunk ch = chunks[blockIdx.x];
     const ChunkSel& cs = csel[(size_t)w * n_chunks + blockIdx.x];
     const bool all = jb.mode == 2;
-    const uint2 cnt = make_uint2(jb.cnt_gt, jb.cnt_eq), pre = make_uint2(jb.gt_before, jb.eq_before);
     const uint32_t keep_eq = jb.keep_eq;
     const uint32_t tau = jb.tau;
     const ChunkView cv(ch);
@@ -509,6 +429,13 @@ k_sel_write(const float* __restrict__ grads, float* __restrict__ state, const Ch
     const uint32_t idx0 = jb.idx0;
     const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const bool st_vec = ((reinterpret_cast<uintptr_t>(st) | reinterpret_cast<uintptr_t>(gr)) & 15u) == 0; // 128-bit access to both
+    // entries above (low half) and equal to tau (high half) in the chunk's slices up to the one of lane i
+    uint32_t upto = lane < (uint32_t)kSlices ? cs.above[lane] | (uint32_t)cs.eq[lane] << 16 : 0u;
+#pragma unroll
+    for (int o = 1; o < kSlices; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, upto, o);
+        if (lane >= (uint32_t)o) upto += y;
+    }
     __shared__ uint8_t s_pos[kThreads / 32][kSparseGroups]; // per warp: the marked groups of a slice, ascending
     __shared__ uint32_t s_stage[DENSE ? kThreads / 32 : 1][DENSE ? 2 * 16 * 32 : 1]; // per warp: a round's indices, values
 
@@ -516,9 +443,9 @@ k_sel_write(const float* __restrict__ grads, float* __restrict__ state, const Ch
         const uint32_t x0 = sl * kSliceElems;
         if (x0 >= cv.len) break;
         // entries equal to tau are kept while their rank among equals (ascending index) is below keep_eq
-        const uint32_t gt_before = pre.x + cs.above[sl], eq_before = pre.y + cs.eq[sl];
-        const uint32_t gt_here = (sl + 1 < (uint32_t)kSlices ? cs.above[sl + 1] : cnt.x) - cs.above[sl];
-        const uint32_t eq_here = (sl + 1 < (uint32_t)kSlices ? cs.eq[sl + 1] : cnt.y) - cs.eq[sl];
+        const uint32_t ahead = sl ? __shfl_sync(0xffffffffu, upto, sl - 1) : 0u, here = __shfl_sync(0xffffffffu, upto, sl) - ahead;
+        const uint32_t gt_before = jb.gt_before + (ahead & 0xffffu), eq_before = jb.eq_before + (ahead >> 16);
+        const uint32_t gt_here = here & 0xffffu, eq_here = here >> 16;
         // eq_mode 0: none of this slice's equals is kept; 1: all are; 2: ranks must be counted
         const int eq_mode = (all || eq_here == 0 || eq_before >= keep_eq) ? 0 : (eq_before + eq_here <= keep_eq ? 1 : 2);
         if (!all && gt_here == 0 && eq_mode == 0) continue; // nothing kept in this slice
