@@ -28,7 +28,7 @@ struct Layout {
     size_t zero_from, h1_cnt, h1_ss, h23_cnt, h23_ss, bh_cnt, bh_sum, in_n, fb, rc, flags;
     // scratch without initial-state requirements
     size_t cell_tab, cell_win, bin_lo, meta, cands, slots, err, tau, keep_eq, shift, sel, jobs, csel,
-        fb_chunks, fb_layers, rc_chunks, rf, rf_chunks, rf_layers, pd, rows, total;
+        fb_chunks, rc_chunks, rf, rf_chunks, pd, rows, total;
 };
 
 } // namespace
@@ -133,11 +133,9 @@ void plan_layout(kimad_ctx* c) {
     y.jobs = take((size_t)c->W * nch * sizeof(ChunkJob));
     y.csel = take((size_t)c->W * nch * sizeof(ChunkSel));
     y.fb_chunks = take(kGroups * align_up((size_t)c->W * nch * sizeof(uint2)));
-    y.fb_layers = take(kGroups * align_up(WL * sizeof(uint2)));
     y.rc_chunks = take(kGroups * align_up((size_t)c->W * nch * sizeof(uint2)));
     y.rf = take(WLK * sizeof(RefineCand));
     y.rf_chunks = take(kGroups * align_up((size_t)c->W * nch * sizeof(uint2)));
-    y.rf_layers = take(kGroups * align_up(WL * sizeof(uint2)));
     y.pd = take((size_t)c->W * c->L * c->pd_stride);
     y.rows = take(c->policy == 0 && !c->rows_in_bins ? WL * c->hist_row * sizeof(float) + 16 : 0);
     y.total = o;
@@ -158,9 +156,7 @@ static int preload_kernels() {
     cudaFuncAttributes a;
 #define KIMAD_PRELOAD(f) CUDA_TRY(cudaFuncGetAttributes(&a, f))
     KIMAD_PRELOAD(k_sample); KIMAD_PRELOAD(k_pass_a<true>); KIMAD_PRELOAD(k_pass_a<false>); KIMAD_PRELOAD(k_resolve_a);
-    KIMAD_PRELOAD(k_refine_hist); KIMAD_PRELOAD(k_refine_resolve);
-    KIMAD_PRELOAD(k_tiny_exact); KIMAD_PRELOAD(k_fb_hist1); KIMAD_PRELOAD(k_fb_hist23<2>); KIMAD_PRELOAD(k_fb_hist23<3>);
-    KIMAD_PRELOAD(k_resolve1); KIMAD_PRELOAD(k_resolve23<2>); KIMAD_PRELOAD(k_resolve23<3>); KIMAD_PRELOAD(k_rebuild_slots);
+    KIMAD_PRELOAD(k_refine); KIMAD_PRELOAD(k_tiny_exact); KIMAD_PRELOAD(k_fb1); KIMAD_PRELOAD(k_fb23<2>); KIMAD_PRELOAD(k_fb23<3>);
     KIMAD_PRELOAD(k_dp<2>); KIMAD_PRELOAD(k_dp<4>); KIMAD_PRELOAD(k_dp<8>); KIMAD_PRELOAD(k_pick); KIMAD_PRELOAD(k_fit_ratio); KIMAD_PRELOAD(k_sel_count);
     KIMAD_PRELOAD(k_sel_offsets<128>); KIMAD_PRELOAD(k_sel_offsets<512>); KIMAD_PRELOAD(k_sel_recount);
     KIMAD_PRELOAD((k_sel_write<false, false>)); KIMAD_PRELOAD((k_sel_write<false, true>));
@@ -414,10 +410,8 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
         const Interval in{c->at<uint32_t>(y.in_n), binlo, bhc, bhs, reg_index, R};
         uint2* fb_chunks = c->at<uint2>(y.fb_chunks + g * align_up((size_t)W * nch * sizeof(uint2)));
         uint2* rc_chunks = c->at<uint2>(y.rc_chunks + g * align_up((size_t)W * nch * sizeof(uint2)));
-        uint2* fb_layers = c->at<uint2>(y.fb_layers + g * align_up((size_t)W * L * sizeof(uint2)));
         RefineCand* rf = c->at<RefineCand>(y.rf);
         uint2* rf_chunks = c->at<uint2>(y.rf_chunks + g * align_up((size_t)W * nch * sizeof(uint2)));
-        uint2* rf_layers = c->at<uint2>(y.rf_layers + g * align_up((size_t)W * L * sizeof(uint2)));
         const dim3 gch(nch, nw), glw(L, nw);
         // the group's runs of the sweep: the run table is sorted by worker
         uint32_t run0 = 0, run1 = 0;
@@ -436,7 +430,7 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
         CUDA_TRY(hand_over(big, small));
         if (R) {
             CUDA_TRY(launch_pdl(k_resolve_a, dim3(R, nw), kBigThreads, 0, small, layers, reg_layers, R, L, ktab, K, meta, cell_win, binlo, bhc, bhs,
-                                err, tau, keq, shf, flags, fb, fb_chunks, fb_layers, rf, rf_chunks, rf_layers, list_cap, w0));
+                                err, tau, keq, shf, flags, fb, fb_chunks, rf, rf_chunks, list_cap, w0));
             c->launches += 1;
         }
         mark(small);
@@ -475,26 +469,24 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
         };
         // refinement and exact radix select for the layers listed by k_resolve_a (the lists are usually empty)
         auto launch_lists = [&](cudaStream_t st) -> int {
-            // small grids: the lists are usually empty, and every kernel of the chain then costs only its launch; the
-            // histogram kernels get four CTAs per SM, enough to stream a large handed-over layer
-            const uint32_t gfb = 4 * 148, glay = std::min<uint32_t>(nw * R, 32u);
-            const dim3 gslot(glay, 1, K);
+            // the lists are usually empty, and a kernel of the chain then costs only its launch; four CTAs per SM are enough to
+            // stream a large handed-over layer
+            const uint32_t gfb = 4 * 148;
+            uint32_t* arrived = c->at<uint32_t>(y.in_n); // (counts the select stage's entries later in the step; zero in between)
             // candidates with a loose bound first (they may still end on the exact path's lists)
-            CUDA_TRY(launch_pdl(k_refine_hist, 6 * 148, blk, 0, st, dbuf, chunks, c->dstride, L, K, fb, rf_chunks, rf, codes, h23c, h23s));
-            CUDA_TRY(launch_pdl(k_refine_resolve, glay, blk, 0, st, layers, L, K, fb, rf_layers, rf, h23c, h23s, err, tau, keq, shf,
-                                codes, fb_chunks, fb_layers, list_cap));
-            CUDA_TRY(launch_pdl(k_fb_hist1, gfb, blk, 0, st, dbuf, chunks, c->dstride, fb, fb_chunks, h1c, h1s, flags, codes));
-            CUDA_TRY(launch_pdl(k_resolve1, glay, blk, 0, st, fb, fb_layers, h1c, h1s, ktab, L, K, cands, slots, codes));
-            CUDA_TRY(launch_pdl(k_fb_hist23<2>, gfb, blk, 0, st, dbuf, chunks, c->dstride, L, K, fb, fb_chunks, slots, h23c, h23s, codes));
-            CUDA_TRY(launch_pdl(k_resolve23<2>, gslot, blk, 0, st, fb, fb_layers, h23c, h23s, L, K, cands, slots, err, tau, keq, shf, codes));
-            CUDA_TRY(launch_pdl(k_rebuild_slots, (nw * R + kThreads - 1) / kThreads, blk, 0, st, fb, fb_layers, L, K, cands, slots));
-            CUDA_TRY(launch_pdl(k_fb_hist23<3>, gfb, blk, 0, st, dbuf, chunks, c->dstride, L, K, fb, fb_chunks, slots, h23c, h23s, codes));
-            CUDA_TRY(launch_pdl(k_resolve23<3>, gslot, blk, 0, st, fb, fb_layers, h23c, h23s, L, K, cands, slots, err, tau, keq, shf, codes));
-            c->launches += 9;
+            CUDA_TRY(launch_pdl(k_refine, 5 * 148, blk, 0, st, dbuf, layers, chunks, c->dstride, L, K, fb, rf_chunks, rf, codes, h23c, h23s,
+                                arrived, err, tau, keq, shf, fb_chunks, list_cap));
+            CUDA_TRY(launch_pdl(k_fb1, gfb, blk, 0, st, dbuf, layers, chunks, c->dstride, L, K, ktab, fb, fb_chunks, h1c, h1s, flags, codes,
+                                arrived, cands, slots));
+            CUDA_TRY(launch_pdl(k_fb23<2>, gfb, blk, 0, st, dbuf, layers, chunks, c->dstride, L, K, fb, fb_chunks, slots, cands, h23c, h23s,
+                                codes, arrived, err, tau, keq, shf));
+            CUDA_TRY(launch_pdl(k_fb23<3>, gfb, blk, 0, st, dbuf, layers, chunks, c->dstride, L, K, fb, fb_chunks, slots, cands, h23c, h23s,
+                                codes, arrived, err, tau, keq, shf));
+            c->launches += 4;
             return KIMAD_OK;
         };
         if (R && !c->timing) {
-            // The lists are usually empty, so the DP is launched at once and goes ahead only if they are; the nine
+            // The lists are usually empty, so the DP is launched at once and goes ahead only if they are; the four
             // list-driven kernels run beside it on a stream of their own, followed by a second launch of the DP that
             // goes ahead only if something was listed.  Their launch latencies leave the step's critical path.
             cudaStream_t lst = c->glist[g];

@@ -19,11 +19,10 @@
 //                layer's size minus the counted entries) and the squares below it.  The candidate's error is certified to 5e-6 relative from the bin's width.  A
 //                threshold in a gap bin (the sample mispredicted) sends the layer to the exact radix path; a bound
 //                that is too loose sends the candidate to the refinement.
-//   k_refine_hist, k_refine_resolve
-//                loose candidates: the entries of the threshold's bin, found by their code byte, are counted in
+//   k_refine     loose candidates: the entries of the threshold's bin, found by their code byte, are counted in
 //                1024 pieces of the bin; error and interval from the pieces (still loose: exact path).
 //   k_tiny_exact layers of at most kTinyMax elements are sorted in shared memory instead.
-//   k_fb_*       exact three-digit radix select over the chunks of the layers handed over (rare).
+//   k_fb1, k_fb23 exact three-digit radix select over the chunks of the layers handed over (rare).
 #pragma once
 #include "kimad_kernels.cuh"
 #include <type_traits>
@@ -69,8 +68,9 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
     uint32_t* s_cb = s_w + 32;                    // [128] per candidate, then per merged group: lowest cell,
     uint32_t* s_ct = s_cb + 128;                  // [128] highest cell,
     uint32_t* s_cs = s_ct + 128;                  // [128] shift
-    __shared__ uint32_t s_m, s_flag, s_ng, s_cg, s_z;
+    __shared__ uint32_t s_m, s_flag, s_ng, s_cg, s_z, s_clip;
     __shared__ unsigned long long s_zz;
+    __shared__ float s_nd[128]; // bins per cell needed, per candidate, then per merged group
     const uint32_t r = blockIdx.x, w = blockIdx.y;
     const uint32_t l = reg_layers[r];
     const size_t wr = (size_t)w * R + r;
@@ -82,7 +82,7 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
     const LayerDesc ld = layers[l];
     const uint32_t n = (uint32_t)ld.n;
     for (int i = threadIdx.x; i < 32768 / 4; i += kBigThreads) reinterpret_cast<uint4*>(h32)[i] = make_uint4(0u, 0u, 0u, 0u);
-    if (threadIdx.x == 0) { s_m = 0; s_flag = 0; s_ng = 0; s_cg = 0; s_z = 0; s_zz = 0ull; }
+    if (threadIdx.x == 0) { s_m = 0; s_flag = 0; s_ng = 0; s_cg = 0; s_z = 0; s_zz = 0ull; s_clip = 0; }
     __syncthreads();
 
     // ---- stratified sample of |grad - g|.  Exact zeros (the untouched rows of a sparse gradient) are counted apart:
@@ -205,6 +205,7 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
     for (uint32_t j = threadIdx.x >> 5; j < K; j += kBigThreads / 32) {
         const uint64_t k = ktab.at(w, (size_t)l * K + j);
         uint32_t o_cb = 1, o_ct = 0, o_cs = 15; // k == n keeps everything: no threshold, no band
+        float o_nd = 1.f;                        // bins per cell it needs
         if (k < n) {
             uint32_t r_lo, r_hi;
             if (whole) {
@@ -230,7 +231,10 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
             // quarter octave further up; clipped at the bottom: no bound from the sample, exact path
             // bands stay among the finite keys (a sample with non-finite values is reported by the curve stage)
             uint32_t c_top = min(cell_of_rank(max(r_lo, 1u)), 65279u);
-            if (r_lo == 0) c_top = min(c_top + 64u, 65279u);
+            if (r_lo == 0) {
+                c_top = min(c_top + 64u, 65279u);
+                if (lane == 0) s_clip = 1;
+            }
             if (r_hi == 0 && !z && lane == 0) s_flag = 1;
             uint32_t c_bot = cell_of_rank(clip_bot ? mz : max(r_hi, 1u));
             if (clip_bot) c_bot = c_bot > 64u ? c_bot - 64u : 0u;
@@ -282,9 +286,10 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
                 uint32_t sh_j = 15;
                 while (sh_j > 5 && (double)(1u << (15 - sh_j)) < bins) --sh_j;
                 o_cb = c_bot; o_ct = c_top; o_cs = sh_j;
+                o_nd = (float)bins;
             }
         }
-        if (lane == 0) { s_cb[j] = o_cb; s_ct[j] = o_ct; s_cs[j] = o_cs; }
+        if (lane == 0) { s_cb[j] = o_cb; s_ct[j] = o_ct; s_cs[j] = o_cs; s_nd[j] = o_nd; }
     }
     __syncthreads();
     // merge overlapping / adjacent bands (they descend in key with j) into groups; groups end up in s_c*[0..ng)
@@ -301,33 +306,56 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
         const uint32_t cmask = (1u << cg) - 1u;
         uint32_t ng = 0;
         uint32_t gb = 1, gt = 0, gs = 15;
+        float gn = 0.f;
         bool open = false;
         for (uint32_t j = 0; j < K; ++j) {
             uint32_t cb = s_cb[j], ct = s_ct[j];
             const uint32_t cs = s_cs[j];
+            const float cn = s_nd[j];
             if (cb > ct) continue;
             cb &= ~cmask; ct |= cmask; // stays below the non-finite cells: 65279 ends a block of 32
             if (open && ct + 1 >= gb) {
-                gb = min(gb, cb); gt = max(gt, ct); gs = min(gs, cs);
+                gb = min(gb, cb); gt = max(gt, ct); gs = min(gs, cs); gn = fmaxf(gn, cn);
             } else {
-                if (open) { s_cb[ng] = gb; s_ct[ng] = gt; s_cs[ng] = gs; ++ng; } // ng <= j: slots already consumed
-                gb = cb; gt = ct; gs = cs; open = true;
+                if (open) { s_cb[ng] = gb; s_ct[ng] = gt; s_cs[ng] = gs; s_nd[ng] = gn; ++ng; } // ng <= j: slots already consumed
+                gb = cb; gt = ct; gs = cs; gn = cn; open = true;
             }
         }
-        if (open) { s_cb[ng] = gb; s_ct[ng] = gt; s_cs[ng] = gs; ++ng; }
-        // if the fine bins do not fit, scale every group's bins per cell down by the same factor (rounded
-        // down to a power of two, at least one bin per cell)
+        if (open) { s_cb[ng] = gb; s_ct[ng] = gt; s_cs[ng] = gs; s_nd[ng] = gn; ++ng; }
         uint64_t fine = 0, cells = 0;
         for (uint32_t g = 0; g < ng; ++g) {
             fine += (uint64_t)(s_ct[g] - s_cb[g] + 1) << (15 - s_cs[g]);
             cells += s_ct[g] - s_cb[g] + 1;
         }
-        if (cells > (uint64_t)kFineBins) {
-            s_flag = 3;
-        } else if (fine > (uint64_t)kFineBins) {
-            uint32_t extra = 1;
-            while ((fine >> extra) > (uint64_t)kFineBins - cells) ++extra; // groups clamped at shift 15 keep 1 bin per cell
-            for (uint32_t g = 0; g < ng; ++g) s_cs[g] = min(15u, s_cs[g] + extra);
+        if (cells > (uint64_t)kFineBins) s_flag = 3;
+        // If the fine bins do not fit, groups are coarsened one step at a time, always the one that stays closest to what its
+        // candidates need (bins per cell are powers of two, so many have more than they need); every group keeps at least
+        // one bin per cell.
+        while (!s_flag && fine > (uint64_t)kFineBins) {
+            uint32_t at = 0;
+            float best = 3.4e38f;
+            for (uint32_t g = 0; g < ng; ++g) {
+                const float after = s_nd[g] * (float)(1u << s_cs[g]); // need over bins per cell, up to a common factor
+                if (s_cs[g] < 15u && after < best) { best = after; at = g; }
+            }
+            fine -= (uint64_t)(s_ct[at] - s_cb[at] + 1) << (14 - s_cs[at]);
+            s_cs[at] += 1;
+        }
+        // Where the rank window of the highest band reached beyond the largest sample, up to four more octaves above the band
+        // get one bin per cell, as far as bins and table entries are left.  A sample without an entry as large as the smallest
+        // candidate's threshold is not rare where large entries lie together (a few rows of a gradient, seven samples
+        // expected), and the exact path costs far more than these bins (1.1 B Llama shape, gradients moved across
+        // the tensors' borders: 4.5 layers of 402 per step on the exact path without them, 1 with one octave).
+        if (s_clip && ng && !s_flag) {
+            const uint32_t left = (uint32_t)((uint64_t)kFineBins - fine);
+            const uint32_t window = (s_ct[0] >> cg) - (s_cb[ng - 1] >> cg) + 3u;
+            uint32_t ext = min(min(1024u, left), window < (uint32_t)kCellTab ? ((uint32_t)kCellTab - window) << cg : 0u) & ~cmask;
+            ext = min(ext, 65279u - s_ct[0]);
+            if (ext) {
+                for (uint32_t g = ng; g; --g) { s_cb[g] = s_cb[g - 1]; s_ct[g] = s_ct[g - 1]; s_cs[g] = s_cs[g - 1]; }
+                s_cb[0] = s_ct[1] + 1u; s_ct[0] = s_ct[1] + ext; s_cs[0] = 15;
+                ++ng;
+            }
         }
         s_ng = ng;
     }
@@ -614,8 +642,7 @@ k_resolve_a(const LayerDesc* __restrict__ layers, const uint32_t* __restrict__ r
             const uint32_t* __restrict__ bin_lo, uint32_t* __restrict__ bh_cnt, unsigned long long* __restrict__ bh_sum,
             float* __restrict__ err_out, uint32_t* __restrict__ tau_out, uint32_t* __restrict__ rank_out,
             uint32_t* __restrict__ shift_out, uint32_t* __restrict__ flags, FbList* __restrict__ fb,
-            uint2* __restrict__ fb_chunks, uint2* __restrict__ fb_layers, RefineCand* __restrict__ rf,
-            uint2* __restrict__ rf_chunks, uint2* __restrict__ rf_layers, uint32_t list_cap, uint32_t w_base) {
+            uint2* __restrict__ fb_chunks, RefineCand* __restrict__ rf, uint2* __restrict__ rf_chunks, uint32_t list_cap, uint32_t w_base) {
     pdl_wait();
     __shared__ uint32_t s_drop[KIMAD_MAX_RATIOS]; // entries not kept by candidate j: n - k_j
     __shared__ int s_loose;
@@ -740,7 +767,7 @@ k_resolve_a(const LayerDesc* __restrict__ layers, const uint32_t* __restrict__ r
     if (bad) { // hand the layer and its chunks to the exact path
         if (threadIdx.x == 0) {
             s_at = atomicAdd(&fb->n_chunks, ld.n_chunks);
-            fb_layers[atomicAdd(&fb->n_layers, 1u)] = make_uint2(w, l);
+            atomicAdd(&fb->n_layers, 1u);
             atomicAdd(&fb->total_layers, 1u);
             atomicAdd(&fb->why[bad - 1], 1u);
         }
@@ -750,7 +777,7 @@ k_resolve_a(const LayerDesc* __restrict__ layers, const uint32_t* __restrict__ r
     } else if (s_loose) { // only loose bounds: refine those candidates
         if (threadIdx.x == 0) {
             s_at = atomicAdd(&fb->rf_chunks, ld.n_chunks);
-            rf_layers[atomicAdd(&fb->rf_layers, 1u)] = make_uint2(w, l);
+            atomicAdd(&fb->rf_layers, 1u);
             atomicAdd(&fb->refined, 1u);
         }
         __syncthreads();
@@ -765,10 +792,101 @@ k_resolve_a(const LayerDesc* __restrict__ layers, const uint32_t* __restrict__ r
 // summed per piece (the level-2/3 arrays of the exact path serve as storage: a layer is never on both paths at once).
 // Costs one pass over the layer's code bytes instead of the exact path's three passes over its inputs.
 // ------------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads, 6)
-k_refine_hist(DSource dbuf, const Chunk* __restrict__ chunks, uint64_t dstride, uint32_t L, uint32_t K,
-              const FbList* __restrict__ fb, const uint2* __restrict__ rf_chunks, const RefineCand* __restrict__ rf,
-              const CodeSpace codes, uint32_t* __restrict__ g_cnt, unsigned long long* __restrict__ g_ss) {
+// The pieces of a layer's loose bins resolved, by the CTA that counted the last of its chunks; the loose candidates one after
+// the other.  Candidates that share a bin were counted into the histogram of the first of them (the lowest j): the later
+// ones read it there.
+__device__ __forceinline__ void refine_resolve_layer(uint32_t l, uint32_t w, size_t wl, size_t wr, const LayerDesc* __restrict__ layers,
+                                                     uint32_t K, FbList* __restrict__ fb, RefineCand* __restrict__ rf,
+                                                     uint32_t* __restrict__ g_cnt, unsigned long long* __restrict__ g_ss,
+                                                     float* __restrict__ err_out, uint32_t* __restrict__ tau_out,
+                                                     uint32_t* __restrict__ rank_out, uint32_t* __restrict__ shift_out,
+                                                     const CodeSpace& codes, uint2* __restrict__ fb_chunks, uint32_t list_cap) {
+    __shared__ uint32_t s_w32[8];
+    __shared__ double s_w64[8];
+    __shared__ int s_bad;
+    __shared__ uint32_t s_at;
+            __syncthreads();
+            if (threadIdx.x == 0) s_bad = 0;
+            __syncthreads();
+            for (uint32_t j = 0; j < K; ++j) {
+                const RefineCand rc = rf[wl * K + j];
+                if (rc.shift == kNoRefine) continue;
+                uint32_t owner = j; // the first loose candidate with this bin holds the pieces
+                for (uint32_t i = 0; i < j; ++i) {
+                    const RefineCand o = rf[wl * K + i];
+                    if (o.shift != kNoRefine && o.klo == rc.klo) { owner = i; break; }
+                }
+                const uint32_t sub = rc.shift > 10u ? rc.shift - 10u : 0u, nsub = 1u << (rc.shift - sub);
+                const uint32_t* gc = g_cnt + (wr * K + owner) * kL23Bins;
+                const unsigned long long* gs = g_ss + (wr * K + owner) * kL23Bins;
+                const double scale = sq_scale(rc.klo >> 23);
+                // four consecutive pieces per thread, ascending keys
+                uint32_t c[4], csum = 0;
+                double q[4], qsum = 0.0;
+    #pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const uint32_t b = 4 * threadIdx.x + i;
+                    c[i] = b < nsub ? __ldcg(gc + b) : 0u;
+                    q[i] = b < nsub ? (double)__ldcg(gs + b) * scale : 0.0;
+                    csum += c[i];
+                    qsum += q[i];
+                }
+                uint32_t tot;
+                uint32_t before = block_excl_scan<uint32_t>(csum, s_w32, &tot);
+                double below = block_excl_scan<double>(qsum, s_w64, nullptr);
+                if (!KIMAD_CHECK(tot == rc.cb, 7)) s_bad = 1;
+                const size_t o = wl * K + j;
+    #pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if (c[i] && rc.drop >= before && rc.drop - before < c[i]) { // the piece that holds the threshold
+                        const uint32_t b = 4 * threadIdx.x + i, klo = rc.klo + (b << sub), d2 = rc.drop - before;
+                        const double vlo = (double)__uint_as_float(klo);
+                        const double upper = q[i] * ((double)d2 / (double)c[i]), lower = (double)d2 * vlo * vlo;
+                        double part = 0.5 * (upper + lower), slack = 0.5 * (upper - lower);
+                        if (d2 == 0 || sub == 0) { part = lower; slack = 0.0; }
+                        const double e = rc.below + below + part;
+                        if (slack > e * 5e-6) {
+                            s_bad = 1;
+                        } else {
+                            err_out[o] = (float)e; tau_out[o] = klo; rank_out[o] = c[i] - d2;
+                            shift_out[o] = sub | codes.code(w, l, klo) << 8;
+                        }
+                    }
+                    before += c[i];
+                    below += q[i];
+                }
+                __syncthreads();
+            }
+            // clean the pieces, close the candidates
+            for (uint32_t j = 0; j < K; ++j) {
+                if (rf[wl * K + j].shift == kNoRefine) continue;
+                for (uint32_t b = threadIdx.x; b < (uint32_t)kL23Bins; b += kThreads) {
+                    g_cnt[(wr * K + j) * kL23Bins + b] = 0;
+                    g_ss[(wr * K + j) * kL23Bins + b] = 0ull;
+                }
+            }
+            __syncthreads();
+            for (uint32_t j = threadIdx.x; j < K; j += kThreads) rf[wl * K + j].shift = kNoRefine;
+            if (s_bad) { // still too loose (a bin with very many entries): the exact path after all
+                const LayerDesc ld = layers[l];
+                if (threadIdx.x == 0) {
+                    s_at = atomicAdd(&fb->n_chunks, ld.n_chunks);
+                    atomicAdd(&fb->n_layers, 1u);
+                    atomicAdd(&fb->total_layers, 1u);
+                    atomicAdd(&fb->why[3], 1u);
+                }
+                __syncthreads();
+                for (uint32_t i = threadIdx.x; i < ld.n_chunks; i += kThreads)
+                    if (KIMAD_CHECK(s_at + i < list_cap, 2)) fb_chunks[s_at + i] = make_uint2(w, ld.first_chunk + i);
+            }
+}
+
+__global__ void __launch_bounds__(kThreads, 5)
+k_refine(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* __restrict__ chunks, uint64_t dstride, uint32_t L, uint32_t K,
+         FbList* __restrict__ fb, const uint2* __restrict__ rf_chunks, RefineCand* __restrict__ rf,
+         const CodeSpace codes, uint32_t* __restrict__ g_cnt, unsigned long long* __restrict__ g_ss, uint32_t* __restrict__ arrived,
+         float* __restrict__ err_out, uint32_t* __restrict__ tau_out, uint32_t* __restrict__ rank_out, uint32_t* __restrict__ shift_out,
+         uint2* __restrict__ fb_chunks, uint32_t list_cap) {
     pdl_wait();
     __shared__ uint32_t s_klo[KIMAD_MAX_RATIOS], s_shift[KIMAD_MAX_RATIOS], s_j[KIMAD_MAX_RATIOS];
     __shared__ uint32_t s_mask[4]; // the 7-bit codes of the loose candidates' bins
@@ -782,23 +900,35 @@ k_refine_hist(DSource dbuf, const Chunk* __restrict__ chunks, uint64_t dstride, 
         if (threadIdx.x < 4) s_mask[threadIdx.x] = 0;
         if (threadIdx.x == 0) s_n = 0;
         __syncthreads();
-        if (threadIdx.x == 0) { // the layer's loose candidates in order of j, every bin once (under its lowest j)
-            uint32_t p = 0;
-            for (uint32_t j = 0; j < K; ++j) {
-                const RefineCand rc = rf[wl * K + j];
-                if (rc.shift == kNoRefine || (p && s_klo[p - 1] == rc.klo)) continue; // thresholds descend with j
-                s_klo[p] = rc.klo; s_shift[p] = rc.shift; s_j[p] = j;
-                ++p;
-                const uint32_t code = codes.code(e.x, ch.layer, rc.klo) & 127u;
-                s_mask[code >> 5] |= 1u << (code & 31u);
+        if (threadIdx.x < 32) { // the layer's loose candidates in order of j, every bin once (under its lowest j); a lane each
+            const uint32_t lane = threadIdx.x;
+            uint32_t p = 0, last = 0; // bins so far, the last one's lower key
+            for (uint32_t j0 = 0; j0 < K; j0 += 32u) {
+                const uint32_t j = j0 + lane;
+                RefineCand r{0, kNoRefine, 0, 0, 0.0};
+                if (j < K) r = rf[wl * K + j];
+                const bool loose = r.shift != kNoRefine;
+                const uint32_t m = __ballot_sync(0xffffffffu, loose), before = m & ((1u << lane) - 1u);
+                const uint32_t left = __shfl_sync(0xffffffffu, r.klo, before ? 31 - __clz(before) : 0);
+                const bool first = loose && (before ? left != r.klo : (p == 0 || last != r.klo)); // thresholds descend with j
+                const uint32_t f = __ballot_sync(0xffffffffu, first);
+                if (first) {
+                    const uint32_t at = p + __popc(f & ((1u << lane) - 1u));
+                    s_klo[at] = r.klo; s_shift[at] = r.shift; s_j[at] = j;
+                    const uint32_t code = codes.code(e.x, ch.layer, r.klo) & 127u;
+                    atomicOr(&s_mask[code >> 5], 1u << (code & 31u));
+                }
+                if (m) last = __shfl_sync(0xffffffffu, r.klo, 31 - __clz(m));
+                p += __popc(f);
             }
-            s_n = p;
+            if (lane == 0) s_n = p;
         }
         __syncthreads();
         const uint32_t nc = s_n;
         const uint32_t m0 = s_mask[0], m1 = s_mask[1], m2 = s_mask[2], m3 = s_mask[3];
         const ChunkView cv(ch);
         const DView dd(dbuf, e.x, dstride, cv.a0);
+        const bool vec = ((reinterpret_cast<uintptr_t>(dd.gr) | reinterpret_cast<uintptr_t>(dd.st)) & 15u) == 0;
         auto wanted = [&](uint32_t code) -> bool {
             const uint32_t word = code < 64u ? (code < 32u ? m0 : m1) : (code < 96u ? m2 : m3);
             return (word >> (code & 31u)) & 1u;
@@ -810,7 +940,7 @@ k_refine_hist(DSource dbuf, const Chunk* __restrict__ chunks, uint64_t dstride, 
                     const size_t at = (wr * K + s_j[p]) * kL23Bins + (d1 >> (sh > 10u ? sh - 10u : 0u));
                     atomicAdd(&g_cnt[at], 1u);
                     atomicAdd(&g_ss[at], (unsigned long long)sq_fixed(key));
-                    break; // bins are disjoint; candidates that share a bin share a piece histogram (see k_refine_resolve)
+                    break; // bins are disjoint; candidates that share a bin share a piece histogram (see refine_resolve_layer)
                 }
             }
         };
@@ -830,115 +960,28 @@ k_refine_hist(DSource dbuf, const Chunk* __restrict__ chunks, uint64_t dstride, 
                 for (uint32_t x = max(e0, cv.first); x < min(e0 + 16u, cv.len); ++x)
                     if (wanted(dd.code[x] & 127u)) hit |= 1u << (x - e0);
             }
-            while (hit) { // completed from the inputs four at a time: their loads are independent
-                uint32_t pos[4];
-                float v[4];
+            if (!hit) continue;
+            // the unit's entries are completed from the inputs with independent loads: eight at a time
+            if (vec && e0 >= cv.first && e0 + 16u <= cv.len) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    pos[i] = hit ? (uint32_t)__ffs(hit) - 1u : 0xffffffffu;
-                    if (hit) hit &= hit - 1u;
+                for (int h = 0; h < 2; ++h) {
+                    if (!((hit >> (8 * h)) & 255u)) continue;
+                    const float4* g4 = reinterpret_cast<const float4*>(dd.gr + e0 + 8 * h);
+                    const float4* t4 = reinterpret_cast<const float4*>(dd.st + e0 + 8 * h);
+                    const float4 ga = __ldg(g4), gb = __ldg(g4 + 1), ta = __ldg(t4), tb = __ldg(t4 + 1);
+                    const float v[8] = {__fsub_rn(ga.x, ta.x), __fsub_rn(ga.y, ta.y), __fsub_rn(ga.z, ta.z), __fsub_rn(ga.w, ta.w),
+                                        __fsub_rn(gb.x, tb.x), __fsub_rn(gb.y, tb.y), __fsub_rn(gb.z, tb.z), __fsub_rn(gb.w, tb.w)};
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+                        if ((hit >> (8 * h + i)) & 1u) place(key_of(v[i]));
                 }
-#pragma unroll
-                for (int i = 0; i < 4; ++i) v[i] = pos[i] != 0xffffffffu ? dd.at(e0 + pos[i]) : 0.f;
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if (pos[i] != 0xffffffffu) place(key_of(v[i]));
+            } else {
+                for (; hit; hit &= hit - 1u) place(key_of(dd.at(e0 + (uint32_t)__ffs(hit) - 1u)));
             }
         }
-    }
-}
-
-// One CTA per refined layer and pass of the loop; its loose candidates one after the other.  Candidates that share a
-// bin were counted into the histogram of the first of them (the lowest j): the later ones read it there.
-__global__ void __launch_bounds__(kThreads)
-k_refine_resolve(const LayerDesc* __restrict__ layers, uint32_t L, uint32_t K, FbList* __restrict__ fb,
-                 const uint2* __restrict__ rf_layers, RefineCand* __restrict__ rf, uint32_t* __restrict__ g_cnt,
-                 unsigned long long* __restrict__ g_ss, float* __restrict__ err_out, uint32_t* __restrict__ tau_out,
-                 uint32_t* __restrict__ rank_out, uint32_t* __restrict__ shift_out, const CodeSpace codes, uint2* __restrict__ fb_chunks,
-                 uint2* __restrict__ fb_layers, uint32_t list_cap) {
-    pdl_wait();
-    __shared__ uint32_t s_w32[8];
-    __shared__ double s_w64[8];
-    __shared__ int s_bad;
-    __shared__ uint32_t s_at;
-    const uint32_t n = fb->rf_layers;
-    for (uint32_t it = blockIdx.x; it < n; it += gridDim.x) {
-        const uint32_t w = rf_layers[it].x, l = rf_layers[it].y;
-        const size_t wl = (size_t)w * L + l, wr = codes.slot(w, l);
-        __syncthreads();
-        if (threadIdx.x == 0) s_bad = 0;
-        __syncthreads();
-        for (uint32_t j = 0; j < K; ++j) {
-            const RefineCand rc = rf[wl * K + j];
-            if (rc.shift == kNoRefine) continue;
-            uint32_t owner = j; // the first loose candidate with this bin holds the pieces
-            for (uint32_t i = 0; i < j; ++i) {
-                const RefineCand o = rf[wl * K + i];
-                if (o.shift != kNoRefine && o.klo == rc.klo) { owner = i; break; }
-            }
-            const uint32_t sub = rc.shift > 10u ? rc.shift - 10u : 0u, nsub = 1u << (rc.shift - sub);
-            const uint32_t* gc = g_cnt + (wr * K + owner) * kL23Bins;
-            const unsigned long long* gs = g_ss + (wr * K + owner) * kL23Bins;
-            const double scale = sq_scale(rc.klo >> 23);
-            // four consecutive pieces per thread, ascending keys
-            uint32_t c[4], csum = 0;
-            double q[4], qsum = 0.0;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const uint32_t b = 4 * threadIdx.x + i;
-                c[i] = b < nsub ? gc[b] : 0u;
-                q[i] = b < nsub ? (double)gs[b] * scale : 0.0;
-                csum += c[i];
-                qsum += q[i];
-            }
-            uint32_t tot;
-            uint32_t before = block_excl_scan<uint32_t>(csum, s_w32, &tot);
-            double below = block_excl_scan<double>(qsum, s_w64, nullptr);
-            if (!KIMAD_CHECK(tot == rc.cb, 7)) s_bad = 1;
-            const size_t o = wl * K + j;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                if (c[i] && rc.drop >= before && rc.drop - before < c[i]) { // the piece that holds the threshold
-                    const uint32_t b = 4 * threadIdx.x + i, klo = rc.klo + (b << sub), d2 = rc.drop - before;
-                    const double vlo = (double)__uint_as_float(klo);
-                    const double upper = q[i] * ((double)d2 / (double)c[i]), lower = (double)d2 * vlo * vlo;
-                    double part = 0.5 * (upper + lower), slack = 0.5 * (upper - lower);
-                    if (d2 == 0 || sub == 0) { part = lower; slack = 0.0; }
-                    const double e = rc.below + below + part;
-                    if (slack > e * 5e-6) {
-                        s_bad = 1;
-                    } else {
-                        err_out[o] = (float)e; tau_out[o] = klo; rank_out[o] = c[i] - d2;
-                        shift_out[o] = sub | codes.code(w, l, klo) << 8;
-                    }
-                }
-                before += c[i];
-                below += q[i];
-            }
-            __syncthreads();
-        }
-        // clean the pieces, close the candidates
-        for (uint32_t j = 0; j < K; ++j) {
-            if (rf[wl * K + j].shift == kNoRefine) continue;
-            for (uint32_t b = threadIdx.x; b < (uint32_t)kL23Bins; b += kThreads) {
-                g_cnt[(wr * K + j) * kL23Bins + b] = 0;
-                g_ss[(wr * K + j) * kL23Bins + b] = 0ull;
-            }
-        }
-        __syncthreads();
-        for (uint32_t j = threadIdx.x; j < K; j += kThreads) rf[wl * K + j].shift = kNoRefine;
-        if (s_bad) { // still too loose (a bin with very many entries): the exact path after all
-            const LayerDesc ld = layers[l];
-            if (threadIdx.x == 0) {
-                s_at = atomicAdd(&fb->n_chunks, ld.n_chunks);
-                fb_layers[atomicAdd(&fb->n_layers, 1u)] = make_uint2(w, l);
-                atomicAdd(&fb->total_layers, 1u);
-                atomicAdd(&fb->why[3], 1u);
-            }
-            __syncthreads();
-            for (uint32_t i = threadIdx.x; i < ld.n_chunks; i += kThreads)
-                if (KIMAD_CHECK(s_at + i < list_cap, 2)) fb_chunks[s_at + i] = make_uint2(w, ld.first_chunk + i);
-        }
+        if (last_of_layer(arrived + wl, layers[ch.layer].n_chunks))
+            refine_resolve_layer(ch.layer, e.x, wl, wr, layers, K, fb, rf, g_cnt, g_ss, err_out, tau_out, rank_out, shift_out, codes,
+                                 fb_chunks, list_cap);
     }
 }
 
@@ -1112,11 +1155,16 @@ k_tiny_exact(const float* __restrict__ grads, const float* __restrict__ state, u
 constexpr int kFbAhead = 4; // elements per thread whose loads are issued together
 
 __global__ void __launch_bounds__(kThreads)
-k_fb_hist1(DSource dbuf, const Chunk* __restrict__ chunks, uint64_t dstride,
-           const FbList* __restrict__ fb, const uint2* __restrict__ fb_chunks, uint32_t* __restrict__ g_cnt,
-           unsigned long long* __restrict__ g_ss, uint32_t* __restrict__ flags, const CodeSpace codes) {
+k_fb1(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* __restrict__ chunks, uint64_t dstride, uint32_t L, uint32_t K,
+      const KTab ktab, const FbList* __restrict__ fb, const uint2* __restrict__ fb_chunks, uint32_t* __restrict__ g_cnt,
+      unsigned long long* __restrict__ g_ss, uint32_t* __restrict__ flags, const CodeSpace codes, uint32_t* __restrict__ arrived,
+      Cand* __restrict__ cands, SlotTab* __restrict__ slots) {
     pdl_wait();
-    __shared__ uint32_t s_cnt[kL1Bins], s_hi[kL1Bins], s_lo[kL1Bins];
+    __shared__ __align__(16) uint32_t s_cnt[kL1Bins];
+    __shared__ __align__(16) double s_below[kL1Bins]; // the two words of the chunk's sums, then the layer's squares
+    __shared__ uint32_t s_w32[8];
+    __shared__ double s_w64[8];
+    uint32_t *s_hi = reinterpret_cast<uint32_t*>(s_below), *s_lo = s_hi + kL1Bins;
     const uint32_t n = fb->n_chunks;
     for (uint32_t it = blockIdx.x; it < n; it += gridDim.x) {
         const uint2 e = fb_chunks[it];
@@ -1156,15 +1204,18 @@ k_fb_hist1(DSource dbuf, const Chunk* __restrict__ chunks, uint64_t dstride,
                 atomicAdd(&gc[b], s_cnt[b]);
                 atomicAdd(&gs[b], ((unsigned long long)s_hi[b] << 16) + s_lo[b]);
             }
-        __syncthreads();
+        const size_t wl = (size_t)e.x * L + ch.layer;
+        if (last_of_layer(arrived + wl, layers[ch.layer].n_chunks))
+            fb_resolve1_layer(ch.layer, e.x, wl, wr, K, g_cnt, g_ss, ktab, cands, slots, s_cnt, s_below, s_w32, s_w64);
     }
 }
 
 template <int LEVEL>
 __global__ void __launch_bounds__(kThreads)
-k_fb_hist23(DSource dbuf, const Chunk* __restrict__ chunks, uint64_t dstride, uint32_t L, uint32_t K,
-            const FbList* __restrict__ fb, const uint2* __restrict__ fb_chunks, const SlotTab* __restrict__ slots,
-            uint32_t* __restrict__ g_cnt, unsigned long long* __restrict__ g_ss, const CodeSpace codes) {
+k_fb23(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* __restrict__ chunks, uint64_t dstride, uint32_t L, uint32_t K,
+       const FbList* __restrict__ fb, const uint2* __restrict__ fb_chunks, SlotTab* __restrict__ slots, Cand* __restrict__ cands,
+       uint32_t* __restrict__ g_cnt, unsigned long long* __restrict__ g_ss, const CodeSpace codes, uint32_t* __restrict__ arrived,
+       float* __restrict__ err_out, uint32_t* __restrict__ tau_out, uint32_t* __restrict__ keep_eq_out, uint32_t* __restrict__ shift_out) {
     pdl_wait();
     __shared__ uint8_t s_first[kL1Bins]; // level-1 bin -> first slot whose prefix starts with it (0xff: none)
     __shared__ uint8_t s_num[kL1Bins];   // ... and how many consecutive slots share that bin (level 3)
@@ -1224,7 +1275,8 @@ k_fb_hist23(DSource dbuf, const Chunk* __restrict__ chunks, uint64_t dstride, ui
             }
         }
         flush();
-        __syncthreads();
+        if (last_of_layer(arrived + wl, layers[ch.layer].n_chunks))
+            fb_resolve23_layer<LEVEL>(ch.layer, e.x, wl, wr, K, g_cnt, g_ss, cands, slots, err_out, tau_out, keep_eq_out, shift_out, codes);
     }
 }
 

@@ -10,9 +10,9 @@
 //   k_resolve_a     (b) Eq. 4 / the "Errors" matrix of Algorithm 3: err_l(k_j) from the bins, certified to the
 //                   curve tolerance; layers that fail the certificate are handed to the exact path [kimad_curve.cuh]
 //   k_tiny_exact    (b) layers of at most 4096 elements, sorted in shared memory                 [kimad_curve.cuh]
-//   k_refine_hist, k_refine_resolve
+//   k_refine
 //                   (b) candidates whose certified bound is too loose: one more look at their bin (usually none)
-//   k_fb_hist1, k_fb_hist23<2|3>, k_resolve1, k_resolve23<2|3>, k_rebuild_slots
+//   k_fb1, k_fb23<2|3>
 //                   (b) exact 11+10+10-bit radix select over the handed-over layers (usually none)
 //                                                                          [kimad_curve.cuh, this file]
 //   k_dp            (c) Algorithm 3 on the budget axis (Eq. 2, Eq. 3, Section 3.2), one CTA per worker [kimad_dp.cuh]
@@ -200,7 +200,7 @@ struct FbList { // layers handed to the exact radix path in this step, and their
                            // outside its band, 3: error bound too loose
     uint32_t loose_j[KIMAD_MAX_RATIOS + 1]; // never reset: which candidate's bound was too loose
     // layers whose only defect is a loose bound are refined instead: one more look at the entries of the bins that
-    // hold the loose candidates' thresholds (k_refine_hist, k_refine_resolve)
+    // hold the loose candidates' thresholds (k_refine)
     uint32_t rf_chunks;
     uint32_t rf_layers;
     uint32_t refined; // never reset: layers that took the refinement
@@ -248,35 +248,36 @@ struct CodeSpace { // how the sweep coded the elements of one (worker, layer)
     }
 };
 
-__global__ void __launch_bounds__(kThreads)
-k_resolve1(const FbList* __restrict__ fb, const uint2* __restrict__ fb_layers, uint32_t* __restrict__ g_cnt,
-           unsigned long long* __restrict__ g_ss, const KTab ktab, uint32_t L, uint32_t K,
-           Cand* __restrict__ cands, SlotTab* __restrict__ slots, const CodeSpace codes) {
-    pdl_wait();
-    __shared__ __align__(16) uint32_t s_incl[kL1Bins];
-    __shared__ __align__(16) double s_below[kL1Bins];
-    __shared__ uint32_t s_w32[8];
-    __shared__ double s_w64[8];
-  for (uint32_t it = blockIdx.x; it < fb->n_layers; it += gridDim.x) {
-    const uint32_t l = fb_layers[it].y, w = fb_layers[it].x;
-    const size_t wl = (size_t)w * L + l;
-    const size_t wr = codes.slot(w, l);
+// Work over chunks of listed layers ends, per layer, with a step that needs all of them: the CTA that finishes the layer's
+// last chunk takes that step.  True (for the whole CTA) in that CTA, which then sees what the others wrote; the counter is
+// back at zero.  Every thread of the CTA calls it after its last write for the chunk.
+__device__ __forceinline__ bool last_of_layer(uint32_t* counter, uint32_t n_chunks) {
+    __shared__ uint32_t s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        s_last = atomicAdd(counter, 1u) + 1u == n_chunks;
+        if (s_last) *counter = 0;
+    }
+    __syncthreads();
+    const bool last = s_last != 0;
+    if (last) __threadfence();
+    return last;
+}
+
+// Level 1 of the exact radix select of one (worker, layer): candidates -> level-1 bins.  By a whole CTA; s_incl and s_below are
+// [kL1Bins].  Leaves the histogram clean.
+__device__ __forceinline__ void fb_resolve1_layer(uint32_t l, uint32_t w, size_t wl, size_t wr, uint32_t K, uint32_t* __restrict__ g_cnt,
+                                                  unsigned long long* __restrict__ g_ss, const KTab& ktab, Cand* __restrict__ cands,
+                                                  SlotTab* __restrict__ slots, uint32_t* s_incl, double* s_below, uint32_t* s_w32,
+                                                  double* s_w64) {
     uint32_t* gc = g_cnt + wr * kL1Bins;
     unsigned long long* gs = g_ss + wr * kL1Bins;
-    {
-        constexpr int PER = kL1Bins / kThreads;
-        uint32_t c[PER];
-        unsigned long long g[PER];
-#pragma unroll
-        for (int i = 0; i < PER; ++i) { c[i] = gc[threadIdx.x + i * kThreads]; g[i] = gs[threadIdx.x + i * kThreads]; }
-#pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            const int b = threadIdx.x + i * kThreads;
-            s_incl[kL1Bins - 1 - b] = c[i];
-            s_below[b] = (double)g[i] * sq_scale((uint32_t)b >> 3);
-            gc[b] = 0; // leave the histogram clean for the next step
-            gs[b] = 0ull;
-        }
+    for (int b = threadIdx.x; b < kL1Bins; b += kThreads) {
+        s_incl[kL1Bins - 1 - b] = __ldcg(gc + b);
+        s_below[b] = (double)__ldcg(gs + b) * sq_scale((uint32_t)b >> 3);
+        gc[b] = 0;
+        gs[b] = 0ull;
     }
     __syncthreads();
     scan_bins<kL1Bins>(s_incl, s_below, s_w32, s_w64);
@@ -304,102 +305,87 @@ k_resolve1(const FbList* __restrict__ fb, const uint2* __restrict__ fb_layers, u
         stab.n = ns;
     }
     __syncthreads();
-  }
 }
 
-// LEVEL 2: refine inside a level-1 bin; LEVEL 3: inside a (level-1, level-2) bin.
-// One CTA per (layer, worker, slot).
+// LEVEL 2: refine inside a level-1 bin; LEVEL 3: inside a (level-1, level-2) bin.  By a whole CTA, a warp per slot: a lane takes
+// 32 consecutive bins.  Leaves the histograms clean.
 template <int LEVEL>
-__global__ void __launch_bounds__(kThreads)
-k_resolve23(const FbList* __restrict__ fb, const uint2* __restrict__ fb_layers, uint32_t* __restrict__ g_cnt,
-            unsigned long long* __restrict__ g_ss, uint32_t L, uint32_t K, Cand* __restrict__ cands,
-            const SlotTab* __restrict__ slots, float* __restrict__ err_out, uint32_t* __restrict__ tau_out,
-            uint32_t* __restrict__ keep_eq_out, uint32_t* __restrict__ shift_out, const CodeSpace codes) {
-    pdl_wait();
-    __shared__ __align__(16) uint32_t s_incl[kL23Bins];
-    __shared__ __align__(16) double s_below[kL23Bins];
-    __shared__ uint32_t s_w32[8];
-    __shared__ double s_w64[8];
-  for (uint32_t it = blockIdx.x; it < fb->n_layers; it += gridDim.x) {
-    const uint32_t l = fb_layers[it].y, w = fb_layers[it].x, s = blockIdx.z;
-    const size_t wl = (size_t)w * L + l;
-    const SlotTab& stab = slots[wl];
-    if (s >= stab.n) continue;
-    Cand* cd = cands + wl * K;
-    const size_t wr = codes.slot(w, l);
-    uint32_t* gc = g_cnt + (wr * K + s) * kL23Bins;
-    unsigned long long* gs = g_ss + (wr * K + s) * kL23Bins;
-    const uint32_t prefix = stab.prefix[s];
-    {
-        constexpr int PER = kL23Bins / kThreads;
-        uint32_t cc[PER];
-        unsigned long long g[PER];
-#pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            cc[i] = gc[threadIdx.x + i * kThreads];
-            g[i] = LEVEL == 2 ? gs[threadIdx.x + i * kThreads] : 0ull;
-        }
-        const double scale = sq_scale(prefix >> 3); // LEVEL 2: prefix = level-1 bin (8 exponent + 3 mantissa bits)
-#pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            const int b = threadIdx.x + i * kThreads;
-            s_incl[kL23Bins - 1 - b] = cc[i];
-            gc[b] = 0;
-            if (LEVEL == 2) {
-                s_below[b] = (double)g[i] * scale;
-                gs[b] = 0ull;
-            } else { // all 31 bits known: the bin's sum of squares is count * value^2
-                const double v = (double)__uint_as_float((prefix << 10) | (uint32_t)b);
-                s_below[b] = (double)cc[i] * v * v;
-            }
-        }
-    }
-    __syncthreads();
-    scan_bins<kL23Bins>(s_incl, s_below, s_w32, s_w64);
-    for (uint32_t j = threadIdx.x; j < K; j += kThreads) {
-        Cand c = cd[j];
-        if (c.slot != s) continue;
-        const int p = find_pos<kL23Bins>(s_incl, c.rank);
-        const uint32_t above = p ? s_incl[p - 1] : 0u;
-        const uint32_t bin = (uint32_t)(kL23Bins - 1 - p);
-        c.prefix = (prefix << 10) | bin;
-        c.gt += above;
-        c.err_low += s_below[bin];
-        if (LEVEL == 2) {
-            c.rank -= above;
-            cd[j] = c;
-        } else {
-            const uint32_t eq = s_incl[p] - above;
-            const uint32_t keep = c.rank - above; // 1 <= keep <= eq
-            const double v = (double)__uint_as_float(c.prefix);
-            const double e = c.err_low + (double)(eq - keep) * v * v;
-            err_out[wl * K + j] = (float)e;
-            tau_out[wl * K + j] = c.prefix;
-            keep_eq_out[wl * K + j] = keep;
-            shift_out[wl * K + j] = codes.code(w, l, c.prefix) << 8;
-        }
-    }
-    __syncthreads();
-  }
-}
-
-// After digit 2: new slots = distinct 21-bit prefixes (non-increasing in j).  One thread per (worker, layer).
-__global__ void __launch_bounds__(kThreads)
-k_rebuild_slots(const FbList* __restrict__ fb, const uint2* __restrict__ fb_layers, uint32_t L, uint32_t K,
-                Cand* __restrict__ cands, SlotTab* __restrict__ slots) {
-    pdl_wait();
-    const uint32_t it = blockIdx.x * kThreads + threadIdx.x;
-    if (it >= fb->n_layers) return;
-    const size_t wl = (size_t)fb_layers[it].x * L + fb_layers[it].y;
-    Cand* cd = cands + (size_t)wl * K;
+__device__ __forceinline__ void fb_resolve23_layer(uint32_t l, uint32_t w, size_t wl, size_t wr, uint32_t K, uint32_t* __restrict__ g_cnt,
+                                                   unsigned long long* __restrict__ g_ss, Cand* __restrict__ cands,
+                                                   SlotTab* __restrict__ slots, float* __restrict__ err_out, uint32_t* __restrict__ tau_out,
+                                                   uint32_t* __restrict__ keep_eq_out, uint32_t* __restrict__ shift_out,
+                                                   const CodeSpace& codes) {
+    const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     SlotTab& stab = slots[wl];
-    uint32_t n2 = 0;
-    for (uint32_t j = 0; j < K; ++j) {
-        const uint32_t pfx = cd[j].prefix;
-        if (n2 == 0 || stab.prefix[n2 - 1] != pfx) stab.prefix[n2++] = pfx;
-        cd[j].slot = n2 - 1;
+    Cand* cd = cands + wl * K;
+    const uint32_t ns = stab.n;
+    for (uint32_t s = wid; s < ns; s += kThreads / 32) {
+        uint32_t* gc = g_cnt + (wr * K + s) * kL23Bins;
+        unsigned long long* gs = g_ss + (wr * K + s) * kL23Bins;
+        const uint32_t prefix = stab.prefix[s], b0 = 32u * lane;
+        const double scale = LEVEL == 2 ? sq_scale(prefix >> 3) : 0.0; // LEVEL 2: prefix = level-1 bin (8 exponent + 3 mantissa bits)
+        auto count = [&](uint32_t b) { return __ldcg(gc + b); };
+        auto squares = [&](uint32_t b, uint32_t c) { // LEVEL 3: all 31 bits known, the sum of squares is count * value^2
+            if (LEVEL == 2) return (double)__ldcg(gs + b) * scale;
+            const double v = (double)__uint_as_float((prefix << 10) | b);
+            return (double)c * v * v;
+        };
+        uint32_t cnt = 0;
+        double sq = 0.0;
+        for (uint32_t b = b0; b < b0 + 32u; ++b) { const uint32_t c = count(b); cnt += c; sq += squares(b, c); }
+        uint32_t upto = cnt; // entries in the lane's bins and those of the lanes above
+        double below = sq;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t yc = __shfl_down_sync(0xffffffffu, upto, o);
+            const double ys = __shfl_up_sync(0xffffffffu, below, o);
+            if (lane + o < 32u) upto += yc;
+            if (lane >= (uint32_t)o) below += ys;
+        }
+        const uint32_t above = upto - cnt;
+        below = __shfl_up_sync(0xffffffffu, below, 1); // exclusive value from the left neighbour: no cancellation
+        if (lane == 0) below = 0.0;
+        for (uint32_t j = 0; j < K; ++j) {
+            if (cd[j].slot != s) continue;
+            const uint32_t rank = cd[j].rank;
+            __syncwarp(); // read by all lanes before one of them writes it
+            if (above < rank && rank <= upto) { // one lane
+                uint32_t b = b0 + 31u, gt = above, c = count(b);
+                while (gt + c < rank) { gt += c; --b; c = count(b); }
+                double e = below;
+                for (uint32_t x = b0; x < b; ++x) e += squares(x, count(x));
+                e += cd[j].err_low;
+                const uint32_t found = (prefix << 10) | b;
+                if (LEVEL == 2) {
+                    cd[j].prefix = found;
+                    cd[j].gt += gt;
+                    cd[j].err_low = e;
+                    cd[j].rank = rank - gt;
+                } else {
+                    const uint32_t keep = rank - gt; // 1 <= keep <= c
+                    const double v = (double)__uint_as_float(found);
+                    err_out[wl * K + j] = (float)(e + (double)(c - keep) * v * v);
+                    tau_out[wl * K + j] = found;
+                    keep_eq_out[wl * K + j] = keep;
+                    shift_out[wl * K + j] = codes.code(w, l, found) << 8;
+                }
+            }
+            __syncwarp();
+        }
+        __syncwarp();
+        for (uint32_t b = lane; b < (uint32_t)kL23Bins; b += 32u) { gc[b] = 0; if (LEVEL == 2) gs[b] = 0ull; }
     }
-    stab.n = n2;
+    __syncthreads();
+    if (LEVEL == 2 && threadIdx.x == 0) { // new slots = distinct 21-bit prefixes (non-increasing in j)
+        uint32_t n2 = 0;
+        for (uint32_t j = 0; j < K; ++j) {
+            const uint32_t pfx = cd[j].prefix;
+            if (n2 == 0 || stab.prefix[n2 - 1] != pfx) stab.prefix[n2++] = pfx;
+            cd[j].slot = n2 - 1;
+        }
+        stab.n = n2;
+    }
+    __syncthreads();
 }
 
 } // namespace kimad
