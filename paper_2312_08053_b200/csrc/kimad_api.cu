@@ -375,14 +375,17 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
                             ktab, K, c->curve_mode == 1 ? 1u : 0u, cell_tab, cell_win, binlo, meta));
         c->launches += 1;
     }
-    if (T) { // tiny layers: sorted in shared memory on the side stream, beside the sample kernel (its CTAs fill what
-             // that kernel leaves idle); joined before the sweep, whose CTAs take most of an SM's shared memory and
-             // could not start on an SM that still holds CTAs of another kernel
+    // Tiny layers: sorted in shared memory on the side stream, beside the sample kernel (its CTAs fill what that kernel leaves
+    // idle).  On large steps joined before the sweep, whose CTAs take most of an SM's shared memory and could not start on an
+    // SM that still holds CTAs of another kernel (0.2 ms on 4 x 124 M elements); on small ones, whose sweep leaves SMs idle
+    // anyway, before the DP, so that the chain from the sample kernel to the curves does not wait for it.
+    const bool join_late = (uint64_t)W * c->N < kPipelineMinElems;
+    if (T) {
         CUDA_TRY(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
         CUDA_TRY(launch_pdl(k_tiny_exact, dim3(T, W), blk, c->tiny_smem, c->side, grads, state, c->stride, layers, tiny_layers, L,
                             ktab, K, err, tau, keq, shf, flags));
         CUDA_TRY(cudaEventRecord(c->ev_join, c->side));
-        CUDA_TRY(cudaStreamWaitEvent(s, c->ev_join, 0));
+        if (!join_late) CUDA_TRY(cudaStreamWaitEvent(s, c->ev_join, 0));
         c->launches += 1;
     }
     mark(s);
@@ -433,6 +436,7 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
                                 err, tau, keq, shf, flags, fb, fb_chunks, rf, rf_chunks, list_cap, w0));
             c->launches += 1;
         }
+        if (T && join_late) CUDA_TRY(cudaStreamWaitEvent(small, c->ev_join, 0));
         mark(small);
         // (c) as a launch sequence on stream st; `when`: 0 always, 1 only if no layer is listed for the refinement or
         // the exact path, 2 only if one is
@@ -609,7 +613,7 @@ int kimad_create(kimad_ctx** out, const uint64_t* layer_sizes, uint32_t n_layers
         c->dstride = (N + 15) / 16 * 16; // every worker's code plane starts on a 16-byte boundary
         if (!plan_choice(c)) { delete c; return KIMAD_ERR_INVALID_ARG; }
         c->curve_mode = o.curve_mode;
-        c->sample_smem = (size_t)(2 * (1024 + 32) + 32768 + 1024 + 2 * kMaxGaps + 32 + 3 * 128) * 4;
+        c->sample_smem = (size_t)(1024 + 32 + 32768 + 1024 + 2 * kMaxGaps + 32 + 3 * 128) * 4;
         c->pass_a_smem = (size_t)(2 * kMaxBins + kCellTab) * 4;
         { // the sweep's runs, one CTA each: every worker's chunk list is cut into pieces of about equal element counts.
           // The sweep of a group of workers ((W + 1) / 2 of them) is one wave of CTAs (148 SMs, one CTA resident per

@@ -59,9 +59,9 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
          int4* __restrict__ cell_win, uint32_t* __restrict__ bin_lo, BandMeta* __restrict__ meta) {
     pdl_wait();
     extern __shared__ __align__(16) uint32_t sh[];
-    double* s_sq = reinterpret_cast<double*>(sh); // [1024] squares (cell midpoints) below each thread segment
-    double* s_wd = s_sq + 1024;                   // [32]
-    uint32_t* h32 = sh + 2 * (1024 + 32);         // [32768] two u16 cell counters per word
+    float* s_sq = reinterpret_cast<float*>(sh);   // [1024] squares (cell midpoints) below each thread segment
+    float* s_wd = s_sq + 1024;                    // [32]
+    uint32_t* h32 = sh + 1024 + 32;               // [32768] two u16 cell counters per word
     uint32_t* s_pre = h32 + 32768;                // [1024] inclusive sample count of the thread segments, from the top
     uint32_t* s_base = s_pre + 1024;              // [2 kMaxGaps] first bin id of every gap region, of every group
     uint32_t* s_w = s_base + 2 * kMaxGaps;        // [32]
@@ -81,6 +81,8 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
     }
     const LayerDesc ld = layers[l];
     const uint32_t n = (uint32_t)ld.n;
+    // the candidate of the thread's warp, asked for ahead of its use (the first one, where a warp takes several)
+    const uint64_t k_first = (threadIdx.x >> 5) < K ? ktab.at(w, (size_t)l * K + (threadIdx.x >> 5)) : 0ull;
     for (int i = threadIdx.x; i < 32768 / 4; i += kBigThreads) reinterpret_cast<uint4*>(h32)[i] = make_uint4(0u, 0u, 0u, 0u);
     if (threadIdx.x == 0) { s_m = 0; s_flag = 0; s_ng = 0; s_cg = 0; s_z = 0; s_zz = 0ull; s_clip = 0; }
     __syncthreads();
@@ -94,7 +96,8 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
     const bool whole = m_units == n_units;
     const uint32_t sq_ = n / (uint32_t)kSampleUnits, sr_ = n % (uint32_t)kSampleUnits; // used when sampled: m_units = kSampleUnits
     uint32_t mine = 0;
-    // a warp reads one unit (128 bytes); eight units per thread are in flight before their keys are counted
+    // a warp reads one unit (128 bytes); eight units per thread are in flight before their keys are counted (this phase runs at
+    // the DRAM's random-access rate on large layers; four and four, counted alternately, took a fifth longer)
     for (uint32_t ib = threadIdx.x / kSampleUnit; ib < m_units; ib += 8 * (kBigThreads / kSampleUnit)) {
         float a[8], b[8];
         bool ok[8];
@@ -138,45 +141,53 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
     auto cell_count = [&](uint32_t cell) { return (h32[cell >> 1] >> (16 * (cell & 1))) & 0xffffu; };
     auto cell_sq = [&](uint32_t cell) { // square of the cell's middle value (planning only: float range is enough)
         const float v = __uint_as_float((cell << 15) | 0x4000u);
-        return (double)(v * v);
+        return v * v;
     };
 
-    // ---- per thread segment (cells 65535 - 64 t - (0..63)): sample count and squares; the reads of a warp are
-    // rotated so that the lanes of a quarter warp hit different banks
+    // ---- per segment t (cells 65535 - 64 t - (0..63)): sample count and squares.  Eight lanes take a segment, four words (two
+    // cells each) per lane; the few segments that hold anything lie side by side, so fours of them are dealt out over the warps.
     uint32_t mz; // sample entries in the histogram: all but the exact zeros
     {
-        uint32_t sum = 0;
-        double sq = 0.0;
-        // the segment is 32 words (two cells each), read four at a time; most words are empty
-        const uint32_t w0 = 32736u - 32u * threadIdx.x; // first word of the segment: cells 2 w0 .. 2 w0 + 63
-        for (uint32_t q0 = 0; q0 < 8; ++q0) {
-            const uint32_t q = (q0 + threadIdx.x) & 7u;
-            const uint4 x4 = reinterpret_cast<const uint4*>(h32)[(w0 >> 2) + q];
-            const uint32_t x[4] = {x4.x, x4.y, x4.z, x4.w};
+        const uint32_t ln = threadIdx.x & 31u, wd = threadIdx.x >> 5;
+        for (uint32_t four = wd; four < (uint32_t)kBigThreads / 4; four += kBigThreads / 32) {
+            const uint32_t seg = 4u * four + (ln >> 3), word = 32736u - 32u * seg + 4u * (ln & 7u);
+            const uint4 x4 = *reinterpret_cast<const uint4*>(h32 + word);
+            uint32_t sum = 0;
+            float sq = 0.f;
+            if (__any_sync(0xffffffffu, (x4.x | x4.y | x4.z | x4.w) != 0u)) {
+                const uint32_t x[4] = {x4.x, x4.y, x4.z, x4.w};
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-                if (x[i]) {
-                    const uint32_t cell = 2u * (w0 + 4u * q + (uint32_t)i), c0 = x[i] & 0xffffu, c1 = x[i] >> 16;
+                for (int i = 0; i < 4; ++i) {
+                    const uint32_t c0 = x[i] & 0xffffu, c1 = x[i] >> 16;
                     sum += c0 + c1;
-                    if (c0) sq += (double)c0 * cell_sq(cell);
-                    if (c1) sq += (double)c1 * cell_sq(cell + 1u);
+                    if (c0) sq += (float)c0 * cell_sq(2u * (word + i));
+                    if (c1) sq += (float)c1 * cell_sq(2u * (word + i) + 1u);
                 }
+#pragma unroll
+                for (int o = 4; o; o >>= 1) {
+                    sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                    sq += __shfl_xor_sync(0xffffffffu, sq, o);
+                }
+            }
+            if ((ln & 7u) == 0) { s_pre[seg] = sum; s_sq[seg] = sq; }
         }
-        double totd;
+        __syncthreads();
+        const uint32_t sum = s_pre[threadIdx.x];
+        const float sq = s_sq[kBigThreads - 1 - threadIdx.x]; // squares are added up from the bottom: no cancellation
         const uint32_t ex = block_excl_scan<uint32_t, kBigThreads>(sum, s_w, &mz);
-        const double exd = block_excl_scan<double, kBigThreads>(sq, s_wd, &totd);
+        const float exd = block_excl_scan<float, kBigThreads>(sq, s_wd, nullptr);
         s_pre[threadIdx.x] = ex + sum;
-        s_sq[threadIdx.x] = totd - exd - sq; // squares in the segments below this one (higher thread index)
+        s_sq[kBigThreads - 1 - threadIdx.x] = exd; // squares in the segments below this one (higher index)
     }
     __syncthreads();
     const uint32_t z = m - mz; // the sample's exact zeros
     // Variance of the sample's zero count, from the spread of the zero counts of the units looked at (the units i with
     // i mod 128 < 32): zeros that come in runs (whole rows) make the sample's share of zeros, and with it the sample
     // rank of every threshold among the other keys, far less certain than independent draws would.
-    double var_z = 0.0;
+    float var_z = 0.f;
     if (z && !whole) {
-        const double ns = (double)((m_units / 128u) * 32u + min(m_units % 128u, 32u)), zs = (double)s_z;
-        var_z = fmax(0.0, ((double)s_zz - zs * zs / ns) / ns) * (double)m_units;
+        const float ns = (float)((m_units / 128u) * 32u + min(m_units % 128u, 32u)), zs = (float)s_z;
+        var_z = fmaxf(0.f, ((float)s_zz - zs * zs / ns) / ns) * (float)m_units;
     }
     // cell holding sample rank rk (1-based, from the top); the whole warp takes part
     const uint32_t lane = threadIdx.x & 31;
@@ -203,7 +214,7 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
 
     // ---- bands: the cells that can hold the k_j-th largest key, and how finely to cut them (one warp per candidate)
     for (uint32_t j = threadIdx.x >> 5; j < K; j += kBigThreads / 32) {
-        const uint64_t k = ktab.at(w, (size_t)l * K + j);
+        const uint64_t k = j < kBigThreads / 32 ? k_first : ktab.at(w, (size_t)l * K + j);
         uint32_t o_cb = 1, o_ct = 0, o_cs = 15; // k == n keeps everything: no threshold, no band
         float o_nd = 1.f;                        // bins per cell it needs
         if (k < n) {
@@ -211,12 +222,12 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
             if (whole) {
                 r_lo = r_hi = (uint32_t)k;
             } else {
-                const double p = (double)k / (double)n;
-                const double rho = p * (double)m, rel = mz ? rho / (double)mz : 0.0;
-                const double sg = sqrt((double)m * p * (1.0 - p) + rel * rel * var_z);
-                const double a = floor(rho - 6.0 * sg - 2.0), b = ceil(rho + 6.0 * sg + 2.0);
-                r_lo = a < 1.0 ? 0u : (uint32_t)a;
-                r_hi = b > (double)m ? 0u : (uint32_t)b;
+                const float p = (float)((double)k / (double)n);
+                const float rho = p * (float)m, rel = mz ? rho / (float)mz : 0.f;
+                const float sg = sqrtf((float)m * p * (1.f - p) + rel * rel * var_z);
+                const float a = floorf(rho - 6.f * sg - 2.f), b = ceilf(rho + 6.f * sg + 2.f);
+                r_lo = a < 1.f ? 0u : (uint32_t)a;
+                r_hi = b > (float)m ? 0u : (uint32_t)b;
             }
             // a rank window wholly among the zeros: the threshold is 0 unless the sample misleads, no band (the curve
             // stage knows the exact number of zeros); a window that reaches into the zeros ends at the lowest cell
@@ -253,10 +264,10 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
                 }
                 // estimate of this candidate's error: squares of everything below the band
                 const uint32_t seg = (65535u - c_bot) >> 6;
-                double below = 0.0;
+                float below = 0.f;
                 for (uint32_t c = 65535u - 64u * seg - 63u + lane; c < c_bot; c += 32) {
                     const uint32_t cc = cell_count(c);
-                    if (cc) below += (double)cc * cell_sq(c);
+                    if (cc) below += (float)cc * cell_sq(c);
                 }
 #pragma unroll
                 for (int o = 16; o; o >>= 1) {
@@ -265,28 +276,28 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
                     below += __shfl_xor_sync(0xffffffffu, below, o);
                 }
                 below += s_sq[seg];
-                const double scale = (double)n / (double)m;
+                const float scale = (float)n / (float)m;
                 // bins per cell: at most ~2048 entries per bin (what the select stage collects and sorts), and
                 // narrow enough that the uncertainty of the bin holding the threshold (its entries times its
                 // spread of squares, 2^-7 of v^2 for a whole cell) stays below ~3e-6 of the error; entries per
                 // cell and v^2 are taken quarter by quarter
-                double dens = 0.0, load = 0.0;
+                float dens = 0.f, load = 0.f;
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const uint32_t qtop = min(c_top, c_bot + (uint32_t)(i + 1) * nq - 1);
-                    const double per_cell = (double)(inq[i] + 1) / (double)nq * scale; // + 1: never plan on an empty sample
+                    const float per_cell = (float)(inq[i] + 1) / (float)nq * scale; // + 1: never plan on an empty sample
                     dens = per_cell > dens ? per_cell : dens;
-                    const double ld = per_cell * cell_sq(qtop);
+                    const float ld = per_cell * cell_sq(qtop);
                     load = ld > load ? ld : load;
                 }
-                double bins = dens / 2048.0;
-                const double e_est = below * scale;
-                const double cert = e_est > 0.0 ? sqrt(load * 0.0078125 / (3e-6 * e_est)) : 1024.0;
+                float bins = dens * (1.f / 2048.f);
+                const float e_est = below * scale;
+                const float cert = e_est > 0.f ? sqrtf(load / e_est * (0.0078125f / 3e-6f)) : 1024.f;
                 if (cert > bins) bins = cert;
                 uint32_t sh_j = 15;
-                while (sh_j > 5 && (double)(1u << (15 - sh_j)) < bins) --sh_j;
+                while (sh_j > 5 && (float)(1u << (15 - sh_j)) < bins) --sh_j;
                 o_cb = c_bot; o_ct = c_top; o_cs = sh_j;
-                o_nd = (float)bins;
+                o_nd = bins;
             }
         }
         if (lane == 0) { s_cb[j] = o_cb; s_ct[j] = o_ct; s_cs[j] = o_cs; s_nd[j] = o_nd; }
@@ -398,41 +409,36 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
         if (threadIdx.x == 0) *mt = BandMeta{tot_bins, used, 2, s_flag};
         return;
     }
-    // (base, shift) of the region that holds a cell, as base << 5 | shift (base may be negative)
-    auto entry_of = [&](uint32_t cell) -> uint32_t {
-        uint32_t a = 0;
-        for (; a < ng; ++a) {
-            const uint32_t g = ng - 1 - a;
-            if (cell > s_ct[g]) continue;
-            if (cell >= s_cb[g]) {
-                const uint32_t cs = s_cs[g];
-                return (uint32_t)(((int)s_base[kMaxGaps + a] - (int)(s_cb[g] << (15 - cs))) * 32) | cs;
-            }
-            break;
-        }
-        return (uint32_t)(((int)s_base[a] - (int)(s_glo[a] >> 5)) * 32) | 20u;
-    };
     uint32_t* tab = cell_tab + wr * kCellTab;
     uint32_t* blo = bin_lo + wr * (kMaxBins + 1);
     // entry i serves the cells (wlo - 1 + i) << cg ...; the first one everything below the window, the last one
     // everything above it
-    for (uint32_t i = threadIdx.x; i < used; i += kBigThreads) tab[i] = entry_of(i + 1 == used ? 65535u : (wlo + i - 1u) << cg);
-    // lower key of every bin: the pieces of the gaps ...
-    for (uint32_t b1 = threadIdx.x; b1 < (uint32_t)kL1Bins; b1 += kBigThreads) {
-        const uint32_t c0 = b1 << 5, c1 = c0 + 31;
-        if (b1 >= 2040u) { blo[s_base[ng + 1] + (b1 - 2040u)] = (b1 << 20) | kGapBit; continue; }
-        for (uint32_t a = 0; a <= ng; ++a) {
-            const uint32_t lo = s_glo[a];
-            const uint32_t hi = a == ng ? 65279u : s_cb[ng - 1 - a] - 1;
-            if (hi + 1 <= lo || hi < c0 || lo > c1) continue;
-            blo[s_base[a] + b1 - (lo >> 5)] = (max(lo, c0) << 15) | kGapBit;
+    // (base, shift) of the region that holds a cell, as base << 5 | shift (base may be negative); the cells of a thread ascend
+    for (uint32_t i = threadIdx.x, a = 0; i < used; i += kBigThreads) {
+        const uint32_t cell = i + 1 == used ? 65535u : (i == 0 && wlo == 0 ? 0u : (wlo + i - 1u) << cg);
+        while (a < ng && cell > s_ct[ng - 1 - a]) ++a;
+        const uint32_t g = ng - 1 - a;
+        if (a < ng && cell >= s_cb[g]) {
+            const uint32_t cs = s_cs[g];
+            tab[i] = (uint32_t)(((int)s_base[kMaxGaps + a] - (int)(s_cb[g] << (15 - cs))) * 32) | cs;
+        } else {
+            tab[i] = (uint32_t)(((int)s_base[a] - (int)(s_glo[a] >> 5)) * 32) | 20u;
         }
     }
-    // ... and the fine bins of the groups
-    for (uint32_t a = 0; a < ng; ++a) {
-        const uint32_t g = ng - 1 - a, cs = s_cs[g], first = s_base[kMaxGaps + a];
-        const uint32_t nf = (s_ct[g] - s_cb[g] + 1) << (15 - cs);
-        for (uint32_t x = threadIdx.x; x < nf; x += kBigThreads) blo[first + x] = (s_cb[g] << 15) + (x << cs);
+    // lower key of every bin; the bins of a thread ascend, and with them the region they lie in
+    for (uint32_t x = threadIdx.x, a = 0; x < tot_bins; x += kBigThreads) {
+        while (a < ng && s_base[a + 1] <= x) ++a;
+        uint32_t key;
+        if (x >= s_base[ng + 1]) {
+            key = ((2040u + x - s_base[ng + 1]) << 20) | kGapBit;
+        } else if (a < ng && x >= s_base[kMaxGaps + a]) {
+            const uint32_t g = ng - 1 - a;
+            key = (s_cb[g] << 15) + ((x - s_base[kMaxGaps + a]) << s_cs[g]);
+        } else {
+            const uint32_t lo = s_glo[a];
+            key = (max(lo, ((lo >> 5) + x - s_base[a]) << 5) << 15) | kGapBit;
+        }
+        blo[x] = key;
     }
     if (threadIdx.x == 0) {
         blo[tot_bins] = 0x80000000u;

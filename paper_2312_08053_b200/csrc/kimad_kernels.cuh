@@ -91,7 +91,7 @@ __device__ __forceinline__ uint32_t pack_key_codes(uint32_t k0, uint32_t k1, uin
 }
 
 // ------------------------------------------------------------------------------------------------
-// block-wide exclusive scans (256 threads), result valid in every thread; `total` optional
+// block-wide exclusive scans (NT threads), result valid in every thread; `total` optional
 // ------------------------------------------------------------------------------------------------
 template <typename T, int NT = kThreads>
 __device__ __forceinline__ T block_excl_scan(T v, T* s_warp /* [NT / 32] */, T* total) {
@@ -106,11 +106,22 @@ __device__ __forceinline__ T block_excl_scan(T v, T* s_warp /* [NT / 32] */, T* 
     if (lane == 31) s_warp[wid] = x;
     __syncthreads();
     T base = 0, tot = 0;
+    if (NT <= 256) {
 #pragma unroll
-    for (int i = 0; i < NT / 32; ++i) {
-        T t = s_warp[i];
-        if (i < wid) base += t;
-        tot += t;
+        for (int i = 0; i < NT / 32; ++i) {
+            const T t = s_warp[i];
+            if (i < wid) base += t;
+            tot += t;
+        }
+    } else { // every warp scans the warps' totals
+        T t = lane < NT / 32 ? s_warp[lane] : T(0);
+#pragma unroll
+        for (int o = 1; o < NT / 32; o <<= 1) {
+            const T y = __shfl_up_sync(0xffffffffu, t, o);
+            if (lane >= o) t += y;
+        }
+        base = wid ? __shfl_sync(0xffffffffu, t, wid - 1) : T(0);
+        tot = __shfl_sync(0xffffffffu, t, NT / 32 - 1);
     }
     if (total) *total = tot;
     // the lane's exclusive value is taken from its left neighbour, not as inclusive - own: a subtraction would
