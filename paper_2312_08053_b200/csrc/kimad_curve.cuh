@@ -39,6 +39,7 @@ constexpr int kMaxBins = kFineBins + kL1Bins + 2 * kMaxGaps; // fine bins + gap 
 constexpr int kMaxShift = 15;                       // a fine bin is 2^shift keys wide, at most a whole cell
 constexpr int kSampleUnit = 32;                     // consecutive elements read together (128 bytes, one warp)
 constexpr int kSampleUnits = 2047;                  // units of a sample (<= 65504 elements: the u16 cell counters cannot overflow)
+constexpr int kWholeUnits = 1024;                   // layers of up to as many units are taken whole
 constexpr int kBigThreads = 1024;
 constexpr uint32_t kGapBit = 1u;                    // bin_lo entries carry this bit when the bin is a gap bin
 
@@ -92,9 +93,11 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
     const float* gr = grads + (size_t)w * stride + ld.begin;
     const float* st = state + (size_t)w * stride + ld.begin;
     const uint32_t n_units = n / kSampleUnit + ((n % kSampleUnit) != 0); // n may be as large as 2^32 - 1
-    const uint32_t m_units = min(n_units, (uint32_t)kSampleUnits);
+    // Half of the layer is enough of a sample: drawn without replacement its ranks are as certain as those of kSampleUnits units
+    // of a large layer.  Up to kWholeUnits the layer is taken whole (exact ranks, bands of one cell).
+    const uint32_t m_units = n_units <= (uint32_t)kWholeUnits ? n_units : min(max(n_units / 2u, (uint32_t)kWholeUnits), (uint32_t)kSampleUnits);
     const bool whole = m_units == n_units;
-    const uint32_t sq_ = n / (uint32_t)kSampleUnits, sr_ = n % (uint32_t)kSampleUnits; // used when sampled: m_units = kSampleUnits
+    const uint32_t sq_ = n / m_units, sr_ = n % m_units; // used when sampled
     uint32_t mine = 0;
     // a warp reads one unit (128 bytes); eight units per thread are in flight before their keys are counted (this phase runs at
     // the DRAM's random-access rate on large layers; four and four, counted alternately, took a fifth longer)
@@ -108,8 +111,8 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
             const uint32_t i = ib + (threadIdx.x & 7u) * (kBigThreads / kSampleUnit);
             my_start = kSampleUnit * i;
             if (!whole && i < m_units) { // unit i somewhere inside stratum i = [i q + i r / m, (i+1) q + (i+1) r / m)
-                const uint32_t s0 = i * sq_ + (i * sr_) / (uint32_t)kSampleUnits;
-                const uint32_t s1 = (i + 1) * sq_ + ((i + 1) * sr_) / (uint32_t)kSampleUnits;
+                const uint32_t s0 = i * sq_ + (i * sr_) / m_units;
+                const uint32_t s1 = (i + 1) * sq_ + ((i + 1) * sr_) / m_units;
                 const uint32_t room = s1 > s0 + kSampleUnit ? s1 - s0 - kSampleUnit : 0;
                 my_start = s0 + __umulhi(hash_u32(i * 0x9e3779b9u + l * 0x85ebca6bu + 1u), room + 1);
             }
@@ -224,7 +227,8 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
             } else {
                 const float p = (float)((double)k / (double)n);
                 const float rho = p * (float)m, rel = mz ? rho / (float)mz : 0.f;
-                const float sg = sqrtf((float)m * p * (1.f - p) + rel * rel * var_z);
+                const float left_out = fmaxf(0.f, 1.f - (float)m / (float)n); // drawn without replacement
+                const float sg = sqrtf((float)m * p * (1.f - p) * left_out + rel * rel * var_z);
                 const float a = floorf(rho - 6.f * sg - 2.f), b = ceilf(rho + 6.f * sg + 2.f);
                 r_lo = a < 1.f ? 0u : (uint32_t)a;
                 r_hi = b > (float)m ? 0u : (uint32_t)b;
