@@ -363,7 +363,7 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
     if (c->policy == 3 && mode != kGivenJ) { // Section 3.1: the one ratio sized to each worker's budget
         for (uint32_t w0 = 0; w0 < W; w0 += kDpWorkersPerLaunch) {
             const uint32_t nw = std::min<uint32_t>(kDpWorkersPerLaunch, W - w0);
-            CUDA_TRY(launch_pdl(k_fit_ratio, nw, blk, 0, s, budgets_of(w0, nw), w0, W, L, c->bpe, c->N, layers,
+            CUDA_TRY(launch_pdl(k_fit_ratio, nw, kFitThreads, 0, s, budgets_of(w0, nw), w0, W, L, c->bpe, c->N, layers,
                                 c->at<uint64_t>(y.ktab_dyn)));
             c->launches += 1;
         }
