@@ -47,6 +47,7 @@ struct kimad_ctx {
     std::vector<unsigned char> static_image;                  // the static tables as they lie in the workspace, one block
     std::vector<size_t> guards;                               // checked build: offsets of the canary words between regions
     uint32_t most_chunks = 0; // of a layer
+    bool odd = false;         // workers may start at different distances from a 128-bit boundary
     uint32_t curve_mode = 0;
     uint32_t policy = 0, cost_model = 0;
     size_t sample_smem = 0, pass_a_smem = 0, tiny_smem = 0;
@@ -304,11 +305,14 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream_v);
     const uint32_t L = c->L, W = c->W, K = c->K;
     const uint32_t nch = (uint32_t)c->chunks.size();
-    const bool vec = ((uintptr_t)grads % 16 == 0) && ((uintptr_t)state % 16 == 0) && (c->stride % 4 == 0);
+    // 128-bit loads need both inputs equally far past a 16-byte boundary; how far may differ from worker to worker where the
+    // chunks leave room for it
+    const bool vec = (((uintptr_t)grads ^ (uintptr_t)state) & 15u) == 0 && ((uintptr_t)grads & (c->odd ? 3u : 15u)) == 0;
+    const Phase phase{vec && c->odd ? (uint32_t)((uintptr_t)grads / 4 & 3u) : 0u, vec && c->odd ? (uint32_t)(c->stride & 3u) : 0u};
 
     const Layout& y = c->lay;
     // one code byte per element, u8 [W][dstride]; exact values are recomputed from grads and state
-    const DSource dbuf{c->at<uint8_t>(y.dbuf), grads, state, c->stride};
+    const DSource dbuf{c->at<uint8_t>(y.dbuf), grads, state, c->stride, c->dstride, phase};
     const Chunk* chunks = c->at<Chunk>(y.chunks);
     const LayerDesc* layers = c->at<LayerDesc>(y.layers);
     // candidates: the grid's table for every worker, or (policy 3) each worker's row of the ratio fitted to its budget
@@ -424,10 +428,10 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
         }
         if (vec)
             CUDA_TRY(launch_pdl(k_pass_a<true>, run1 - run0, kBigThreads, c->pass_a_smem, big, grads, state, dbuf.code, chunks, runs + run0,
-                                c->stride, c->dstride, reg_index, R, cell_tab, cell_win, meta, bhc, bhs));
+                                c->stride, c->dstride, phase, reg_index, R, cell_tab, cell_win, meta, bhc, bhs));
         else
             CUDA_TRY(launch_pdl(k_pass_a<false>, run1 - run0, kBigThreads, c->pass_a_smem, big, grads, state, dbuf.code, chunks, runs + run0,
-                                c->stride, c->dstride, reg_index, R, cell_tab, cell_win, meta, bhc, bhs));
+                                c->stride, c->dstride, phase, reg_index, R, cell_tab, cell_win, meta, bhc, bhs));
         c->launches += 1;
         mark(big);
         CUDA_TRY(hand_over(big, small));
@@ -478,13 +482,13 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
             const uint32_t gfb = 4 * 148;
             uint32_t* arrived = c->at<uint32_t>(y.in_n); // (counts the select stage's entries later in the step; zero in between)
             // candidates with a loose bound first (they may still end on the exact path's lists)
-            CUDA_TRY(launch_pdl(k_refine, 5 * 148, blk, 0, st, dbuf, layers, chunks, c->dstride, L, K, fb, rf_chunks, rf, codes, h23c, h23s,
+            CUDA_TRY(launch_pdl(k_refine, 5 * 148, blk, 0, st, dbuf, layers, chunks, L, K, fb, rf_chunks, rf, codes, h23c, h23s,
                                 arrived, err, tau, keq, shf, fb_chunks, list_cap));
-            CUDA_TRY(launch_pdl(k_fb1, gfb, blk, 0, st, dbuf, layers, chunks, c->dstride, L, K, ktab, fb, fb_chunks, h1c, h1s, flags, codes,
+            CUDA_TRY(launch_pdl(k_fb1, gfb, blk, 0, st, dbuf, layers, chunks, L, K, ktab, fb, fb_chunks, h1c, h1s, flags, codes,
                                 arrived, cands, slots));
-            CUDA_TRY(launch_pdl(k_fb23<2>, gfb, blk, 0, st, dbuf, layers, chunks, c->dstride, L, K, fb, fb_chunks, slots, cands, h23c, h23s,
+            CUDA_TRY(launch_pdl(k_fb23<2>, gfb, blk, 0, st, dbuf, layers, chunks, L, K, fb, fb_chunks, slots, cands, h23c, h23s,
                                 codes, arrived, err, tau, keq, shf));
-            CUDA_TRY(launch_pdl(k_fb23<3>, gfb, blk, 0, st, dbuf, layers, chunks, c->dstride, L, K, fb, fb_chunks, slots, cands, h23c, h23s,
+            CUDA_TRY(launch_pdl(k_fb23<3>, gfb, blk, 0, st, dbuf, layers, chunks, L, K, fb, fb_chunks, slots, cands, h23c, h23s,
                                 codes, arrived, err, tau, keq, shf));
             c->launches += 4;
             return KIMAD_OK;
@@ -509,22 +513,22 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
         mark(small);
         CUDA_TRY(hand_over(small, big));
         // (d), (e), (f)
-        CUDA_TRY(launch_pdl(k_sel_count, gch, blk, 0, big, dbuf, chunks, nch, c->dstride, L, sel, layers, csel, in, rc, w0));
+        CUDA_TRY(launch_pdl(k_sel_count, gch, blk, 0, big, dbuf, chunks, nch, L, sel, layers, csel, in, rc, w0));
         mark(big);
         CUDA_TRY(hand_over(big, small));
         {
             auto launch = [&](auto kern, uint32_t threads) {
                 return launch_named("k_sel_offsets", kern, glw, threads, 0, small, layers, chunks, nch, L, sel, csel, jobs, in, fb, rc,
-                                    rc_chunks, list_cap, w0);
+                                    rc_chunks, list_cap, phase, w0);
             };
             CUDA_TRY(c->most_chunks > 256 ? launch(k_sel_offsets<512>, 512) : launch(k_sel_offsets<128>, 128));
         }
-        CUDA_TRY(launch_pdl(k_sel_recount, 148, blk, 0, small, dbuf, layers, chunks, nch, c->dstride, L, sel, csel, jobs, in, rc, rc_chunks));
+        CUDA_TRY(launch_pdl(k_sel_recount, 148, blk, 0, small, dbuf, layers, chunks, nch, L, sel, csel, jobs, in, rc, rc_chunks));
         mark(small);
         CUDA_TRY(hand_over(small, big));
         {
             auto launch = [&](auto kern) {
-                return launch_named("k_sel_write", kern, gch, blk, 0, big, grads, state, chunks, nch, c->dstride, c->stride, csel,
+                return launch_named("k_sel_write", kern, gch, blk, 0, big, grads, state, chunks, nch, c->stride, phase, csel,
                                     jobs, c->cap, out->idx, out->val, w0);
             };
             if (c->value_dtype == 1) CUDA_TRY(dense_write ? launch(k_sel_write<true, true>) : launch(k_sel_write<true, false>));
@@ -577,6 +581,10 @@ int kimad_create(kimad_ctx** out, const uint64_t* layer_sizes, uint32_t n_layers
         c->grid.assign(ratio_grid, ratio_grid + n_ratios);
         c->ktab.resize((size_t)n_layers * n_ratios);
         uint64_t N = 0;
+        for (uint32_t l = 0; l < n_layers; ++l) N += layer_sizes[l];
+        c->odd = n_workers > 1 && (o.worker_stride ? o.worker_stride : N) % 4 != 0;
+        const uint64_t window = c->odd ? kChunkElemsOdd : kChunkElems;
+        N = 0;
         for (uint32_t l = 0; l < n_layers; ++l) {
             const uint64_t n = layer_sizes[l];
             if (n == 0 || n > 0xffffffffull) { delete c; return KIMAD_ERR_INVALID_ARG; }
@@ -590,7 +598,7 @@ int kimad_create(kimad_ctx** out, const uint64_t* layer_sizes, uint32_t n_layers
             // chunk table: aligned windows of the flat vector intersected with this layer
             LayerDesc ld{N, n, (uint32_t)c->chunks.size(), 0};
             for (uint64_t p = N; p < N + n;) {
-                const uint64_t e = std::min(N + n, (p / kChunkElems + 1) * kChunkElems);
+                const uint64_t e = std::min(N + n, (p / window + 1) * window);
                 c->chunks.push_back(Chunk{l, 0, p, e});
                 p = e;
             }
@@ -610,7 +618,7 @@ int kimad_create(kimad_ctx** out, const uint64_t* layer_sizes, uint32_t n_layers
         c->stride = o.worker_stride ? o.worker_stride : N;
         c->cap = o.max_packed_elems ? o.max_packed_elems : N;
         if (c->stride < N || c->chunks.size() > 0x7fffffffull) { delete c; return KIMAD_ERR_INVALID_ARG; }
-        c->dstride = (N + 15) / 16 * 16; // every worker's code plane starts on a 16-byte boundary
+        c->dstride = (N + 3 + 15) / 16 * 16; // every worker's code plane starts on a 16-byte boundary (and up to 3 codes in)
         if (!plan_choice(c)) { delete c; return KIMAD_ERR_INVALID_ARG; }
         c->curve_mode = o.curve_mode;
         c->sample_smem = (size_t)(1024 + 32 + 32768 + 1024 + 2 * kMaxGaps + 32 + 3 * 128) * 4;

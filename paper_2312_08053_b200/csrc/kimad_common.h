@@ -26,9 +26,13 @@ __device__ unsigned int g_kimad_check_word;
 
 namespace kimad {
 
-// A chunk is the part of one layer that falls inside one aligned window of kChunkElems elements of
-// the flat per-worker vector.  One CTA streams one chunk.
+// A chunk is the part of one layer that falls inside one aligned window of the flat per-worker vector.  One CTA streams
+// one chunk.  Contexts whose workers start at different distances from a 128-bit boundary (unpadded strides) have windows of
+// kChunkElemsOdd elements: a chunk that starts up to three elements past a boundary then still has at most kChunkElems from
+// the boundary on, and windows start on 128-byte lines of the code plane (with windows of 32752 the counting sweep took
+// 12-20 % longer).
 constexpr uint64_t kChunkElems = 32768;
+constexpr uint64_t kChunkElemsOdd = 32640;
 constexpr int kDpWorkersPerLaunch = 32;
 
 struct Chunk {

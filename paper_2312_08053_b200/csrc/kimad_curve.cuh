@@ -463,7 +463,7 @@ constexpr int kRunDesc = 64;             // chunk descriptors staged in shared m
 template <bool VEC>
 __global__ void __launch_bounds__(kBigThreads, 1)
 k_pass_a(const float* __restrict__ grads, const float* __restrict__ state, uint8_t* __restrict__ d_code,
-         const Chunk* __restrict__ chunks, const SweepRun* __restrict__ runs, uint64_t stride, uint64_t dstride,
+         const Chunk* __restrict__ chunks, const SweepRun* __restrict__ runs, uint64_t stride, uint64_t dstride, const Phase phases,
          const uint32_t* __restrict__ reg_index /* [L], 0xffffffff: tiny layer */, uint32_t R,
          const uint32_t* __restrict__ cell_tab, const int4* __restrict__ cell_win, const BandMeta* __restrict__ meta,
          uint32_t* __restrict__ bh_cnt, unsigned long long* __restrict__ bh_sum) {
@@ -474,12 +474,19 @@ k_pass_a(const float* __restrict__ grads, const float* __restrict__ state, uint8
     uint32_t* tab = sh + 2 * kMaxBins; // [kCellTab]
     // the run, its first chunk descriptors and the clean histogram do not depend on the kernels before this one
     const SweepRun run = runs[blockIdx.x];
+    auto chunk_at = [&](uint32_t c) { // in positions counted from the worker's 128-bit boundary
+        Chunk ch = chunks[c];
+        const uint32_t phase = VEC ? phases.at(run.w) : 0u;
+        ch.begin += phase;
+        ch.end += phase;
+        return ch;
+    };
     for (int i = threadIdx.x; i < 2 * kMaxBins; i += kBigThreads) sh[i] = 0;
-    for (uint32_t i = threadIdx.x; i < min(run.c1 - run.c0, (uint32_t)kRunDesc); i += kBigThreads) s_desc[i] = chunks[run.c0 + i];
+    for (uint32_t i = threadIdx.x; i < min(run.c1 - run.c0, (uint32_t)kRunDesc); i += kBigThreads) s_desc[i] = chunk_at(run.c0 + i);
     pdl_wait();
     __syncthreads();
-    const float* gr0 = grads + (size_t)run.w * stride;
-    const float* st0 = state + (size_t)run.w * stride;
+    const float* gr0 = grads + (size_t)run.w * stride - (VEC ? phases.at(run.w) : 0u);
+    const float* st0 = state + (size_t)run.w * stride - (VEC ? phases.at(run.w) : 0u);
     uint8_t* dc0 = d_code + (size_t)run.w * dstride;
     int cur_layer = -1;
     // slot of the current layer's histogram; 0xffffffff: none (tiny or handed-over layer); bit 30 (kSkipZeros): the
@@ -554,7 +561,7 @@ k_pass_a(const float* __restrict__ grads, const float* __restrict__ state, uint8
         const uint32_t di = (c - run.c0) % (uint32_t)kRunDesc;
         if (di == 0 && c != run.c0) { // next window of descriptors
             __syncthreads();
-            for (uint32_t i = threadIdx.x; i < min(run.c1 - c, (uint32_t)kRunDesc); i += kBigThreads) s_desc[i] = chunks[c + i];
+            for (uint32_t i = threadIdx.x; i < min(run.c1 - c, (uint32_t)kRunDesc); i += kBigThreads) s_desc[i] = chunk_at(c + i);
             __syncthreads();
         }
         Chunk ch = s_desc[di];
@@ -584,7 +591,7 @@ k_pass_a(const float* __restrict__ grads, const float* __restrict__ state, uint8
             __syncthreads();
         }
         const bool active = wr != 0xffffffffu;
-        const ChunkView cv(ch);
+        const ChunkView cv(ch, 0);
         uint8_t* dc = dc0 + cv.a0;
         {
             const uint32_t q_lo = (cv.first + 3) >> 2, q_hi = cv.len >> 2; // whole quads [q_lo, q_hi)
@@ -892,7 +899,7 @@ __device__ __forceinline__ void refine_resolve_layer(uint32_t l, uint32_t w, siz
 }
 
 __global__ void __launch_bounds__(kThreads, 5)
-k_refine(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* __restrict__ chunks, uint64_t dstride, uint32_t L, uint32_t K,
+k_refine(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* __restrict__ chunks, uint32_t L, uint32_t K,
          FbList* __restrict__ fb, const uint2* __restrict__ rf_chunks, RefineCand* __restrict__ rf,
          const CodeSpace codes, uint32_t* __restrict__ g_cnt, unsigned long long* __restrict__ g_ss, uint32_t* __restrict__ arrived,
          float* __restrict__ err_out, uint32_t* __restrict__ tau_out, uint32_t* __restrict__ rank_out, uint32_t* __restrict__ shift_out,
@@ -936,8 +943,8 @@ k_refine(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* __rest
         __syncthreads();
         const uint32_t nc = s_n;
         const uint32_t m0 = s_mask[0], m1 = s_mask[1], m2 = s_mask[2], m3 = s_mask[3];
-        const ChunkView cv(ch);
-        const DView dd(dbuf, e.x, dstride, cv.a0);
+        const ChunkView cv(ch, dbuf.phase.at(e.x));
+        const DView dd(dbuf, e.x, cv.a0);
         const bool vec = ((reinterpret_cast<uintptr_t>(dd.gr) | reinterpret_cast<uintptr_t>(dd.st)) & 15u) == 0;
         auto wanted = [&](uint32_t code) -> bool {
             const uint32_t word = code < 64u ? (code < 32u ? m0 : m1) : (code < 96u ? m2 : m3);
@@ -958,7 +965,7 @@ k_refine(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* __rest
         for (uint32_t u = threadIdx.x; u < units; u += kThreads) {
             const uint32_t e0 = 16u * u;
             uint32_t hit = 0; // the unit's elements whose code is one of the loose bins' codes
-            if (e0 >= cv.first && e0 + 16u <= cv.len) {
+            if (e0 + 16u > cv.first) { // (a unit at the chunk's edge holds codes of the neighbouring chunk, too)
                 const uint4 a = __ldcs(reinterpret_cast<const uint4*>(dd.code) + u);
                 const uint32_t x[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
@@ -966,9 +973,8 @@ k_refine(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* __rest
 #pragma unroll
                     for (int b = 0; b < 4; ++b)
                         if (wanted((x[i] >> (8 * b)) & 127u)) hit |= 1u << (4 * i + b);
-            } else {
-                for (uint32_t x = max(e0, cv.first); x < min(e0 + 16u, cv.len); ++x)
-                    if (wanted(dd.code[x] & 127u)) hit |= 1u << (x - e0);
+                if (e0 < cv.first) hit &= ~0u << (cv.first - e0);
+                if (e0 + 16u > cv.len) hit &= ~(~0u << (cv.len - e0));
             }
             if (!hit) continue;
             // the unit's entries are completed from the inputs with independent loads: eight at a time
@@ -1165,7 +1171,7 @@ k_tiny_exact(const float* __restrict__ grads, const float* __restrict__ state, u
 constexpr int kFbAhead = 4; // elements per thread whose loads are issued together
 
 __global__ void __launch_bounds__(kThreads)
-k_fb1(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* __restrict__ chunks, uint64_t dstride, uint32_t L, uint32_t K,
+k_fb1(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* __restrict__ chunks, uint32_t L, uint32_t K,
       const KTab ktab, const FbList* __restrict__ fb, const uint2* __restrict__ fb_chunks, uint32_t* __restrict__ g_cnt,
       unsigned long long* __restrict__ g_ss, uint32_t* __restrict__ flags, const CodeSpace codes, uint32_t* __restrict__ arrived,
       Cand* __restrict__ cands, SlotTab* __restrict__ slots) {
@@ -1179,8 +1185,8 @@ k_fb1(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* __restric
     for (uint32_t it = blockIdx.x; it < n; it += gridDim.x) {
         const uint2 e = fb_chunks[it];
         const Chunk ch = chunks[e.y];
-        const ChunkView cv(ch);
-        const DView dd(dbuf, e.x, dstride, cv.a0);
+        const ChunkView cv(ch, dbuf.phase.at(e.x));
+        const DView dd(dbuf, e.x, cv.a0);
         for (int b = threadIdx.x; b < kL1Bins; b += kThreads) { s_cnt[b] = 0; s_hi[b] = 0; s_lo[b] = 0; }
         __syncthreads();
         // a thread sees at most kChunkElems / kThreads elements of a chunk: its two partial sums stay below 2^32
@@ -1222,7 +1228,7 @@ k_fb1(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* __restric
 
 template <int LEVEL>
 __global__ void __launch_bounds__(kThreads)
-k_fb23(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* __restrict__ chunks, uint64_t dstride, uint32_t L, uint32_t K,
+k_fb23(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* __restrict__ chunks, uint32_t L, uint32_t K,
        const FbList* __restrict__ fb, const uint2* __restrict__ fb_chunks, SlotTab* __restrict__ slots, Cand* __restrict__ cands,
        uint32_t* __restrict__ g_cnt, unsigned long long* __restrict__ g_ss, const CodeSpace codes, uint32_t* __restrict__ arrived,
        float* __restrict__ err_out, uint32_t* __restrict__ tau_out, uint32_t* __restrict__ keep_eq_out, uint32_t* __restrict__ shift_out) {
@@ -1247,8 +1253,8 @@ k_fb23(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* __restri
                 s_num[b1]++;
             }
         __syncthreads();
-        const ChunkView cv(ch);
-        const DView dd(dbuf, e.x, dstride, cv.a0);
+        const ChunkView cv(ch, dbuf.phase.at(e.x));
+        const DView dd(dbuf, e.x, cv.a0);
         const size_t wr = codes.slot(e.x, ch.layer);
         uint32_t* gc = g_cnt + wr * K * kL23Bins;
         unsigned long long* gs = g_ss + wr * K * kL23Bins;

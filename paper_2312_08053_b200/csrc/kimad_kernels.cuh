@@ -49,13 +49,19 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // Aligned view of a chunk for 128-bit loads of the inputs (quads of elements) and of the code plane (sixteen
 // codes): units start at a0 = begin & ~15; only the first and the last ones can be partial.  All offsets are
 // 32-bit and relative to a0.
+// Where a worker's vectors start at an odd element (unpadded strides, an offset base), both inputs are `phase` elements past a
+// 128-bit boundary.  Positions counted from that boundary (element + phase) are aligned as the memory is; the code plane is laid
+// out in them, and chunks are cut into quads and units of sixteen there.
+struct Phase {
+    uint32_t first, step; // elements past the boundary of worker 0; what the stride adds per worker (0, 0: inputs that are
+                          // not equally far past one, which are read element by element)
+    __device__ __forceinline__ uint32_t at(uint32_t w) const { return (first + w * step) & 3u; }
+};
 struct ChunkView {
-    uint64_t a0;
+    uint64_t a0;         // aligned start: element + phase
     uint32_t first, len; // valid element offsets are [first, len)
-    __device__ __forceinline__ explicit ChunkView(const Chunk& ch)
-        : a0(ch.begin & ~15ull), first((uint32_t)(ch.begin - (ch.begin & ~15ull))), len((uint32_t)(ch.end - (ch.begin & ~15ull))) {}
-    __device__ __forceinline__ uint32_t quads() const { return (len + 3) >> 2; }
-    __device__ __forceinline__ bool quad_full(uint32_t q) const { return 4 * q >= first && 4 * q + 4 <= len; }
+    __device__ __forceinline__ ChunkView(const Chunk& ch, uint32_t phase)
+        : a0((ch.begin + phase) & ~15ull), first((uint32_t)(ch.begin + phase - a0)), len((uint32_t)(ch.end + phase - a0)) {}
 };
 
 // The difference vector d = grad - g is never stored.  The sweep leaves one BYTE per element (u8 [W][dstride]): a
@@ -69,14 +75,17 @@ struct DSource {
     uint8_t* code;
     const float* grads;
     const float* state;
-    uint64_t stride; // elements between workers in grads / state
+    uint64_t stride;  // elements between workers in grads / state
+    uint64_t dstride; // ... in the code plane
+    Phase phase;
 };
 struct DView { // one worker's data at a chunk's aligned start
     const uint8_t* code;
     const float* gr;
     const float* st;
-    __device__ __forceinline__ DView(const DSource& p, uint32_t w, uint64_t dstride, uint64_t a0)
-        : code(p.code + (size_t)w * dstride + a0), gr(p.grads + (size_t)w * p.stride + a0), st(p.state + (size_t)w * p.stride + a0) {}
+    __device__ __forceinline__ DView(const DSource& p, uint32_t w, uint64_t a0)
+        : code(p.code + (size_t)w * p.dstride + a0), gr(p.grads + (size_t)w * p.stride + a0 - p.phase.at(w)),
+          st(p.state + (size_t)w * p.stride + a0 - p.phase.at(w)) {}
     __device__ __forceinline__ float at(uint32_t e) const { return __fsub_rn(gr[e], st[e]); }
 };
 // code of layers without a histogram: the upper seven bits of the 31-bit key

@@ -71,7 +71,7 @@ struct Recount {
 // Counting sweep: a CTA per chunk, warp w takes the slices w and w + 8.
 // ------------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(kThreads, 6)
-k_sel_count(DSource dbuf, const Chunk* __restrict__ chunks, uint32_t n_chunks, uint64_t dstride, uint32_t L,
+k_sel_count(DSource dbuf, const Chunk* __restrict__ chunks, uint32_t n_chunks, uint32_t L,
             const Sel* __restrict__ sel, const LayerDesc* __restrict__ layers, ChunkSel* __restrict__ csel, const Interval in,
             Recount* __restrict__ rc, uint32_t w_base) {
     pdl_wait();
@@ -83,7 +83,7 @@ k_sel_count(DSource dbuf, const Chunk* __restrict__ chunks, uint32_t n_chunks, u
     const Sel s = sel[wl];
     const LayerDesc ld = layers[ch.layer];
     ChunkSel* out = csel + (size_t)w * n_chunks + blockIdx.x;
-    const ChunkView cv(ch);
+    const ChunkView cv(ch, dbuf.phase.at(w));
     const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) rc->n_chunks = 0; // consumed by the step before
     if (s.k == 0 || (uint64_t)s.k == ld.n) { // nothing / everything kept: no need to look at the data
@@ -99,7 +99,7 @@ k_sel_count(DSource dbuf, const Chunk* __restrict__ chunks, uint32_t n_chunks, u
     const uint32_t rel = blockIdx.x - ld.first_chunk;
     if (threadIdx.x == 0) s_n = 0;
     __syncthreads();
-    const DView dd(dbuf, w, dstride, cv.a0);
+    const DView dd(dbuf, w, cv.a0);
     auto append = [&](uint32_t at, uint32_t rec) { // one entry of the layer's interval, the at-th
         const size_t wr = in.slot(w, ch.layer);
         if (at < (uint32_t)kListCap) in.list(wr)[at] = make_uint2(rel, rec);
@@ -134,29 +134,44 @@ k_sel_count(DSource dbuf, const Chunk* __restrict__ chunks, uint32_t n_chunks, u
         // a 32-element group is a pair of lanes
         constexpr int ROWS = kSliceElems / 512;
         const uint32_t u0 = sl * (kSliceElems / 16) + lane; // this lane's 16-element unit in row 0
-        uint4 a[ROWS];
+        // EDGE: the slice reaches over an end of the chunk; its units there hold codes of the neighbouring chunk, or bytes that
+        // nobody wrote
+        auto count = [&](auto edge_c) {
+            constexpr bool EDGE = decltype(edge_c)::value;
+            uint4 a[ROWS];
 #pragma unroll
-        for (int r = 0; r < ROWS; ++r) {
-            const uint32_t e0 = 16 * (u0 + r * 32);
-            if (e0 >= cv.first && e0 + 16 <= cv.len) a[r] = __ldcs(reinterpret_cast<const uint4*>(dd.code) + u0 + r * 32);
-        }
+            for (int r = 0; r < ROWS; ++r) {
+                const uint32_t e0 = 16 * (u0 + r * 32);
+                if (EDGE) a[r] = make_uint4(0u, 0u, 0u, 0u);
+                if (!EDGE || (e0 + 16 > cv.first && e0 < cv.len)) a[r] = __ldcs(reinterpret_cast<const uint4*>(dd.code) + u0 + r * 32);
+            }
 #pragma unroll
-        for (int r = 0; r < ROWS; ++r) {
-            const uint32_t e0 = 16 * (u0 + r * 32);
-            bool f = false; // this lane holds an entry that is not below the interval
-            if (e0 >= cv.first && e0 + 16 <= cv.len) {
-                const uint32_t x[4] = {a[r].x, a[r].y, a[r].z, a[r].w};
+            for (int r = 0; r < ROWS; ++r) {
+                const uint32_t e0 = 16 * (u0 + r * 32);
+                bool f = false; // this lane holds an entry that is not below the interval
+                uint32_t in = 0xffffu; // elements of the unit that are the chunk's
+                uint32_t x[4] = {a[r].x, a[r].y, a[r].z, a[r].w};
+                if (EDGE) {
+                    if (e0 < cv.first) in = e0 + 16 > cv.first ? in & (~0u << (cv.first - e0)) : 0u;
+                    if (e0 + 16 > cv.len) in = e0 < cv.len ? in & ~(~0u << (cv.len - e0)) : 0u;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) x[j] &= 0x7f7f7f7fu;
+                }
                 uint32_t ge[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) ge[j] = (x[j] + add_ge) & 0x80808080u;
-                if (ge[0] | ge[1] | ge[2] | ge[3]) { // with a sparse budget few lanes hold a code that is not below the interval's
+                if ((ge[0] | ge[1] | ge[2] | ge[3]) && in) { // with a sparse budget few lanes hold a code that is not below the interval's
                     uint32_t hit = 0; // rare: the unit's entries with the interval's own code, bit k -> element k
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        const uint32_t gt = (x[j] + add_gt) & 0x80808080u;
+                        uint32_t gt = (x[j] + add_gt) & 0x80808080u, border = ge[j] ^ gt; // bit 8 k + 7 -> element k of this word
+                        if (EDGE) {
+                            const uint32_t v = in >> (4 * j), m = ((v & 1u) << 7) | ((v & 2u) << 14) | ((v & 4u) << 21) | ((v & 8u) << 28);
+                            gt &= m;
+                            border &= m;
+                        }
                         above += __popc(gt);
                         f |= gt != 0; // entries with the interval's code mark the group only if they are not below it
-                        const uint32_t border = ge[j] ^ gt; // bit 8 k + 7 -> element k of this word
                         hit |= (((border >> 7) & 1u) | ((border >> 14) & 2u) | ((border >> 21) & 4u) | ((border >> 28) & 8u)) << (4 * j);
                     }
                     while (hit) { // completed from the inputs two at a time: their loads are independent
@@ -169,20 +184,19 @@ k_sel_count(DSource dbuf, const Chunk* __restrict__ chunks, uint32_t n_chunks, u
                         if (p1 != p0) f |= visit(key_of(v1));
                     }
                 }
-            } else if (e0 < cv.len) { // ragged first or last unit of the chunk
-                for (uint32_t e = e0; e < e0 + 16; ++e)
-                    if (e >= cv.first && e < cv.len) f |= visit(key_of(dd.at(e)));
+                uint32_t m = __ballot_sync(0xffffffffu, f);
+                if (m) { // pairs of lanes -> 16 group bits of this row
+                    m = (m | (m >> 1)) & 0x55555555u;
+                    m = (m | (m >> 1)) & 0x33333333u;
+                    m = (m | (m >> 2)) & 0x0f0f0f0fu;
+                    m = (m | (m >> 4)) & 0x00ff00ffu;
+                    m = (m | (m >> 8)) & 0x0000ffffu;
+                    mask |= (uint64_t)m << (16 * r);
+                }
             }
-            uint32_t m = __ballot_sync(0xffffffffu, f);
-            if (m) { // pairs of lanes -> 16 group bits of this row
-                m = (m | (m >> 1)) & 0x55555555u;
-                m = (m | (m >> 1)) & 0x33333333u;
-                m = (m | (m >> 2)) & 0x0f0f0f0fu;
-                m = (m | (m >> 4)) & 0x00ff00ffu;
-                m = (m | (m >> 8)) & 0x0000ffffu;
-                mask |= (uint64_t)m << (16 * r);
-            }
-        }
+        };
+        if (sl * kSliceElems >= cv.first && (sl + 1) * kSliceElems <= cv.len) count(std::false_type{});
+        else count(std::true_type{});
 #pragma unroll
         for (int o = 16; o; o >>= 1) above += __shfl_xor_sync(0xffffffffu, above, o);
         if (lane == 0) { out->above[sl] = (uint16_t)above; out->eq[sl] = (uint16_t)(above >> 16); out->mask[sl] = mask; }
@@ -200,7 +214,8 @@ k_sel_count(DSource dbuf, const Chunk* __restrict__ chunks, uint32_t n_chunks, u
 // layer's threshold.  The whole CTA works on it.
 template <int NT>
 __device__ __forceinline__ void sel_scan_layer(const LayerDesc& ld, const Sel& s, const Chunk* __restrict__ chunks,
-                                               const ChunkSel* cs /* the layer's */, ChunkJob* __restrict__ jb, uint32_t* s_w) {
+                                               uint32_t phase, const ChunkSel* cs /* the layer's */, ChunkJob* __restrict__ jb,
+                                               uint32_t* s_w) {
     const bool all = (uint64_t)s.k == ld.n;
     uint32_t run_g = 0, run_e = 0;
     for (uint32_t base = 0; base < ld.n_chunks; base += NT) {
@@ -221,13 +236,13 @@ __device__ __forceinline__ void sel_scan_layer(const LayerDesc& ld, const Sel& s
         const uint32_t eg = block_excl_scan<uint32_t, NT>(g, s_w, &tg);
         const uint32_t ee = block_excl_scan<uint32_t, NT>(q, s_w, &te);
         if (i < ld.n_chunks) {
-            const ChunkView cv(chunks[ld.first_chunk + i]);
+            const ChunkView cv(chunks[ld.first_chunk + i], phase);
             ChunkJob j;
             j.tau = s.tau;
             j.keep_eq = s.keep_eq;
             j.gt_before = run_g + eg;
             j.eq_before = run_e + ee;
-            j.idx0 = (uint32_t)(cv.a0 - ld.begin);
+            j.idx0 = (uint32_t)(cv.a0 - phase - ld.begin);
             j.base = s.base;
             const bool none = s.k == 0 || (!all && g == 0 && (q == 0 || j.eq_before >= s.keep_eq));
             j.mode = none ? 0u : (all ? 2u : 1u);
@@ -246,7 +261,7 @@ template <int NT>
 __global__ void __launch_bounds__(NT)
 k_sel_offsets(const LayerDesc* __restrict__ layers, const Chunk* __restrict__ chunks, uint32_t n_chunks, uint32_t L,
               Sel* __restrict__ sel, ChunkSel* __restrict__ csel, ChunkJob* __restrict__ jobs, const Interval in, FbList* __restrict__ fb,
-              Recount* __restrict__ rc, uint2* __restrict__ rc_chunks, uint32_t list_cap, uint32_t w_base) {
+              Recount* __restrict__ rc, uint2* __restrict__ rc_chunks, uint32_t list_cap, const Phase phase, uint32_t w_base) {
     pdl_wait();
     __shared__ uint32_t s_w[NT / 32], s_h[256], s_digit, s_gt, s_at;
     __shared__ uint16_t s_key[kListCap];
@@ -347,13 +362,13 @@ k_sel_offsets(const LayerDesc* __restrict__ layers, const Chunk* __restrict__ ch
             return;
         }
     }
-    sel_scan_layer<NT>(ld, s, chunks, cs, jobs + (size_t)w * n_chunks + ld.first_chunk, s_w);
+    sel_scan_layer<NT>(ld, s, chunks, phase.at(w), cs, jobs + (size_t)w * n_chunks + ld.first_chunk, s_w);
 }
 
 // Exact per-slice (gt, eq) of the listed chunks: warp w recounts the slices w and w + 8.  The CTA that finishes the last
 // chunk of a layer makes the layer's job records (Interval::n counts the finished ones).
 __global__ void __launch_bounds__(kThreads)
-k_sel_recount(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* __restrict__ chunks, uint32_t n_chunks, uint64_t dstride,
+k_sel_recount(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* __restrict__ chunks, uint32_t n_chunks,
               uint32_t L, const Sel* __restrict__ sel, ChunkSel* __restrict__ csel, ChunkJob* __restrict__ jobs, const Interval in,
               const Recount* __restrict__ rc, const uint2* __restrict__ rc_chunks) {
     pdl_wait();
@@ -365,8 +380,8 @@ k_sel_recount(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* _
         const Chunk ch = chunks[e.y];
         const size_t wl = (size_t)e.x * L + ch.layer;
         const Sel s = sel[wl];
-        const ChunkView cv(ch);
-        const DView dd(dbuf, e.x, dstride, cv.a0);
+        const ChunkView cv(ch, dbuf.phase.at(e.x));
+        const DView dd(dbuf, e.x, cv.a0);
         ChunkSel* out = csel + (size_t)e.x * n_chunks + e.y;
         for (uint32_t sl = wid; sl < (uint32_t)kSlices; sl += kThreads / 32) {
             uint32_t gt = 0, eq = 0;
@@ -390,7 +405,7 @@ k_sel_recount(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* _
         __syncthreads();
         if (s_last) {
             __threadfence();
-            sel_scan_layer<kThreads>(ld, s, chunks, csel + (size_t)e.x * n_chunks + ld.first_chunk,
+            sel_scan_layer<kThreads>(ld, s, chunks, dbuf.phase.at(e.x), csel + (size_t)e.x * n_chunks + ld.first_chunk,
                                      jobs + (size_t)e.x * n_chunks + ld.first_chunk, s_w);
             if (threadIdx.x == 0) in.n[wl] = 0;
         }
@@ -407,7 +422,7 @@ k_sel_recount(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* _
 template <bool BF16, bool DENSE>
 __global__ void __launch_bounds__(kThreads, DENSE ? 3 : 8)
 k_sel_write(const float* __restrict__ grads, float* __restrict__ state, const Chunk* __restrict__ chunks,
-            uint32_t n_chunks, uint64_t dstride, uint64_t stride, const ChunkSel* __restrict__ csel,
+            uint32_t n_chunks, uint64_t stride, const Phase phase, const ChunkSel* __restrict__ csel,
             const ChunkJob* __restrict__ jobs, uint64_t cap, uint32_t* __restrict__ out_idx, void* __restrict__ out_val,
             uint32_t w_base) {
     pdl_wait();
@@ -419,10 +434,10 @@ k_sel_write(const float* __restrict__ grads, float* __restrict__ state, const Ch
     const bool all = jb.mode == 2;
     const uint32_t keep_eq = jb.keep_eq;
     const uint32_t tau = jb.tau;
-    const ChunkView cv(ch);
+    const ChunkView cv(ch, phase.at(w));
     // d is recomputed from the inputs; every element of the estimator is read before this kernel updates it
-    const float* gr = grads + (size_t)w * stride + cv.a0;
-    float* st = state + (size_t)w * stride + cv.a0;
+    const float* gr = grads + (size_t)w * stride + cv.a0 - phase.at(w);
+    float* st = state + (size_t)w * stride + cv.a0 - phase.at(w);
     uint32_t* oi = out_idx + (size_t)w * cap + jb.base;
     float* ov32 = reinterpret_cast<float*>(out_val) + (size_t)w * cap + jb.base;
     __nv_bfloat16* ov16 = reinterpret_cast<__nv_bfloat16*>(out_val) + (size_t)w * cap + jb.base;
