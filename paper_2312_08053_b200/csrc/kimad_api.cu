@@ -795,10 +795,10 @@ int kimad_apply_packed(const kimad_ctx* c, const kimad_packed* msg, float* est_d
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     const LayerDesc* layers = reinterpret_cast<const LayerDesc*>(c->ws + c->lay.layers);
     const dim3 grid(148 * 4, c->W);
-    if (c->value_dtype == 1)
-        k_apply_packed<true><<<grid, kThreads, 0, s>>>(msg->idx, msg->val, msg->offs, layers, c->L, c->cap, c->stride, est_dev);
-    else
-        k_apply_packed<false><<<grid, kThreads, 0, s>>>(msg->idx, msg->val, msg->offs, layers, c->L, c->cap, c->stride, est_dev);
+    auto launch = [&](auto kern) {
+        return launch_named("k_apply_packed", kern, grid, kThreads, 0, s, msg->idx, msg->val, msg->offs, layers, c->L, c->cap, c->stride, est_dev);
+    };
+    CUDA_TRY(c->value_dtype == 1 ? launch(k_apply_packed<true>) : launch(k_apply_packed<false>));
     CUDA_TRY(cudaGetLastError());
     return KIMAD_OK;
 }
@@ -815,10 +815,8 @@ int kimad_aggregate(float* x_dev, const float* est_dev, uint64_t stride, uint32_
                      (stride % 4 == 0);
     const uint64_t units = vec ? (n + 3) / 4 : n;
     const uint32_t grid = (uint32_t)std::min<uint64_t>((units + kThreads - 1) / kThreads, 148ull * 16);
-    if (vec)
-        k_aggregate<true><<<grid, kThreads, 0, s>>>(x_dev, est_dev, stride, n_workers, n, wt, gamma);
-    else
-        k_aggregate<false><<<grid, kThreads, 0, s>>>(x_dev, est_dev, stride, n_workers, n, wt, gamma);
+    auto launch = [&](auto kern) { return launch_named("k_aggregate", kern, grid, kThreads, 0, s, x_dev, est_dev, stride, n_workers, n, wt, gamma); };
+    CUDA_TRY(vec ? launch(k_aggregate<true>) : launch(k_aggregate<false>));
     CUDA_TRY(cudaGetLastError());
     return KIMAD_OK;
 }
