@@ -43,8 +43,12 @@ __device__ __forceinline__ uint32_t key_of(float d) { return __float_as_uint(d) 
 
 // Kernels launched with programmatic stream serialisation may be scheduled before their predecessor in the
 // stream has finished (which hides their launch latency); they wait here, before touching anything it wrote.
-// A no-op for an ordinary launch.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// A no-op for an ordinary launch.  From then on the next kernel in the stream may be scheduled as SMs come free: its CTAs
+// start and wait here in their turn, which takes most of a launch off every link of the chain.
+__device__ __forceinline__ void pdl_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 
 // Aligned view of a chunk for 128-bit loads of the inputs (quads of elements) and of the code plane (sixteen
 // codes): units start at a0 = begin & ~15; only the first and the last ones can be partial.  All offsets are
