@@ -156,7 +156,7 @@ constexpr uint64_t kPipelineMinElems = 1ull << 25; // W N from which a step is r
 static int preload_kernels() {
     cudaFuncAttributes a;
 #define KIMAD_PRELOAD(f) CUDA_TRY(cudaFuncGetAttributes(&a, f))
-    KIMAD_PRELOAD(k_sample); KIMAD_PRELOAD(k_pass_a<true>); KIMAD_PRELOAD(k_pass_a<false>); KIMAD_PRELOAD(k_resolve_a);
+    KIMAD_PRELOAD(k_sample); KIMAD_PRELOAD(k_pass_a<true>); KIMAD_PRELOAD(k_pass_a<false>); KIMAD_PRELOAD(k_resolve_a<true>); KIMAD_PRELOAD(k_resolve_a<false>);
     KIMAD_PRELOAD(k_refine); KIMAD_PRELOAD(k_tiny_exact); KIMAD_PRELOAD(k_fb1); KIMAD_PRELOAD(k_fb23<2>); KIMAD_PRELOAD(k_fb23<3>);
     KIMAD_PRELOAD(k_dp<2>); KIMAD_PRELOAD(k_dp<4>); KIMAD_PRELOAD(k_dp<8>); KIMAD_PRELOAD(k_pick); KIMAD_PRELOAD(k_fit_ratio); KIMAD_PRELOAD(k_sel_count);
     KIMAD_PRELOAD(k_sel_offsets<128>); KIMAD_PRELOAD(k_sel_offsets<512>); KIMAD_PRELOAD(k_sel_recount);
@@ -435,9 +435,15 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
         c->launches += 1;
         mark(big);
         CUDA_TRY(hand_over(big, small));
+        const ListArgs la{dbuf, layers, chunks, L, K, ktab, fb, rf, h1c, h1s, h23c, h23s, cands, slots, flags, err, tau, keq, shf, codes,
+                          c->at<uint32_t>(y.in_n)}; // (in_n counts the select stage's entries later in the step; zero in between)
+        const bool lists = c->most_chunks > (c->curve_mode == 1 ? kInlineChunksExact : kInlineChunks);
         if (R) {
-            CUDA_TRY(launch_pdl(k_resolve_a, dim3(R, nw), kBigThreads, 0, small, layers, reg_layers, R, L, ktab, K, meta, cell_win, binlo, bhc, bhs,
-                                err, tau, keq, shf, flags, fb, fb_chunks, rf, rf_chunks, list_cap, w0));
+            auto launch = [&](auto kern) {
+                return launch_named("k_resolve_a", kern, dim3(R, nw), kBigThreads, 0, small, layers, reg_layers, R, L, ktab, K, meta, cell_win,
+                                    binlo, bhc, bhs, err, tau, keq, shf, flags, fb, fb_chunks, rf, rf_chunks, list_cap, w0, la);
+            };
+            CUDA_TRY(lists ? launch(k_resolve_a<true>) : launch(k_resolve_a<false>));
             c->launches += 1;
         }
         if (T && join_late) CUDA_TRY(cudaStreamWaitEvent(small, c->ev_join, 0));
@@ -480,20 +486,15 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
             // the lists are usually empty, and a kernel of the chain then costs only its launch; four CTAs per SM are enough to
             // stream a large handed-over layer
             const uint32_t gfb = 4 * 148;
-            uint32_t* arrived = c->at<uint32_t>(y.in_n); // (counts the select stage's entries later in the step; zero in between)
             // candidates with a loose bound first (they may still end on the exact path's lists)
-            CUDA_TRY(launch_pdl(k_refine, 5 * 148, blk, 0, st, dbuf, layers, chunks, L, K, fb, rf_chunks, rf, codes, h23c, h23s,
-                                arrived, err, tau, keq, shf, fb_chunks, list_cap));
-            CUDA_TRY(launch_pdl(k_fb1, gfb, blk, 0, st, dbuf, layers, chunks, L, K, ktab, fb, fb_chunks, h1c, h1s, flags, codes,
-                                arrived, cands, slots));
-            CUDA_TRY(launch_pdl(k_fb23<2>, gfb, blk, 0, st, dbuf, layers, chunks, L, K, fb, fb_chunks, slots, cands, h23c, h23s,
-                                codes, arrived, err, tau, keq, shf));
-            CUDA_TRY(launch_pdl(k_fb23<3>, gfb, blk, 0, st, dbuf, layers, chunks, L, K, fb, fb_chunks, slots, cands, h23c, h23s,
-                                codes, arrived, err, tau, keq, shf));
+            CUDA_TRY(launch_pdl(k_refine, 5 * 148, blk, 0, st, la, rf_chunks, fb_chunks, list_cap));
+            CUDA_TRY(launch_pdl(k_fb1, gfb, blk, 0, st, la, fb_chunks));
+            CUDA_TRY(launch_pdl(k_fb23<2>, gfb, blk, 0, st, la, fb_chunks));
+            CUDA_TRY(launch_pdl(k_fb23<3>, gfb, blk, 0, st, la, fb_chunks));
             c->launches += 4;
             return KIMAD_OK;
         };
-        if (R && !c->timing) {
+        if (R && lists && !c->timing) {
             // The lists are usually empty, so the DP is launched at once and goes ahead only if they are; the four
             // list-driven kernels run beside it on a stream of their own, followed by a second launch of the DP that
             // goes ahead only if something was listed.  Their launch latencies leave the step's critical path.
@@ -506,7 +507,7 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
             CUDA_TRY(cudaEventRecord(c->ev_list[g][1], lst));
             CUDA_TRY(cudaStreamWaitEvent(small, c->ev_list[g][1], 0));
         } else {
-            if (R) { const int rc = launch_lists(small); if (rc != KIMAD_OK) return rc; }
+            if (R && lists) { const int rc = launch_lists(small); if (rc != KIMAD_OK) return rc; }
             mark(small);
             { const int rc = launch_dp(small, 0); if (rc != KIMAD_OK) return rc; }
         }

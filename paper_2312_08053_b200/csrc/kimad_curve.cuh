@@ -651,15 +651,411 @@ k_pass_a(const float* __restrict__ grads, const float* __restrict__ state, uint8
 }
 
 // ------------------------------------------------------------------------------------------------
+// The slow paths of a layer: refinement of loose candidates, exact radix select.  Both go over the layer's chunks and
+// end with a step that needs all of them.  Layers of large contexts are listed with their chunks (k_refine, k_fb1, k_fb23), which
+// costs every step four launches, a second launch of the DP and two event waits although the lists are usually empty.  Where no
+// layer has more than kInlineChunks chunks the curve kernel's CTA takes them itself (layer_by_itself): 62 tensors of up to
+// 147 K elements 116.5 -> 112 us a step, a small model through a built-in workspace 98 -> 86 us.  A layer that does need the
+// exact path costs 110 (list: 166) us with one chunk, 136 (166) with two, 197 (168) with four, 317 (172) with eight; hence the
+// second bound for contexts that take it always.
+// ------------------------------------------------------------------------------------------------
+constexpr uint32_t kInlineChunks = 8, kInlineChunksExact = 2;
+struct ListArgs {
+    DSource src;
+    const LayerDesc* layers;
+    const Chunk* chunks;
+    uint32_t L, K;
+    KTab ktab;
+    FbList* fb;
+    RefineCand* rf;     // [W][L][K]
+    uint32_t* h1_cnt;   // [W][R][kL1Bins]
+    unsigned long long* h1_ss;
+    uint32_t* h23_cnt;  // [W][R][K][kL23Bins]
+    unsigned long long* h23_ss;
+    Cand* cands;        // [W][L][K]
+    SlotTab* slots;     // [W][L]
+    uint32_t* flags;
+    float* err;         // [W][L][K], and the three below
+    uint32_t *tau, *keep_eq, *shift;
+    CodeSpace codes;
+    uint32_t* arrived;  // [W][L] finished chunks of a listed layer; zero in between
+};
+
+// ------------------------------------------------------------------------------------------------
+// Refinement of loose candidates: the bin that holds such a candidate's threshold is cut into up to 1024 pieces, and
+// the entries of the bin -- found by their code byte, completed from the inputs -- are counted and their squares
+// summed per piece (the level-2/3 arrays of the exact path serve as storage: a layer is never on both paths at once).
+// Costs one pass over the layer's code bytes instead of the exact path's three passes over its inputs.
+// ------------------------------------------------------------------------------------------------
+template <int NT>
+__device__ __forceinline__ void refine_chunk(const ListArgs& a, uint32_t w, const Chunk& ch, size_t wl, size_t wr) {
+    __shared__ uint32_t s_klo[KIMAD_MAX_RATIOS], s_shift[KIMAD_MAX_RATIOS], s_j[KIMAD_MAX_RATIOS];
+    __shared__ uint32_t s_mask[4]; // the 7-bit codes of the loose candidates' bins
+    __shared__ uint32_t s_n;
+    __syncthreads();
+    if (threadIdx.x < 4) s_mask[threadIdx.x] = 0;
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    if (threadIdx.x < 32) { // the layer's loose candidates in order of j, every bin once (under its lowest j); a lane each
+        const uint32_t lane = threadIdx.x;
+        uint32_t p = 0, last = 0; // bins so far, the last one's lower key
+        for (uint32_t j0 = 0; j0 < a.K; j0 += 32u) {
+            const uint32_t j = j0 + lane;
+            RefineCand r{0, kNoRefine, 0, 0, 0.0};
+            if (j < a.K) r = a.rf[wl * a.K + j];
+            const bool loose = r.shift != kNoRefine;
+            const uint32_t m = __ballot_sync(0xffffffffu, loose), before = m & ((1u << lane) - 1u);
+            const uint32_t left = __shfl_sync(0xffffffffu, r.klo, before ? 31 - __clz(before) : 0);
+            const bool first = loose && (before ? left != r.klo : (p == 0 || last != r.klo)); // thresholds descend with j
+            const uint32_t f = __ballot_sync(0xffffffffu, first);
+            if (first) {
+                const uint32_t at = p + __popc(f & ((1u << lane) - 1u));
+                s_klo[at] = r.klo; s_shift[at] = r.shift; s_j[at] = j;
+                const uint32_t code = a.codes.code(w, ch.layer, r.klo) & 127u;
+                atomicOr(&s_mask[code >> 5], 1u << (code & 31u));
+            }
+            if (m) last = __shfl_sync(0xffffffffu, r.klo, 31 - __clz(m));
+            p += __popc(f);
+        }
+        if (lane == 0) s_n = p;
+    }
+    __syncthreads();
+    const uint32_t nc = s_n;
+    const uint32_t m0 = s_mask[0], m1 = s_mask[1], m2 = s_mask[2], m3 = s_mask[3];
+    const ChunkView cv(ch, a.src.phase.at(w));
+    const DView dd(a.src, w, cv.a0);
+    const bool vec = ((reinterpret_cast<uintptr_t>(dd.gr) | reinterpret_cast<uintptr_t>(dd.st)) & 15u) == 0;
+    auto wanted = [&](uint32_t code) -> bool {
+        const uint32_t word = code < 64u ? (code < 32u ? m0 : m1) : (code < 96u ? m2 : m3);
+        return (word >> (code & 31u)) & 1u;
+    };
+    auto place = [&](uint32_t key) { // the entry's piece, if it lies in one of the loose bins
+        for (uint32_t p = 0; p < nc; ++p) {
+            const uint32_t d1 = key - s_klo[p], sh = s_shift[p];
+            if (d1 < (1u << sh)) {
+                const size_t at = (wr * a.K + s_j[p]) * kL23Bins + (d1 >> (sh > 10u ? sh - 10u : 0u));
+                atomicAdd(&a.h23_cnt[at], 1u);
+                atomicAdd(&a.h23_ss[at], (unsigned long long)sq_fixed(key));
+                break; // bins are disjoint; candidates that share a bin share a piece histogram (see refine_resolve_layer)
+            }
+        }
+    };
+    const uint32_t units = (cv.len + 15u) >> 4;
+    for (uint32_t u = threadIdx.x; u < units; u += NT) {
+        const uint32_t e0 = 16u * u;
+        uint32_t hit = 0; // the unit's elements whose code is one of the loose bins'
+        if (e0 + 16u > cv.first) { // (a unit at the chunk's edge holds codes of the neighbouring chunk, too)
+            const uint4 c4 = __ldcs(reinterpret_cast<const uint4*>(dd.code) + u);
+            const uint32_t x[4] = {c4.x, c4.y, c4.z, c4.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int b = 0; b < 4; ++b)
+                    if (wanted((x[i] >> (8 * b)) & 127u)) hit |= 1u << (4 * i + b);
+            if (e0 < cv.first) hit &= ~0u << (cv.first - e0);
+            if (e0 + 16u > cv.len) hit &= ~(~0u << (cv.len - e0));
+        }
+        if (!hit) continue;
+        // the unit's entries are completed from the inputs with independent loads: eight at a time
+        if (vec && e0 >= cv.first && e0 + 16u <= cv.len) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if (!((hit >> (8 * h)) & 255u)) continue;
+                const float4* g4 = reinterpret_cast<const float4*>(dd.gr + e0 + 8 * h);
+                const float4* t4 = reinterpret_cast<const float4*>(dd.st + e0 + 8 * h);
+                const float4 ga = __ldg(g4), gb = __ldg(g4 + 1), ta = __ldg(t4), tb = __ldg(t4 + 1);
+                const float v[8] = {__fsub_rn(ga.x, ta.x), __fsub_rn(ga.y, ta.y), __fsub_rn(ga.z, ta.z), __fsub_rn(ga.w, ta.w),
+                                    __fsub_rn(gb.x, tb.x), __fsub_rn(gb.y, tb.y), __fsub_rn(gb.z, tb.z), __fsub_rn(gb.w, tb.w)};
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if ((hit >> (8 * h + i)) & 1u) place(key_of(v[i]));
+            }
+        } else {
+            for (; hit; hit &= hit - 1u) place(key_of(dd.at(e0 + (uint32_t)__ffs(hit) - 1u)));
+        }
+    }
+}
+
+// The pieces of a layer's loose bins resolved; the loose candidates one after the other.  Candidates that share a bin were
+// counted into the histogram of the first of them (the lowest j): the later ones read it there.  True where a bound is still
+// too loose (a bin with very many entries): the layer needs the exact path after all.
+template <int NT>
+__device__ __forceinline__ bool refine_resolve_layer(const ListArgs& a, uint32_t l, uint32_t w, size_t wl, size_t wr) {
+    __shared__ uint32_t s_w32[NT / 32];
+    __shared__ double s_w64[NT / 32];
+    __shared__ int s_bad;
+    __syncthreads();
+    if (threadIdx.x == 0) s_bad = 0;
+    __syncthreads();
+    for (uint32_t j = 0; j < a.K; ++j) {
+        const RefineCand rc = a.rf[wl * a.K + j];
+        if (rc.shift == kNoRefine) continue;
+        uint32_t owner = j; // the first loose candidate with this bin holds the pieces
+        for (uint32_t i = 0; i < j; ++i) {
+            const RefineCand o = a.rf[wl * a.K + i];
+            if (o.shift != kNoRefine && o.klo == rc.klo) { owner = i; break; }
+        }
+        const uint32_t sub = rc.shift > 10u ? rc.shift - 10u : 0u, nsub = 1u << (rc.shift - sub);
+        const uint32_t* gc = a.h23_cnt + (wr * a.K + owner) * kL23Bins;
+        const unsigned long long* gs = a.h23_ss + (wr * a.K + owner) * kL23Bins;
+        const double scale = sq_scale(rc.klo >> 23);
+        // four consecutive pieces per thread, ascending keys
+        uint32_t c[4], csum = 0;
+        double q[4], qsum = 0.0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t b = 4 * threadIdx.x + i;
+            c[i] = b < nsub ? __ldcg(gc + b) : 0u;
+            q[i] = b < nsub ? (double)__ldcg(gs + b) * scale : 0.0;
+            csum += c[i];
+            qsum += q[i];
+        }
+        uint32_t tot;
+        uint32_t before = block_excl_scan<uint32_t, NT>(csum, s_w32, &tot);
+        double below = block_excl_scan<double, NT>(qsum, s_w64, nullptr);
+        if (!KIMAD_CHECK(tot == rc.cb, 7)) s_bad = 1;
+        const size_t o = wl * a.K + j;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (c[i] && rc.drop >= before && rc.drop - before < c[i]) { // the piece that holds the threshold
+                const uint32_t b = 4 * threadIdx.x + i, klo = rc.klo + (b << sub), d2 = rc.drop - before;
+                const double vlo = (double)__uint_as_float(klo);
+                const double upper = q[i] * ((double)d2 / (double)c[i]), lower = (double)d2 * vlo * vlo;
+                double part = 0.5 * (upper + lower), slack = 0.5 * (upper - lower);
+                if (d2 == 0 || sub == 0) { part = lower; slack = 0.0; }
+                const double e = rc.below + below + part;
+                if (slack > e * 5e-6) {
+                    s_bad = 1;
+                } else {
+                    a.err[o] = (float)e; a.tau[o] = klo; a.keep_eq[o] = c[i] - d2;
+                    a.shift[o] = sub | a.codes.code(w, l, klo) << 8;
+                }
+            }
+            before += c[i];
+            below += q[i];
+        }
+        __syncthreads();
+    }
+    // clean the pieces, close the candidates
+    for (uint32_t j = 0; j < a.K; ++j) {
+        if (a.rf[wl * a.K + j].shift == kNoRefine) continue;
+        for (uint32_t b = threadIdx.x; b < (uint32_t)kL23Bins; b += NT) {
+            a.h23_cnt[(wr * a.K + j) * kL23Bins + b] = 0;
+            a.h23_ss[(wr * a.K + j) * kL23Bins + b] = 0ull;
+        }
+    }
+    __syncthreads();
+    for (uint32_t j = threadIdx.x; j < a.K; j += NT) a.rf[wl * a.K + j].shift = kNoRefine;
+    return s_bad != 0;
+}
+
+// ------------------------------------------------------------------------------------------------
+// exact radix path over the handed-over chunks.  The list is usually empty, but a handed-over layer may be large and
+// may hold one key millions of times (the exact zeros of a sparse gradient): every thread therefore adds up the run
+// of consecutive elements of its own that fall into one bin and issues its atomics when the bin changes, and keeps
+// four elements' loads in flight.
+// ------------------------------------------------------------------------------------------------
+constexpr int kFbAhead = 4; // elements per thread whose loads are issued together
+
+// s_cnt, s_below [kL1Bins]; s_below holds the two words of the chunk's sums
+template <int NT>
+__device__ __forceinline__ void fb1_chunk(const ListArgs& a, uint32_t w, const Chunk& ch, size_t wr, uint32_t* s_cnt, double* s_below) {
+    uint32_t *s_hi = reinterpret_cast<uint32_t*>(s_below), *s_lo = s_hi + kL1Bins;
+    __syncthreads(); // (the arrays may still be read from the chunk or layer before)
+    const ChunkView cv(ch, a.src.phase.at(w));
+    const DView dd(a.src, w, cv.a0);
+    for (int b = threadIdx.x; b < kL1Bins; b += NT) { s_cnt[b] = 0; s_hi[b] = 0; s_lo[b] = 0; }
+    __syncthreads();
+    // a thread sees at most kChunkElems / NT elements of a chunk: its two partial sums stay below 2^32
+    uint32_t cur = 0, cn = 0, chi = 0, clo = 0;
+    bool nonfinite = false;
+    auto flush = [&]() {
+        if (cn) { atomicAdd(&s_cnt[cur], cn); atomicAdd(&s_hi[cur], chi); atomicAdd(&s_lo[cur], clo); }
+    };
+    for (uint32_t x0 = cv.first + threadIdx.x; x0 < cv.len; x0 += kFbAhead * NT) {
+        float v[kFbAhead];
+#pragma unroll
+        for (int u = 0; u < kFbAhead; ++u) v[u] = x0 + u * NT < cv.len ? dd.at(x0 + u * NT) : 0.f;
+#pragma unroll
+        for (int u = 0; u < kFbAhead; ++u) {
+            if (x0 + u * NT >= cv.len) break;
+            const uint32_t key = key_of(v[u]);
+            const uint32_t sq = (uint32_t)sq_fixed(key);
+            if ((key >> 20) != cur) { flush(); cur = key >> 20; cn = 0; chi = 0; clo = 0; }
+            ++cn; chi += sq >> 16; clo += sq & 0xffffu;
+            nonfinite |= key >= 0x7f800000u;
+        }
+    }
+    flush();
+    if (nonfinite) atomicOr(&a.flags[w], 1u);
+    __syncthreads();
+    uint32_t* gc = a.h1_cnt + wr * kL1Bins;
+    unsigned long long* gs = a.h1_ss + wr * kL1Bins;
+    for (int b = threadIdx.x; b < kL1Bins; b += NT)
+        if (s_cnt[b]) {
+            atomicAdd(&gc[b], s_cnt[b]);
+            atomicAdd(&gs[b], ((unsigned long long)s_hi[b] << 16) + s_lo[b]);
+        }
+}
+
+template <int LEVEL, int NT>
+__device__ __forceinline__ void fb23_chunk(const ListArgs& a, uint32_t w, const Chunk& ch, size_t wl, size_t wr) {
+    __shared__ uint8_t s_first[kL1Bins]; // level-1 bin -> first slot whose prefix starts with it (0xff: none)
+    __shared__ uint8_t s_num[kL1Bins];   // ... and how many consecutive slots share that bin (level 3)
+    __shared__ uint32_t s_prefix[KIMAD_MAX_RATIOS];
+    __syncthreads(); // (they may still be read from the chunk before)
+    const SlotTab& stab = a.slots[wl];
+    const uint32_t ns = stab.n;
+    for (int b = threadIdx.x; b < kL1Bins; b += NT) { s_first[b] = 0xff; s_num[b] = 0; }
+    for (uint32_t s = threadIdx.x; s < ns; s += NT) s_prefix[s] = stab.prefix[s];
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (uint32_t s = 0; s < ns; ++s) {
+            const uint32_t b1 = LEVEL == 2 ? s_prefix[s] : (s_prefix[s] >> 10);
+            if (s_first[b1] == 0xff) s_first[b1] = (uint8_t)s;
+            s_num[b1]++;
+        }
+    __syncthreads();
+    const ChunkView cv(ch, a.src.phase.at(w));
+    const DView dd(a.src, w, cv.a0);
+    uint32_t* gc = a.h23_cnt + wr * a.K * kL23Bins;
+    unsigned long long* gs = a.h23_ss + wr * a.K * kL23Bins;
+    uint32_t cur = 0xffffffffu, cn = 0; // (slot, bin) of the thread's current run, its entries and squares
+    unsigned long long csq = 0;
+    auto flush = [&]() {
+        if (cn) {
+            atomicAdd(&gc[cur], cn);
+            if (LEVEL == 2) atomicAdd(&gs[cur], csq);
+        }
+    };
+    for (uint32_t x0 = cv.first + threadIdx.x; x0 < cv.len; x0 += kFbAhead * NT) {
+        float v[kFbAhead];
+#pragma unroll
+        for (int u = 0; u < kFbAhead; ++u) v[u] = x0 + u * NT < cv.len ? dd.at(x0 + u * NT) : 0.f;
+#pragma unroll
+        for (int u = 0; u < kFbAhead; ++u) {
+            if (x0 + u * NT >= cv.len) break;
+            const uint32_t key = key_of(v[u]);
+            const uint32_t f = s_first[key >> 20];
+            if (f == 0xff) continue;
+            uint32_t at = 0xffffffffu;
+            if (LEVEL == 2) {
+                at = f * (uint32_t)kL23Bins + ((key >> 10) & 1023u);
+            } else {
+                const uint32_t nn = s_num[key >> 20], p21 = key >> 10;
+                for (uint32_t s = f; s < f + nn; ++s)
+                    if (s_prefix[s] == p21) { at = s * (uint32_t)kL23Bins + (key & 1023u); break; }
+                if (at == 0xffffffffu) continue;
+            }
+            if (at != cur) { flush(); cur = at; cn = 0; csq = 0; }
+            ++cn;
+            if (LEVEL == 2) csq += (unsigned long long)sq_fixed(key);
+        }
+    }
+    flush();
+}
+
+template <int LEVEL, int NT>
+__device__ __forceinline__ void fb23_resolve(const ListArgs& a, uint32_t l, uint32_t w, size_t wl, size_t wr) {
+    fb_resolve23_layer<LEVEL, NT>(l, w, wl, wr, a.K, a.h23_cnt, a.h23_ss, a.cands, a.slots, a.err, a.tau, a.keep_eq, a.shift, a.codes);
+}
+
+// All of it for one layer, by one CTA of kBigThreads threads.  exact: the exact path at once, else the refinement first.
+__device__ __noinline__ void layer_by_itself(const ListArgs& a, uint32_t l, uint32_t w, bool exact) {
+    constexpr int NT = kBigThreads;
+    __shared__ __align__(16) uint32_t s_cnt[kL1Bins];
+    __shared__ __align__(16) double s_below[kL1Bins];
+    __shared__ uint32_t s_w32[NT / 32];
+    __shared__ double s_w64[NT / 32];
+    const LayerDesc ld = a.layers[l];
+    const size_t wl = (size_t)w * a.L + l, wr = a.codes.slot(w, l);
+    auto each_chunk = [&](auto f) {
+        for (uint32_t i = 0; i < ld.n_chunks; ++i) f(a.chunks[ld.first_chunk + i]);
+        __threadfence();
+        __syncthreads();
+    };
+    if (!exact) {
+        each_chunk([&](const Chunk& ch) { refine_chunk<NT>(a, w, ch, wl, wr); });
+        if (!refine_resolve_layer<NT>(a, l, w, wl, wr)) return;
+        if (threadIdx.x == 0) { atomicAdd(&a.fb->total_layers, 1u); atomicAdd(&a.fb->why[3], 1u); }
+    }
+    each_chunk([&](const Chunk& ch) { fb1_chunk<NT>(a, w, ch, wr, s_cnt, s_below); });
+    fb_resolve1_layer<NT>(l, w, wl, wr, a.K, a.h1_cnt, a.h1_ss, a.ktab, a.cands, a.slots, s_cnt, s_below, s_w32, s_w64);
+    each_chunk([&](const Chunk& ch) { fb23_chunk<2, NT>(a, w, ch, wl, wr); });
+    fb23_resolve<2, NT>(a, l, w, wl, wr);
+    each_chunk([&](const Chunk& ch) { fb23_chunk<3, NT>(a, w, ch, wl, wr); });
+    fb23_resolve<3, NT>(a, l, w, wl, wr);
+}
+
+__global__ void __launch_bounds__(kThreads, 5)
+k_refine(const ListArgs a, const uint2* __restrict__ rf_chunks, uint2* __restrict__ fb_chunks, uint32_t list_cap) {
+    pdl_wait();
+    __shared__ uint32_t s_at;
+    const uint32_t n = a.fb->rf_chunks;
+    for (uint32_t it = blockIdx.x; it < n; it += gridDim.x) {
+        const uint2 e = rf_chunks[it];
+        const Chunk ch = a.chunks[e.y];
+        const LayerDesc ld = a.layers[ch.layer];
+        const size_t wl = (size_t)e.x * a.L + ch.layer, wr = a.codes.slot(e.x, ch.layer);
+        refine_chunk<kThreads>(a, e.x, ch, wl, wr);
+        if (last_of_layer(a.arrived + wl, ld.n_chunks) && refine_resolve_layer<kThreads>(a, ch.layer, e.x, wl, wr)) { // to the exact path after all
+            if (threadIdx.x == 0) {
+                s_at = atomicAdd(&a.fb->n_chunks, ld.n_chunks);
+                atomicAdd(&a.fb->n_layers, 1u);
+                atomicAdd(&a.fb->total_layers, 1u);
+                atomicAdd(&a.fb->why[3], 1u);
+            }
+            __syncthreads();
+            for (uint32_t i = threadIdx.x; i < ld.n_chunks; i += kThreads)
+                if (KIMAD_CHECK(s_at + i < list_cap, 2)) fb_chunks[s_at + i] = make_uint2(e.x, ld.first_chunk + i);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kThreads)
+k_fb1(const ListArgs a, const uint2* __restrict__ fb_chunks) {
+    pdl_wait();
+    __shared__ __align__(16) uint32_t s_cnt[kL1Bins];
+    __shared__ __align__(16) double s_below[kL1Bins];
+    __shared__ uint32_t s_w32[8];
+    __shared__ double s_w64[8];
+    const uint32_t n = a.fb->n_chunks;
+    for (uint32_t it = blockIdx.x; it < n; it += gridDim.x) {
+        const uint2 e = fb_chunks[it];
+        const Chunk ch = a.chunks[e.y];
+        const size_t wl = (size_t)e.x * a.L + ch.layer, wr = a.codes.slot(e.x, ch.layer);
+        fb1_chunk<kThreads>(a, e.x, ch, wr, s_cnt, s_below);
+        if (last_of_layer(a.arrived + wl, a.layers[ch.layer].n_chunks))
+            fb_resolve1_layer<kThreads>(ch.layer, e.x, wl, wr, a.K, a.h1_cnt, a.h1_ss, a.ktab, a.cands, a.slots, s_cnt, s_below, s_w32, s_w64);
+    }
+}
+
+template <int LEVEL>
+__global__ void __launch_bounds__(kThreads)
+k_fb23(const ListArgs a, const uint2* __restrict__ fb_chunks) {
+    pdl_wait();
+    const uint32_t n = a.fb->n_chunks;
+    for (uint32_t it = blockIdx.x; it < n; it += gridDim.x) {
+        const uint2 e = fb_chunks[it];
+        const Chunk ch = a.chunks[e.y];
+        const size_t wl = (size_t)e.x * a.L + ch.layer, wr = a.codes.slot(e.x, ch.layer);
+        fb23_chunk<LEVEL, kThreads>(a, e.x, ch, wl, wr);
+        if (last_of_layer(a.arrived + wl, a.layers[ch.layer].n_chunks)) fb23_resolve<LEVEL, kThreads>(a, ch.layer, e.x, wl, wr);
+    }
+}
+
+// ------------------------------------------------------------------------------------------------
 // k_resolve_a: one CTA per (regular layer, worker)
 // ------------------------------------------------------------------------------------------------
+template <bool LISTS> // false: no layer has more than kInlineChunks chunks; the slow paths are taken here
 __global__ void __launch_bounds__(kBigThreads)
 k_resolve_a(const LayerDesc* __restrict__ layers, const uint32_t* __restrict__ reg_layers, uint32_t R, uint32_t L,
             const KTab ktab, uint32_t K, const BandMeta* __restrict__ meta, const int4* __restrict__ cell_win,
             const uint32_t* __restrict__ bin_lo, uint32_t* __restrict__ bh_cnt, unsigned long long* __restrict__ bh_sum,
             float* __restrict__ err_out, uint32_t* __restrict__ tau_out, uint32_t* __restrict__ rank_out,
             uint32_t* __restrict__ shift_out, uint32_t* __restrict__ flags, FbList* __restrict__ fb,
-            uint2* __restrict__ fb_chunks, RefineCand* __restrict__ rf, uint2* __restrict__ rf_chunks, uint32_t list_cap, uint32_t w_base) {
+            uint2* __restrict__ fb_chunks, RefineCand* __restrict__ rf, uint2* __restrict__ rf_chunks, uint32_t list_cap, uint32_t w_base,
+            const __grid_constant__ ListArgs la) {
     pdl_wait();
     __shared__ uint32_t s_drop[KIMAD_MAX_RATIOS]; // entries not kept by candidate j: n - k_j
     __shared__ int s_loose;
@@ -781,6 +1177,15 @@ k_resolve_a(const LayerDesc* __restrict__ layers, const uint32_t* __restrict__ r
     __syncthreads();
     const int bad = s_bad;
     __shared__ uint32_t s_at;
+    if constexpr (!LISTS) {
+        if (!bad && !s_loose) return;
+        if (threadIdx.x == 0) {
+            if (bad) { atomicAdd(&fb->total_layers, 1u); atomicAdd(&fb->why[bad - 1], 1u); }
+            else atomicAdd(&fb->refined, 1u);
+        }
+        layer_by_itself(la, l, w, bad != 0);
+        return;
+    }
     if (bad) { // hand the layer and its chunks to the exact path
         if (threadIdx.x == 0) {
             s_at = atomicAdd(&fb->n_chunks, ld.n_chunks);
@@ -800,204 +1205,6 @@ k_resolve_a(const LayerDesc* __restrict__ layers, const uint32_t* __restrict__ r
         __syncthreads();
         for (uint32_t i = threadIdx.x; i < ld.n_chunks; i += kBigThreads)
             if (KIMAD_CHECK(s_at + i < list_cap, 2)) rf_chunks[s_at + i] = make_uint2(w, ld.first_chunk + i);
-    }
-}
-
-// ------------------------------------------------------------------------------------------------
-// Refinement of loose candidates: the bin that holds such a candidate's threshold is cut into up to 1024 pieces, and
-// the entries of the bin -- found by their code byte, completed from the inputs -- are counted and their squares
-// summed per piece (the level-2/3 arrays of the exact path serve as storage: a layer is never on both paths at once).
-// Costs one pass over the layer's code bytes instead of the exact path's three passes over its inputs.
-// ------------------------------------------------------------------------------------------------
-// The pieces of a layer's loose bins resolved, by the CTA that counted the last of its chunks; the loose candidates one after
-// the other.  Candidates that share a bin were counted into the histogram of the first of them (the lowest j): the later
-// ones read it there.
-__device__ __forceinline__ void refine_resolve_layer(uint32_t l, uint32_t w, size_t wl, size_t wr, const LayerDesc* __restrict__ layers,
-                                                     uint32_t K, FbList* __restrict__ fb, RefineCand* __restrict__ rf,
-                                                     uint32_t* __restrict__ g_cnt, unsigned long long* __restrict__ g_ss,
-                                                     float* __restrict__ err_out, uint32_t* __restrict__ tau_out,
-                                                     uint32_t* __restrict__ rank_out, uint32_t* __restrict__ shift_out,
-                                                     const CodeSpace& codes, uint2* __restrict__ fb_chunks, uint32_t list_cap) {
-    __shared__ uint32_t s_w32[8];
-    __shared__ double s_w64[8];
-    __shared__ int s_bad;
-    __shared__ uint32_t s_at;
-            __syncthreads();
-            if (threadIdx.x == 0) s_bad = 0;
-            __syncthreads();
-            for (uint32_t j = 0; j < K; ++j) {
-                const RefineCand rc = rf[wl * K + j];
-                if (rc.shift == kNoRefine) continue;
-                uint32_t owner = j; // the first loose candidate with this bin holds the pieces
-                for (uint32_t i = 0; i < j; ++i) {
-                    const RefineCand o = rf[wl * K + i];
-                    if (o.shift != kNoRefine && o.klo == rc.klo) { owner = i; break; }
-                }
-                const uint32_t sub = rc.shift > 10u ? rc.shift - 10u : 0u, nsub = 1u << (rc.shift - sub);
-                const uint32_t* gc = g_cnt + (wr * K + owner) * kL23Bins;
-                const unsigned long long* gs = g_ss + (wr * K + owner) * kL23Bins;
-                const double scale = sq_scale(rc.klo >> 23);
-                // four consecutive pieces per thread, ascending keys
-                uint32_t c[4], csum = 0;
-                double q[4], qsum = 0.0;
-    #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const uint32_t b = 4 * threadIdx.x + i;
-                    c[i] = b < nsub ? __ldcg(gc + b) : 0u;
-                    q[i] = b < nsub ? (double)__ldcg(gs + b) * scale : 0.0;
-                    csum += c[i];
-                    qsum += q[i];
-                }
-                uint32_t tot;
-                uint32_t before = block_excl_scan<uint32_t>(csum, s_w32, &tot);
-                double below = block_excl_scan<double>(qsum, s_w64, nullptr);
-                if (!KIMAD_CHECK(tot == rc.cb, 7)) s_bad = 1;
-                const size_t o = wl * K + j;
-    #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    if (c[i] && rc.drop >= before && rc.drop - before < c[i]) { // the piece that holds the threshold
-                        const uint32_t b = 4 * threadIdx.x + i, klo = rc.klo + (b << sub), d2 = rc.drop - before;
-                        const double vlo = (double)__uint_as_float(klo);
-                        const double upper = q[i] * ((double)d2 / (double)c[i]), lower = (double)d2 * vlo * vlo;
-                        double part = 0.5 * (upper + lower), slack = 0.5 * (upper - lower);
-                        if (d2 == 0 || sub == 0) { part = lower; slack = 0.0; }
-                        const double e = rc.below + below + part;
-                        if (slack > e * 5e-6) {
-                            s_bad = 1;
-                        } else {
-                            err_out[o] = (float)e; tau_out[o] = klo; rank_out[o] = c[i] - d2;
-                            shift_out[o] = sub | codes.code(w, l, klo) << 8;
-                        }
-                    }
-                    before += c[i];
-                    below += q[i];
-                }
-                __syncthreads();
-            }
-            // clean the pieces, close the candidates
-            for (uint32_t j = 0; j < K; ++j) {
-                if (rf[wl * K + j].shift == kNoRefine) continue;
-                for (uint32_t b = threadIdx.x; b < (uint32_t)kL23Bins; b += kThreads) {
-                    g_cnt[(wr * K + j) * kL23Bins + b] = 0;
-                    g_ss[(wr * K + j) * kL23Bins + b] = 0ull;
-                }
-            }
-            __syncthreads();
-            for (uint32_t j = threadIdx.x; j < K; j += kThreads) rf[wl * K + j].shift = kNoRefine;
-            if (s_bad) { // still too loose (a bin with very many entries): the exact path after all
-                const LayerDesc ld = layers[l];
-                if (threadIdx.x == 0) {
-                    s_at = atomicAdd(&fb->n_chunks, ld.n_chunks);
-                    atomicAdd(&fb->n_layers, 1u);
-                    atomicAdd(&fb->total_layers, 1u);
-                    atomicAdd(&fb->why[3], 1u);
-                }
-                __syncthreads();
-                for (uint32_t i = threadIdx.x; i < ld.n_chunks; i += kThreads)
-                    if (KIMAD_CHECK(s_at + i < list_cap, 2)) fb_chunks[s_at + i] = make_uint2(w, ld.first_chunk + i);
-            }
-}
-
-__global__ void __launch_bounds__(kThreads, 5)
-k_refine(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* __restrict__ chunks, uint32_t L, uint32_t K,
-         FbList* __restrict__ fb, const uint2* __restrict__ rf_chunks, RefineCand* __restrict__ rf,
-         const CodeSpace codes, uint32_t* __restrict__ g_cnt, unsigned long long* __restrict__ g_ss, uint32_t* __restrict__ arrived,
-         float* __restrict__ err_out, uint32_t* __restrict__ tau_out, uint32_t* __restrict__ rank_out, uint32_t* __restrict__ shift_out,
-         uint2* __restrict__ fb_chunks, uint32_t list_cap) {
-    pdl_wait();
-    __shared__ uint32_t s_klo[KIMAD_MAX_RATIOS], s_shift[KIMAD_MAX_RATIOS], s_j[KIMAD_MAX_RATIOS];
-    __shared__ uint32_t s_mask[4]; // the 7-bit codes of the loose candidates' bins
-    __shared__ uint32_t s_n;
-    const uint32_t n = fb->rf_chunks;
-    for (uint32_t it = blockIdx.x; it < n; it += gridDim.x) {
-        const uint2 e = rf_chunks[it];
-        const Chunk ch = chunks[e.y];
-        const size_t wl = (size_t)e.x * L + ch.layer, wr = codes.slot(e.x, ch.layer);
-        __syncthreads();
-        if (threadIdx.x < 4) s_mask[threadIdx.x] = 0;
-        if (threadIdx.x == 0) s_n = 0;
-        __syncthreads();
-        if (threadIdx.x < 32) { // the layer's loose candidates in order of j, every bin once (under its lowest j); a lane each
-            const uint32_t lane = threadIdx.x;
-            uint32_t p = 0, last = 0; // bins so far, the last one's lower key
-            for (uint32_t j0 = 0; j0 < K; j0 += 32u) {
-                const uint32_t j = j0 + lane;
-                RefineCand r{0, kNoRefine, 0, 0, 0.0};
-                if (j < K) r = rf[wl * K + j];
-                const bool loose = r.shift != kNoRefine;
-                const uint32_t m = __ballot_sync(0xffffffffu, loose), before = m & ((1u << lane) - 1u);
-                const uint32_t left = __shfl_sync(0xffffffffu, r.klo, before ? 31 - __clz(before) : 0);
-                const bool first = loose && (before ? left != r.klo : (p == 0 || last != r.klo)); // thresholds descend with j
-                const uint32_t f = __ballot_sync(0xffffffffu, first);
-                if (first) {
-                    const uint32_t at = p + __popc(f & ((1u << lane) - 1u));
-                    s_klo[at] = r.klo; s_shift[at] = r.shift; s_j[at] = j;
-                    const uint32_t code = codes.code(e.x, ch.layer, r.klo) & 127u;
-                    atomicOr(&s_mask[code >> 5], 1u << (code & 31u));
-                }
-                if (m) last = __shfl_sync(0xffffffffu, r.klo, 31 - __clz(m));
-                p += __popc(f);
-            }
-            if (lane == 0) s_n = p;
-        }
-        __syncthreads();
-        const uint32_t nc = s_n;
-        const uint32_t m0 = s_mask[0], m1 = s_mask[1], m2 = s_mask[2], m3 = s_mask[3];
-        const ChunkView cv(ch, dbuf.phase.at(e.x));
-        const DView dd(dbuf, e.x, cv.a0);
-        const bool vec = ((reinterpret_cast<uintptr_t>(dd.gr) | reinterpret_cast<uintptr_t>(dd.st)) & 15u) == 0;
-        auto wanted = [&](uint32_t code) -> bool {
-            const uint32_t word = code < 64u ? (code < 32u ? m0 : m1) : (code < 96u ? m2 : m3);
-            return (word >> (code & 31u)) & 1u;
-        };
-        auto place = [&](uint32_t key) { // the entry's piece, if it lies in one of the loose bins
-            for (uint32_t p = 0; p < nc; ++p) {
-                const uint32_t d1 = key - s_klo[p], sh = s_shift[p];
-                if (d1 < (1u << sh)) {
-                    const size_t at = (wr * K + s_j[p]) * kL23Bins + (d1 >> (sh > 10u ? sh - 10u : 0u));
-                    atomicAdd(&g_cnt[at], 1u);
-                    atomicAdd(&g_ss[at], (unsigned long long)sq_fixed(key));
-                    break; // bins are disjoint; candidates that share a bin share a piece histogram (see refine_resolve_layer)
-                }
-            }
-        };
-        const uint32_t units = (cv.len + 15u) >> 4;
-        for (uint32_t u = threadIdx.x; u < units; u += kThreads) {
-            const uint32_t e0 = 16u * u;
-            uint32_t hit = 0; // the unit's elements whose code is one of the loose bins' codes
-            if (e0 + 16u > cv.first) { // (a unit at the chunk's edge holds codes of the neighbouring chunk, too)
-                const uint4 a = __ldcs(reinterpret_cast<const uint4*>(dd.code) + u);
-                const uint32_t x[4] = {a.x, a.y, a.z, a.w};
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int b = 0; b < 4; ++b)
-                        if (wanted((x[i] >> (8 * b)) & 127u)) hit |= 1u << (4 * i + b);
-                if (e0 < cv.first) hit &= ~0u << (cv.first - e0);
-                if (e0 + 16u > cv.len) hit &= ~(~0u << (cv.len - e0));
-            }
-            if (!hit) continue;
-            // the unit's entries are completed from the inputs with independent loads: eight at a time
-            if (vec && e0 >= cv.first && e0 + 16u <= cv.len) {
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    if (!((hit >> (8 * h)) & 255u)) continue;
-                    const float4* g4 = reinterpret_cast<const float4*>(dd.gr + e0 + 8 * h);
-                    const float4* t4 = reinterpret_cast<const float4*>(dd.st + e0 + 8 * h);
-                    const float4 ga = __ldg(g4), gb = __ldg(g4 + 1), ta = __ldg(t4), tb = __ldg(t4 + 1);
-                    const float v[8] = {__fsub_rn(ga.x, ta.x), __fsub_rn(ga.y, ta.y), __fsub_rn(ga.z, ta.z), __fsub_rn(ga.w, ta.w),
-                                        __fsub_rn(gb.x, tb.x), __fsub_rn(gb.y, tb.y), __fsub_rn(gb.z, tb.z), __fsub_rn(gb.w, tb.w)};
-#pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        if ((hit >> (8 * h + i)) & 1u) place(key_of(v[i]));
-                }
-            } else {
-                for (; hit; hit &= hit - 1u) place(key_of(dd.at(e0 + (uint32_t)__ffs(hit) - 1u)));
-            }
-        }
-        if (last_of_layer(arrived + wl, layers[ch.layer].n_chunks))
-            refine_resolve_layer(ch.layer, e.x, wl, wr, layers, K, fb, rf, g_cnt, g_ss, err_out, tau_out, rank_out, shift_out, codes,
-                                 fb_chunks, list_cap);
     }
 }
 
@@ -1159,140 +1366,6 @@ k_tiny_exact(const float* __restrict__ grads, const float* __restrict__ state, u
         tau_out[o] = t;
         rank_out[o] = k - (uint32_t)lo;
         shift_out[o] = code_of_key(t) << 8;
-    }
-}
-
-// ------------------------------------------------------------------------------------------------
-// exact radix path over the handed-over chunks.  The list is usually empty, but a handed-over layer may be large and
-// may hold one key millions of times (the exact zeros of a sparse gradient): every thread therefore adds up the run
-// of consecutive elements of its own that fall into one bin and issues its atomics when the bin changes, and keeps
-// four elements' loads in flight.
-// ------------------------------------------------------------------------------------------------
-constexpr int kFbAhead = 4; // elements per thread whose loads are issued together
-
-__global__ void __launch_bounds__(kThreads)
-k_fb1(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* __restrict__ chunks, uint32_t L, uint32_t K,
-      const KTab ktab, const FbList* __restrict__ fb, const uint2* __restrict__ fb_chunks, uint32_t* __restrict__ g_cnt,
-      unsigned long long* __restrict__ g_ss, uint32_t* __restrict__ flags, const CodeSpace codes, uint32_t* __restrict__ arrived,
-      Cand* __restrict__ cands, SlotTab* __restrict__ slots) {
-    pdl_wait();
-    __shared__ __align__(16) uint32_t s_cnt[kL1Bins];
-    __shared__ __align__(16) double s_below[kL1Bins]; // the two words of the chunk's sums, then the layer's squares
-    __shared__ uint32_t s_w32[8];
-    __shared__ double s_w64[8];
-    uint32_t *s_hi = reinterpret_cast<uint32_t*>(s_below), *s_lo = s_hi + kL1Bins;
-    const uint32_t n = fb->n_chunks;
-    for (uint32_t it = blockIdx.x; it < n; it += gridDim.x) {
-        const uint2 e = fb_chunks[it];
-        const Chunk ch = chunks[e.y];
-        const ChunkView cv(ch, dbuf.phase.at(e.x));
-        const DView dd(dbuf, e.x, cv.a0);
-        for (int b = threadIdx.x; b < kL1Bins; b += kThreads) { s_cnt[b] = 0; s_hi[b] = 0; s_lo[b] = 0; }
-        __syncthreads();
-        // a thread sees at most kChunkElems / kThreads elements of a chunk: its two partial sums stay below 2^32
-        uint32_t cur = 0, cn = 0, chi = 0, clo = 0;
-        bool nonfinite = false;
-        auto flush = [&]() {
-            if (cn) { atomicAdd(&s_cnt[cur], cn); atomicAdd(&s_hi[cur], chi); atomicAdd(&s_lo[cur], clo); }
-        };
-        for (uint32_t x0 = cv.first + threadIdx.x; x0 < cv.len; x0 += kFbAhead * kThreads) {
-            float v[kFbAhead];
-#pragma unroll
-            for (int u = 0; u < kFbAhead; ++u) v[u] = x0 + u * kThreads < cv.len ? dd.at(x0 + u * kThreads) : 0.f;
-#pragma unroll
-            for (int u = 0; u < kFbAhead; ++u) {
-                if (x0 + u * kThreads >= cv.len) break;
-                const uint32_t key = key_of(v[u]);
-                const uint32_t sq = (uint32_t)sq_fixed(key);
-                if ((key >> 20) != cur) { flush(); cur = key >> 20; cn = 0; chi = 0; clo = 0; }
-                ++cn; chi += sq >> 16; clo += sq & 0xffffu;
-                nonfinite |= key >= 0x7f800000u;
-            }
-        }
-        flush();
-        if (nonfinite) atomicOr(&flags[e.x], 1u);
-        __syncthreads();
-        const size_t wr = codes.slot(e.x, ch.layer);
-        uint32_t* gc = g_cnt + wr * kL1Bins;
-        unsigned long long* gs = g_ss + wr * kL1Bins;
-        for (int b = threadIdx.x; b < kL1Bins; b += kThreads)
-            if (s_cnt[b]) {
-                atomicAdd(&gc[b], s_cnt[b]);
-                atomicAdd(&gs[b], ((unsigned long long)s_hi[b] << 16) + s_lo[b]);
-            }
-        const size_t wl = (size_t)e.x * L + ch.layer;
-        if (last_of_layer(arrived + wl, layers[ch.layer].n_chunks))
-            fb_resolve1_layer(ch.layer, e.x, wl, wr, K, g_cnt, g_ss, ktab, cands, slots, s_cnt, s_below, s_w32, s_w64);
-    }
-}
-
-template <int LEVEL>
-__global__ void __launch_bounds__(kThreads)
-k_fb23(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* __restrict__ chunks, uint32_t L, uint32_t K,
-       const FbList* __restrict__ fb, const uint2* __restrict__ fb_chunks, SlotTab* __restrict__ slots, Cand* __restrict__ cands,
-       uint32_t* __restrict__ g_cnt, unsigned long long* __restrict__ g_ss, const CodeSpace codes, uint32_t* __restrict__ arrived,
-       float* __restrict__ err_out, uint32_t* __restrict__ tau_out, uint32_t* __restrict__ keep_eq_out, uint32_t* __restrict__ shift_out) {
-    pdl_wait();
-    __shared__ uint8_t s_first[kL1Bins]; // level-1 bin -> first slot whose prefix starts with it (0xff: none)
-    __shared__ uint8_t s_num[kL1Bins];   // ... and how many consecutive slots share that bin (level 3)
-    __shared__ uint32_t s_prefix[KIMAD_MAX_RATIOS];
-    const uint32_t n = fb->n_chunks;
-    for (uint32_t it = blockIdx.x; it < n; it += gridDim.x) {
-        const uint2 e = fb_chunks[it];
-        const Chunk ch = chunks[e.y];
-        const size_t wl = (size_t)e.x * L + ch.layer;
-        const SlotTab& stab = slots[wl];
-        const uint32_t ns = stab.n;
-        for (int b = threadIdx.x; b < kL1Bins; b += kThreads) { s_first[b] = 0xff; s_num[b] = 0; }
-        for (uint32_t s = threadIdx.x; s < ns; s += kThreads) s_prefix[s] = stab.prefix[s];
-        __syncthreads();
-        if (threadIdx.x == 0)
-            for (uint32_t s = 0; s < ns; ++s) {
-                const uint32_t b1 = LEVEL == 2 ? s_prefix[s] : (s_prefix[s] >> 10);
-                if (s_first[b1] == 0xff) s_first[b1] = (uint8_t)s;
-                s_num[b1]++;
-            }
-        __syncthreads();
-        const ChunkView cv(ch, dbuf.phase.at(e.x));
-        const DView dd(dbuf, e.x, cv.a0);
-        const size_t wr = codes.slot(e.x, ch.layer);
-        uint32_t* gc = g_cnt + wr * K * kL23Bins;
-        unsigned long long* gs = g_ss + wr * K * kL23Bins;
-        uint32_t cur = 0xffffffffu, cn = 0; // (slot, bin) of the thread's current run, its entries and squares
-        unsigned long long csq = 0;
-        auto flush = [&]() {
-            if (cn) {
-                atomicAdd(&gc[cur], cn);
-                if (LEVEL == 2) atomicAdd(&gs[cur], csq);
-            }
-        };
-        for (uint32_t x0 = cv.first + threadIdx.x; x0 < cv.len; x0 += kFbAhead * kThreads) {
-            float v[kFbAhead];
-#pragma unroll
-            for (int u = 0; u < kFbAhead; ++u) v[u] = x0 + u * kThreads < cv.len ? dd.at(x0 + u * kThreads) : 0.f;
-#pragma unroll
-            for (int u = 0; u < kFbAhead; ++u) {
-                if (x0 + u * kThreads >= cv.len) break;
-                const uint32_t key = key_of(v[u]);
-                const uint32_t f = s_first[key >> 20];
-                if (f == 0xff) continue;
-                uint32_t at = 0xffffffffu;
-                if (LEVEL == 2) {
-                    at = f * (uint32_t)kL23Bins + ((key >> 10) & 1023u);
-                } else {
-                    const uint32_t nn = s_num[key >> 20], p21 = key >> 10;
-                    for (uint32_t s = f; s < f + nn; ++s)
-                        if (s_prefix[s] == p21) { at = s * (uint32_t)kL23Bins + (key & 1023u); break; }
-                    if (at == 0xffffffffu) continue;
-                }
-                if (at != cur) { flush(); cur = at; cn = 0; csq = 0; }
-                ++cn;
-                if (LEVEL == 2) csq += (unsigned long long)sq_fixed(key);
-            }
-        }
-        flush();
-        if (last_of_layer(arrived + wl, layers[ch.layer].n_chunks))
-            fb_resolve23_layer<LEVEL>(ch.layer, e.x, wl, wr, K, g_cnt, g_ss, cands, slots, err_out, tau_out, keep_eq_out, shift_out, codes);
     }
 }
 

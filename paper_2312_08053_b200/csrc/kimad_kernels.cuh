@@ -167,26 +167,23 @@ __device__ __forceinline__ double sq_scale(uint32_t e) { // 2^(2 (max(e,1) - 150
 // ------------------------------------------------------------------------------------------------
 // In-place: on return s_incl[p] (p = position counted from the TOP bin, p = NB-1-bin) holds the
 // inclusive count of keys in bins >= that bin; s_below[bin] holds the sum of ss over bins < bin.
-template <int NB>
+template <int NB, int NT>
 __device__ __forceinline__ void scan_bins(uint32_t* s_incl /* in: counts by position */, double* s_below /* in: ss by bin */,
                                           uint32_t* s_w32, double* s_w64) {
-    constexpr int PER = NB / kThreads;
-    static_assert(PER % 4 == 0, "16-byte shared-memory accesses");
+    constexpr int PER = NB / NT;
+    static_assert(PER % 2 == 0, "8-byte shared-memory accesses");
     uint32_t loc[PER];
     uint32_t sum = 0;
-    uint4* v4 = reinterpret_cast<uint4*>(s_incl + threadIdx.x * PER);
+    uint2* v2 = reinterpret_cast<uint2*>(s_incl + threadIdx.x * PER);
 #pragma unroll
-    for (int i = 0; i < PER / 4; ++i) {
-        const uint4 t = v4[i];
-        loc[4 * i] = t.x; loc[4 * i + 1] = t.y; loc[4 * i + 2] = t.z; loc[4 * i + 3] = t.w;
-    }
+    for (int i = 0; i < PER / 2; ++i) { const uint2 t = v2[i]; loc[2 * i] = t.x; loc[2 * i + 1] = t.y; }
 #pragma unroll
     for (int i = 0; i < PER; ++i) sum += loc[i];
-    uint32_t ex = block_excl_scan<uint32_t>(sum, s_w32, nullptr);
+    uint32_t ex = block_excl_scan<uint32_t, NT>(sum, s_w32, nullptr);
 #pragma unroll
     for (int i = 0; i < PER; ++i) { ex += loc[i]; loc[i] = ex; }
 #pragma unroll
-    for (int i = 0; i < PER / 4; ++i) v4[i] = make_uint4(loc[4 * i], loc[4 * i + 1], loc[4 * i + 2], loc[4 * i + 3]);
+    for (int i = 0; i < PER / 2; ++i) v2[i] = make_uint2(loc[2 * i], loc[2 * i + 1]);
     if (s_below) {
         double dl[PER];
         double ds = 0.0;
@@ -195,7 +192,7 @@ __device__ __forceinline__ void scan_bins(uint32_t* s_incl /* in: counts by posi
         for (int i = 0; i < PER / 2; ++i) { const double2 t = d2[i]; dl[2 * i] = t.x; dl[2 * i + 1] = t.y; }
 #pragma unroll
         for (int i = 0; i < PER; ++i) ds += dl[i];
-        double de = block_excl_scan<double>(ds, s_w64, nullptr);
+        double de = block_excl_scan<double, NT>(ds, s_w64, nullptr);
 #pragma unroll
         for (int i = 0; i < PER; ++i) { const double t = dl[i]; dl[i] = de; de += t; }
 #pragma unroll
@@ -291,22 +288,23 @@ __device__ __forceinline__ bool last_of_layer(uint32_t* counter, uint32_t n_chun
 
 // Level 1 of the exact radix select of one (worker, layer): candidates -> level-1 bins.  By a whole CTA; s_incl and s_below are
 // [kL1Bins].  Leaves the histogram clean.
+template <int NT>
 __device__ __forceinline__ void fb_resolve1_layer(uint32_t l, uint32_t w, size_t wl, size_t wr, uint32_t K, uint32_t* __restrict__ g_cnt,
                                                   unsigned long long* __restrict__ g_ss, const KTab& ktab, Cand* __restrict__ cands,
                                                   SlotTab* __restrict__ slots, uint32_t* s_incl, double* s_below, uint32_t* s_w32,
                                                   double* s_w64) {
     uint32_t* gc = g_cnt + wr * kL1Bins;
     unsigned long long* gs = g_ss + wr * kL1Bins;
-    for (int b = threadIdx.x; b < kL1Bins; b += kThreads) {
+    for (int b = threadIdx.x; b < kL1Bins; b += NT) {
         s_incl[kL1Bins - 1 - b] = __ldcg(gc + b);
         s_below[b] = (double)__ldcg(gs + b) * sq_scale((uint32_t)b >> 3);
         gc[b] = 0;
         gs[b] = 0ull;
     }
     __syncthreads();
-    scan_bins<kL1Bins>(s_incl, s_below, s_w32, s_w64);
+    scan_bins<kL1Bins, NT>(s_incl, s_below, s_w32, s_w64);
     Cand* cd = cands + wl * K;
-    for (uint32_t j = threadIdx.x; j < K; j += kThreads) {
+    for (uint32_t j = threadIdx.x; j < K; j += NT) {
         const uint32_t k = (uint32_t)ktab.at(w, (size_t)l * K + j);
         const int p = find_pos<kL1Bins>(s_incl, k);
         const uint32_t above = p ? s_incl[p - 1] : 0u;
@@ -333,7 +331,7 @@ __device__ __forceinline__ void fb_resolve1_layer(uint32_t l, uint32_t w, size_t
 
 // LEVEL 2: refine inside a level-1 bin; LEVEL 3: inside a (level-1, level-2) bin.  By a whole CTA, a warp per slot: a lane takes
 // 32 consecutive bins.  Leaves the histograms clean.
-template <int LEVEL>
+template <int LEVEL, int NT>
 __device__ __forceinline__ void fb_resolve23_layer(uint32_t l, uint32_t w, size_t wl, size_t wr, uint32_t K, uint32_t* __restrict__ g_cnt,
                                                    unsigned long long* __restrict__ g_ss, Cand* __restrict__ cands,
                                                    SlotTab* __restrict__ slots, float* __restrict__ err_out, uint32_t* __restrict__ tau_out,
@@ -343,7 +341,7 @@ __device__ __forceinline__ void fb_resolve23_layer(uint32_t l, uint32_t w, size_
     SlotTab& stab = slots[wl];
     Cand* cd = cands + wl * K;
     const uint32_t ns = stab.n;
-    for (uint32_t s = wid; s < ns; s += kThreads / 32) {
+    for (uint32_t s = wid; s < ns; s += NT / 32) {
         uint32_t* gc = g_cnt + (wr * K + s) * kL23Bins;
         unsigned long long* gs = g_ss + (wr * K + s) * kL23Bins;
         const uint32_t prefix = stab.prefix[s], b0 = 32u * lane;
