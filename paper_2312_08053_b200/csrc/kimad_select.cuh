@@ -3,7 +3,7 @@
 // After the DP every (worker, layer) knows a key interval [lo, lo + 2^shift) that contains its
 // threshold and the rank of the threshold inside that interval (shift = 0 when the curve stage already
 // resolved all 31 bits).  k_sel_count, one sweep over the byte codes the curve stage left, counts, per 2048-element
-// slice, the entries above the interval, lists the few entries inside it per layer and marks the 32-element groups that
+// slice, the entries above the interval, lists the few entries inside it per layer and marks the 16-element groups that
 // can hold a kept entry; k_sel_offsets (a CTA per layer) takes the exact threshold from the listed entries and leaves one
 // job record per chunk with the chunk's output offset; k_sel_write compacts in index order and updates the estimator,
 // reading only the marked groups of sparse slices.  A layer with more entries in its interval than its list holds counts
@@ -18,14 +18,13 @@ namespace kimad {
 // the sweeps of this stage a warp works on a slice by itself, so no sweep needs a block-wide barrier.
 constexpr int kSliceElems = 2048;
 constexpr int kSlices = 16;
-constexpr int kSparseGroups = 32; // the write sweep reads a slice group by group when at most this many are marked
 constexpr int kListCap = 4096;    // entries inside the interval listed per layer
 constexpr int kStageCap = 128;    // ... of which a CTA of the counting sweep gathers as many before it appends them
 
 struct ChunkSel { // per (worker, chunk)
     uint16_t above[kSlices];   // per slice: entries whose key lies above the interval, after k_sel_offsets above the threshold
     uint16_t eq[kSlices];      // per slice: entries equal to the threshold
-    uint64_t mask[kSlices];    // per slice: bit g set when the 32-element group g may hold a kept entry (key >= the
+    uint4 mask[kSlices];       // per slice: bit g set when the 16-element group g may hold a kept entry (key >= the
                                // interval's lower end); a superset of the groups the write sweep has to read
 };
 
@@ -68,7 +67,7 @@ struct Recount {
 };
 
 // ------------------------------------------------------------------------------------------------
-// Counting sweep: a CTA per chunk, warp w takes the slices w and w + 8.
+// Counting sweep: one or two CTAs per chunk, a warp takes one or two slices.
 // ------------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(kThreads, 6)
 k_sel_count(DSource dbuf, const Chunk* __restrict__ chunks, uint32_t n_chunks, uint32_t L,
@@ -110,9 +109,9 @@ k_sel_count(DSource dbuf, const Chunk* __restrict__ chunks, uint32_t n_chunks, u
     // completed from the inputs.  Codes are 7-bit numbers, so "x >= t" for the four bytes of a word is bit 7 of
     // every byte of x + (0x80 - t) * 0x01010101.
     const uint32_t add_gt = (0x80u - (s.code + 1u)) * 0x01010101u, add_ge = (0x80u - s.code) * 0x01010101u;
-    for (uint32_t sl = wid; sl < (uint32_t)kSlices; sl += kThreads / 32) {
+    for (uint32_t sl = wid + blockIdx.z * (kThreads / 32); sl < (uint32_t)kSlices; sl += gridDim.z * (kThreads / 32)) {
         uint32_t above = 0; // low half: entries above the interval; high half: entries equal to an exact threshold
-        uint64_t mask = 0;
+        uint32_t mask[kSliceElems / 512];
         auto visit = [&](uint32_t key) -> bool { // true: the key is not below the interval
             const uint32_t d1 = key - lo; // wraps to >= 2^31 for keys below the interval
             if (d1 < width) {
@@ -130,8 +129,7 @@ k_sel_count(DSource dbuf, const Chunk* __restrict__ chunks, uint32_t n_chunks, u
             }
             return d1 < 0x80000000u;
         };
-        // a lane takes sixteen consecutive codes (one 128-bit load) of each of the slice's four rows of 512 elements;
-        // a 32-element group is a pair of lanes
+        // a lane takes sixteen consecutive codes (one 128-bit load) of each of the slice's four rows of 512 elements: a group
         constexpr int ROWS = kSliceElems / 512;
         const uint32_t u0 = sl * (kSliceElems / 16) + lane; // this lane's 16-element unit in row 0
         // EDGE: the slice reaches over an end of the chunk; its units there hold codes of the neighbouring chunk, or bytes that
@@ -184,22 +182,14 @@ k_sel_count(DSource dbuf, const Chunk* __restrict__ chunks, uint32_t n_chunks, u
                         if (p1 != p0) f |= visit(key_of(v1));
                     }
                 }
-                uint32_t m = __ballot_sync(0xffffffffu, f);
-                if (m) { // pairs of lanes -> 16 group bits of this row
-                    m = (m | (m >> 1)) & 0x55555555u;
-                    m = (m | (m >> 1)) & 0x33333333u;
-                    m = (m | (m >> 2)) & 0x0f0f0f0fu;
-                    m = (m | (m >> 4)) & 0x00ff00ffu;
-                    m = (m | (m >> 8)) & 0x0000ffffu;
-                    mask |= (uint64_t)m << (16 * r);
-                }
+                mask[r] = __ballot_sync(0xffffffffu, f);
             }
         };
         if (sl * kSliceElems >= cv.first && (sl + 1) * kSliceElems <= cv.len) count(std::false_type{});
         else count(std::true_type{});
 #pragma unroll
         for (int o = 16; o; o >>= 1) above += __shfl_xor_sync(0xffffffffu, above, o);
-        if (lane == 0) { out->above[sl] = (uint16_t)above; out->eq[sl] = (uint16_t)(above >> 16); out->mask[sl] = mask; }
+        if (lane == 0) { out->above[sl] = (uint16_t)above; out->eq[sl] = (uint16_t)(above >> 16); out->mask[sl] = make_uint4(mask[0], mask[1], mask[2], mask[3]); }
     }
     __syncthreads();
     const uint32_t n_in = min(s_n, (uint32_t)kStageCap);
@@ -422,8 +412,12 @@ k_sel_recount(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* _
 // ------------------------------------------------------------------------------------------------
 // DENSE: tuned for steps whose budget keeps more than a few per cent of the entries (the host picks the
 // instantiation from the budgets; both are correct for any input).
+// A slice is read group by group where at most kSparseGroups of its 128 groups are marked.  Write stage with 48 / 64 / 96 / 128:
+// sparse (4 x 124 M, 0.6 % kept) 148 / 141 / 137 / 138 us, (1.1 B, half of it zero) 145 / 145 / 144 / 150; dense (4 x 124 M, 16 %)
+// 558 / 553 / 561 / 728, (8 x 25.6 M, 5 %) 201 / 200 / 213 / 244.  Groups of 32 elements instead of 16 (steps): 1201 -> 1178 us
+// (4 x 124 M, 0.6 %), 4740 -> 4620 (2 x 1.1 B, 0.7 %), 925 -> 910 (8 x 25.6 M).
 template <bool BF16, bool DENSE>
-__global__ void __launch_bounds__(kThreads, DENSE ? 4 : 8)
+__global__ void __launch_bounds__(kThreads, DENSE ? 3 : 8)
 k_sel_write(const float* __restrict__ grads, float* __restrict__ state, const Chunk* __restrict__ chunks,
             uint32_t n_chunks, uint64_t stride, const Phase phase, const ChunkSel* __restrict__ csel,
             const ChunkJob* __restrict__ jobs, uint64_t cap, uint32_t* __restrict__ out_idx, void* __restrict__ out_val,
@@ -454,10 +448,11 @@ k_sel_write(const float* __restrict__ grads, float* __restrict__ state, const Ch
         const uint32_t y = __shfl_up_sync(0xffffffffu, upto, o);
         if (lane >= (uint32_t)o) upto += y;
     }
+    constexpr uint32_t kSparseGroups = DENSE ? 64 : 96;
     __shared__ uint8_t s_pos[kThreads / 32][kSparseGroups]; // per warp: the marked groups of a slice, ascending
     __shared__ uint32_t s_stage[DENSE ? kThreads / 32 : 1][DENSE ? 2 * 16 * 32 : 1]; // per warp: a round's indices, values
 
-    for (uint32_t sl = wid; sl < (uint32_t)kSlices; sl += kThreads / 32) {
+    for (uint32_t sl = wid + blockIdx.z * (kThreads / 32); sl < (uint32_t)kSlices; sl += gridDim.z * (kThreads / 32)) {
         const uint32_t x0 = sl * kSliceElems;
         if (x0 >= cv.len) break;
         // entries equal to tau are kept while their rank among equals (ascending index) is below keep_eq
@@ -469,19 +464,23 @@ k_sel_write(const float* __restrict__ grads, float* __restrict__ state, const Ch
         if (!all && gt_here == 0 && eq_mode == 0) continue; // nothing kept in this slice
         uint32_t eq_seen = eq_before;
         uint32_t pos = gt_before + min(eq_before, keep_eq); // position of the slice's first kept entry in the layer
-        const uint64_t gm = cs.mask[sl];
-        const uint32_t n_groups = __popcll(gm);
-        if (!all && n_groups <= (uint32_t)kSparseGroups) {
-            // sparse slice: read only the 32-element groups the counting sweep marked; a quarter warp per group,
-            // four groups per pass, in ascending order, so that lane order is index order
+        const uint4 gm = cs.mask[sl];
+        const uint32_t n_groups = __popc(gm.x) + __popc(gm.y) + __popc(gm.z) + __popc(gm.w);
+        if (!all && n_groups <= kSparseGroups) {
+            // sparse slice: read only the 16-element groups the counting sweep marked; four lanes per group,
+            // eight groups per pass, in ascending order, so that lane order is index order
             uint8_t* sp = s_pos[wid];
-            const uint32_t lo32 = (uint32_t)gm, hi32 = (uint32_t)(gm >> 32), lt = (1u << lane) - 1u;
+            const uint32_t lt = (1u << lane) - 1u, g4[4] = {gm.x, gm.y, gm.z, gm.w};
             __syncwarp();
-            if ((lo32 >> lane) & 1u) sp[__popc(lo32 & lt)] = (uint8_t)lane;
-            if ((hi32 >> lane) & 1u) sp[__popc(lo32) + __popc(hi32 & lt)] = (uint8_t)(32u + lane);
+            uint32_t at = 0;
+#pragma unroll
+            for (uint32_t q = 0; q < 4; ++q) {
+                if ((g4[q] >> lane) & 1u) sp[at + __popc(g4[q] & lt)] = (uint8_t)(32u * q + lane);
+                at += __popc(g4[q]);
+            }
             __syncwarp();
-            for (uint32_t it = 0; it < n_groups; it += 4) {
-                const uint32_t r = it + (lane >> 3);
+            for (uint32_t it = 0; it < n_groups; it += 8) {
+                const uint32_t r = it + (lane >> 2);
                 uint32_t keepm = 0, eqm = 0, e0 = 0;
                 auto classify = [&](float v, int i) {
                     const uint32_t key = key_of(v);
@@ -490,7 +489,7 @@ k_sel_write(const float* __restrict__ grads, float* __restrict__ state, const Ch
                 };
                 float vq[4] = {0.f, 0.f, 0.f, 0.f}, sq[4] = {0.f, 0.f, 0.f, 0.f}; // d and the state of this lane's quad
                 if (r < n_groups) {
-                    e0 = x0 + (uint32_t)sp[r] * 32u + (lane & 7u) * 4u;
+                    e0 = x0 + (uint32_t)sp[r] * 16u + (lane & 3u) * 4u;
                     if (e0 >= cv.first && e0 + 4 <= cv.len) {
                         // the state is requested together with d: a kept entry's update then waits for one
                         // memory round trip, not two
