@@ -20,7 +20,7 @@
 // much as the cells they address), by the chain of latencies per exchange on short ones, and by the cold start of the
 // records and of the backtracking's rows.  Against one CTA with a barrier per layer, every candidate's index carried along
 // and back-pointers for every cell: GPT-2 small's 148 layers, 16 candidates, D = 1000: 163 -> 69 us; 1995 blocks of it,
-// D = 3990: 12.4 -> 1.87 ms; ResNet-18's 62 layers, 7 candidates: 60 -> 32 us.
+// D = 3990: 12.4 -> 1.76 ms; ResNet-18's 62 layers, 7 candidates: 60 -> 32 us.
 //
 // Waits are on warps of the same CTA and are bounded: a wait that runs out marks the worker's result KIMAD_ERR_TIMEOUT and
 // the remaining waits are skipped.
@@ -64,19 +64,20 @@ __device__ __forceinline__ void lds_cells(float (&x)[CPT][N], int k, uint32_t ad
     }
 }
 __device__ __forceinline__ float min3(float a, float b, float c) { float m; asm("min.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(a), "f"(b), "f"(c)); return m; }
-// orders the accesses before it and after it for the threads of the CTA (the progress counters need no more than this;
-// __threadfence_block is the sequentially consistent fence and costs several times as much here)
-__device__ __forceinline__ void fence_cta() { asm volatile("fence.acq_rel.cta;" ::: "memory"); }
-// bounded wait of a warp: until every lane's counter has reached the lane's target
-__device__ __forceinline__ void progress_wait(const volatile uint32_t* counter, int target, volatile uint32_t* failed) {
-    if (!__all_sync(0xffffffffu, (int)*counter >= target)) {
+// A warp's progress: published by one lane after __syncwarp, which orders the warp's accesses before it, and waited for
+// (bounded) by a warp until every lane's counter has reached the lane's target.  Release and acquire on the counters themselves:
+// with a fence before and after plain accesses the 1995 blocks took 1.87 instead of 1.76 ms.
+__device__ __forceinline__ void progress_set(uint32_t* counter, uint32_t x) { asm volatile("st.release.cta.shared.u32 [%0], %1;" ::"r"(smem_u32(counter)), "r"(x) : "memory"); }
+__device__ __forceinline__ int progress_get(uint32_t counter) { int x; asm volatile("ld.acquire.cta.shared.u32 %0, [%1];" : "=r"(x) : "r"(counter) : "memory"); return x; }
+__device__ __forceinline__ void progress_wait(const uint32_t* counter, int target, volatile uint32_t* failed) {
+    const uint32_t at = smem_u32(counter);
+    if (!__all_sync(0xffffffffu, progress_get(at) >= target)) {
         const long long start = clock64();
-        while (!__all_sync(0xffffffffu, (int)*counter >= target)) {
+        while (!__all_sync(0xffffffffu, progress_get(at) >= target)) {
             if (clock64() - start > kDpWaitClocks) *failed = 1u;
             if (__any_sync(0xffffffffu, *failed != 0u)) break;
         }
     }
-    fence_cta();
     __syncwarp();
 }
 
@@ -358,7 +359,7 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
     const bool busy = wcell < width;
     // Progress: a warp publishes s + 1 when its part of row s is written; it is then done with reading row s - 1.
     if (t < 32u) s_prog[t] = t < T / 32u && t * (32u * CPT) < width ? 0u : 0x7fffffffu; // no work: never holds anybody up
-    volatile uint32_t* prog = s_prog;
+    uint32_t* prog = s_prog;
     volatile uint32_t* failed = &s_failed;
     const uint32_t n_chunks = (L + CL - 1) / CL;
     auto stage_tab = [&](uint32_t ch) { // the first records of a chunk of layers
@@ -398,7 +399,7 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
                 if (cell0 + 32u * q < width) row[cell0 + 32u * q] = v[q];
             if (t == 0) s_ex[seq] = (uint16_t)(l0 + i);
             __syncwarp();
-            if (lane == 0) { fence_cta(); prog[wid] = seq + 1u; }
+            if (lane == 0) progress_set(prog + wid, seq + 1u);
             const uint32_t* er = rec + kr;
             uint4 u4 = *reinterpret_cast<const uint4*>(rec), e4 = *reinterpret_cast<const uint4*>(er);
             // Two cells per thread (short rows: bound by the chain of latencies per layer): up to sixteen candidates' records
