@@ -56,7 +56,7 @@ extern "C" {
 #define KIMAD_ERR_WORKSPACE (-2) /* workspace missing, too small or misaligned                        */
 #define KIMAD_ERR_CAPACITY (-3)  /* a worker selected more entries than max_packed_elems             */
 #define KIMAD_ERR_NONFINITE (-4) /* Inf/NaN met in grad - g (only reported when check_finite != 0)   */
-#define KIMAD_ERR_TIMEOUT (-5)   /* reserved: no kernel of this library waits on another             */
+#define KIMAD_ERR_TIMEOUT (-5)   /* in stats: a bounded wait inside the knapsack kernel ran out      */
 #define KIMAD_ERR_CUDA (-6)      /* a CUDA runtime call failed                                       */
 #define KIMAD_ERR_NOMEM (-7)     /* host allocation failed                                           */
 #define KIMAD_ERR_TOO_LARGE (-8) /* kimad_step_builtin_scratch: scratch need above the built-in array */
