@@ -1,5 +1,6 @@
 // Plain structs and integer helpers shared by the host planner and the kernels of the CUDA library.
 #pragma once
+#include <math.h>
 #include <stdint.h>
 
 #include "kimad.h"
@@ -105,6 +106,42 @@ inline double candidate_cost(uint64_t n, uint64_t k, uint32_t bpe, uint32_t cost
     bool dense;
     const double x = (double)(candidate_bytes(n, k, bpe, cost_model, &dense) * (uint64_t)D);
     return dense ? -x : x;
+}
+
+// ---- Planning of the sweep's bins from the sample (k_sample).  A fine bin is 2^shift keys wide, between kMinShift and a cell.
+constexpr uint32_t kMinShift = 5, kCellShift = 15;
+constexpr float kMostBins = 1024.f; // ... and a cell is cut into at most that many
+
+// Bins per cell that a candidate needs: at most ~2048 entries per bin (`dens`: entries per cell), and bins narrow enough that the
+// uncertainty of the one holding the threshold (its entries times its spread of squares, 2^-7 of v^2 for a whole cell;
+// `load`: entries per cell times v^2) stays below ~3e-6 of the error.  Finite whatever the estimates are, and never more than a cell
+// can be cut into: an error that vanishes in binary32 beside `load` asks for all a cell can get.
+KIMAD_HD float bins_needed(float dens, float load, float error) {
+    const float cert = error > 0.f ? sqrtf(load / error * (0.0078125f / 3e-6f)) : kMostBins;
+    const float bins = fmaxf(dens * (1.f / 2048.f), cert);
+    return bins < kMostBins ? bins : kMostBins; // (also where it is not a number)
+}
+
+// Where the groups of bands together have more fine bins than there is room for (`fine` of them, `most` allowed), groups are
+// coarsened one step at a time, always the one that stays closest to what its candidates need (bins per cell are powers of two, so many
+// have more than they need); every group keeps at least one bin per cell.  Group g has the cells bot[g] .. top[g], bins of
+// 2^shift[g] keys and needs need[g] bins per cell.  Every round halves a group's bins, so at most 10 n rounds are taken whatever
+// the needs are; false: one bin per cell everywhere is still too much.
+KIMAD_HD bool coarsen_groups(const uint32_t* bot, const uint32_t* top, uint32_t* shift, const float* need, uint32_t n, uint64_t fine,
+                             uint64_t most, uint64_t* left) {
+    while (fine > most) {
+        uint32_t at = n;
+        float best = 0.f;
+        for (uint32_t g = 0; g < n; ++g) {
+            const float after = need[g] * (float)(1u << shift[g]); // need over bins per cell, up to a common factor
+            if (shift[g] < kCellShift && (at == n || after < best)) { best = after; at = g; }
+        }
+        if (at == n) return false;
+        fine -= (uint64_t)(top[at] - bot[at] + 1u) << (kCellShift - 1u - shift[at]);
+        shift[at] += 1u;
+    }
+    *left = most - fine;
+    return true;
 }
 
 } // namespace kimad

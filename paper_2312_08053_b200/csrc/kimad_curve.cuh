@@ -69,7 +69,7 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
     uint32_t* s_cb = s_w + 32;                    // [128] per candidate, then per merged group: lowest cell,
     uint32_t* s_ct = s_cb + 128;                  // [128] highest cell,
     uint32_t* s_cs = s_ct + 128;                  // [128] shift
-    __shared__ uint32_t s_m, s_flag, s_ng, s_cg, s_z, s_clip;
+    __shared__ uint32_t s_flag, s_ng, s_cg, s_z, s_clip, s_top;
     __shared__ unsigned long long s_zz;
     __shared__ float s_nd[128]; // bins per cell needed, per candidate, then per merged group
     const uint32_t r = blockIdx.x, w = blockIdx.y;
@@ -85,7 +85,7 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
     // the candidate of the thread's warp, asked for ahead of its use (the first one, where a warp takes several)
     const uint64_t k_first = (threadIdx.x >> 5) < K ? ktab.at(w, (size_t)l * K + (threadIdx.x >> 5)) : 0ull;
     for (int i = threadIdx.x; i < 32768 / 4; i += kBigThreads) reinterpret_cast<uint4*>(h32)[i] = make_uint4(0u, 0u, 0u, 0u);
-    if (threadIdx.x == 0) { s_m = 0; s_flag = 0; s_ng = 0; s_cg = 0; s_z = 0; s_zz = 0ull; s_clip = 0; }
+    if (threadIdx.x == 0) { s_flag = 0; s_ng = 0; s_cg = 0; s_z = 0; s_zz = 0ull; s_clip = 0; s_top = 0; }
     __syncthreads();
 
     // ---- stratified sample of |grad - g|.  Exact zeros (the untouched rows of a sparse gradient) are counted apart:
@@ -98,7 +98,8 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
     const uint32_t m_units = n_units <= (uint32_t)kWholeUnits ? n_units : min(max(n_units / 2u, (uint32_t)kWholeUnits), (uint32_t)kSampleUnits);
     const bool whole = m_units == n_units;
     const uint32_t sq_ = n / m_units, sr_ = n % m_units; // used when sampled
-    uint32_t mine = 0;
+    const uint32_t m = whole ? n : kSampleUnit * m_units; // sample size (a stratum is no shorter than a unit), exact zeros included
+    uint32_t top_key = 0;                                  // largest finite key
     // a warp reads one unit (128 bytes); eight units per thread are in flight before their keys are counted (this phase runs at
     // the DRAM's random-access rate on large layers; four and four, counted alternately, took a fifth longer)
     for (uint32_t ib = threadIdx.x / kSampleUnit; ib < m_units; ib += 8 * (kBigThreads / kSampleUnit)) {
@@ -134,16 +135,19 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
             }
             if (ok[u]) {
                 if (key) atomicAdd(&h32[key >> 16], 1u << (16 * ((key >> 15) & 1)));
-                ++mine;
+                top_key = max(top_key, key < 0x7f800000u ? key : 0u);
             }
         }
     }
-    atomicAdd(&s_m, mine);
+    top_key = __reduce_max_sync(0xffffffffu, top_key);
+    if ((threadIdx.x & 31) == 0) atomicMax(&s_top, top_key);
     __syncthreads();
-    const uint32_t m = s_m; // sample size, exact zeros included
     auto cell_count = [&](uint32_t cell) { return (h32[cell >> 1] >> (16 * (cell & 1))) & 0xffffu; };
-    auto cell_sq = [&](uint32_t cell) { // square of the cell's middle value (planning only: float range is enough)
-        const float v = __uint_as_float((cell << 15) | 0x4000u);
+    // Square of the cell's middle value, in units that put the sample's largest value into [2^40, 2^41): sums of squares over the
+    // layer stay finite, and squares of values down to 2^-113 of the largest one are there.  Only ratios of sums are used.
+    const float unit = __uint_as_float(min(254u, 294u - max(s_top >> 23, 1u)) << 23);
+    auto cell_sq = [&](uint32_t cell) {
+        const float v = __uint_as_float((cell << 15) | 0x4000u) * unit;
         return v * v;
     };
 
@@ -281,10 +285,7 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
                 }
                 below += s_sq[seg];
                 const float scale = (float)n / (float)m;
-                // bins per cell: at most ~2048 entries per bin (what the select stage collects and sorts), and
-                // narrow enough that the uncertainty of the bin holding the threshold (its entries times its
-                // spread of squares, 2^-7 of v^2 for a whole cell) stays below ~3e-6 of the error; entries per
-                // cell and v^2 are taken quarter by quarter
+                // entries per cell and v^2 are taken quarter by quarter
                 float dens = 0.f, load = 0.f;
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
@@ -294,12 +295,9 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
                     const float ld = per_cell * cell_sq(qtop);
                     load = ld > load ? ld : load;
                 }
-                float bins = dens * (1.f / 2048.f);
-                const float e_est = below * scale;
-                const float cert = e_est > 0.f ? sqrtf(load / e_est * (0.0078125f / 3e-6f)) : 1024.f;
-                if (cert > bins) bins = cert;
-                uint32_t sh_j = 15;
-                while (sh_j > 5 && (float)(1u << (15 - sh_j)) < bins) --sh_j;
+                const float bins = bins_needed(dens, load, below * scale); // (about 2048 entries of a bin are listed by the select stage)
+                uint32_t sh_j = kCellShift;
+                while (sh_j > kMinShift && (float)(1u << (kCellShift - sh_j)) < bins) --sh_j;
                 o_cb = c_bot; o_ct = c_top; o_cs = sh_j;
                 o_nd = bins;
             }
@@ -343,28 +341,16 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
             cells += s_ct[g] - s_cb[g] + 1;
         }
         if (cells > (uint64_t)kFineBins) s_flag = 3;
-        // If the fine bins do not fit, groups are coarsened one step at a time, always the one that stays closest to what its
-        // candidates need (bins per cell are powers of two, so many have more than they need); every group keeps at least
-        // one bin per cell.
-        while (!s_flag && fine > (uint64_t)kFineBins) {
-            uint32_t at = 0;
-            float best = 3.4e38f;
-            for (uint32_t g = 0; g < ng; ++g) {
-                const float after = s_nd[g] * (float)(1u << s_cs[g]); // need over bins per cell, up to a common factor
-                if (s_cs[g] < 15u && after < best) { best = after; at = g; }
-            }
-            fine -= (uint64_t)(s_ct[at] - s_cb[at] + 1) << (14 - s_cs[at]);
-            s_cs[at] += 1;
-        }
+        uint64_t left = 0; // fine bins not given away
+        if (!s_flag && !coarsen_groups(s_cb, s_ct, s_cs, s_nd, ng, fine, (uint64_t)kFineBins, &left)) s_flag = 3;
         // Where the rank window of the highest band reached beyond the largest sample, up to four more octaves above the band
         // get one bin per cell, as far as bins and table entries are left.  A sample without an entry as large as the smallest
         // candidate's threshold is not rare where large entries lie together (a few rows of a gradient, seven samples
         // expected), and the exact path costs far more than these bins (1.1 B Llama shape, gradients moved across
         // the tensors' borders: 4.5 layers of 402 per step on the exact path without them, 1 with one octave).
         if (s_clip && ng && !s_flag) {
-            const uint32_t left = (uint32_t)((uint64_t)kFineBins - fine);
             const uint32_t window = (s_ct[0] >> cg) - (s_cb[ng - 1] >> cg) + 3u;
-            uint32_t ext = min(min(1024u, left), window < (uint32_t)kCellTab ? ((uint32_t)kCellTab - window) << cg : 0u) & ~cmask;
+            uint32_t ext = min(min(1024u, (uint32_t)left), window < (uint32_t)kCellTab ? ((uint32_t)kCellTab - window) << cg : 0u) & ~cmask;
             ext = min(ext, 65279u - s_ct[0]);
             if (ext) {
                 for (uint32_t g = ng; g; --g) { s_cb[g] = s_cb[g - 1]; s_ct[g] = s_ct[g - 1]; s_cs[g] = s_cs[g - 1]; }

@@ -1,0 +1,68 @@
+"""Planning of the sweep's bins (kimad_common.h) compiled for the host: it ends, with finite needs and as many bins as fit,
+whatever the estimates it starts from."""
+import ctypes
+import math
+import os
+import random
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CODE = r'''
+#include "kimad_common.h"
+extern "C" float need_of(float dens, float load, float error) { return kimad::bins_needed(dens, load, error); }
+extern "C" int coarsen(const uint32_t* bot, const uint32_t* top, uint32_t* shift, const float* need, uint32_t n, uint64_t most, uint64_t* left) {
+    uint64_t fine = 0;
+    for (uint32_t g = 0; g < n; ++g) fine += (uint64_t)(top[g] - bot[g] + 1) << (kimad::kCellShift - shift[g]);
+    return kimad::coarsen_groups(bot, top, shift, need, n, fine, most, left);
+}
+'''
+
+
+@pytest.fixture(scope="module")
+def planner(tmp_path_factory):
+    d = tmp_path_factory.mktemp("planner")
+    (d / "planner.cpp").write_text(CODE)
+    so = str(d / "planner.so")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I", os.path.join(ROOT, "include"),
+                    "-I", os.path.join(ROOT, "paper_2312_08053_b200", "csrc"), "-o", so, str(d / "planner.cpp")], check=True)
+    lib = ctypes.CDLL(so)
+    lib.need_of.restype = ctypes.c_float
+    lib.need_of.argtypes = [ctypes.c_float] * 3
+    return lib
+
+
+def test_needs_are_finite(planner):
+    values = [0.0, 1e-45, 1e-38, 1e-20, 1.0, 2048.0, 1e20, 3e38, math.inf, math.nan]
+    for dens in values:
+        for load in values:
+            for error in values:
+                x = planner.need_of(dens, load, error)
+                assert 0.0 <= x <= 1024.0, (dens, load, error, x)
+    assert planner.need_of(4096.0, 0.0, 1.0) == 2.0
+
+
+def test_coarsening_ends(planner):
+    rng = random.Random(1)
+    odd = [math.inf, math.nan, 0.0, 1e-30, 1024.0, 3e38]
+    for _ in range(500):
+        n = rng.randint(1, 128)
+        cells = [int(math.exp(rng.uniform(0, math.log(12288 / n)))) for _ in range(n)]
+        bot, top, at = [], [], 70000
+        for c in cells:
+            at -= c + rng.randint(0, 3)
+            bot.append(at)
+            top.append(at + c - 1)
+        shift = [rng.randint(5, 15) for _ in range(n)]
+        need = [rng.choice(odd) if rng.random() < 0.5 else math.exp(rng.uniform(-10, 10)) for _ in range(n)]
+        most = rng.choice([12288, sum(cells), max(1, sum(cells) // 2)])
+        u32, f32 = ctypes.c_uint32 * n, ctypes.c_float * n
+        s, left = u32(*shift), ctypes.c_uint64(0)
+        ok = planner.coarsen(u32(*bot), u32(*top), s, f32(*need), ctypes.c_uint32(n), ctypes.c_uint64(most), ctypes.byref(left))
+        fine = sum(c << (15 - x) for c, x in zip(cells, s))
+        assert all(a <= b <= 15 for a, b in zip(shift, s))
+        if ok:
+            assert fine + left.value == most
+        else:
+            assert all(x == 15 for x in s) and fine > most
