@@ -625,7 +625,7 @@ int kimad_create(kimad_ctx** out, const uint64_t* layer_sizes, uint32_t n_layers
         c->dstride = (N + 3 + 15) / 16 * 16; // every worker's code plane starts on a 16-byte boundary (and up to 3 codes in)
         if (!plan_choice(c)) { delete c; return KIMAD_ERR_INVALID_ARG; }
         c->curve_mode = o.curve_mode;
-        c->sample_smem = (size_t)(1024 + 32 + 32768 + 1024 + 2 * kMaxGaps + 32 + 3 * 128) * 4;
+        c->sample_smem = (size_t)(1024 + 32 + 32768 + 1024 + 2 * kBaseWords + 32 + 3 * 128) * 4;
         c->pass_a_smem = (size_t)(2 * kMaxBins + kCellTab) * 4;
         { // the sweep's runs, one CTA each: every worker's chunk list is cut into pieces of about equal element counts.
           // The sweep of a group of workers ((W + 1) / 2 of them) is one wave of CTAs (148 SMs, one CTA resident per

@@ -35,7 +35,9 @@ constexpr int kTinyMax = 4096;
 #endif
 constexpr int kFineBins = KIMAD_FINE_BINS;          // fine bins per (worker, layer)
 constexpr int kMaxGaps = KIMAD_MAX_RATIOS + 2;      // gap regions: below / between / above the band groups, + non-finite keys
+constexpr int kBaseWords = kMaxGaps + 2;            // first bin of every gap and of the keys that are not finite; the number of bins
 constexpr int kMaxBins = kFineBins + kL1Bins + 2 * kMaxGaps; // fine bins + gap regions cut at every 11-bit prefix
+static_assert(kBaseWords > KIMAD_MAX_RATIOS + 1 + 2, "a group of bands per candidate and one above them");
 constexpr int kMaxShift = 15;                       // a fine bin is 2^shift keys wide, at most a whole cell
 constexpr int kSampleUnit = 32;                     // consecutive elements read together (128 bytes, one warp)
 constexpr int kSampleUnits = 2047;                  // units of a sample (<= 65504 elements: the u16 cell counters cannot overflow)
@@ -64,8 +66,8 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
     float* s_wd = s_sq + 1024;                    // [32]
     uint32_t* h32 = sh + 1024 + 32;               // [32768] two u16 cell counters per word
     uint32_t* s_pre = h32 + 32768;                // [1024] inclusive sample count of the thread segments, from the top
-    uint32_t* s_base = s_pre + 1024;              // [2 kMaxGaps] first bin id of every gap region, of every group
-    uint32_t* s_w = s_base + 2 * kMaxGaps;        // [32]
+    uint32_t* s_base = s_pre + 1024;              // [2 kBaseWords] first bin id of every gap region, of every group
+    uint32_t* s_w = s_base + 2 * kBaseWords;      // [32]
     uint32_t* s_cb = s_w + 32;                    // [128] per candidate, then per merged group: lowest cell,
     uint32_t* s_ct = s_cb + 128;                  // [128] highest cell,
     uint32_t* s_cs = s_ct + 128;                  // [128] shift
@@ -380,7 +382,7 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
             if (hi + 1 > lo) id += (hi >> 5) - (lo >> 5) + 1;
             if (a < ng) {
                 const uint32_t g = ng - 1 - a;
-                s_base[kMaxGaps + a] = id; // first fine bin of group a
+                s_base[kBaseWords + a] = id; // first fine bin of group a
                 id += (s_ct[g] - s_cb[g] + 1) << (15 - s_cs[g]);
             }
         }
@@ -410,7 +412,7 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
         const uint32_t g = ng - 1 - a;
         if (a < ng && cell >= s_cb[g]) {
             const uint32_t cs = s_cs[g];
-            tab[i] = (uint32_t)(((int)s_base[kMaxGaps + a] - (int)(s_cb[g] << (15 - cs))) * 32) | cs;
+            tab[i] = (uint32_t)(((int)s_base[kBaseWords + a] - (int)(s_cb[g] << (15 - cs))) * 32) | cs;
         } else {
             tab[i] = (uint32_t)(((int)s_base[a] - (int)(s_glo[a] >> 5)) * 32) | 20u;
         }
@@ -421,9 +423,9 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
         uint32_t key;
         if (x >= s_base[ng + 1]) {
             key = ((2040u + x - s_base[ng + 1]) << 20) | kGapBit;
-        } else if (a < ng && x >= s_base[kMaxGaps + a]) {
+        } else if (a < ng && x >= s_base[kBaseWords + a]) {
             const uint32_t g = ng - 1 - a;
-            key = (s_cb[g] << 15) + ((x - s_base[kMaxGaps + a]) << s_cs[g]);
+            key = (s_cb[g] << 15) + ((x - s_base[kBaseWords + a]) << s_cs[g]);
         } else {
             const uint32_t lo = s_glo[a];
             key = (max(lo, ((lo >> 5) + x - s_base[a]) << 5) << 15) | kGapBit;

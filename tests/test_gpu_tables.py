@@ -81,6 +81,20 @@ def test_codes_of_layers_without_a_histogram():
         r.compare_step(grads, state, budget, 1.0)
 
 
+@pytest.mark.parametrize("n", [4097, 20000, 32768])
+def test_a_band_for_every_one_of_127_candidates(n):
+    """As many groups of bands as candidates are allowed, none of which keeps the whole layer: magnitudes spread so far that every
+    threshold lies in a band of its own."""
+    rng = np.random.default_rng(n)
+    grid = [float(v) for v in np.linspace(0.005, 0.99, 127)]
+    x = np.exp(rng.uniform(-30, 30, (1, n))) * rng.choice((-1.0, 1.0), (1, n))
+    r = Runner([n], 1, grid, 1000, 0)
+    grads = torch.from_numpy(x.astype(np.float32)).cuda()
+    res = r.compare_step(grads, torch.zeros_like(grads), [0.4 * 8 * n], 1.0)
+    assert res["same_k"]
+    assert _meta(r)[0, 0, 2:].tolist() == [0, 127 + 2]  # swept with its histogram; groups + 2
+
+
 def _row_sparse(rng, W, rows, cols, zero_frac, tail):
     """[W][rows * cols + tail]: a matrix whose untouched rows are exactly zero (an embedding gradient), then a dense tail."""
     x = rng.standard_normal((W, rows * cols + tail)).astype(np.float32)
