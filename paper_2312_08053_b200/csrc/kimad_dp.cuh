@@ -229,7 +229,7 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
      float* __restrict__ hist_all /* [W] at hist_stride words, [exchanges][hist_row] each */, size_t hist_stride, uint32_t hist_row) {
     pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ uint32_t s_prog[32], s_failed, s_reach, s_cell, s_left;
+    __shared__ uint32_t s_prog[32], s_failed, s_reach, s_cell, s_left, s_signed;
     __shared__ unsigned long long s_sum;
     __shared__ float s_redv[kDpMaxThreads / 32], s_total;
     __shared__ uint32_t s_redb[kDpMaxThreads / 32];
@@ -255,7 +255,7 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
     if (a.check_finite && (a.flags[w] & 1u)) status = KIMAD_ERR_NONFINITE;
     else if (c >= a.full_bytes) status = KIMAD_STATUS_PLATEAU;
     else if (c == 0) status = KIMAD_STATUS_INFEASIBLE;
-    if (t == 0) { s_failed = 0; s_sum = 0; s_reach = 0; }
+    if (t == 0) { s_failed = 0; s_sum = 0; s_reach = 0; s_signed = 0; }
     __syncthreads(); // (and the flags are read before the end of the choice resets them)
 
     // ---- the layers' records; 8, 16 or 32 lanes per layer, the loads of the next layers ahead of the current ones' work
@@ -267,6 +267,7 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
         const uint32_t rounds = (kr + G - 1u) / G; // above 1: more than 32 candidates
         unsigned long long sum = 0;
         uint32_t reach = 0;
+        bool negative = false;
         // budget_cells = (bytes D + c - 1) / c in binary64: everything is an integer below 2^50 (bytes < 2^35, D < 2^13, c below
         // the sum of the layers' sizes), the quotient from the reciprocal is off by one at most and the remainder is exact
         const double cd = (double)c, inv_c = 1.0 / cd, c_1 = cd - 1.0, most = (double)(D + 1u);
@@ -304,6 +305,7 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
                     if (oks) far = __shfl_sync(gmask, du, 31 - __clz(oks));
                     nu += __popc(oks);
                     emin = fminf(emin, ok ? e : kInf);
+                    negative |= ok && e < 0.f;
                     // of two neighbours with the same cells the first is left out unless its error is the smaller one
                     const float e_right = __shfl_down_sync(0xffffffffu, e, 1);
                     const uint32_t u_right = __shfl_down_sync(0xffffffffu, u, 1);
@@ -335,6 +337,7 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
                 }
             }
         }
+        if (negative) s_signed = 1u;
         if (jj == 0 && sum) { atomicAdd(&s_sum, sum); atomicMax(&s_reach, reach); }
     }
     __syncthreads();
@@ -501,6 +504,14 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
         // the first candidate that attains the minimum, and the cell it came from.
         __syncthreads(); // everybody has read the number of exchanges
         if (t == 0) s_cell = bb;
+        // Errors that the curve stage computes are not negative, and neither are their sums: they order as their bits do.
+        const bool any_sign = s_signed != 0u;
+        auto warp_min = [](float x, auto any) {
+            if (!decltype(any)::value) return __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(x)));
+#pragma unroll
+            for (int o = 16; o; o >>= 1) x = fminf(x, __shfl_xor_sync(0xffffffffu, x, o));
+            return x;
+        };
         __syncthreads();
         for (uint32_t left = n_ex; left;) {
             const uint32_t b0 = s_cell, lo = (b0 - min(b0, reach + 256u)) & ~3u;
@@ -532,20 +543,24 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
                     const uint32_t lane_j = min(lane, kr - 1u);
                     uint32_t nu = rec[2u * kr], far = rec[2u * kr + 2u], off = (0u - rec[lane_j]) >> 2;
                     float e = __uint_as_float(rec[kr + lane_j]);
-                    while (i < nx) {
-                        if (lo && b - lo < far) break; // left the window: staged anew from here (never on the first exchange)
-                        const bool fits = lane < nu && off <= b;
-                        const float sum = fits ? __fadd_rn(row[b - off], e) : kInf;
-                        const uint32_t mine = lane << 16 | off;
-                        row += 4u * per16; rec += 4u * per16; // (the last ones read lie inside the buffer: work_bytes is below its end)
-                        nu = rec[2u * kr]; far = rec[2u * kr + 2u]; off = (0u - rec[lane_j]) >> 2;
-                        e = __uint_as_float(rec[kr + lane_j]);
-                        const float best = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(sum))); // (sums of squares: not negative)
-                        const uint32_t win = __reduce_min_sync(0xffffffffu, fits && sum == best ? mine : 0xffffffffu); // the first of them
-                        if (lane == (i & 31u)) { my_j = win >> 16; my_best = best; }
-                        b -= win & 0xffffu;
-                        if ((++i & 31u) == 0) keep(32u, i);
-                    }
+                    auto walk = [&](auto any) {
+                        while (i < nx) {
+                            if (lo && b - lo < far) break; // left the window: staged anew from here (never on the first exchange)
+                            const bool fits = lane < nu && off <= b;
+                            const float sum = fits ? __fadd_rn(row[b - off], e) : kInf;
+                            const uint32_t mine = lane << 16 | off;
+                            row += 4u * per16; rec += 4u * per16; // (the last ones read lie inside the buffer: work_bytes is below its end)
+                            nu = rec[2u * kr]; far = rec[2u * kr + 2u]; off = (0u - rec[lane_j]) >> 2;
+                            e = __uint_as_float(rec[kr + lane_j]);
+                            const float best = warp_min(sum, any);
+                            const uint32_t win = __reduce_min_sync(0xffffffffu, fits && sum == best ? mine : 0xffffffffu); // the first of them
+                            if (lane == (i & 31u)) { my_j = win >> 16; my_best = best; }
+                            b -= win & 0xffffu;
+                            if ((++i & 31u) == 0) keep(32u, i);
+                        }
+                    };
+                    if (any_sign) walk(std::true_type{}); // (not a test per exchange: that took 1.6 us on 148 layers, 10 on 1995)
+                    else walk(std::false_type{});
                     keep(i & 31u, i);
                 } else {
                     for (; i < nx; ++i, rec += 4u * per16) {
@@ -565,7 +580,7 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
                             }
                             best = fminf(best, sum[h]);
                         }
-                        best = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(best)));
+                        best = any_sign ? warp_min(best, std::true_type{}) : warp_min(best, std::false_type{});
 #pragma unroll
                         for (int h = 3; h >= 0; --h) {
                             const uint32_t eq = __ballot_sync(0xffffffffu, sum[h] == best);

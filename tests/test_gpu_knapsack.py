@@ -5,7 +5,9 @@ import numpy as np
 import pytest
 import torch
 
-from tests._harness import Runner
+from oracle import kimad_oracle as ko
+from paper_2312_08053_b200 import binding as kb
+from tests._harness import Runner, u32
 
 pytestmark = pytest.mark.gpu
 
@@ -28,3 +30,27 @@ def test_decisions_match_the_oracle(L, K, D):
     for frac in (1.02, 3.0, 20.0):  # from hardly feasible to wide; one worker's budget is cut below
         bw = [frac * least, 1.7 * frac * least, 0.4 * frac * least]
         r.compare_step(torch.from_numpy(x).cuda(), torch.zeros((3, N), dtype=torch.float32, device="cuda"), bw, 1.0)
+
+
+@pytest.mark.parametrize("L,K,D", [(40, 9, 1000), (25, 40, 300), (60, 16, 2500)])
+def test_given_errors_of_any_sign(L, K, D):
+    """A curve given from outside may hold negative values (and infinite ones): the search only compares sums."""
+    rng = np.random.default_rng(L)
+    sizes = [int(v) for v in rng.integers(20, 900, L)]
+    N, W = sum(sizes), 2
+    r = Runner(sizes, W, list(np.geomspace(0.01, 1.0, K)), D, 0)
+    g = rng.standard_normal((W, N)).astype(np.float32)
+    err = rng.standard_normal((W, L, K)).astype(np.float32)
+    err[1, ::7] = -abs(err[1, ::7])
+    err[0, ::5, K // 2] = np.inf
+    err[0, 3] = 0.0
+    for frac in (0.05, 0.3):
+        bw = [frac * 8 * N, 0.7 * frac * 8 * N]
+        state = torch.zeros((W, N), dtype=torch.float32, device="cuda")
+        kb.kimad_debug_step_with_err(r.ctx, torch.from_numpy(g).cuda(), state, bw, 1.0, r.out, torch.from_numpy(err).cuda())
+        ref = ko.step(sizes, W, r.grid, D, 0, g, np.zeros_like(g), bw, 1.0, inject_err=err)
+        st = r.out.stats_host()
+        assert np.array_equal(st["status"], ref.status) and not ref.status.any()
+        assert np.array_equal(u32(r.out.j), ref.j)
+        assert np.array_equal(st["total_err"], ref.total_err)
+        assert np.array_equal(u32(state), ref.state.view(np.uint32))
