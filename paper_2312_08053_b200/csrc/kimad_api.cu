@@ -527,7 +527,8 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
             };
             CUDA_TRY(c->most_chunks > 256 ? launch(k_sel_offsets<512>, 512) : launch(k_sel_offsets<128>, 128));
         }
-        CUDA_TRY(launch_pdl(k_sel_recount, 148, blk, 0, small, dbuf, layers, chunks, nch, L, sel, csel, jobs, in, rc, rc_chunks));
+        // (a warp per chunk; usually there is nothing to do)
+        CUDA_TRY(launch_pdl(k_sel_recount, std::min(148u, (nch * nw + 7) / 8), blk, 0, small, dbuf, layers, chunks, nch, L, sel, csel, jobs, in, rc, rc_chunks));
         mark(small);
         CUDA_TRY(hand_over(small, big));
         {

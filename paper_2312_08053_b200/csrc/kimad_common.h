@@ -64,6 +64,11 @@ struct SlotTab {
     uint32_t prefix[KIMAD_MAX_RATIOS];
 };
 
+// Entries inside a layer's key interval that the select stage lists in one place; the curve stage marks an interval that may
+// hold more (kSelMany, beside the code of its keys).
+constexpr uint32_t kListCap = 4096;
+constexpr uint32_t kSelMany = 256;
+
 // What the select kernels need to know about one (worker, layer) after the DP.  The threshold lies in
 // the key interval [tau, tau + 2^shift) and is the keep_eq-th largest key inside it; k_sel_offsets
 // narrows that to the exact threshold (shift = 0) and to the number of ties kept.
@@ -74,7 +79,7 @@ struct Sel {
     uint32_t shift;   // log2 of the interval width (<= 10)
     uint32_t tau_low; // exact threshold minus the interval's lower key
     uint32_t code;    // the code (byte plane of the sweep) of the keys of the interval: entries with a larger code lie
-                      // above the interval, entries with a smaller one below
+                      // above the interval, entries with a smaller one below; | kSelMany
     uint64_t base;    // first output position of the layer in the worker's packed buffers
 };
 

@@ -816,7 +816,7 @@ __device__ __forceinline__ bool refine_resolve_layer(const ListArgs& a, uint32_t
                     s_bad = 1;
                 } else {
                     a.err[o] = (float)e; a.tau[o] = klo; a.keep_eq[o] = c[i] - d2;
-                    a.shift[o] = sub | a.codes.code(w, l, klo) << 8;
+                    a.shift[o] = sub | (a.codes.code(w, l, klo) | (sub && c[i] > kListCap ? kSelMany : 0u)) << 8;
                 }
             }
             before += c[i];
@@ -1156,7 +1156,9 @@ k_resolve_a(const LayerDesc* __restrict__ layers, const uint32_t* __restrict__ r
             err_out[o] = (float)e;
             tau_out[o] = klo;
             rank_out[o] = cb - drop;
-            shift_out[o] = (31 - __clz(width)) | (bin >> ls) << 8; // with the code of the bin's entries
+            // with the code of the bin's entries (zeros that the sweep left out lie in the bin of key 0)
+            const bool many = cb > kListCap || (klo == 0u && zeros);
+            shift_out[o] = (31 - __clz(width)) | ((bin >> ls) | (many ? kSelMany : 0u)) << 8;
         }
         __syncthreads();
         for (uint32_t bb = threadIdx.x; bb < nb; bb += kBigThreads) // clean for the next step

@@ -93,7 +93,7 @@ struct ChooseArgs {
     const LayerDesc* layers;
     KTab ktab;
     const float* err;          // [W][L][K]
-    const uint32_t *tau, *keep_eq, *shift; // shift: log2 of the interval's width | code of its keys << 8
+    const uint32_t *tau, *keep_eq, *shift; // shift: log2 of the interval's width | (code of its keys | kSelMany) << 8
     uint32_t* flags;
     Sel* sel;
     uint32_t *out_k, *out_j;

@@ -6,9 +6,10 @@
 // slice, the entries above the interval, lists the few entries inside it per layer and marks the 16-element groups that
 // can hold a kept entry; k_sel_offsets (a CTA per layer) takes the exact threshold from the listed entries and leaves one
 // job record per chunk with the chunk's output offset; k_sel_write compacts in index order and updates the estimator,
-// reading only the marked groups of sparse slices.  A layer with more entries in its interval than its list holds counts
-// the rest in a histogram of single keys; its chunks are counted once more against the exact threshold (k_sel_recount,
-// usually nothing to do).  No kernel waits on another: offsets come from stored counts.
+// reading only the marked groups of sparse slices.  Of a layer with more entries in its interval than its list holds (values
+// that came from 16 or 8 bits repeat) every key of the interval is counted, and every slice keeps a list of its own, where its codes
+// were; the slices' counts then follow from those (k_sel_recount, usually nothing to do).  No kernel waits on another: offsets
+// come from stored counts.
 #pragma once
 #include "kimad_curve.cuh"
 
@@ -18,12 +19,12 @@ namespace kimad {
 // the sweeps of this stage a warp works on a slice by itself, so no sweep needs a block-wide barrier.
 constexpr int kSliceElems = 2048;
 constexpr int kSlices = 16;
-constexpr int kListCap = 4096;    // entries inside the interval listed per layer
 constexpr int kStageCap = 128;    // ... of which a CTA of the counting sweep gathers as many before it appends them
 
 struct ChunkSel { // per (worker, chunk)
     uint16_t above[kSlices];   // per slice: entries whose key lies above the interval, after k_sel_offsets above the threshold
-    uint16_t eq[kSlices];      // per slice: entries equal to the threshold
+    uint16_t eq[kSlices];      // per slice: entries equal to the threshold; until k_sel_recount, where every slice has a list of its
+                               // own: entries inside the interval
     uint4 mask[kSlices];       // per slice: bit g set when the 16-element group g may hold a kept entry (key >= the
                                // interval's lower end); a superset of the groups the write sweep has to read
 };
@@ -42,9 +43,9 @@ struct ChunkJob {
 
 // Entries inside the intervals.  Only layers swept with a histogram have an interval wider than one key; their bin tables
 // and bin histograms are free after the DP, and hold the layer's list (kListCap records {chunk of the layer, slice << 16 |
-// key - lo}) and, beyond that many entries, the count of every key of the interval (clean before and after).
+// key - lo}) or, for intervals that may hold more, the count of every key of the interval (clean before and after).
 struct Interval {
-    uint32_t* n;        // [W][L] entries inside the interval; zero between steps
+    uint32_t* n;        // [W][L] entries in the layer's list, then finished chunks of k_sel_recount; zero between steps
     uint32_t* bin_lo;   // [W][R][kMaxBins + 1]
     uint32_t* bh_cnt;   // [W][R][kMaxBins]
     unsigned long long* bh_sum;
@@ -58,9 +59,21 @@ struct Interval {
         return d < (uint32_t)kMaxBins ? bh_cnt + wr * kMaxBins + d : reinterpret_cast<uint32_t*>(bh_sum + wr * kMaxBins) + (d - kMaxBins);
     }
 };
-static_assert(kListCap * 8 + 8 <= (kMaxBins + 1) * 4 && 3 * kMaxBins >= (1 << kMaxShift), "list and key counts fit the bin arrays");
+static_assert(kListCap * 8 + 8 <= (uint32_t)(kMaxBins + 1) * 4 && 3 * kMaxBins >= (1 << kMaxShift), "list and key counts fit the bin arrays");
 
-// chunks of layers whose interval held more entries than the list
+// The list of a slice: distances (key - lo) of its entries inside the interval, laid over the slice's own codes once its warp has
+// read them (units of sixteen codes that the slice shares with another chunk stay).  Nobody reads a code after the counting sweep.
+struct SliceList {
+    uint16_t* at;
+    uint32_t cap; // entries; a slice with more is counted from the inputs
+    __device__ __forceinline__ SliceList(const DSource& p, uint32_t w, const ChunkView& cv, uint32_t sl) {
+        const uint32_t b = max((cv.first + 15u) & ~15u, sl * kSliceElems), e = min(cv.len & ~15u, (sl + 1) * kSliceElems);
+        at = reinterpret_cast<uint16_t*>(p.code + (size_t)w * p.dstride + cv.a0 + b);
+        cap = e > b ? (e - b) / 2 : 0u;
+    }
+};
+
+// chunks of layers whose slices have lists of their own
 struct Recount {
     uint32_t n_chunks;
     uint32_t _pad[3];
@@ -77,7 +90,7 @@ k_sel_count(DSource dbuf, const Chunk* __restrict__ chunks, uint32_t n_chunks, u
             const Sel* __restrict__ sel, const LayerDesc* __restrict__ layers, ChunkSel* __restrict__ csel, const Interval in,
             Recount* __restrict__ rc, uint32_t w_base) {
     pdl_wait();
-    __shared__ uint32_t s_n, s_at;
+    __shared__ uint32_t s_n, s_at, s_in[kThreads / 32]; // s_in: entries in the list of the warp's slice
     __shared__ uint32_t s_low[kStageCap];
     const Chunk ch = chunks[blockIdx.x];
     const uint32_t w = w_base + blockIdx.y;
@@ -97,30 +110,35 @@ k_sel_count(DSource dbuf, const Chunk* __restrict__ chunks, uint32_t n_chunks, u
         return;
     }
     const uint32_t lo = s.tau, width = 1u << s.shift;
-    const bool exact = s.shift == 0;
-    const uint32_t rel = blockIdx.x - ld.first_chunk;
+    const bool exact = s.shift == 0, many = !exact && (s.code & kSelMany) != 0;
+    const uint32_t rel = blockIdx.x - ld.first_chunk, code = s.code & 127u;
     if (threadIdx.x == 0) s_n = 0;
     __syncthreads();
     const DView dd(dbuf, w, cv.a0);
     auto append = [&](uint32_t at, uint32_t rec) { // one entry of the layer's interval, the at-th
-        const size_t wr = in.slot(w, ch.layer);
-        if (at < (uint32_t)kListCap) in.list(wr)[at] = make_uint2(rel, rec);
-        else if (KIMAD_CHECK((rec & 0xffffu) < width, 1)) atomicAdd(in.key_count(wr, rec & 0xffffu), 1u);
+        if (at < kListCap) in.list(in.slot(w, ch.layer))[at] = make_uint2(rel, rec);
     };
     // Codes first: an entry whose code (the byte the sweep left for it) is larger than the code of the interval's
     // keys lies above the interval, one with a smaller code below; only entries with the interval's own code are
     // completed from the inputs.  Codes are 7-bit numbers, so "x >= t" for the four bytes of a word is bit 7 of
     // every byte of x + (0x80 - t) * 0x01010101.
-    const uint32_t add_gt = (0x80u - (s.code + 1u)) * 0x01010101u, add_ge = (0x80u - s.code) * 0x01010101u;
+    const uint32_t add_gt = (0x80u - (code + 1u)) * 0x01010101u, add_ge = (0x80u - code) * 0x01010101u;
     for (uint32_t sl = wid + blockIdx.z * (kThreads / 32); sl < (uint32_t)kSlices; sl += gridDim.z * (kThreads / 32)) {
-        uint32_t above = 0; // low half: entries above the interval; high half: entries equal to an exact threshold
+        // low half: entries above the interval; high half: entries equal to an exact threshold, or in the slice's own list
+        uint32_t above = 0;
         uint32_t mask[kSliceElems / 512];
-        auto visit = [&](uint32_t key) -> bool { // true: the key is not below the interval
+        auto visit = [&](uint32_t key, auto many_c) -> bool { // true: the key is not below the interval
             const uint32_t d1 = key - lo; // wraps to >= 2^31 for keys below the interval
             if (d1 < width) {
-                // an exact threshold needs no list, only the slice's number of equal entries (there may be millions of
-                // them: the exact zeros of a sparse gradient)
-                if (exact) {
+                if (decltype(many_c)::value) {
+                    above += 0x10000u;
+                    const SliceList mine(dbuf, w, cv, sl);
+                    const uint32_t p = atomicAdd(&s_in[wid], 1u);
+                    if (p < mine.cap) mine.at[p] = (uint16_t)d1;
+                    if (KIMAD_CHECK(d1 < (1u << kMaxShift), 1)) atomicAdd(in.key_count(in.slot(w, ch.layer), d1), 1u);
+                } else if (exact) {
+                    // an exact threshold needs no list, only the slice's number of equal entries (there may be millions of
+                    // them: the exact zeros of a sparse gradient)
                     above += 0x10000u;
                 } else {
                     const uint32_t p = atomicAdd(&s_n, 1u);
@@ -137,14 +155,20 @@ k_sel_count(DSource dbuf, const Chunk* __restrict__ chunks, uint32_t n_chunks, u
         const uint32_t u0 = sl * (kSliceElems / 16) + lane; // this lane's 16-element unit in row 0
         // EDGE: the slice reaches over an end of the chunk; its units there hold codes of the neighbouring chunk, or bytes that
         // nobody wrote
-        auto count = [&](auto edge_c) {
-            constexpr bool EDGE = decltype(edge_c)::value;
+        // MANY: every slice has a list of its own
+        auto count = [&](auto edge_c, auto many_c) {
+            constexpr bool EDGE = decltype(edge_c)::value, MANY = decltype(many_c)::value;
             uint4 a[ROWS];
 #pragma unroll
             for (int r = 0; r < ROWS; ++r) {
                 const uint32_t e0 = 16 * (u0 + r * 32);
                 if (EDGE) a[r] = make_uint4(0u, 0u, 0u, 0u);
                 if (!EDGE || (e0 + 16 > cv.first && e0 < cv.len)) a[r] = __ldcs(reinterpret_cast<const uint4*>(dd.code) + u0 + r * 32);
+            }
+            if (MANY) { // the list takes the place of the codes
+                __syncwarp();
+                if (lane == 0) s_in[wid] = 0;
+                __syncwarp();
             }
 #pragma unroll
             for (int r = 0; r < ROWS; ++r) {
@@ -190,15 +214,16 @@ k_sel_count(DSource dbuf, const Chunk* __restrict__ chunks, uint32_t n_chunks, u
                     while (border) { // completed from the inputs two at a time: their loads are independent
                         const uint32_t p0 = take(), p1 = border ? take() : p0;
                         const float v0 = dd.at(p0), v1 = dd.at(p1);
-                        f |= visit(key_of(v0));
-                        if (p1 != p0) f |= visit(key_of(v1));
+                        f |= visit(key_of(v0), many_c);
+                        if (p1 != p0) f |= visit(key_of(v1), many_c);
                     }
                 }
                 mask[r] = __ballot_sync(0xffffffffu, f);
             }
         };
-        if (sl * kSliceElems >= cv.first && (sl + 1) * kSliceElems <= cv.len) count(std::false_type{});
-        else count(std::true_type{});
+        if (many) count(std::true_type{}, std::true_type{});
+        else if (sl * kSliceElems >= cv.first && (sl + 1) * kSliceElems <= cv.len) count(std::false_type{}, std::false_type{});
+        else count(std::true_type{}, std::false_type{});
 #pragma unroll
         for (int o = 16; o; o >>= 1) above += __shfl_xor_sync(0xffffffffu, above, o);
         if (lane == 0) { out->above[sl] = (uint16_t)above; out->eq[sl] = (uint16_t)(above >> 16); out->mask[sl] = make_uint4(mask[0], mask[1], mask[2], mask[3]); }
@@ -281,8 +306,8 @@ k_sel_offsets(const LayerDesc* __restrict__ layers, const Chunk* __restrict__ ch
     if (s.k != 0 && (uint64_t)s.k != ld.n && s.shift != 0) {
         const size_t wr = in.slot(w, l);
         const uint2* list = in.list(wr);
-        const uint32_t total = in.n[wl], cnt = min(total, (uint32_t)kListCap);
-        const bool over = total > (uint32_t)kListCap;
+        const uint32_t cnt = min(in.n[wl], kListCap);
+        const bool over = (s.code & kSelMany) != 0;
         if (!over) {
             for (uint32_t i = threadIdx.x; i < cnt; i += NT) s_key[i] = (uint16_t)(list[i].y & 0xffffu);
             uint32_t rank = s.keep_eq, hi_digit = 0, greater = 0; // rank <= cnt by construction
@@ -328,10 +353,7 @@ k_sel_offsets(const LayerDesc* __restrict__ layers, const Chunk* __restrict__ ch
                 atomicAdd(c, 1u << (16u * (sl & 1u)));
             }
             __threadfence(); // the counts are read back below by other threads of this CTA
-        } else { // every key of the interval was counted, but for the listed entries
-            for (uint32_t i = threadIdx.x; i < cnt; i += NT) atomicAdd(in.key_count(wr, list[i].y & 0xffffu), 1u);
-            __threadfence();
-            __syncthreads();
+        } else { // every key of the interval was counted
             // thread t takes the keys [k0, k1), descending with t
             const uint32_t width = 1u << s.shift, per = (width + NT - 1) / NT;
             const uint32_t k1 = threadIdx.x * per < width ? width - threadIdx.x * per : 0u, k0 = k1 > per ? k1 - per : 0u;
@@ -367,47 +389,82 @@ k_sel_offsets(const LayerDesc* __restrict__ layers, const Chunk* __restrict__ ch
     sel_scan_layer<NT>(ld, s, chunks, phase.at(w), cs, jobs + (size_t)w * n_chunks + ld.first_chunk, s_w);
 }
 
-// Exact per-slice (gt, eq) of the listed chunks: warp w recounts the slices w and w + 8.  The CTA that finishes the last
-// chunk of a layer makes the layer's job records (Interval::n counts the finished ones).
+// Exact per-slice (gt, eq) of the listed chunks, a warp per chunk: from the slices' lists, or from the inputs where a slice has more
+// entries inside the interval than its list holds.  The CTA that finishes the last chunk of a layer makes the layer's job records
+// (Interval::n counts the finished ones).  Bound by latency: the first 32 entries of all lists of a chunk are requested together.
+// Values of bf16 gradients (4 x 124 M, 0.6 % kept): offsets 1226 us with every chunk counted
+// again from the inputs, 77 so, and 22 where nothing repeats.
 __global__ void __launch_bounds__(kThreads)
 k_sel_recount(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* __restrict__ chunks, uint32_t n_chunks,
               uint32_t L, const Sel* __restrict__ sel, ChunkSel* __restrict__ csel, ChunkJob* __restrict__ jobs, const Interval in,
               const Recount* __restrict__ rc, const uint2* __restrict__ rc_chunks) {
     pdl_wait();
-    __shared__ uint32_t s_w[kThreads / 32], s_last;
+    constexpr uint32_t kWarps = kThreads / 32;
+    __shared__ uint32_t s_w[kWarps], s_last[kWarps]; // s_last: the warp's chunk was the last one of its layer
     const uint32_t n = rc->n_chunks;
     const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (uint32_t it = blockIdx.x; it < n; it += gridDim.x) {
-        const uint2 e = rc_chunks[it];
-        const Chunk ch = chunks[e.y];
-        const size_t wl = (size_t)e.x * L + ch.layer;
-        const Sel s = sel[wl];
-        const ChunkView cv(ch, dbuf.phase.at(e.x));
-        const DView dd(dbuf, e.x, cv.a0);
-        ChunkSel* out = csel + (size_t)e.x * n_chunks + e.y;
-        for (uint32_t sl = wid; sl < (uint32_t)kSlices; sl += kThreads / 32) {
-            uint32_t gt = 0, eq = 0;
-            const uint32_t x0 = max(cv.first, sl * kSliceElems), x1 = min(cv.len, (sl + 1) * kSliceElems);
-            for (uint32_t x = x0 + lane; x < x1; x += 32) {
-                const uint32_t key = key_of(dd.at(x));
-                gt += key > s.tau;
-                eq += key == s.tau;
+    for (uint32_t base = blockIdx.x * kWarps; base < n; base += gridDim.x * kWarps) {
+        if (lane == 0) s_last[wid] = 0;
+        if (base + wid < n) {
+            const uint2 e = rc_chunks[base + wid];
+            const Chunk ch = chunks[e.y];
+            const size_t wl = (size_t)e.x * L + ch.layer;
+            const Sel s = sel[wl];
+            const ChunkView cv(ch, dbuf.phase.at(e.x));
+            ChunkSel* out = csel + (size_t)e.x * n_chunks + e.y;
+            const uint32_t my_in = lane < (uint32_t)kSlices ? out->eq[lane] : 0u; // lane i: slice i
+            uint32_t my_gt = lane < (uint32_t)kSlices ? out->above[lane] : 0u, my_eq = 0;
+            uint32_t first[kSlices]; // the slices' first entries, a lane each
+#pragma unroll
+            for (int sl = 0; sl < kSlices; ++sl) {
+                const SliceList list(dbuf, e.x, cv, sl);
+                const uint32_t n_in = __shfl_sync(0xffffffffu, my_in, sl);
+                first[sl] = lane < n_in && n_in <= list.cap ? list.at[lane] : 0xffffffffu;
             }
 #pragma unroll
-            for (int o = 16; o; o >>= 1) {
-                gt += __shfl_xor_sync(0xffffffffu, gt, o);
-                eq += __shfl_xor_sync(0xffffffffu, eq, o);
+            for (int sl = 0; sl < kSlices; ++sl) {
+                const SliceList list(dbuf, e.x, cv, sl);
+                const uint32_t n_in = __shfl_sync(0xffffffffu, my_in, sl);
+                if (n_in == 0) continue;
+                uint32_t gt = 0, eq = 0;
+                if (n_in <= list.cap) {
+                    auto count = [&](uint32_t d) {
+                        gt += __popc(__ballot_sync(0xffffffffu, d != 0xffffffffu && d > s.tau_low));
+                        eq += __popc(__ballot_sync(0xffffffffu, d == s.tau_low));
+                    };
+                    count(first[sl]);
+                    for (uint32_t i = 32; i < n_in; i += 32) count(i + lane < n_in ? list.at[i + lane] : 0xffffffffu);
+                    gt += __shfl_sync(0xffffffffu, my_gt, sl);
+                } else {
+                    const DView dd(dbuf, e.x, cv.a0);
+                    const uint32_t x0 = max(cv.first, sl * kSliceElems), x1 = min(cv.len, (sl + 1) * kSliceElems);
+                    for (uint32_t x = x0 + lane; x < x1; x += 32) {
+                        const uint32_t key = key_of(dd.at(x));
+                        gt += key > s.tau;
+                        eq += key == s.tau;
+                    }
+#pragma unroll
+                    for (int o = 16; o; o >>= 1) {
+                        gt += __shfl_xor_sync(0xffffffffu, gt, o);
+                        eq += __shfl_xor_sync(0xffffffffu, eq, o);
+                    }
+                }
+                if (lane == (uint32_t)sl) { my_gt = gt; my_eq = eq; }
             }
-            if (lane == 0) { out->above[sl] = (uint16_t)gt; out->eq[sl] = (uint16_t)eq; }
-        }
-        const LayerDesc ld = layers[ch.layer];
-        __threadfence();
-        __syncthreads();
-        if (threadIdx.x == 0) s_last = atomicAdd(in.n + wl, 1u) + 1u == ld.n_chunks;
-        __syncthreads();
-        if (s_last) {
+            if (lane < (uint32_t)kSlices) { out->above[lane] = (uint16_t)my_gt; out->eq[lane] = (uint16_t)my_eq; }
             __threadfence();
-            sel_scan_layer<kThreads>(ld, s, chunks, dbuf.phase.at(e.x), csel + (size_t)e.x * n_chunks + ld.first_chunk,
+            __syncwarp();
+            if (lane == 0) s_last[wid] = atomicAdd(in.n + wl, 1u) + 1u == layers[ch.layer].n_chunks;
+        }
+        __syncthreads();
+        for (uint32_t i = 0; i < kWarps; ++i) {
+            if (!s_last[i]) continue;
+            const uint2 e = rc_chunks[base + i];
+            const uint32_t l = chunks[e.y].layer;
+            const size_t wl = (size_t)e.x * L + l;
+            const LayerDesc ld = layers[l];
+            __threadfence();
+            sel_scan_layer<kThreads>(ld, sel[wl], chunks, dbuf.phase.at(e.x), csel + (size_t)e.x * n_chunks + ld.first_chunk,
                                      jobs + (size_t)e.x * n_chunks + ld.first_chunk, s_w);
             if (threadIdx.x == 0) in.n[wl] = 0;
         }
