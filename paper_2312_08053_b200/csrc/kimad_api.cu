@@ -235,8 +235,7 @@ static bool plan_choice(kimad_ctx* c) {
     size_t used = ((size_t)2 * (2 * c->D + 3) + c->L) * 4;
     if (c->policy == 2) {
         used += (size_t)c->L * Kp * 8;
-        // (a word per layer and 16 bytes more than the tables take: which contexts are accepted is part of the interface)
-        if (used + (size_t)c->L * 4 + 16 > kDpSmemMax) return false;
+        if (used > kDpSmemMax) return false;
         const size_t pd_bytes = (size_t)c->L * q.pd_row_bytes;
         q.pd_in_smem = used + pd_bytes <= kDpSmemMax ? 1u : 0u;
         if (q.pd_in_smem) used += pd_bytes;

@@ -75,16 +75,6 @@ def test_create_rejects_bad_arguments():
         assert e.value.code == kb.KIMAD_ERR_INVALID_ARG
 
 
-def test_error_axis_is_refused_where_its_tables_are_too_large():
-    """Policy 2 with 33 candidates and 1000 cells: 724 layers are accepted and no more."""
-    grid = [(j + 1) / 33 for j in range(33)]
-    kb.kimad_destroy(kb.kimad_create([10] * 724, 1, grid, D=1000, policy=2))
-    for n in (725, 734):
-        with pytest.raises(kb.KimadError) as e:
-            kb.kimad_create([10] * n, 1, grid, D=1000, policy=2)
-        assert e.value.code == kb.KIMAD_ERR_INVALID_ARG
-
-
 def test_step_without_workspace_is_refused():
     ctx = kb.kimad_create([8], 1, [1.0])
     out = kb.kimad_packed(1, 1, 1, 1, 1, 1)
