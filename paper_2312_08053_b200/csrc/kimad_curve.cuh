@@ -643,9 +643,9 @@ k_pass_a(const float* __restrict__ grads, const float* __restrict__ state, uint8
 // end with a step that needs all of them.  Layers of large contexts are listed with their chunks (k_refine, k_fb1, k_fb23), which
 // costs every step four launches, a second launch of the DP and two event waits although the lists are usually empty.  Where no
 // layer has more than kInlineChunks chunks the curve kernel's CTA takes them itself (layer_by_itself): 62 tensors of up to
-// 147 K elements 116.5 -> 112 us a step, a small model through a built-in workspace 98 -> 86 us.  A layer that does need the
-// exact path costs 110 (list: 166) us with one chunk, 136 (166) with two, 197 (168) with four, 317 (172) with eight; hence the
-// second bound for contexts that take it always.
+// 147 K elements 116.5 -> 112 us a step, a small model through a built-in workspace 98 -> 86 us.  With one layer of thirty
+// candidates on the exact path a step takes 190 us with two chunks, 242 with four, 268 with five and about 340 with eight, 234 over
+// lists with nine; hence the second bound for contexts that take it always.
 // ------------------------------------------------------------------------------------------------
 constexpr uint32_t kInlineChunks = 8, kInlineChunksExact = 2;
 struct ListArgs {
@@ -764,66 +764,74 @@ __device__ __forceinline__ void refine_chunk(const ListArgs& a, uint32_t w, cons
     }
 }
 
-// The pieces of a layer's loose bins resolved; the loose candidates one after the other.  Candidates that share a bin were
-// counted into the histogram of the first of them (the lowest j): the later ones read it there.  True where a bound is still
-// too loose (a bin with very many entries): the layer needs the exact path after all.
+// The pieces of a layer's loose bins resolved, a warp per candidate and a lane per 32 consecutive pieces (ascending keys).  Candidates
+// that share a bin were counted into the histogram of the first of them (the lowest j): the later ones read it there.  True where a
+// bound is still too loose (a bin with very many entries): the layer needs the exact path after all.
 template <int NT>
 __device__ __forceinline__ bool refine_resolve_layer(const ListArgs& a, uint32_t l, uint32_t w, size_t wl, size_t wr) {
-    __shared__ uint32_t s_w32[NT / 32];
-    __shared__ double s_w64[NT / 32];
     __shared__ int s_bad;
+    const uint32_t lane = threadIdx.x & 31;
     __syncthreads();
     if (threadIdx.x == 0) s_bad = 0;
     __syncthreads();
-    for (uint32_t j = 0; j < a.K; ++j) {
+    for (uint32_t j = threadIdx.x >> 5; j < a.K; j += NT / 32) {
         const RefineCand rc = a.rf[wl * a.K + j];
         if (rc.shift == kNoRefine) continue;
         uint32_t owner = j; // the first loose candidate with this bin holds the pieces
-        for (uint32_t i = 0; i < j; ++i) {
-            const RefineCand o = a.rf[wl * a.K + i];
-            if (o.shift != kNoRefine && o.klo == rc.klo) { owner = i; break; }
+        for (uint32_t i0 = 0; i0 < j && owner == j; i0 += 32u) {
+            bool same = false;
+            if (i0 + lane < j) {
+                const RefineCand o = a.rf[wl * a.K + i0 + lane];
+                same = o.shift != kNoRefine && o.klo == rc.klo;
+            }
+            const uint32_t m = __ballot_sync(0xffffffffu, same);
+            if (m) owner = i0 + __ffs(m) - 1u;
         }
-        const uint32_t sub = rc.shift > 10u ? rc.shift - 10u : 0u, nsub = 1u << (rc.shift - sub);
-        const uint32_t* gc = a.h23_cnt + (wr * a.K + owner) * kL23Bins;
+        const uint32_t sub = rc.shift > 10u ? rc.shift - 10u : 0u, b0 = 32u * lane;
+        const uint32_t* gc = a.h23_cnt + (wr * a.K + owner) * kL23Bins; // (pieces beyond 2^(shift - sub) are zero)
         const unsigned long long* gs = a.h23_ss + (wr * a.K + owner) * kL23Bins;
         const double scale = sq_scale(rc.klo >> 23);
-        // four consecutive pieces per thread, ascending keys
-        uint32_t c[4], csum = 0;
-        double q[4], qsum = 0.0;
+        uint32_t c[32], csum = 0;
+        load_counts(c, gc, b0);
+        const double qsum = add_squares(0.0, gs, b0, 32u, scale);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const uint32_t b = 4 * threadIdx.x + i;
-            c[i] = b < nsub ? __ldcg(gc + b) : 0u;
-            q[i] = b < nsub ? (double)__ldcg(gs + b) * scale : 0.0;
-            csum += c[i];
-            qsum += q[i];
+        for (int i = 0; i < 32; ++i) csum += c[i];
+        uint32_t upto = csum; // entries in the lane's pieces and those of the lanes below
+        double below = qsum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t yc = __shfl_up_sync(0xffffffffu, upto, o);
+            const double ys = __shfl_up_sync(0xffffffffu, below, o);
+            if (lane >= (uint32_t)o) { upto += yc; below += ys; }
         }
-        uint32_t tot;
-        uint32_t before = block_excl_scan<uint32_t, NT>(csum, s_w32, &tot);
-        double below = block_excl_scan<double, NT>(qsum, s_w64, nullptr);
+        below = __shfl_up_sync(0xffffffffu, below, 1); // exclusive value from the left neighbour: no cancellation
+        if (lane == 0) below = 0.0;
+        const uint32_t tot = __shfl_sync(0xffffffffu, upto, 31);
         if (!KIMAD_CHECK(tot == rc.cb, 7)) s_bad = 1;
         const size_t o = wl * a.K + j;
+        if (upto - csum <= rc.drop && rc.drop < upto) { // one lane: the piece that holds the threshold is one of its own
+            uint32_t i = 0, before = upto - csum, ci = 0;
+            bool open = true;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            if (c[i] && rc.drop >= before && rc.drop - before < c[i]) { // the piece that holds the threshold
-                const uint32_t b = 4 * threadIdx.x + i, klo = rc.klo + (b << sub), d2 = rc.drop - before;
-                const double vlo = (double)__uint_as_float(klo);
-                const double upper = q[i] * ((double)d2 / (double)c[i]), lower = (double)d2 * vlo * vlo;
-                double part = 0.5 * (upper + lower), slack = 0.5 * (upper - lower);
-                if (d2 == 0 || sub == 0) { part = lower; slack = 0.0; }
-                const double e = rc.below + below + part;
-                if (slack > e * 5e-6) {
-                    s_bad = 1;
-                } else {
-                    a.err[o] = (float)e; a.tau[o] = klo; a.keep_eq[o] = c[i] - d2;
-                    a.shift[o] = sub | (a.codes.code(w, l, klo) | (sub && c[i] > kListCap ? kSelMany : 0u)) << 8;
-                }
+            for (int x = 0; x < 32; ++x) {
+                if (open && rc.drop - before < c[x]) { open = false; i = x; ci = c[x]; }
+                if (open) before += c[x];
             }
-            before += c[i];
-            below += q[i];
+            const uint32_t b = b0 + i, klo = rc.klo + (b << sub), d2 = rc.drop - before;
+            const double vlo = (double)__uint_as_float(klo), qi = (double)__ldcg(gs + b) * scale;
+            const double upper = qi * ((double)d2 / (double)ci), lower = (double)d2 * vlo * vlo;
+            double part = 0.5 * (upper + lower), slack = 0.5 * (upper - lower);
+            if (d2 == 0 || sub == 0) { part = lower; slack = 0.0; }
+            const double e = rc.below + add_squares(below, gs, b0, i, scale) + part;
+            if (slack > e * 5e-6) {
+                s_bad = 1;
+            } else {
+                a.err[o] = (float)e; a.tau[o] = klo; a.keep_eq[o] = ci - d2;
+                a.shift[o] = sub | (a.codes.code(w, l, klo) | (sub && ci > kListCap ? kSelMany : 0u)) << 8;
+            }
         }
-        __syncthreads();
     }
+    __syncthreads(); // the pieces have been read
     // clean the pieces, close the candidates
     for (uint32_t j = 0; j < a.K; ++j) {
         if (a.rf[wl * a.K + j].shift == kNoRefine) continue;
@@ -841,9 +849,9 @@ __device__ __forceinline__ bool refine_resolve_layer(const ListArgs& a, uint32_t
 // exact radix path over the handed-over chunks.  The list is usually empty, but a handed-over layer may be large and
 // may hold one key millions of times (the exact zeros of a sparse gradient): every thread therefore adds up the run
 // of consecutive elements of its own that fall into one bin and issues its atomics when the bin changes, and keeps
-// four elements' loads in flight.
+// eight elements' loads in flight (every layer of GPT-2 small on this path: 2254 us a step, with four 2319).
 // ------------------------------------------------------------------------------------------------
-constexpr int kFbAhead = 4; // elements per thread whose loads are issued together
+constexpr int kFbAhead = 8; // elements per thread whose loads are issued together
 
 // s_cnt, s_below [kL1Bins]; s_below holds the two words of the chunk's sums
 template <int NT>
@@ -897,12 +905,15 @@ __device__ __forceinline__ void fb23_chunk(const ListArgs& a, uint32_t w, const 
     for (int b = threadIdx.x; b < kL1Bins; b += NT) { s_first[b] = 0xff; s_num[b] = 0; }
     for (uint32_t s = threadIdx.x; s < ns; s += NT) s_prefix[s] = stab.prefix[s];
     __syncthreads();
-    if (threadIdx.x == 0)
-        for (uint32_t s = 0; s < ns; ++s) {
-            const uint32_t b1 = LEVEL == 2 ? s_prefix[s] : (s_prefix[s] >> 10);
-            if (s_first[b1] == 0xff) s_first[b1] = (uint8_t)s;
-            s_num[b1]++;
-        }
+    auto bin1 = [&](uint32_t s) { return LEVEL == 2 ? s_prefix[s] : s_prefix[s] >> 10; };
+    for (uint32_t s = threadIdx.x; s < ns; s += NT) { // slots that share a level-1 bin follow each other
+        const uint32_t b1 = bin1(s);
+        if (s && bin1(s - 1u) == b1) continue;
+        uint32_t n = 1;
+        while (s + n < ns && bin1(s + n) == b1) ++n;
+        s_first[b1] = (uint8_t)s;
+        s_num[b1] = (uint8_t)n;
+    }
     __syncthreads();
     const ChunkView cv(ch, a.src.phase.at(w));
     const DView dd(a.src, w, cv.a0);
@@ -975,18 +986,37 @@ __device__ __noinline__ void layer_by_itself(const ListArgs& a, uint32_t l, uint
     fb23_resolve<3, NT>(a, l, w, wl, wr);
 }
 
+// A CTA's share of a list: consecutive entries, which are mostly of one layer (a layer's chunks follow each other), so that a layer's
+// counter and the fence before it are touched once per CTA and not per chunk.  work(w, chunk, wl, wr) per entry, finish(w, layer, wl, wr)
+// in the CTA that finishes a layer.
+template <typename Work, typename Finish>
+__device__ __forceinline__ void over_list(const ListArgs& a, const uint2* __restrict__ list, uint32_t n, Work work, Finish finish) {
+    const uint32_t per = (n + gridDim.x - 1u) / gridDim.x, end = min(n, (blockIdx.x + 1u) * per);
+    uint32_t done = 0;
+    for (uint32_t it = blockIdx.x * per; it < end; ++it) {
+        const uint2 e = list[it];
+        const Chunk ch = a.chunks[e.y];
+        const size_t wl = (size_t)e.x * a.L + ch.layer, wr = a.codes.slot(e.x, ch.layer);
+        work(e.x, ch, wl, wr);
+        ++done;
+        if (it + 1u < end) {
+            const uint2 next = list[it + 1u];
+            if (next.x == e.x && a.chunks[next.y].layer == ch.layer) continue;
+        }
+        if (last_of_layer(a.arrived + wl, done, a.layers[ch.layer].n_chunks)) finish(e.x, ch.layer, wl, wr);
+        done = 0;
+    }
+}
+
 __global__ void __launch_bounds__(kThreads, 5)
 k_refine(const ListArgs a, const uint2* __restrict__ rf_chunks, uint2* __restrict__ fb_chunks, uint32_t list_cap) {
     pdl_wait();
     __shared__ uint32_t s_at;
-    const uint32_t n = a.fb->rf_chunks;
-    for (uint32_t it = blockIdx.x; it < n; it += gridDim.x) {
-        const uint2 e = rf_chunks[it];
-        const Chunk ch = a.chunks[e.y];
-        const LayerDesc ld = a.layers[ch.layer];
-        const size_t wl = (size_t)e.x * a.L + ch.layer, wr = a.codes.slot(e.x, ch.layer);
-        refine_chunk<kThreads>(a, e.x, ch, wl, wr);
-        if (last_of_layer(a.arrived + wl, ld.n_chunks) && refine_resolve_layer<kThreads>(a, ch.layer, e.x, wl, wr)) { // to the exact path after all
+    over_list(a, rf_chunks, a.fb->rf_chunks,
+        [&](uint32_t w, const Chunk& ch, size_t wl, size_t wr) { refine_chunk<kThreads>(a, w, ch, wl, wr); },
+        [&](uint32_t w, uint32_t l, size_t wl, size_t wr) {
+            if (!refine_resolve_layer<kThreads>(a, l, w, wl, wr)) return;
+            const LayerDesc ld = a.layers[l]; // to the exact path after all
             if (threadIdx.x == 0) {
                 s_at = atomicAdd(&a.fb->n_chunks, ld.n_chunks);
                 atomicAdd(&a.fb->n_layers, 1u);
@@ -995,41 +1025,33 @@ k_refine(const ListArgs a, const uint2* __restrict__ rf_chunks, uint2* __restric
             }
             __syncthreads();
             for (uint32_t i = threadIdx.x; i < ld.n_chunks; i += kThreads)
-                if (KIMAD_CHECK(s_at + i < list_cap, 2)) fb_chunks[s_at + i] = make_uint2(e.x, ld.first_chunk + i);
-        }
-    }
+                if (KIMAD_CHECK(s_at + i < list_cap, 2)) fb_chunks[s_at + i] = make_uint2(w, ld.first_chunk + i);
+            __syncthreads(); // s_at may be written again
+        });
 }
 
-__global__ void __launch_bounds__(kThreads)
+// (four CTAs per SM: the step that follows a layer's last chunk would take twice the registers)
+__global__ void __launch_bounds__(kThreads, 4)
 k_fb1(const ListArgs a, const uint2* __restrict__ fb_chunks) {
     pdl_wait();
     __shared__ __align__(16) uint32_t s_cnt[kL1Bins];
     __shared__ __align__(16) double s_below[kL1Bins];
     __shared__ uint32_t s_w32[8];
     __shared__ double s_w64[8];
-    const uint32_t n = a.fb->n_chunks;
-    for (uint32_t it = blockIdx.x; it < n; it += gridDim.x) {
-        const uint2 e = fb_chunks[it];
-        const Chunk ch = a.chunks[e.y];
-        const size_t wl = (size_t)e.x * a.L + ch.layer, wr = a.codes.slot(e.x, ch.layer);
-        fb1_chunk<kThreads>(a, e.x, ch, wr, s_cnt, s_below);
-        if (last_of_layer(a.arrived + wl, a.layers[ch.layer].n_chunks))
-            fb_resolve1_layer<kThreads>(ch.layer, e.x, wl, wr, a.K, a.h1_cnt, a.h1_ss, a.ktab, a.cands, a.slots, s_cnt, s_below, s_w32, s_w64);
-    }
+    over_list(a, fb_chunks, a.fb->n_chunks,
+        [&](uint32_t w, const Chunk& ch, size_t, size_t wr) { fb1_chunk<kThreads>(a, w, ch, wr, s_cnt, s_below); },
+        [&](uint32_t w, uint32_t l, size_t wl, size_t wr) {
+            fb_resolve1_layer<kThreads>(l, w, wl, wr, a.K, a.h1_cnt, a.h1_ss, a.ktab, a.cands, a.slots, s_cnt, s_below, s_w32, s_w64);
+        });
 }
 
 template <int LEVEL>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 4)
 k_fb23(const ListArgs a, const uint2* __restrict__ fb_chunks) {
     pdl_wait();
-    const uint32_t n = a.fb->n_chunks;
-    for (uint32_t it = blockIdx.x; it < n; it += gridDim.x) {
-        const uint2 e = fb_chunks[it];
-        const Chunk ch = a.chunks[e.y];
-        const size_t wl = (size_t)e.x * a.L + ch.layer, wr = a.codes.slot(e.x, ch.layer);
-        fb23_chunk<LEVEL, kThreads>(a, e.x, ch, wl, wr);
-        if (last_of_layer(a.arrived + wl, a.layers[ch.layer].n_chunks)) fb23_resolve<LEVEL, kThreads>(a, ch.layer, e.x, wl, wr);
-    }
+    over_list(a, fb_chunks, a.fb->n_chunks,
+        [&](uint32_t w, const Chunk& ch, size_t wl, size_t wr) { fb23_chunk<LEVEL, kThreads>(a, w, ch, wl, wr); },
+        [&](uint32_t w, uint32_t l, size_t wl, size_t wr) { fb23_resolve<LEVEL, kThreads>(a, l, w, wl, wr); });
 }
 
 // ------------------------------------------------------------------------------------------------

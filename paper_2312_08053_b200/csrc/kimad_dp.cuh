@@ -507,10 +507,13 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
         // Errors that the curve stage computes are not negative, and neither are their sums: they order as their bits do.
         const bool any_sign = s_signed != 0u;
         auto warp_min = [](float x, auto any) {
-            if (!decltype(any)::value) return __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(x)));
+            if constexpr (decltype(any)::value) {
 #pragma unroll
-            for (int o = 16; o; o >>= 1) x = fminf(x, __shfl_xor_sync(0xffffffffu, x, o));
-            return x;
+                for (int o = 16; o; o >>= 1) x = fminf(x, __shfl_xor_sync(0xffffffffu, x, o));
+                return x;
+            } else {
+                return __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(x)));
+            }
         };
         __syncthreads();
         for (uint32_t left = n_ex; left;) {

@@ -271,19 +271,55 @@ struct CodeSpace { // how the sweep coded the elements of one (worker, layer)
 
 // Work over chunks of listed layers ends, per layer, with a step that needs all of them: the CTA that finishes the layer's
 // last chunk takes that step.  True (for the whole CTA) in that CTA, which then sees what the others wrote; the counter is
-// back at zero.  Every thread of the CTA calls it after its last write for the chunk.
-__device__ __forceinline__ bool last_of_layer(uint32_t* counter, uint32_t n_chunks) {
+// back at zero.  Every thread of the CTA calls it after its last write for the `done` chunks.
+__device__ __forceinline__ bool last_of_layer(uint32_t* counter, uint32_t done, uint32_t n_chunks) {
     __shared__ uint32_t s_last;
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) {
-        s_last = atomicAdd(counter, 1u) + 1u == n_chunks;
+        s_last = atomicAdd(counter, done) + done == n_chunks;
         if (s_last) *counter = 0;
     }
     __syncthreads();
     const bool last = s_last != 0;
     if (last) __threadfence();
     return last;
+}
+
+// The 32 counts from b0 on (a lane's share of a histogram of kL23Bins), requested together.
+__device__ __forceinline__ void load_counts(uint32_t (&c)[32], const uint32_t* gc, uint32_t b0) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const uint4 x = __ldcg(reinterpret_cast<const uint4*>(gc + b0) + q);
+        c[4 * q] = x.x; c[4 * q + 1] = x.y; c[4 * q + 2] = x.z; c[4 * q + 3] = x.w;
+    }
+}
+// `from` and the first `upto` of the 32 sums of squares from b0 on, added in order.
+__device__ __forceinline__ double add_squares(double from, const unsigned long long* gs, uint32_t b0, uint32_t upto, double scale) {
+#pragma unroll 8
+    for (uint32_t q = 0; q < 16; ++q) {
+        if (2u * q >= upto) break;
+        const ulonglong2 x = __ldcg(reinterpret_cast<const ulonglong2*>(gs + b0) + q);
+        from += (double)x.x * scale;
+        if (2u * q + 1u < upto) from += (double)x.y * scale;
+    }
+    return from;
+}
+// Slots of a layer's candidates: one per distinct prefix, in candidate order (prefixes do not increase with the candidate).  By a warp.
+__device__ __forceinline__ void assign_slots(Cand* cd, SlotTab& stab, uint32_t K) {
+    const uint32_t lane = threadIdx.x & 31;
+    uint32_t n = 0, last = 0;
+    for (uint32_t j0 = 0; j0 < K; j0 += 32u) {
+        const uint32_t j = j0 + lane, pfx = j < K ? cd[j].prefix : 0u;
+        const uint32_t left = __shfl_up_sync(0xffffffffu, pfx, 1);
+        const bool first = j < K && (lane ? left != pfx : (n == 0u || last != pfx));
+        const uint32_t m = __ballot_sync(0xffffffffu, first), slot = n + __popc(m & (0xffffffffu >> (31u - lane))) - 1u;
+        if (first) stab.prefix[slot] = pfx;
+        if (j < K) cd[j].slot = slot;
+        last = __shfl_sync(0xffffffffu, pfx, min(K - 1u - j0, 31u));
+        n += __popc(m);
+    }
+    if (lane == 0) stab.n = n;
 }
 
 // Level 1 of the exact radix select of one (worker, layer): candidates -> level-1 bins.  By a whole CTA; s_incl and s_below are
@@ -317,20 +353,13 @@ __device__ __forceinline__ void fb_resolve1_layer(uint32_t l, uint32_t w, size_t
         cd[j] = c;
     }
     __syncthreads();
-    if (threadIdx.x == 0) { // distinct prefixes, in candidate order (prefix is non-increasing in j)
-        SlotTab& stab = slots[wl];
-        uint32_t ns = 0;
-        for (uint32_t j = 0; j < K; ++j) {
-            if (ns == 0 || stab.prefix[ns - 1] != cd[j].prefix) stab.prefix[ns++] = cd[j].prefix;
-            cd[j].slot = ns - 1;
-        }
-        stab.n = ns;
-    }
+    if (threadIdx.x < 32) assign_slots(cd, slots[wl], K);
     __syncthreads();
 }
 
 // LEVEL 2: refine inside a level-1 bin; LEVEL 3: inside a (level-1, level-2) bin.  By a whole CTA, a warp per slot: a lane takes
-// 32 consecutive bins.  Leaves the histograms clean.
+// 32 consecutive bins, whose counts it keeps.  Leaves the histograms clean.  Bound by the latency of a few rounds of loads per slot;
+// with bins read one at a time, again for every candidate, it was the longest part of a layer's exact path.
 template <int LEVEL, int NT>
 __device__ __forceinline__ void fb_resolve23_layer(uint32_t l, uint32_t w, size_t wl, size_t wr, uint32_t K, uint32_t* __restrict__ g_cnt,
                                                    unsigned long long* __restrict__ g_ss, Cand* __restrict__ cands,
@@ -346,15 +375,18 @@ __device__ __forceinline__ void fb_resolve23_layer(uint32_t l, uint32_t w, size_
         unsigned long long* gs = g_ss + (wr * K + s) * kL23Bins;
         const uint32_t prefix = stab.prefix[s], b0 = 32u * lane;
         const double scale = LEVEL == 2 ? sq_scale(prefix >> 3) : 0.0; // LEVEL 2: prefix = level-1 bin (8 exponent + 3 mantissa bits)
-        auto count = [&](uint32_t b) { return __ldcg(gc + b); };
-        auto squares = [&](uint32_t b, uint32_t c) { // LEVEL 3: all 31 bits known, the sum of squares is count * value^2
-            if (LEVEL == 2) return (double)__ldcg(gs + b) * scale;
-            const double v = (double)__uint_as_float((prefix << 10) | b);
-            return (double)c * v * v;
-        };
-        uint32_t cnt = 0;
+        auto value = [&](uint32_t b) { return (double)__uint_as_float((prefix << 10) | b); };
+        uint32_t c[32], cnt = 0;
+        load_counts(c, gc, b0);
         double sq = 0.0;
-        for (uint32_t b = b0; b < b0 + 32u; ++b) { const uint32_t c = count(b); cnt += c; sq += squares(b, c); }
+        if (LEVEL == 2) {
+            sq = add_squares(sq, gs, b0, 32u, scale);
+#pragma unroll
+            for (int i = 0; i < 32; ++i) cnt += c[i];
+        } else { // all 31 bits known, the sum of squares is count * value^2
+#pragma unroll
+            for (int i = 0; i < 32; ++i) { const double v = value(b0 + i); cnt += c[i]; sq += (double)c[i] * v * v; }
+        }
         uint32_t upto = cnt; // entries in the lane's bins and those of the lanes above
         double below = sq;
 #pragma unroll
@@ -367,46 +399,54 @@ __device__ __forceinline__ void fb_resolve23_layer(uint32_t l, uint32_t w, size_
         const uint32_t above = upto - cnt;
         below = __shfl_up_sync(0xffffffffu, below, 1); // exclusive value from the left neighbour: no cancellation
         if (lane == 0) below = 0.0;
-        for (uint32_t j = 0; j < K; ++j) {
-            if (cd[j].slot != s) continue;
-            const uint32_t rank = cd[j].rank;
-            __syncwarp(); // read by all lanes before one of them writes it
-            if (above < rank && rank <= upto) { // one lane
-                uint32_t b = b0 + 31u, gt = above, c = count(b);
-                while (gt + c < rank) { gt += c; --b; c = count(b); }
-                double e = below;
-                for (uint32_t x = b0; x < b; ++x) e += squares(x, count(x));
-                e += cd[j].err_low;
-                const uint32_t found = (prefix << 10) | b;
-                if (LEVEL == 2) {
-                    cd[j].prefix = found;
-                    cd[j].gt += gt;
-                    cd[j].err_low = e;
-                    cd[j].rank = rank - gt;
-                } else {
-                    const uint32_t keep = rank - gt; // 1 <= keep <= c
-                    const double v = (double)__uint_as_float(found);
-                    err_out[wl * K + j] = (float)(e + (double)(c - keep) * v * v);
-                    tau_out[wl * K + j] = found;
-                    keep_eq_out[wl * K + j] = keep;
-                    shift_out[wl * K + j] = codes.code(w, l, found) << 8;
+        for (uint32_t j0 = 0; j0 < K; j0 += 32u) { // the slot's candidates, asked for by a lane each
+            const bool in = j0 + lane < K;
+            const uint32_t my_rank = in ? cd[j0 + lane].rank : 0u;
+            uint32_t here = __ballot_sync(0xffffffffu, in && cd[j0 + lane].slot == s);
+            for (; here; here &= here - 1u) {
+                const uint32_t j = j0 + __ffs(here) - 1u, rank = __shfl_sync(0xffffffffu, my_rank, j - j0);
+                if (above < rank && rank <= upto) { // one lane
+                    uint32_t i = 0, gt = above, found_c = 0; // its bin that holds the rank, counted from the top
+                    bool open = true;
+#pragma unroll
+                    for (int x = 31; x >= 0; --x) {
+                        if (open && gt + c[x] >= rank) { open = false; i = x; found_c = c[x]; }
+                        if (open) gt += c[x];
+                    }
+                    double e = below;
+                    if (LEVEL == 2) {
+                        e = add_squares(e, gs, b0, i, scale);
+                    } else {
+#pragma unroll
+                        for (int x = 0; x < 31; ++x)
+                            if ((uint32_t)x < i) { const double v = value(b0 + x); e += (double)c[x] * v * v; }
+                    }
+                    e += cd[j].err_low;
+                    const uint32_t found = (prefix << 10) | (b0 + i);
+                    if (LEVEL == 2) {
+                        cd[j].prefix = found;
+                        cd[j].gt += gt;
+                        cd[j].err_low = e;
+                        cd[j].rank = rank - gt;
+                    } else {
+                        const uint32_t keep = rank - gt; // 1 <= keep <= found_c
+                        const double v = (double)__uint_as_float(found);
+                        err_out[wl * K + j] = (float)(e + (double)(found_c - keep) * v * v);
+                        tau_out[wl * K + j] = found;
+                        keep_eq_out[wl * K + j] = keep;
+                        shift_out[wl * K + j] = codes.code(w, l, found) << 8;
+                    }
                 }
+                __syncwarp();
             }
-            __syncwarp();
         }
         __syncwarp();
-        for (uint32_t b = lane; b < (uint32_t)kL23Bins; b += 32u) { gc[b] = 0; if (LEVEL == 2) gs[b] = 0ull; }
+        for (uint32_t b = lane; b < (uint32_t)kL23Bins / 4; b += 32u) reinterpret_cast<uint4*>(gc)[b] = make_uint4(0u, 0u, 0u, 0u);
+        if (LEVEL == 2)
+            for (uint32_t b = lane; b < (uint32_t)kL23Bins / 2; b += 32u) reinterpret_cast<ulonglong2*>(gs)[b] = make_ulonglong2(0ull, 0ull);
     }
     __syncthreads();
-    if (LEVEL == 2 && threadIdx.x == 0) { // new slots = distinct 21-bit prefixes (non-increasing in j)
-        uint32_t n2 = 0;
-        for (uint32_t j = 0; j < K; ++j) {
-            const uint32_t pfx = cd[j].prefix;
-            if (n2 == 0 || stab.prefix[n2 - 1] != pfx) stab.prefix[n2++] = pfx;
-            cd[j].slot = n2 - 1;
-        }
-        stab.n = n2;
-    }
+    if (LEVEL == 2 && threadIdx.x < 32) assign_slots(cd, stab, K); // new slots = distinct 21-bit prefixes
     __syncthreads();
 }
 
