@@ -175,8 +175,8 @@ static std::vector<LaunchRec>* g_launch_trace = nullptr;
 
 // Launch with programmatic stream serialisation (the kernel must start with pdl_wait()).
 template <typename... KArgs, typename... Args>
-static cudaError_t launch_named(const char* name, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                                Args... args) {
+static cudaError_t launch_clusters(const char* name, uint32_t cluster_z, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                                   cudaStream_t s, Args... args) {
     LaunchRec rec{name, s, nullptr, nullptr};
     if (g_launch_trace) {
         if (cudaEventCreate(&rec.a) != cudaSuccess || cudaEventCreate(&rec.b) != cudaSuccess) return cudaErrorUnknown;
@@ -187,17 +187,25 @@ static cudaError_t launch_named(const char* name, void (*kern)(KArgs...), dim3 g
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = 1;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = cluster_z;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster_z > 1 ? 2 : 1;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
     if (g_launch_trace) {
         cudaEventRecord(rec.b, s);
         g_launch_trace->push_back(rec);
     }
     return e;
+}
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_named(const char* name, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
+    return launch_clusters(name, 1, kern, grid, block, smem, s, args...);
 }
 #define launch_pdl(kern, ...) launch_named(#kern, kern, __VA_ARGS__)
 
@@ -440,10 +448,14 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
         CUDA_TRY(hand_over(big, small));
         const ListArgs la{dbuf, layers, chunks, L, K, ktab, fb, rf, h1c, h1s, h23c, h23s, cands, slots, flags, err, tau, keq, shf, codes,
                           c->at<uint32_t>(y.in_n)}; // (in_n counts the select stage's entries later in the step; zero in between)
-        const bool lists = c->most_chunks > (c->curve_mode == 1 ? kInlineChunksExact : kInlineChunks);
+        // the slow paths inside the curve kernel, by clusters of cz CTAs along its grid's third axis, or over lists
+        const uint32_t cluster = inline_cluster(c->most_chunks);
+        const bool lists = c->most_chunks > (c->curve_mode == 1 ? kInlineChunksExact : kInlineChunks) ||
+                           (cluster > 1 && (uint64_t)R * nw * cluster > kInlineCtas);
+        const uint32_t cz = lists ? 1u : cluster;
         if (R) {
             auto launch = [&](auto kern) {
-                return launch_named("k_resolve_a", kern, dim3(R, nw), kBigThreads, 0, small, layers, reg_layers, R, L, ktab, K, meta, cell_win,
+                return launch_clusters("k_resolve_a", cz, kern, dim3(R, nw, cz), kBigThreads, 0, small, layers, reg_layers, R, L, ktab, K, meta, cell_win,
                                     binlo, bhc, bhs, err, tau, keq, shf, flags, fb, fb_chunks, rf, rf_chunks, list_cap, w0, la);
             };
             CUDA_TRY(lists ? launch(k_resolve_a<true>) : launch(k_resolve_a<false>));

@@ -642,12 +642,16 @@ k_pass_a(const float* __restrict__ grads, const float* __restrict__ state, uint8
 // The slow paths of a layer: refinement of loose candidates, exact radix select.  Both go over the layer's chunks and
 // end with a step that needs all of them.  Layers of large contexts are listed with their chunks (k_refine, k_fb1, k_fb23), which
 // costs every step four launches, a second launch of the DP and two event waits although the lists are usually empty.  Where no
-// layer has more than kInlineChunks chunks the curve kernel's CTA takes them itself (layer_by_itself): 62 tensors of up to
+// layer has more than kInlineChunks chunks the curve kernel takes them itself (layer_by_itself): 62 tensors of up to
 // 147 K elements 116.5 -> 112 us a step, a small model through a built-in workspace 98 -> 86 us.  With one layer of thirty
-// candidates on the exact path a step takes 190 us with two chunks, 242 with four, 268 with five and about 340 with eight, 234 over
-// lists with nine; hence the second bound for contexts that take it always.
+// candidates on the exact path a step takes 190 us with two chunks, 242 with four, 268 with five and about 340 with eight by one CTA,
+// 234 over lists with nine; hence the second bound for contexts that take it always.  Beyond four chunks a cluster of two or four CTAs
+// takes a layer (227 us with five chunks, 209 with eight); the clusters of all layers have to be resident at once (a CTA fills
+// an SM), though those whose layer needs nothing only wait, else the lists are used.
 // ------------------------------------------------------------------------------------------------
-constexpr uint32_t kInlineChunks = 8, kInlineChunksExact = 2;
+constexpr uint32_t kInlineChunks = 8, kInlineChunksExact = 2; // the latter where every layer takes the exact path
+constexpr uint32_t kInlineCtas = 128;                          // of a launch of clusters
+KIMAD_HD uint32_t inline_cluster(uint32_t most_chunks) { return most_chunks <= 4 ? 1u : (most_chunks <= 6 ? 2u : 4u); }
 struct ListArgs {
     DSource src;
     const LayerDesc* layers;
@@ -959,8 +963,13 @@ __device__ __forceinline__ void fb23_resolve(const ListArgs& a, uint32_t l, uint
     fb_resolve23_layer<LEVEL, NT>(l, w, wl, wr, a.K, a.h23_cnt, a.h23_ss, a.cands, a.slots, a.err, a.tau, a.keep_eq, a.shift, a.codes);
 }
 
-// All of it for one layer, by one CTA of kBigThreads threads.  exact: the exact path at once, else the refinement first.
-__device__ __noinline__ void layer_by_itself(const ListArgs& a, uint32_t l, uint32_t w, bool exact) {
+// A cluster's CTAs meet; what one of them wrote before is seen by all of them after.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
+// All of it for one layer, by a cluster of n CTAs of kBigThreads threads: the chunks are dealt out to them, the steps that need all
+// chunks are the first one's.  exact: the exact path at once, else the refinement first.  word: the cluster's verdict, zero afterwards.
+__device__ __noinline__ void layer_by_itself(const ListArgs& a, uint32_t l, uint32_t w, bool exact, uint32_t rank, uint32_t n, uint32_t* word) {
     constexpr int NT = kBigThreads;
     __shared__ __align__(16) uint32_t s_cnt[kL1Bins];
     __shared__ __align__(16) double s_below[kL1Bins];
@@ -968,22 +977,42 @@ __device__ __noinline__ void layer_by_itself(const ListArgs& a, uint32_t l, uint
     __shared__ double s_w64[NT / 32];
     const LayerDesc ld = a.layers[l];
     const size_t wl = (size_t)w * a.L + l, wr = a.codes.slot(w, l);
-    auto each_chunk = [&](auto f) {
-        for (uint32_t i = 0; i < ld.n_chunks; ++i) f(a.chunks[ld.first_chunk + i]);
+    auto meet = [&]() {
         __threadfence();
         __syncthreads();
+        if (n > 1u) {
+            cluster_arrive();
+            cluster_wait();
+        }
+    };
+    auto each_chunk = [&](auto f) {
+        for (uint32_t i = rank; i < ld.n_chunks; i += n) f(a.chunks[ld.first_chunk + i]);
+        meet();
     };
     if (!exact) {
         each_chunk([&](const Chunk& ch) { refine_chunk<NT>(a, w, ch, wl, wr); });
-        if (!refine_resolve_layer<NT>(a, l, w, wl, wr)) return;
-        if (threadIdx.x == 0) { atomicAdd(&a.fb->total_layers, 1u); atomicAdd(&a.fb->why[3], 1u); }
+        bool loose = false;
+        if (rank == 0) {
+            loose = refine_resolve_layer<NT>(a, l, w, wl, wr);
+            if (threadIdx.x == 0) {
+                if (n > 1u) *word = loose ? 1u : 0u;
+                if (loose) { atomicAdd(&a.fb->total_layers, 1u); atomicAdd(&a.fb->why[3], 1u); }
+            }
+        }
+        meet();
+        if (rank) loose = __ldcg(word) != 0u;
+        if (!loose) return;
     }
     each_chunk([&](const Chunk& ch) { fb1_chunk<NT>(a, w, ch, wr, s_cnt, s_below); });
-    fb_resolve1_layer<NT>(l, w, wl, wr, a.K, a.h1_cnt, a.h1_ss, a.ktab, a.cands, a.slots, s_cnt, s_below, s_w32, s_w64);
+    if (rank == 0) fb_resolve1_layer<NT>(l, w, wl, wr, a.K, a.h1_cnt, a.h1_ss, a.ktab, a.cands, a.slots, s_cnt, s_below, s_w32, s_w64);
+    meet();
     each_chunk([&](const Chunk& ch) { fb23_chunk<2, NT>(a, w, ch, wl, wr); });
-    fb23_resolve<2, NT>(a, l, w, wl, wr);
+    if (rank == 0) fb23_resolve<2, NT>(a, l, w, wl, wr);
+    meet();
     each_chunk([&](const Chunk& ch) { fb23_chunk<3, NT>(a, w, ch, wl, wr); });
+    if (rank) return;
     fb23_resolve<3, NT>(a, l, w, wl, wr);
+    if (n > 1u && threadIdx.x == 0) *word = 0; // (read by all of the cluster before the last meeting)
 }
 
 // A CTA's share of a list: consecutive entries, which are mostly of one layer (a layer's chunks follow each other), so that a layer's
@@ -1057,7 +1086,7 @@ k_fb23(const ListArgs a, const uint2* __restrict__ fb_chunks) {
 // ------------------------------------------------------------------------------------------------
 // k_resolve_a: one CTA per (regular layer, worker)
 // ------------------------------------------------------------------------------------------------
-template <bool LISTS> // false: no layer has more than kInlineChunks chunks; the slow paths are taken here
+template <bool LISTS> // false: no layer has more than kInlineChunks chunks; the slow paths are taken here, by the clusters along z
 __global__ void __launch_bounds__(kBigThreads)
 k_resolve_a(const LayerDesc* __restrict__ layers, const uint32_t* __restrict__ reg_layers, uint32_t R, uint32_t L,
             const KTab ktab, uint32_t K, const BandMeta* __restrict__ meta, const int4* __restrict__ cell_win,
@@ -1078,6 +1107,16 @@ k_resolve_a(const LayerDesc* __restrict__ layers, const uint32_t* __restrict__ r
     const uint32_t r = blockIdx.x, w = w_base + blockIdx.y;
     const uint32_t l = reg_layers[r];
     const size_t wr = (size_t)w * R + r, wl = (size_t)w * L + l;
+    if constexpr (!LISTS) {
+        if (blockIdx.z) { // the first CTA of the cluster decides
+            cluster_arrive();
+            cluster_wait();
+            uint32_t* word = la.arrived + wl;
+            const uint32_t verdict = __ldcg(word);
+            if (verdict) layer_by_itself(la, l, w, verdict == 2u, blockIdx.z, gridDim.z, word);
+            return;
+        }
+    }
     const BandMeta mt = meta[wr];
     const LayerDesc ld = layers[l];
     if (threadIdx.x == 0) { s_bad = mt.flagged; s_loose = 0; }
@@ -1182,20 +1221,31 @@ k_resolve_a(const LayerDesc* __restrict__ layers, const uint32_t* __restrict__ r
             const bool many = cb > kListCap || (klo == 0u && zeros);
             shift_out[o] = (31 - __clz(width)) | ((bin >> ls) | (many ? kSelMany : 0u)) << 8;
         }
-        __syncthreads();
-        for (uint32_t bb = threadIdx.x; bb < nb; bb += kBigThreads) // clean for the next step
-            if (gc[bb]) { gc[bb] = 0; gs[bb] = 0ull; }
     }
     __syncthreads();
     const int bad = s_bad;
+    const uint32_t verdict = bad ? 2u : (s_loose ? 1u : 0u);
+    if constexpr (!LISTS) { // the cluster's other CTAs need not wait for what follows
+        if (gridDim.z > 1u) {
+            if (verdict && threadIdx.x == 0) la.arrived[wl] = verdict;
+            cluster_arrive();
+        }
+    }
+    if (!mt.flagged) { // clean for the next step
+        uint32_t* gc = bh_cnt + wr * kMaxBins;
+        unsigned long long* gs = bh_sum + wr * kMaxBins;
+        for (uint32_t bb = threadIdx.x; bb < mt.n_bins; bb += kBigThreads)
+            if (gc[bb]) { gc[bb] = 0; gs[bb] = 0ull; }
+    }
     __shared__ uint32_t s_at;
     if constexpr (!LISTS) {
-        if (!bad && !s_loose) return;
+        if (gridDim.z > 1u) cluster_wait();
+        if (!verdict) return;
         if (threadIdx.x == 0) {
             if (bad) { atomicAdd(&fb->total_layers, 1u); atomicAdd(&fb->why[bad - 1], 1u); }
             else atomicAdd(&fb->refined, 1u);
         }
-        layer_by_itself(la, l, w, bad != 0);
+        layer_by_itself(la, l, w, bad != 0, 0u, gridDim.z, la.arrived + wl);
         return;
     }
     if (bad) { // hand the layer and its chunks to the exact path
@@ -1208,7 +1258,7 @@ k_resolve_a(const LayerDesc* __restrict__ layers, const uint32_t* __restrict__ r
         __syncthreads();
         for (uint32_t i = threadIdx.x; i < ld.n_chunks; i += kBigThreads)
             if (KIMAD_CHECK(s_at + i < list_cap, 2)) fb_chunks[s_at + i] = make_uint2(w, ld.first_chunk + i);
-    } else if (s_loose) { // only loose bounds: refine those candidates
+    } else if (verdict) { // only loose bounds: refine those candidates
         if (threadIdx.x == 0) {
             s_at = atomicAdd(&fb->rf_chunks, ld.n_chunks);
             atomicAdd(&fb->rf_layers, 1u);
