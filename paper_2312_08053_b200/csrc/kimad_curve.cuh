@@ -46,6 +46,12 @@ constexpr int kBigThreads = 1024;
 constexpr uint32_t kGapBit = 1u;                    // bin_lo entries carry this bit when the bin is a gap bin
 
 
+struct WarpLanes {
+    uint32_t lane = threadIdx.x & 31u, lanes = 32;
+    __device__ __forceinline__ uint32_t sum(uint32_t x) const { return __reduce_add_sync(0xffffffffu, x); }
+    __device__ __forceinline__ void sync() const { __syncwarp(); }
+};
+
 __device__ __forceinline__ uint32_t hash_u32(uint32_t x) {
     x ^= x >> 16; x *= 0x7feb352du; x ^= x >> 15; x *= 0x846ca68bu; x ^= x >> 16;
     return x;
@@ -71,7 +77,7 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
     uint32_t* s_cb = s_w + 32;                    // [128] per candidate, then per merged group: lowest cell,
     uint32_t* s_ct = s_cb + 128;                  // [128] highest cell,
     uint32_t* s_cs = s_ct + 128;                  // [128] shift
-    __shared__ uint32_t s_flag, s_ng, s_cg, s_z, s_clip, s_top;
+    __shared__ uint32_t s_flag, s_ng, s_cg, s_z, s_clip, s_top, s_fine;
     __shared__ unsigned long long s_zz;
     __shared__ float s_nd[128]; // bins per cell needed, per candidate, then per merged group
     const uint32_t r = blockIdx.x, w = blockIdx.y;
@@ -87,7 +93,7 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
     // the candidate of the thread's warp, asked for ahead of its use (the first one, where a warp takes several)
     const uint64_t k_first = (threadIdx.x >> 5) < K ? ktab.at(w, (size_t)l * K + (threadIdx.x >> 5)) : 0ull;
     for (int i = threadIdx.x; i < 32768 / 4; i += kBigThreads) reinterpret_cast<uint4*>(h32)[i] = make_uint4(0u, 0u, 0u, 0u);
-    if (threadIdx.x == 0) { s_flag = 0; s_ng = 0; s_cg = 0; s_z = 0; s_zz = 0ull; s_clip = 0; s_top = 0; }
+    if (threadIdx.x == 0) { s_flag = 0; s_ng = 0; s_cg = 0; s_z = 0; s_zz = 0ull; s_clip = 0; s_top = 0; s_fine = 0; }
     __syncthreads();
 
     // ---- stratified sample of |grad - g|.  Exact zeros (the untouched rows of a sparse gradient) are counted apart:
@@ -343,16 +349,30 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
             cells += s_ct[g] - s_cb[g] + 1;
         }
         if (cells > (uint64_t)kFineBins) s_flag = 3;
-        uint64_t left = 0; // fine bins not given away
-        if (!s_flag && !coarsen_groups(s_cb, s_ct, s_cs, s_nd, ng, fine, (uint64_t)kFineBins, &left)) s_flag = 3;
+        s_fine = (uint32_t)fine; // (below 2^24 unless flagged)
+        s_ng = ng;
+    }
+    uint32_t left = 0; // fine bins not given away
+    if (threadIdx.x < 32) {
+        __syncwarp();
+        if (!s_flag) {
+            const bool fit = coarsen_groups(WarpLanes{}, s_cb, s_ct, s_cs, s_nd, s_ng, s_fine, (uint32_t)kFineBins, &left);
+            __syncwarp();
+            if (!fit && threadIdx.x == 0) s_flag = 3;
+        }
+        __syncwarp();
+    }
+    if (threadIdx.x == 0 && !s_flag) {
+        uint32_t ng = s_ng;
+        const uint32_t cg = s_cg, cmask = (1u << cg) - 1u;
         // Where the rank window of the highest band reached beyond the largest sample, up to four more octaves above the band
         // get one bin per cell, as far as bins and table entries are left.  A sample without an entry as large as the smallest
         // candidate's threshold is not rare where large entries lie together (a few rows of a gradient, seven samples
         // expected), and the exact path costs far more than these bins (1.1 B Llama shape, gradients moved across
         // the tensors' borders: 4.5 layers of 402 per step on the exact path without them, 1 with one octave).
-        if (s_clip && ng && !s_flag) {
+        if (s_clip && ng) {
             const uint32_t window = (s_ct[0] >> cg) - (s_cb[ng - 1] >> cg) + 3u;
-            uint32_t ext = min(min(1024u, (uint32_t)left), window < (uint32_t)kCellTab ? ((uint32_t)kCellTab - window) << cg : 0u) & ~cmask;
+            uint32_t ext = min(min(1024u, left), window < (uint32_t)kCellTab ? ((uint32_t)kCellTab - window) << cg : 0u) & ~cmask;
             ext = min(ext, 65279u - s_ct[0]);
             if (ext) {
                 for (uint32_t g = ng; g; --g) { s_cb[g] = s_cb[g - 1]; s_ct[g] = s_ct[g - 1]; s_cs[g] = s_cs[g - 1]; }
