@@ -159,7 +159,7 @@ static int preload_kernels() {
     KIMAD_PRELOAD(k_sample); KIMAD_PRELOAD(k_pass_a<true>); KIMAD_PRELOAD(k_pass_a<false>); KIMAD_PRELOAD(k_resolve_a<true>); KIMAD_PRELOAD(k_resolve_a<false>);
     KIMAD_PRELOAD(k_refine); KIMAD_PRELOAD(k_tiny_exact); KIMAD_PRELOAD(k_fb1); KIMAD_PRELOAD(k_fb23<2>); KIMAD_PRELOAD(k_fb23<3>);
     KIMAD_PRELOAD(k_dp<2>); KIMAD_PRELOAD(k_dp<4>); KIMAD_PRELOAD(k_dp<8>); KIMAD_PRELOAD(k_pick); KIMAD_PRELOAD(k_fit_ratio); KIMAD_PRELOAD(k_sel_count);
-    KIMAD_PRELOAD(k_sel_offsets<128>); KIMAD_PRELOAD(k_sel_offsets<512>); KIMAD_PRELOAD(k_sel_recount);
+    KIMAD_PRELOAD((k_sel_offsets<128, true>)); KIMAD_PRELOAD((k_sel_offsets<128, false>)); KIMAD_PRELOAD((k_sel_offsets<512, false>)); KIMAD_PRELOAD(k_sel_recount);
     KIMAD_PRELOAD((k_sel_write<false, false>)); KIMAD_PRELOAD((k_sel_write<false, true>));
     KIMAD_PRELOAD((k_sel_write<true, false>)); KIMAD_PRELOAD((k_sel_write<true, true>));
     KIMAD_PRELOAD(k_apply_packed<false>); KIMAD_PRELOAD(k_apply_packed<true>);
@@ -534,13 +534,19 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
         CUDA_TRY(hand_over(big, small));
         {
             auto launch = [&](auto kern, uint32_t threads) {
-                return launch_named("k_sel_offsets", kern, glw, threads, 0, small, layers, chunks, nch, L, sel, csel, jobs, in, fb, rc,
-                                    rc_chunks, list_cap, phase, w0);
+                return launch_named("k_sel_offsets", kern, glw, threads, 0, small, dbuf, layers, chunks, nch, L, sel, csel, jobs, in, fb, rc,
+                                    rc_chunks, list_cap, w0);
             };
-            CUDA_TRY(c->most_chunks > 256 ? launch(k_sel_offsets<512>, 512) : launch(k_sel_offsets<128>, 128));
+            if (c->most_chunks <= kInlineChunks) {
+                CUDA_TRY(launch(k_sel_offsets<128, true>, 128));
+            } else {
+                CUDA_TRY(c->most_chunks > 256 ? launch(k_sel_offsets<512, false>, 512) : launch(k_sel_offsets<128, false>, 128));
+                // (a warp per chunk; usually there is nothing to do)
+                CUDA_TRY(launch_pdl(k_sel_recount, std::min(148u, (nch * nw + 7) / 8), blk, 0, small, dbuf, layers, chunks, nch, L, sel, csel, jobs,
+                                    in, rc, rc_chunks));
+                c->launches += 1;
+            }
         }
-        // (a warp per chunk; usually there is nothing to do)
-        CUDA_TRY(launch_pdl(k_sel_recount, std::min(148u, (nch * nw + 7) / 8), blk, 0, small, dbuf, layers, chunks, nch, L, sel, csel, jobs, in, rc, rc_chunks));
         mark(small);
         CUDA_TRY(hand_over(small, big));
         {
@@ -552,7 +558,7 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
             else CUDA_TRY(dense_write ? launch(k_sel_write<false, true>) : launch(k_sel_write<false, false>));
         }
         mark(big);
-        c->launches += 4;
+        c->launches += 3;
         if (two) CUDA_TRY(cudaEventRecord(c->ev_done[g], big));
     }
     if (two)

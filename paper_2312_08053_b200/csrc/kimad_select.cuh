@@ -280,15 +280,69 @@ __device__ __forceinline__ void sel_scan_layer(const LayerDesc& ld, const Sel& s
     }
 }
 
+// Exact per-slice (gt, eq) of a chunk whose slices have lists of their own, by a warp: from the lists, or from the inputs where a slice
+// has more entries inside the interval than its list holds.  The first 32 entries of AHEAD lists are requested together.
+template <int AHEAD>
+__device__ __forceinline__ void recount_chunk(const DSource& dbuf, uint32_t w, const Chunk& ch, const Sel& s, ChunkSel* out) {
+    const uint32_t lane = threadIdx.x & 31;
+    const ChunkView cv(ch, dbuf.phase.at(w));
+    const uint32_t my_in = lane < (uint32_t)kSlices ? out->eq[lane] : 0u; // lane i: slice i
+    uint32_t my_gt = lane < (uint32_t)kSlices ? out->above[lane] : 0u, my_eq = 0;
+#pragma unroll 1
+    for (int sl0 = 0; sl0 < kSlices; sl0 += AHEAD) {
+        uint32_t first[AHEAD]; // the slices' first entries, a lane each
+#pragma unroll
+        for (int i = 0; i < AHEAD; ++i) {
+            const SliceList list(dbuf, w, cv, sl0 + i);
+            const uint32_t n_in = __shfl_sync(0xffffffffu, my_in, sl0 + i);
+            first[i] = lane < n_in && n_in <= list.cap ? list.at[lane] : 0xffffffffu;
+        }
+#pragma unroll
+        for (int i = 0; i < AHEAD; ++i) {
+            const uint32_t sl = sl0 + i;
+            const SliceList list(dbuf, w, cv, sl);
+            const uint32_t n_in = __shfl_sync(0xffffffffu, my_in, sl);
+            if (n_in == 0) continue;
+            uint32_t gt = 0, eq = 0;
+            if (n_in <= list.cap) {
+                auto count = [&](uint32_t d) {
+                    gt += __popc(__ballot_sync(0xffffffffu, d != 0xffffffffu && d > s.tau_low));
+                    eq += __popc(__ballot_sync(0xffffffffu, d == s.tau_low));
+                };
+                count(first[i]);
+                for (uint32_t x = 32; x < n_in; x += 32) count(x + lane < n_in ? list.at[x + lane] : 0xffffffffu);
+                gt += __shfl_sync(0xffffffffu, my_gt, sl);
+            } else {
+                const DView dd(dbuf, w, cv.a0);
+                const uint32_t x0 = max(cv.first, sl * kSliceElems), x1 = min(cv.len, (sl + 1) * kSliceElems);
+                for (uint32_t x = x0 + lane; x < x1; x += 32) {
+                    const uint32_t key = key_of(dd.at(x));
+                    gt += key > s.tau;
+                    eq += key == s.tau;
+                }
+#pragma unroll
+                for (int o = 16; o; o >>= 1) {
+                    gt += __shfl_xor_sync(0xffffffffu, gt, o);
+                    eq += __shfl_xor_sync(0xffffffffu, eq, o);
+                }
+            }
+            if (lane == sl) { my_gt = gt; my_eq = eq; }
+        }
+    }
+    if (lane < (uint32_t)kSlices) { out->above[lane] = (uint16_t)my_gt; out->eq[lane] = (uint16_t)my_eq; }
+}
+
 // Exact threshold and job records, one CTA per (layer, worker).  The listed entries (16-bit distances from the interval's
 // lower key) are ranked by two 8-bit digits; each then joins its slice's counts.  Bound by the latency of a few dependent
 // rounds per layer: NT = 512 where a layer has thousands of chunks, 128 where none has more than 256 (1995 layers of two
-// chunks: 40 us with 512 threads, which need two waves of CTAs).
-template <int NT>
-__global__ void __launch_bounds__(NT)
-k_sel_offsets(const LayerDesc* __restrict__ layers, const Chunk* __restrict__ chunks, uint32_t n_chunks, uint32_t L,
+// two chunks: 40 us with 512 threads, which need two waves of CTAs).
+// HERE: layers with repeated values count their chunks here (at most kInlineChunks of them: a kernel less in the step's chain);
+// else they are listed for k_sel_recount.  (Ten CTAs of 128 threads per SM.)
+template <int NT, bool HERE>
+__global__ void __launch_bounds__(NT, NT == 512 ? 3 : 10)
+k_sel_offsets(const DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* __restrict__ chunks, uint32_t n_chunks, uint32_t L,
               Sel* __restrict__ sel, ChunkSel* __restrict__ csel, ChunkJob* __restrict__ jobs, const Interval in, FbList* __restrict__ fb,
-              Recount* __restrict__ rc, uint2* __restrict__ rc_chunks, uint32_t list_cap, const Phase phase, uint32_t w_base) {
+              Recount* __restrict__ rc, uint2* __restrict__ rc_chunks, uint32_t list_cap, uint32_t w_base) {
     pdl_wait();
     __shared__ uint32_t s_w[NT / 32], s_h[256], s_digit, s_gt, s_at;
     __shared__ uint16_t s_key[kListCap];
@@ -374,25 +428,27 @@ k_sel_offsets(const LayerDesc* __restrict__ layers, const Chunk* __restrict__ ch
             s.tau_low = s_digit;
             s.keep_eq -= s_gt;
             for (uint32_t k = k0; k < k1; ++k) *in.key_count(wr, k) = 0; // clean for the next use
-            if (threadIdx.x == 0) s_at = atomicAdd(&rc->n_chunks, ld.n_chunks);
+            if (!HERE && threadIdx.x == 0) s_at = atomicAdd(&rc->n_chunks, ld.n_chunks);
         }
         s.tau += s.tau_low;
         s.shift = 0;
         __syncthreads();
         if (threadIdx.x == 0) { sel[wl] = s; in.n[wl] = 0; }
-        if (over) { // its chunks are counted again
+        if (over && HERE) {
+            for (uint32_t i = threadIdx.x >> 5; i < ld.n_chunks; i += NT / 32) recount_chunk<4>(dbuf, w, chunks[ld.first_chunk + i], s, cs + i);
+            __threadfence();
+            __syncthreads();
+        } else if (over) { // its chunks are counted again
             for (uint32_t i = threadIdx.x; i < ld.n_chunks; i += NT)
                 if (KIMAD_CHECK(s_at + i < list_cap, 2)) rc_chunks[s_at + i] = make_uint2(w, ld.first_chunk + i);
             return;
         }
     }
-    sel_scan_layer<NT>(ld, s, chunks, phase.at(w), cs, jobs + (size_t)w * n_chunks + ld.first_chunk, s_w);
+    sel_scan_layer<NT>(ld, s, chunks, dbuf.phase.at(w), cs, jobs + (size_t)w * n_chunks + ld.first_chunk, s_w);
 }
 
-// Exact per-slice (gt, eq) of the listed chunks, a warp per chunk: from the slices' lists, or from the inputs where a slice has more
-// entries inside the interval than its list holds.  The CTA that finishes the last chunk of a layer makes the layer's job records
-// (Interval::n counts the finished ones).  Bound by latency: the first 32 entries of all lists of a chunk are requested together.
-// Values of bf16 gradients (4 x 124 M, 0.6 % kept): offsets 1226 us with every chunk counted
+// The listed chunks, a warp each.  The CTA that finishes the last chunk of a layer makes the layer's job records (Interval::n counts the
+// finished ones).  Bound by latency.  Values of bf16 gradients (4 x 124 M, 0.6 % kept): offsets 1226 us with every chunk counted
 // again from the inputs, 77 so, and 22 where nothing repeats.
 __global__ void __launch_bounds__(kThreads)
 k_sel_recount(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* __restrict__ chunks, uint32_t n_chunks,
@@ -410,48 +466,7 @@ k_sel_recount(DSource dbuf, const LayerDesc* __restrict__ layers, const Chunk* _
             const Chunk ch = chunks[e.y];
             const size_t wl = (size_t)e.x * L + ch.layer;
             const Sel s = sel[wl];
-            const ChunkView cv(ch, dbuf.phase.at(e.x));
-            ChunkSel* out = csel + (size_t)e.x * n_chunks + e.y;
-            const uint32_t my_in = lane < (uint32_t)kSlices ? out->eq[lane] : 0u; // lane i: slice i
-            uint32_t my_gt = lane < (uint32_t)kSlices ? out->above[lane] : 0u, my_eq = 0;
-            uint32_t first[kSlices]; // the slices' first entries, a lane each
-#pragma unroll
-            for (int sl = 0; sl < kSlices; ++sl) {
-                const SliceList list(dbuf, e.x, cv, sl);
-                const uint32_t n_in = __shfl_sync(0xffffffffu, my_in, sl);
-                first[sl] = lane < n_in && n_in <= list.cap ? list.at[lane] : 0xffffffffu;
-            }
-#pragma unroll
-            for (int sl = 0; sl < kSlices; ++sl) {
-                const SliceList list(dbuf, e.x, cv, sl);
-                const uint32_t n_in = __shfl_sync(0xffffffffu, my_in, sl);
-                if (n_in == 0) continue;
-                uint32_t gt = 0, eq = 0;
-                if (n_in <= list.cap) {
-                    auto count = [&](uint32_t d) {
-                        gt += __popc(__ballot_sync(0xffffffffu, d != 0xffffffffu && d > s.tau_low));
-                        eq += __popc(__ballot_sync(0xffffffffu, d == s.tau_low));
-                    };
-                    count(first[sl]);
-                    for (uint32_t i = 32; i < n_in; i += 32) count(i + lane < n_in ? list.at[i + lane] : 0xffffffffu);
-                    gt += __shfl_sync(0xffffffffu, my_gt, sl);
-                } else {
-                    const DView dd(dbuf, e.x, cv.a0);
-                    const uint32_t x0 = max(cv.first, sl * kSliceElems), x1 = min(cv.len, (sl + 1) * kSliceElems);
-                    for (uint32_t x = x0 + lane; x < x1; x += 32) {
-                        const uint32_t key = key_of(dd.at(x));
-                        gt += key > s.tau;
-                        eq += key == s.tau;
-                    }
-#pragma unroll
-                    for (int o = 16; o; o >>= 1) {
-                        gt += __shfl_xor_sync(0xffffffffu, gt, o);
-                        eq += __shfl_xor_sync(0xffffffffu, eq, o);
-                    }
-                }
-                if (lane == (uint32_t)sl) { my_gt = gt; my_eq = eq; }
-            }
-            if (lane < (uint32_t)kSlices) { out->above[lane] = (uint16_t)my_gt; out->eq[lane] = (uint16_t)my_eq; }
+            recount_chunk<kSlices>(dbuf, e.x, ch, s, csel + (size_t)e.x * n_chunks + e.y);
             __threadfence();
             __syncwarp();
             if (lane == 0) s_last[wid] = atomicAdd(in.n + wl, 1u) + 1u == layers[ch.layer].n_chunks;
