@@ -13,10 +13,10 @@
 
 // Checked build (-DKIMAD_CHECKED): indices into the workspace and the output buffers are tested before use; a failed
 // test sets its bit in a status word that the host reads (kimad_debug_check) and the access is skipped -- nothing
-// traps.  Bits: 0 sweep: bin outside the layer's histogram; 1 counting sweep: bin outside the in-interval histogram;
-// 2 a work list (exact path, recount) appended beyond its capacity; 3 write sweep: packed
-// position beyond the capacity; 4 write sweep: element index outside its layer; 5 DP: cell or back-pointer outside
-// its row; 6 curve: bin outside the layer's histogram; 7 curve: the pieces of a refined bin do not add up to the bin.
+// traps.  Bits: 0 sweep: bin outside the layer's histogram; 1 counting sweep: key outside its interval;
+// 2 a work list (exact path, recount) appended beyond its capacity; 3 write sweep: packed position beyond the capacity or element
+// outside its chunk; 4 knapsack: a record, row or exchange outside the memory it lies in; 5 knapsack: a cell outside its row;
+// 6 selection: a listed entry outside its layer's chunks; 7 curve: the pieces of a refined bin do not add up to the bin.
 // In the ordinary build KIMAD_CHECK(cond, bit) is `true`.
 #if defined(KIMAD_CHECKED) && defined(__CUDACC__)
 __device__ unsigned int g_kimad_check_word;

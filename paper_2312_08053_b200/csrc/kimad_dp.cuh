@@ -251,6 +251,9 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
     uint32_t* tab = tab_all + w * tab_stride;
     float* hist = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(hist_all + w * hist_stride) + 15u) & ~(uintptr_t)15u);
 
+    // the records and the rows fit where they are put
+    if (t == 0) (void)KIMAD_CHECK((size_t)L * 2u * rw <= tab_stride && (size_t)L * hist_row + (hist - (hist_all + w * hist_stride)) <= hist_stride &&
+                                  D - L + 1u <= hist_row, 4);
     int status = KIMAD_OK;
     if (a.check_finite && (a.flags[w] & 1u)) status = KIMAD_ERR_NONFINITE;
     else if (c >= a.full_bytes) status = KIMAD_STATUS_PLATEAU;
@@ -354,6 +357,7 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
     // a row has +inf in front of it, for the cells below its start
     const uint32_t margin = (reach + 3u) & ~3u, slot_words = margin + ((width + 3u) & ~3u);
     const uint32_t n_ring = min((uint32_t)kDpMaxRing, (plan.work_bytes - 8u * CL * rw) / (4u * slot_words)); // (at least 2)
+    if (t == 0) (void)KIMAD_CHECK(n_ring >= 2u && 8u * CL * rw + 4u * n_ring * slot_words <= plan.work_bytes, 4);
     for (uint32_t i = t; i < n_ring * margin; i += T) ring[(i / margin) * slot_words + i % margin] = kInf;
 
 
@@ -400,7 +404,7 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
 #pragma unroll
             for (int q = 0; q < CPT; ++q)
                 if (cell0 + 32u * q < width) row[cell0 + 32u * q] = v[q];
-            if (t == 0) s_ex[seq] = (uint16_t)(l0 + i);
+            if (t == 0 && KIMAD_CHECK(seq < L && l0 + i < L, 4)) s_ex[seq] = (uint16_t)(l0 + i);
             __syncwarp();
             if (lane == 0) progress_set(prog + wid, seq + 1u);
             const uint32_t* er = rec + kr;
@@ -425,6 +429,10 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
             // the warps below have written their part of this row; the others are done with the slot of the next one
             progress_wait(prog + lane, lane < wid ? (int)seq + 1 : (lane == wid ? 0 : (int)seq + 3 - (int)n_ring), failed);
             const uint32_t addr = smem_u32(row + cell0);
+            // a candidate's cells: no further below the row's start than its margin (the last warp's, past the row's end, stay in the CTA's memory)
+            auto at = [&](uint32_t off) {
+                return addr + (KIMAD_CHECK((int)cell0 + ((int)off >> 2) >= -(int)margin && row + cell0 + 32u * (CPT - 1) < reinterpret_cast<float*>(smem_raw + plan.smem), 5) ? off : 0u);
+            };
             const int top = -4 * (int)(wcell + 32u * CPT - 1u); // offset from the warp's last cell to the row's start
 #pragma unroll
             for (int q = 0; q < CPT; ++q) {
@@ -436,7 +444,7 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
                 constexpr int N = decltype(count)::value;
                 float x[CPT][N];
 #pragma unroll
-                for (int k = 0; k < N; ++k) lds_cells<CPT, N>(x, k, addr + u[k]);
+                for (int k = 0; k < N; ++k) lds_cells<CPT, N>(x, k, at(u[k]));
 #pragma unroll
                 for (int q = 0; q < CPT; ++q) {
 #pragma unroll
@@ -454,7 +462,7 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
                 const float e[4] = {__uint_as_float(e4.x), __uint_as_float(e4.y), __uint_as_float(e4.z), __uint_as_float(e4.w)};
                 float x[CPT][4]; // cells beyond the row (last warp) read what lies behind it and are never stored
 #pragma unroll
-                for (int k = 0; k < 4; ++k) lds_cells<CPT, 4>(x, k, addr + u[k]);
+                for (int k = 0; k < 4; ++k) lds_cells<CPT, 4>(x, k, at(u[k]));
                 bool more = j0 < nd;
                 if (more) {
                     u4 = *reinterpret_cast<const uint4*>(rec + j0);
@@ -549,7 +557,7 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
                     auto walk = [&](auto any) {
                         while (i < nx) {
                             if (lo && b - lo < far) break; // left the window: staged anew from here (never on the first exchange)
-                            const bool fits = lane < nu && off <= b;
+                            const bool fits = lane < nu && off <= b && KIMAD_CHECK(b - off >= lo && b <= b0, 5);
                             const float sum = fits ? __fadd_rn(row[b - off], e) : kInf;
                             const uint32_t mine = lane << 16 | off;
                             row += 4u * per16; rec += 4u * per16; // (the last ones read lie inside the buffer: work_bytes is below its end)
@@ -558,7 +566,7 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
                             const float best = warp_min(sum, any);
                             const uint32_t win = __reduce_min_sync(0xffffffffu, fits && sum == best ? mine : 0xffffffffu); // the first of them
                             if (lane == (i & 31u)) { my_j = win >> 16; my_best = best; }
-                            b -= win & 0xffffu;
+                            b -= KIMAD_CHECK(win != 0xffffffffu, 5) ? win & 0xffffu : 0u;
                             if ((++i & 31u) == 0) keep(32u, i);
                         }
                     };
@@ -579,7 +587,7 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
                             sum[h] = kInf;
                             if (x < nu) {
                                 off[h] = (0u - rec[x]) >> 2;
-                                if (off[h] <= b) sum[h] = __fadd_rn(row[b - off[h]], __uint_as_float(rec[kr + x]));
+                                if (off[h] <= b && KIMAD_CHECK(b - off[h] >= lo && b <= b0, 5)) sum[h] = __fadd_rn(row[b - off[h]], __uint_as_float(rec[kr + x]));
                             }
                             best = fminf(best, sum[h]);
                         }

@@ -402,7 +402,7 @@ k_sel_offsets(const DSource dbuf, const LayerDesc* __restrict__ layers, const Ch
             for (uint32_t i = threadIdx.x; i < cnt; i += NT) {
                 const uint2 e = list[i];
                 const uint32_t k = e.y & 0xffffu, sl = e.y >> 16;
-                if (k < s.tau_low) continue;
+                if (k < s.tau_low || !KIMAD_CHECK(e.x < ld.n_chunks && sl < (uint32_t)kSlices, 6)) continue;
                 uint32_t* c = reinterpret_cast<uint32_t*>(k > s.tau_low ? cs[e.x].above : cs[e.x].eq) + (sl >> 1);
                 atomicAdd(c, 1u << (16u * (sl & 1u)));
             }
