@@ -300,6 +300,11 @@ int kimad_debug_stage_times(kimad_ctx* ctx, float* host_ms);
  * always run as one group. */
 int kimad_debug_set_schedule(kimad_ctx* ctx, int mode);
 
+/* Limit, in SM clocks, of the waits inside the knapsack kernel (its warps wait for one another; default and maximum 2^31,
+ * about a second).  For tests: a wait that runs out makes the worker's result KIMAD_ERR_TIMEOUT, with nothing selected
+ * and the estimator unchanged; the context stays usable.  Errors: INVALID_ARG. */
+int kimad_debug_set_wait_limit(kimad_ctx* ctx, uint64_t clocks);
+
 /* kimad_step with a pair of CUDA events around every kernel launch; synchronises the device before and after and
  * writes one line per launch to text (host, text_len bytes, NUL-terminated, truncated if too short): kernel, ordinal
  * of its stream (in order of first use: 0 is the step's stream), start and end in milliseconds after the step was

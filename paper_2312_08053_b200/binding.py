@@ -109,6 +109,8 @@ def load():
     L.kimad_debug_stage_times.argtypes = [vp, vp]
     L.kimad_debug_set_schedule.restype = C.c_int
     L.kimad_debug_set_schedule.argtypes = [vp, C.c_int]
+    L.kimad_debug_set_wait_limit.restype = C.c_int
+    L.kimad_debug_set_wait_limit.argtypes = [vp, u64]
     L.kimad_debug_trace_step.restype = C.c_int
     L.kimad_debug_trace_step.argtypes = [vp, vp, vp, C.POINTER(dbl), dbl, vp, vp, C.c_char_p, C.c_size_t]
     L.kimad_debug_get_band_meta.restype = C.c_int
@@ -324,6 +326,11 @@ def kimad_debug_enable_stage_timing(ctx: Ctx, enable: bool) -> None:
 def kimad_debug_set_schedule(ctx: Ctx, mode: int) -> None:
     """0: two worker groups for large steps, 1: whenever W >= 2, 2: one group."""
     _check(load().kimad_debug_set_schedule(ctx.handle, int(mode)), "kimad_debug_set_schedule")
+
+
+def kimad_debug_set_wait_limit(ctx: Ctx, clocks: int) -> None:
+    """Limit of the knapsack kernel's waits in SM clocks (see kimad.h); 2^31 by default."""
+    _check(load().kimad_debug_set_wait_limit(ctx.handle, int(clocks)), "kimad_debug_set_wait_limit")
 
 
 def kimad_debug_trace_step(ctx: Ctx, grads, state, bandwidth_bytes_per_s, t_target_s, out: "Packed", stream=None) -> str:

@@ -268,6 +268,7 @@ static bool plan_choice(kimad_ctx* c) {
     if (tab + 2 * slot > most) return false;
     p.work_bytes = (uint32_t)std::min(most, (std::max<size_t>(tab + kDpMaxRing * slot, 96 * 1024) + 15) & ~(size_t)15);
     p.smem = (uint32_t)(p.work_bytes + tail + beyond);
+    p.wait_clocks = kDpWaitClocks;
     return 8 * (size_t)c->L <= p.work_bytes;
 }
 
@@ -766,6 +767,12 @@ int kimad_debug_trace_step(kimad_ctx* c, const float* grads_dev, float* state_de
 int kimad_debug_set_schedule(kimad_ctx* c, int mode) {
     if (!c || mode < 0 || mode > 2) return KIMAD_ERR_INVALID_ARG;
     c->pipeline_mode = mode;
+    return KIMAD_OK;
+}
+
+int kimad_debug_set_wait_limit(kimad_ctx* c, uint64_t clocks) {
+    if (!c || clocks > (uint64_t)kDpWaitClocks) return KIMAD_ERR_INVALID_ARG;
+    c->dp_plan.wait_clocks = (long long)clocks;
     return KIMAD_OK;
 }
 

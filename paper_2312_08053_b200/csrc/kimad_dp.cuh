@@ -34,7 +34,7 @@ namespace kimad {
 constexpr int kDpMaxThreads = 1024;
 constexpr int kDpMaxRing = 8;                  // rows in flight at most
 constexpr uint32_t kDpMaxChunkLayers = 256;    // layers whose records are staged at a time (two buffers)
-constexpr long long kDpWaitClocks = 1ll << 31; // about a second; an exchange takes about a microsecond
+constexpr long long kDpWaitClocks = 1ll << 31; // limit of a wait unless set otherwise: about a second (an exchange takes about a microsecond)
 constexpr uint32_t kDpSameBit = 0x10000u;      // head: all usable candidates of the layer take the same number of cells
 
 // Plan of a launch (host).  A layer has two records of rw = 2 kr + 4 words (kr = K rounded up to 8): {byte offsets of the
@@ -48,6 +48,7 @@ struct DpPlan {
     uint32_t chunk_layers;
     uint32_t work_bytes;
     uint32_t smem; // dynamic shared memory in all
+    long long wait_clocks; // limit of a wait
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -69,12 +70,12 @@ __device__ __forceinline__ float min3(float a, float b, float c) { float m; asm(
 // with a fence before and after plain accesses the 1995 blocks took 1.87 instead of 1.76 ms.
 __device__ __forceinline__ void progress_set(uint32_t* counter, uint32_t x) { asm volatile("st.release.cta.shared.u32 [%0], %1;" ::"r"(smem_u32(counter)), "r"(x) : "memory"); }
 __device__ __forceinline__ int progress_get(uint32_t counter) { int x; asm volatile("ld.acquire.cta.shared.u32 %0, [%1];" : "=r"(x) : "r"(counter) : "memory"); return x; }
-__device__ __forceinline__ void progress_wait(const uint32_t* counter, int target, volatile uint32_t* failed) {
+__device__ __forceinline__ void progress_wait(const uint32_t* counter, int target, volatile uint32_t* failed, long long limit) {
     const uint32_t at = smem_u32(counter);
     if (!__all_sync(0xffffffffu, progress_get(at) >= target)) {
         const long long start = clock64();
         while (!__all_sync(0xffffffffu, progress_get(at) >= target)) {
-            if (clock64() - start > kDpWaitClocks) *failed = 1u;
+            if (clock64() - start > limit) *failed = 1u;
             if (__any_sync(0xffffffffu, *failed != 0u)) break;
         }
     }
@@ -427,7 +428,7 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
                 }
             }
             // the warps below have written their part of this row; the others are done with the slot of the next one
-            progress_wait(prog + lane, lane < wid ? (int)seq + 1 : (lane == wid ? 0 : (int)seq + 3 - (int)n_ring), failed);
+            progress_wait(prog + lane, lane < wid ? (int)seq + 1 : (lane == wid ? 0 : (int)seq + 3 - (int)n_ring), failed, plan.wait_clocks);
             const uint32_t addr = smem_u32(row + cell0);
             // a candidate's cells: no further below the row's start than its margin (the last warp's, past the row's end, stay in the CTA's memory)
             auto at = [&](uint32_t off) {

@@ -54,3 +54,26 @@ def test_given_errors_of_any_sign(L, K, D):
         assert np.array_equal(u32(r.out.j), ref.j)
         assert np.array_equal(st["total_err"], ref.total_err)
         assert np.array_equal(u32(state), ref.state.view(np.uint32))
+
+
+@pytest.mark.parametrize("schedule", [0, 1])
+def test_a_wait_that_runs_out(schedule):
+    """With no patience at all the warps' first wait that is not met ends the search: nothing is selected, nothing changes, and
+    the next step on the same context is the oracle's."""
+    rng = np.random.default_rng(4)
+    sizes = [int(v) for v in rng.integers(200, 6000, 120)]
+    N, W = sum(sizes), 3
+    r = Runner(sizes, W, list(np.geomspace(0.01, 1.0, 12)), 1000, 0, schedule=schedule)
+    grads = torch.from_numpy(rng.standard_normal((W, N)).astype(np.float32)).cuda()
+    state = torch.from_numpy(rng.standard_normal((W, N)).astype(np.float32)).cuda()
+    before = state.clone()
+    kb.kimad_debug_set_wait_limit(r.ctx, 0)
+    status, k = r.gpu_step(grads, state, [0.2 * 8 * N] * W, 1.0)
+    assert status == kb.KIMAD_ERR_TIMEOUT
+    st = r.out.stats_host()
+    assert (st["status"] == kb.KIMAD_ERR_TIMEOUT).all() and not st["n_selected"].any() and not st["used_bytes"].any()
+    assert not k.any() and not u32(r.out.j).any() and not r.out.offs.any() and torch.equal(state, before)
+    kb.kimad_debug_set_wait_limit(r.ctx, 1 << 31)
+    assert r.compare_step(grads, state, [0.2 * 8 * N] * W, 1.0)["status"] == kb.KIMAD_OK
+    with pytest.raises(kb.KimadError):
+        kb.kimad_debug_set_wait_limit(r.ctx, (1 << 31) + 1)
