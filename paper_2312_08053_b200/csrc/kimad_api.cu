@@ -451,9 +451,9 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
                           c->at<uint32_t>(y.in_n)}; // (in_n counts the select stage's entries later in the step; zero in between)
         // the slow paths inside the curve kernel, by clusters of cz CTAs along its grid's third axis, or over lists
         const uint32_t cluster = inline_cluster(c->most_chunks);
-        const bool lists = c->most_chunks > (c->curve_mode == 1 ? kInlineChunksExact : kInlineChunks) ||
-                           (cluster > 1 && (uint64_t)R * nw * cluster > kInlineCtas);
-        const uint32_t cz = lists ? 1u : cluster;
+        const bool resident = (uint64_t)R * nw * cluster <= kInlineCtas;
+        const bool lists = c->most_chunks > (c->curve_mode == 1 ? kInlineChunksExact : (resident ? kInlineChunks : kInlineChunksAlone));
+        const uint32_t cz = lists || !resident ? 1u : cluster;
         if (R) {
             auto launch = [&](auto kern) {
                 return launch_clusters("k_resolve_a", cz, kern, dim3(R, nw, cz), kBigThreads, 0, small, layers, reg_layers, R, L, ktab, K, meta, cell_win,

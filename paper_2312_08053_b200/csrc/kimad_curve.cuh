@@ -665,11 +665,13 @@ k_pass_a(const float* __restrict__ grads, const float* __restrict__ state, uint8
 // layer has more than kInlineChunks chunks the curve kernel takes them itself (layer_by_itself): 62 tensors of up to
 // 147 K elements 116.5 -> 112 us a step, a small model through a built-in workspace 98 -> 86 us.  With one layer of thirty
 // candidates on the exact path a step takes 190 us with two chunks, 242 with four, 268 with five and about 340 with eight by one CTA,
-// 234 over lists with nine; hence the second bound for contexts that take it always.  Beyond four chunks a cluster of two or four CTAs
-// takes a layer (227 us with five chunks, 209 with eight); the clusters of all layers have to be resident at once (a CTA fills
-// an SM), though those whose layer needs nothing only wait, else the lists are used.
+// 234 over lists with nine; hence the bound for contexts that take it always.  Beyond four chunks a cluster of two or four CTAs
+// takes a layer (227 us with five chunks, 209 with eight).  The clusters of all layers have to be resident at once (a CTA fills
+// an SM), though those whose layer needs nothing only wait; where they are not, one CTA takes layers of up to six chunks (293 us: the
+// lists would cost every step without such a layer 4 to 5 us) and the lists take more.
 // ------------------------------------------------------------------------------------------------
-constexpr uint32_t kInlineChunks = 8, kInlineChunksExact = 2; // the latter where every layer takes the exact path
+constexpr uint32_t kInlineChunks = 8, kInlineChunksAlone = 6; // with clusters, with a CTA per layer where those are too many
+constexpr uint32_t kInlineChunksExact = 2;                     // ... where every layer takes the exact path
 constexpr uint32_t kInlineCtas = 128;                          // of a launch of clusters
 KIMAD_HD uint32_t inline_cluster(uint32_t most_chunks) { return most_chunks <= 4 ? 1u : (most_chunks <= 6 ? 2u : 4u); }
 struct ListArgs {

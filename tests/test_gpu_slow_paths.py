@@ -44,10 +44,10 @@ def test_exact_path_of_small_contexts(n):
     assert kb.kimad_debug_exact_path_layers(r.ctx) == 2 * 4 * W  # two layers; every comparison runs two steps
 
 
-@pytest.mark.parametrize("n,others,W", [(32769, 0, 1), (131072, 0, 2), (131073, 1, 1), (196609, 0, 1), (262144, 2, 3), (140000, 40, 2), (300001, 0, 1)])
+@pytest.mark.parametrize("n,others,W", [(32769, 0, 1), (131072, 0, 2), (131073, 1, 1), (196609, 0, 1), (262144, 2, 3), (140000, 40, 2), (240000, 40, 2), (300001, 0, 1)])
 def test_bands_that_do_not_fit(n, others, W):
     """Magnitudes over 150 octaves and thirty candidates: the bands do not fit the tables and every layer takes the exact path, by one
-    CTA (up to four chunks), by clusters of two and four, or over lists (too many layers for clusters, more than eight chunks)."""
+    CTA (up to four chunks; up to six with too many layers for clusters), by clusters of two and four, or over lists."""
     rng = np.random.default_rng(n)
     sizes, grid = [n] + [n + 7 * i for i in range(others)] + [3000], [(j + 0.5) / 30 for j in range(30)]
     N = sum(sizes)
