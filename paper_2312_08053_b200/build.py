@@ -13,6 +13,7 @@ SOURCES = [os.path.join(_HERE, "csrc", "kimad_api.cu")]
 HEADERS = [os.path.join(_HERE, "csrc", "kimad_kernels.cuh"), os.path.join(_HERE, "csrc", "kimad_select.cuh"),
            os.path.join(_HERE, "csrc", "kimad_curve.cuh"), os.path.join(_HERE, "csrc", "kimad_common.h"),
            os.path.join(_HERE, "csrc", "kimad_receiver.cuh"), os.path.join(_HERE, "csrc", "kimad_dp.cuh"),
+           os.path.join(_HERE, "csrc", "kimad_dp_window.cuh"),
            os.path.join(_ROOT, "include", "kimad.h")]
 
 

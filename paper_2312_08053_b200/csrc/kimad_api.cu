@@ -1,6 +1,7 @@
 // Host side of the C ABI declared in include/kimad.h: context, static planner (candidate table,
 // chunk table, workspace layout) and the per-step launch sequence.  No device memory is allocated
 // here; the caller's workspace is carved into the regions listed in `Layout`.
+#include <algorithm>
 #include <cmath>
 #include <cstdlib>
 #include <cstdio>
@@ -266,7 +267,13 @@ static bool plan_choice(kimad_ctx* c) {
     const size_t beyond = 32 * 8 * 4; // the last warp reads past the row's last cell, at most so far
     const size_t most = (kDpSmemMax - tail - beyond) & ~(size_t)15;
     if (tab + 2 * slot > most) return false;
-    p.work_bytes = (uint32_t)std::min(most, (std::max<size_t>(tab + kDpMaxRing * slot, 96 * 1024) + 15) & ~(size_t)15);
+    // the search over windows: its tables and steps back, in shared memory where the records are staged at once
+    const bool one = p.chunk_layers >= c->L;
+    const size_t fixed = sizeof(WindowScratch) + window_op_bytes(p.chunk_layers, p.kr) + sizeof(WindowOp) + 6 * (size_t)c->L + 32;
+    const size_t want = tab + fixed + (one ? (size_t)c->L * (kWindowTables + kWindowMost) : kWindowPiece);
+    const bool window = c->L >= window_layers(c->dp_cells) && want <= most;
+    p.work_bytes = (uint32_t)std::min(most, (std::max<size_t>({tab + kDpMaxRing * slot, 96 * 1024, window ? want : 0}) + 15) & ~(size_t)15);
+    p.window = window ? (uint32_t)(p.work_bytes - tab) : 0u;
     p.smem = (uint32_t)(p.work_bytes + tail + beyond);
     p.wait_clocks = kDpWaitClocks;
     return 8 * (size_t)c->L <= p.work_bytes;

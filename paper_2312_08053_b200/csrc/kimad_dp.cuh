@@ -16,7 +16,10 @@
 //     exchanged rows go to the workspace, and the winning candidates -- the first that attains the minimum -- are found on
 //     the chosen path alone, last layer first, by repeating the one cell's sums.
 //
-// Bound by instruction issue and shared-memory reads of one SM on wide axes (a record's uniform 128-bit reads cost about as
+// With many layers the few cells of every row that the chosen path can visit are worked out first (kimad_dp_window.cuh), and whole
+// rows are for what that does not decide.
+//
+// Whole rows: bound by instruction issue and shared-memory reads of one SM on wide axes (a record's uniform 128-bit reads cost about as
 // much as the cells they address), by the chain of latencies per exchange on short ones, and by the cold start of the
 // records and of the backtracking's rows.  Against one CTA with a barrier per layer, every candidate's index carried along
 // and back-pointers for every cell: GPT-2 small's 148 layers, 16 candidates, D = 1000: 163 -> 69 us; 1995 blocks of it,
@@ -48,6 +51,7 @@ struct DpPlan {
     uint32_t chunk_layers;
     uint32_t work_bytes;
     uint32_t smem; // dynamic shared memory in all
+    uint32_t window; // bytes of work_bytes behind the records for the search over windows (kimad_dp_window.cuh); 0: whole rows only
     long long wait_clocks; // limit of a wait
 };
 
@@ -81,6 +85,10 @@ __device__ __forceinline__ void progress_wait(const uint32_t* counter, int targe
     }
     __syncwarp();
 }
+
+} // namespace kimad
+#include "kimad_dp_window.cuh"
+namespace kimad {
 
 // ------------------------------------------------------------------------------------------------
 // What follows the choice of a candidate per layer, by one CTA: totals, capacity check, output offsets, statistics and
@@ -262,6 +270,21 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
     if (t == 0) { s_failed = 0; s_sum = 0; s_reach = 0; s_signed = 0; }
     __syncthreads(); // (and the flags are read before the end of the choice resets them)
 
+    // ---- windows of the rows first.  (Where the limit of the waits is set, the recursion whose warps wait for each other is what is asked for.)
+    if (status == KIMAD_OK && plan.window && plan.wait_clocks == kDpWaitClocks) {
+        auto at = [&](const void* p) { return (uint32_t)(reinterpret_cast<const unsigned char*>(p) - smem_raw); };
+        const WindowArgs wa{L, K, D, kr, rw, c, cost, a.err + (size_t)w * L * K, CL, 8u * CL * rw, plan.window, tab,
+                            reinterpret_cast<unsigned char*>(hist), (hist_stride - (size_t)(hist - (hist_all + w * hist_stride))) * 4u, at(s_p), at(s_ex), at(s_j)};
+        float value;
+        if (CL >= L ? window_search<true>(wa, &value) : window_search<false>(wa, &value)) {
+            if (t == 0) s_total = value;
+            __syncthreads();
+            choose_finish(a, w, c, status, false, &s_total, s_j, s_k, s_e);
+            return;
+        }
+        __syncthreads();
+    }
+
     // ---- the layers' records; 8, 16 or 32 lanes per layer, the loads of the next layers ahead of the current ones' work
     const uint32_t G = kr <= 8u ? 8u : (kr <= 16u ? 16u : 32u), per = 32u / G; // lanes per layer, layers per warp
     const uint32_t sub = lane / G, jj = lane % G, stride = (T >> 5) * per;
@@ -272,9 +295,7 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
         unsigned long long sum = 0;
         uint32_t reach = 0;
         bool negative = false;
-        // budget_cells = (bytes D + c - 1) / c in binary64: everything is an integer below 2^50 (bytes < 2^35, D < 2^13, c below
-        // the sum of the layers' sizes), the quotient from the reciprocal is off by one at most and the remainder is exact
-        const double cd = (double)c, inv_c = 1.0 / cd, c_1 = cd - 1.0, most = (double)(D + 1u);
+        const CellsOf cells_of(c, D);
         for (uint32_t l4 = wid * per; l4 < L; l4 += AHEAD * stride) {
             double x_[AHEAD];
             float e_[AHEAD];
@@ -296,10 +317,7 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
                 for (uint32_t r = 0; r < rounds; ++r) {
                     const uint32_t j = r * G + jj;
                     if (r) fetch(l, j, x_[i], e_[i]);
-                    const double num = fabs(x_[i]) + c_1;
-                    uint32_t u = (uint32_t)fmin(num * inv_c, most);
-                    const double rest = fma(-(double)u, cd, num);
-                    u = min(rest < 0.0 ? u - 1u : (rest >= cd ? u + 1u : u), D + 1u);
+                    const uint32_t u = cells_of(x_[i]);
                     const bool in = have && j < K, ok = in && u <= D; // sizes ascend with j: the usable candidates come first
                     const float e = x_[i] < 0.0 ? 0.f : e_[i];        // a layer sent densely (negative cost) loses nothing
                     if (r == 0) { u0 = __shfl_sync(0xffffffffu, u, sub * G); e0 = __shfl_sync(0xffffffffu, e, sub * G); }
