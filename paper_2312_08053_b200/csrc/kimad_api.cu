@@ -44,7 +44,7 @@ struct kimad_ctx {
     std::vector<Chunk> chunks;
     std::vector<LayerDesc> layers;
     std::vector<uint32_t> reg_layers, tiny_layers, reg_index; // layers above / up to kTinyMax elements
-    std::vector<SweepRun> runs;                               // the sweep's CTAs: static runs of chunks, balanced by elements
+    std::vector<SweepRun> runs;                               // the sweep's CTAs: static runs of chunks, balanced by cost
     std::vector<unsigned char> static_image;                  // the static tables as they lie in the workspace, one block
     std::vector<size_t> guards;                               // checked build: offsets of the canary words between regions
     uint32_t most_chunks = 0; // of a layer
@@ -150,6 +150,11 @@ void plan_layout(kimad_ctx* c) {
 
 constexpr size_t kDpSmemMax = 225 * 1024; // dynamic shared memory k_dp and k_pick may ask for
 constexpr uint64_t kSweepRunElems = 4ull << 20; // elements a CTA of the sweep takes at most (as long as four waves suffice)
+// What a run of the sweep pays for every layer it enters (table load, refill of the loads' pipeline, flush of the histogram), in elements
+// swept meanwhile: runs are balanced by elements plus so many per layer.  With 0 / 8 / 16 / 24 / 32 K the sweep of 8 x 25.6 M elements
+// in 53 layers of more than 4096 takes 451 / 414 / 386 / 374 / 373 us, of 4 x 11.7 M in 21 109 / 99 / 91 / 90 / 94, of 4 x 124 M in 50
+// 787 / 781 / 780 / 785 / 781.
+constexpr uint64_t kSweepLayerElems = 24576;
 constexpr uint64_t kPipelineMinElems = 1ull << 25; // W N from which a step is run as two groups of workers
 
 // Kernels are loaded on their first launch; loading one takes about a millisecond.  Touching every kernel a
@@ -654,7 +659,7 @@ int kimad_create(kimad_ctx** out, const uint64_t* layer_sizes, uint32_t n_layers
         c->curve_mode = o.curve_mode;
         c->sample_smem = (size_t)(1024 + 32 + 32768 + 1024 + 2 * kBaseWords + 32 + 3 * 128) * 4;
         c->pass_a_smem = (size_t)(2 * kMaxBins + kCellTab) * 4;
-        { // the sweep's runs, one CTA each: every worker's chunk list is cut into pieces of about equal element counts.
+        { // the sweep's runs, one CTA each: every worker's chunk list is cut into pieces of about equal cost (kSweepLayerElems).
           // The sweep of a group of workers ((W + 1) / 2 of them) is one wave of CTAs (148 SMs, one CTA resident per
           // SM), or up to four waves when a run would otherwise exceed kSweepRunElems: long static runs end
           // unevenly, and later waves even that out.
@@ -662,15 +667,35 @@ int kimad_create(kimad_ctx** out, const uint64_t* layer_sizes, uint32_t n_layers
             const uint32_t gw = (c->W + 1) / 2; // workers in the larger group (1 for a single worker)
             const uint64_t waves = std::min<uint64_t>(4, std::max<uint64_t>(1, (N * gw + 148ull * kSweepRunElems - 1) / (148ull * kSweepRunElems)));
             const uint32_t per_w = std::max<uint32_t>(1u, std::min<uint32_t>(nch, (uint32_t)((waves * 148u + gw - 1) / gw)));
-            for (uint32_t w = 0; w < c->W; ++w) {
-                uint64_t acc = 0;
-                uint32_t g = 0, start = 0;
+            // runs of a worker when none may cost more than `most`
+            auto cut = [&](uint64_t most, std::vector<uint32_t>* starts) {
+                uint64_t cost = 0;
+                uint32_t n = 0, layer = 0;
                 for (uint32_t f = 0; f < nch; ++f) {
-                    if (g + 1 < per_w && f > start && acc >= (N * (uint64_t)(g + 1)) / per_w) { c->runs.push_back(SweepRun{w, start, f}); start = f; ++g; }
-                    acc += c->chunks[f].end - c->chunks[f].begin;
+                    const Chunk& ch = c->chunks[f];
+                    const uint64_t swept = ch.end - ch.begin, entry = c->reg_index[ch.layer] != 0xffffffffu ? kSweepLayerElems : 0;
+                    const uint64_t more = swept + (f && ch.layer == layer ? 0 : entry);
+                    if (f == 0 || cost + more > most) {
+                        cost = swept + entry;
+                        if (starts) starts->push_back(f);
+                        ++n;
+                    } else {
+                        cost += more;
+                    }
+                    layer = ch.layer;
                 }
-                c->runs.push_back(SweepRun{w, start, nch});
+                return n;
+            };
+            uint64_t low = N / per_w, high = N + (uint64_t)c->reg_layers.size() * kSweepLayerElems; // too little (or just right), enough
+            while (high - low > 64) {
+                const uint64_t mid = low + (high - low) / 2;
+                if (cut(mid, nullptr) <= per_w) high = mid;
+                else low = mid;
             }
+            std::vector<uint32_t> starts;
+            cut(high, &starts);
+            for (uint32_t w = 0; w < c->W; ++w)
+                for (size_t i = 0; i < starts.size(); ++i) c->runs.push_back(SweepRun{w, starts[i], i + 1 < starts.size() ? starts[i + 1] : nch});
         }
         c->tiny_smem = (size_t)kTinyMax * (8 + 4);
         plan_layout(c);
