@@ -13,7 +13,7 @@
 //   k_pass_a     the sweep: d = grad - g (one code byte per element goes to scratch), bin = base + (key >> shift)
 //                with (base, shift) = table(cell(key)), two u32 shared-memory atomics per element: the count, and
 //                the exact integer sum of squares in a u32 word whose (rare) carries go straight to the 64-bit sum
-//                in global memory.  CTAs own static runs of chunks balanced by elements.
+//                in global memory.  CTAs own static runs of chunks of equal cost.
 //   k_resolve_a  per (worker, layer): totals of every group of 32 bins, a scan over the groups, then a warp per
 //                candidate finds the group and the bin that hold its threshold (zeros left out by the sweep = the
 //                layer's size minus the counted entries) and the squares below it.  The candidate's error is certified to 5e-6 relative from the bin's width.  A
@@ -462,7 +462,7 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
 }
 
 // ------------------------------------------------------------------------------------------------
-// k_pass_a: every CTA owns one static run of consecutive chunks of one worker (runs balanced by elements, a few
+// k_pass_a: every CTA owns one static run of consecutive chunks of one worker (runs balanced by cost, a few
 // per SM); histogram words and the cell table of the current layer live in shared memory
 // ------------------------------------------------------------------------------------------------
 struct SweepRun { uint32_t w, c0, c1; }; // chunks [c0, c1) of worker w
@@ -501,6 +501,7 @@ k_pass_a(const float* __restrict__ grads, const float* __restrict__ state, uint8
     // layer's exact zeros are left out of the histogram
     constexpr uint32_t kSkipZeros = 0x40000000u;
     uint32_t wr = 0xffffffffu;
+    __shared__ uint32_t s_bins; // of the current layer's histogram
     bool dirty = false;
     int wlo_m1 = 0, whi_p1 = 0;  // cells of the table's first and last entry, in units of 2^(cshift - 15) cells
     uint32_t cshift = 15, lshift = 0; // keys per table entry, bins per code (log2)
@@ -508,15 +509,25 @@ k_pass_a(const float* __restrict__ grads, const float* __restrict__ state, uint8
     auto flush = [&]() {
         __syncthreads();
         const uint32_t slot = wr & ~kSkipZeros;
-        const uint32_t n_bins = meta[slot].n_bins;
+        const uint32_t n_bins = s_bins;
         uint32_t* gc = bh_cnt + (size_t)slot * kMaxBins;
         unsigned long long* gs = bh_sum + (size_t)slot * kMaxBins;
-        for (uint32_t i = threadIdx.x; i < n_bins; i += kBigThreads) {
-            const uint32_t c = h_cnt[i];
-            if (c) {
-                atomicAdd(&gc[i], c);
-                atomicAdd(&gs[i], (unsigned long long)h_lo[i]);
-                h_cnt[i] = 0; h_lo[i] = 0;
+        for (uint32_t i0 = threadIdx.x; i0 < n_bins; i0 += 4 * kBigThreads) { // four bins at a time
+            uint32_t c[4], lo[4];
+#pragma unroll
+            for (uint32_t q = 0; q < 4; ++q) {
+                const uint32_t i = min(i0 + q * kBigThreads, (uint32_t)kMaxBins - 1u);
+                c[q] = i0 + q * kBigThreads < n_bins ? h_cnt[i] : 0u;
+                lo[q] = h_lo[i];
+            }
+#pragma unroll
+            for (uint32_t q = 0; q < 4; ++q) {
+                const uint32_t i = i0 + q * kBigThreads;
+                if (c[q]) {
+                    atomicAdd(&gc[i], c[q]);
+                    atomicAdd(&gs[i], (unsigned long long)lo[q]);
+                    h_cnt[i] = 0; h_lo[i] = 0;
+                }
             }
         }
         __syncthreads();
@@ -590,10 +601,11 @@ k_pass_a(const float* __restrict__ grads, const float* __restrict__ state, uint8
             if (r != 0xffffffffu && !meta[run.w * R + r].flagged) {
                 wr = run.w * R + r;
                 const int4 win = cell_win[wr];
-                wlo_m1 = win.x; whi_p1 = win.y; cshift = (uint32_t)win.z; lshift = (uint32_t)win.w & 31u;
-                const uint32_t* g2 = cell_tab + (size_t)wr * kCellTab;
                 const uint32_t used = meta[wr].n_cells;
-                for (uint32_t i = threadIdx.x; i < used; i += kBigThreads) tab[i] = g2[i];
+                wlo_m1 = win.x; whi_p1 = win.y; cshift = (uint32_t)win.z; lshift = (uint32_t)win.w & 31u;
+                if (threadIdx.x == 0) s_bins = meta[wr].n_bins;
+                static_assert(kCellTab == 4 * kBigThreads && 2 * kMaxBins % 4 == 0, "the table in one round of 128-bit loads");
+                if (4 * threadIdx.x < used) reinterpret_cast<uint4*>(tab)[threadIdx.x] = reinterpret_cast<const uint4*>(cell_tab + (size_t)wr * kCellTab)[threadIdx.x];
                 if ((uint32_t)win.w & 256u) wr |= kSkipZeros;
             }
             __syncthreads();
