@@ -164,7 +164,8 @@ static int preload_kernels() {
 #define KIMAD_PRELOAD(f) CUDA_TRY(cudaFuncGetAttributes(&a, f))
     KIMAD_PRELOAD(k_sample); KIMAD_PRELOAD(k_pass_a<true>); KIMAD_PRELOAD(k_pass_a<false>); KIMAD_PRELOAD(k_resolve_a<true>); KIMAD_PRELOAD(k_resolve_a<false>);
     KIMAD_PRELOAD(k_refine); KIMAD_PRELOAD(k_tiny_exact); KIMAD_PRELOAD(k_fb1); KIMAD_PRELOAD(k_fb23<2>); KIMAD_PRELOAD(k_fb23<3>);
-    KIMAD_PRELOAD(k_dp<2>); KIMAD_PRELOAD(k_dp<4>); KIMAD_PRELOAD(k_dp<8>); KIMAD_PRELOAD(k_pick); KIMAD_PRELOAD(k_fit_ratio); KIMAD_PRELOAD(k_sel_count);
+    KIMAD_PRELOAD((k_dp<2, false>)); KIMAD_PRELOAD((k_dp<4, false>)); KIMAD_PRELOAD((k_dp<8, false>));
+    KIMAD_PRELOAD((k_dp<2, true>)); KIMAD_PRELOAD((k_dp<4, true>)); KIMAD_PRELOAD((k_dp<8, true>)); KIMAD_PRELOAD(k_pick); KIMAD_PRELOAD(k_fit_ratio); KIMAD_PRELOAD(k_sel_count);
     KIMAD_PRELOAD((k_sel_offsets<128, true>)); KIMAD_PRELOAD((k_sel_offsets<128, false>)); KIMAD_PRELOAD((k_sel_offsets<512, false>)); KIMAD_PRELOAD(k_sel_recount);
     KIMAD_PRELOAD((k_sel_write<false, false>)); KIMAD_PRELOAD((k_sel_write<false, true>));
     KIMAD_PRELOAD((k_sel_write<true, false>)); KIMAD_PRELOAD((k_sel_write<true, true>));
@@ -292,9 +293,9 @@ static int prepare_device(kimad_ctx* c) {
     CUDA_TRY(cudaGetDevice(&dev));
     if (dev < 0 || dev >= KIMAD_BUILTIN_MAX_DEVICES) return KIMAD_ERR_INVALID_ARG;
     if (!ready[dev]) {
-        CUDA_TRY(cudaFuncSetAttribute(k_dp<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDpSmemMax));
-        CUDA_TRY(cudaFuncSetAttribute(k_dp<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDpSmemMax));
-        CUDA_TRY(cudaFuncSetAttribute(k_dp<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDpSmemMax));
+        auto dp_smem = [](auto kern) { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDpSmemMax); };
+        CUDA_TRY(dp_smem(k_dp<2, false>)); CUDA_TRY(dp_smem(k_dp<4, false>)); CUDA_TRY(dp_smem(k_dp<8, false>));
+        CUDA_TRY(dp_smem(k_dp<2, true>)); CUDA_TRY(dp_smem(k_dp<4, true>)); CUDA_TRY(dp_smem(k_dp<8, true>));
         CUDA_TRY(cudaFuncSetAttribute(k_pick, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDpSmemMax));
         CUDA_TRY(cudaFuncSetAttribute(k_sample, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->sample_smem));
         CUDA_TRY(cudaFuncSetAttribute(k_pass_a<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->pass_a_smem));
@@ -500,7 +501,8 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
                                             rows, row_stride, c->hist_row);
                     };
                     const uint32_t per = dp_cells_per_thread(c->dp_cells);
-                    CUDA_TRY(per == 2 ? launch(k_dp<2>) : (per == 4 ? launch(k_dp<4>) : launch(k_dp<8>)));
+                    if (p.window) CUDA_TRY(per == 2 ? launch(k_dp<2, true>) : (per == 4 ? launch(k_dp<4, true>) : launch(k_dp<8, true>)));
+                    else CUDA_TRY(per == 2 ? launch(k_dp<2, false>) : (per == 4 ? launch(k_dp<4, false>) : launch(k_dp<8, false>)));
                 } else {
                     const int pick = mode == kGivenJ ? 1 : (c->policy == 1 ? 2 : (c->policy == 2 ? 3 : 4));
                     CUDA_TRY(launch_pdl(k_pick, nwa, kPickThreads, c->pick_smem, st, budgets_of(wa, nwa), wa, ca, pick, c->pick_plan, j_dev, pd));

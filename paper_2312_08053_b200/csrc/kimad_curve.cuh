@@ -52,6 +52,11 @@ struct WarpLanes {
     __device__ __forceinline__ void sync() const { __syncwarp(); }
 };
 
+__device__ __forceinline__ uint32_t select(uint32_t c, uint32_t x, uint32_t y) { // c != 0 ? x : y, without a branch
+    uint32_t r;
+    asm("{.reg .pred p; setp.ne.u32 p, %1, 0; selp.b32 %0, %2, %3, p;}" : "=r"(r) : "r"(c), "r"(x), "r"(y));
+    return r;
+}
 __device__ __forceinline__ uint32_t hash_u32(uint32_t x) {
     x ^= x >> 16; x *= 0x7feb352du; x ^= x >> 15; x *= 0x846ca68bu; x ^= x >> 16;
     return x;
@@ -207,8 +212,12 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
     // cell holding sample rank rk (1-based, from the top); the whole warp takes part
     const uint32_t lane = threadIdx.x & 31;
     auto cell_of_rank = [&](uint32_t rk) {
-        int lo = 0, hi = kBigThreads - 1;
-        while (lo < hi) { const int mid = (lo + hi) >> 1; if (s_pre[mid] >= rk) hi = mid; else lo = mid + 1; }
+        // the first segment that reaches the rank: 32 segments' ends, then the segments of one of those 32 (as a bisection, ten rounds)
+        static_assert(kBigThreads == 1024, "two rounds of 32");
+        const uint32_t ends = __ballot_sync(0xffffffffu, s_pre[32u * lane + 31u] >= rk);
+        const uint32_t part = ends ? __ffs(ends) - 1u : 31u;
+        const uint32_t here = __ballot_sync(0xffffffffu, s_pre[32u * part + lane] >= rk);
+        const int lo = 32 * (int)part + (here ? __ffs(here) - 1 : 31);
         const uint32_t before = lo ? s_pre[lo - 1] : 0u;
         const uint32_t top = 65535u - 64u * lo;
         // lanes take cells top - 2 lane and top - 2 lane - 1; inclusive counts along the lanes
@@ -314,43 +323,62 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
     }
     __syncthreads();
     // merge overlapping / adjacent bands (they descend in key with j) into groups; groups end up in s_c*[0..ng)
-    if (threadIdx.x == 0 && !s_flag) {
+    // (by a warp that holds the candidates, 32 at a time: one thread that read them from shared memory took 1.9 us)
+    if (threadIdx.x < 32 && !s_flag) {
         // The sweep reads a key's region from a table over the cells between the lowest and the highest band.  If
         // that window has more cells than the table has entries, an entry stands for 2^cg cells and the bands
         // are widened to whole entries (more fine bins; the common case is cg = 0).
         uint32_t lo_all = 0xffffffffu, hi_all = 0, cg = 0;
-        for (uint32_t j = 0; j < K; ++j)
+        for (uint32_t j = lane; j < K; j += 32u)
             if (s_cb[j] <= s_ct[j]) { lo_all = min(lo_all, s_cb[j]); hi_all = max(hi_all, s_ct[j]); }
+        lo_all = __reduce_min_sync(0xffffffffu, lo_all);
+        hi_all = __reduce_max_sync(0xffffffffu, hi_all);
         if (lo_all <= hi_all)
             while ((hi_all >> cg) - (lo_all >> cg) + 3 > (uint32_t)kCellTab) ++cg;
-        s_cg = cg;
         const uint32_t cmask = (1u << cg) - 1u;
-        uint32_t ng = 0;
+        // The group that is open goes to slot ng, again with every band that joins it (ng <= j: slots already consumed).
+        uint32_t ng = 0, open = 0;
         uint32_t gb = 1, gt = 0, gs = 15;
         float gn = 0.f;
-        bool open = false;
-        for (uint32_t j = 0; j < K; ++j) {
-            uint32_t cb = s_cb[j], ct = s_ct[j];
-            const uint32_t cs = s_cs[j];
-            const float cn = s_nd[j];
-            if (cb > ct) continue;
-            cb &= ~cmask; ct |= cmask; // stays below the non-finite cells: 65279 ends a block of 32
-            if (open && ct + 1 >= gb) {
-                gb = min(gb, cb); gt = max(gt, ct); gs = min(gs, cs); gn = fmaxf(gn, cn);
-            } else {
-                if (open) { s_cb[ng] = gb; s_ct[ng] = gt; s_cs[ng] = gs; s_nd[ng] = gn; ++ng; } // ng <= j: slots already consumed
-                gb = cb; gt = ct; gs = cs; gn = cn; open = true;
+        for (uint32_t j0 = 0; j0 < K; j0 += 32u) {
+            const uint32_t jl = min(j0 + lane, K - 1u);
+            const uint32_t my_cb = s_cb[jl], my_ct = s_ct[jl], my_cs = s_cs[jl], upto = min(32u, K - j0);
+            const float my_nd = s_nd[jl];
+            __syncwarp();
+#pragma unroll 4
+            for (uint32_t i = 0; i < upto; ++i) {
+                uint32_t cb = __shfl_sync(0xffffffffu, my_cb, i), ct = __shfl_sync(0xffffffffu, my_ct, i);
+                const uint32_t cs = __shfl_sync(0xffffffffu, my_cs, i);
+                const float cn = __shfl_sync(0xffffffffu, my_nd, i);
+                const uint32_t valid = cb <= ct;
+                cb &= ~cmask; ct |= cmask; // stays below the non-finite cells: 65279 ends a block of 32
+                const uint32_t join = open & (uint32_t)(ct + 1 >= gb);
+                ng += valid & open & (join ^ 1u);
+                // joined, first of a group, left out: written out as selections (branches took as long as one thread that walked the list)
+                gb = select(valid, select(join, min(gb, cb), cb), gb);
+                gt = select(valid, select(join, max(gt, ct), ct), gt);
+                gs = select(valid, select(join, min(gs, cs), cs), gs);
+                gn = __uint_as_float(select(valid, select(join, __float_as_uint(fmaxf(gn, cn)), __float_as_uint(cn)), __float_as_uint(gn)));
+                open |= valid;
+                if (lane == 0) { s_cb[ng] = gb; s_ct[ng] = gt; s_cs[ng] = gs; s_nd[ng] = gn; }
             }
+            __syncwarp();
         }
-        if (open) { s_cb[ng] = gb; s_ct[ng] = gt; s_cs[ng] = gs; s_nd[ng] = gn; ++ng; }
-        uint64_t fine = 0, cells = 0;
-        for (uint32_t g = 0; g < ng; ++g) {
-            fine += (uint64_t)(s_ct[g] - s_cb[g] + 1) << (15 - s_cs[g]);
-            cells += s_ct[g] - s_cb[g] + 1;
+        ng += open;
+        uint32_t fine = 0, cells = 0;
+        for (uint32_t g = lane; g < ng; g += 32u) {
+            const uint32_t c = s_ct[g] - s_cb[g] + 1;
+            fine += c << (15 - s_cs[g]);
+            cells += c;
         }
-        if (cells > (uint64_t)kFineBins) s_flag = 3;
-        s_fine = (uint32_t)fine; // (below 2^24 unless flagged)
-        s_ng = ng;
+        fine = __reduce_add_sync(0xffffffffu, fine);
+        cells = __reduce_add_sync(0xffffffffu, cells);
+        if (lane == 0) {
+            s_cg = cg;
+            if (cells > (uint32_t)kFineBins) s_flag = 3;
+            s_fine = fine; // (below 2^24 unless flagged)
+            s_ng = ng;
+        }
     }
     uint32_t left = 0; // fine bins not given away
     if (threadIdx.x < 32) {
@@ -392,22 +420,37 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
     // Every region -- a gap or a group of fine bins -- maps a key to its bin as base + (key >> shift) with one
     // (base, shift) pair: shift 20 for the gap pieces, the group's bin width for the fine bins.
     uint32_t* s_glo = s_pre; // [kMaxGaps] reuse: the rank prefix is no longer needed
-    if (threadIdx.x == 0 && !s_flag) {
+    if (threadIdx.x < 32 && !s_flag) {
         uint32_t id = 0;
-        for (uint32_t a = 0; a <= ng; ++a) {
-            const uint32_t lo = a == 0 ? 0u : s_ct[ng - a] + 1;              // lowest cell of the gap
-            const uint32_t hi = a == ng ? 65279u : s_cb[ng - 1 - a] - 1;      // highest cell (may be lo - 1: empty)
-            s_base[a] = id;
-            s_glo[a] = lo;
-            if (hi + 1 > lo) id += (hi >> 5) - (lo >> 5) + 1;
-            if (a < ng) {
-                const uint32_t g = ng - 1 - a;
-                s_base[kBaseWords + a] = id; // first fine bin of group a
-                id += (s_ct[g] - s_cb[g] + 1) << (15 - s_cs[g]);
+        for (uint32_t a0 = 0; a0 <= ng; a0 += 32u) { // a lane per gap and the group above it
+            const uint32_t a = a0 + lane;
+            uint32_t gap = 0, bins = 0;
+            if (a <= ng) {
+                const uint32_t lo = a == 0 ? 0u : s_ct[ng - a] + 1;          // lowest cell of the gap
+                const uint32_t hi = a == ng ? 65279u : s_cb[ng - 1 - a] - 1;  // highest cell (may be lo - 1: empty)
+                s_glo[a] = lo;
+                if (hi + 1 > lo) gap = (hi >> 5) - (lo >> 5) + 1;
+                if (a < ng) {
+                    const uint32_t g = ng - 1 - a;
+                    bins = (s_ct[g] - s_cb[g] + 1) << (15 - s_cs[g]);
+                }
             }
+            uint32_t incl = gap + bins;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= (uint32_t)o) incl += y;
+            }
+            if (a <= ng) {
+                s_base[a] = id + incl - gap - bins;
+                if (a < ng) s_base[kBaseWords + a] = id + incl - bins; // first fine bin of group a
+            }
+            id += __shfl_sync(0xffffffffu, incl, 31);
         }
-        s_base[ng + 1] = id;     // keys with exponent 255: the pieces 2040..2047
-        s_base[ng + 2] = id + 8; // number of bins
+        if (lane == 0) {
+            s_base[ng + 1] = id;     // keys with exponent 255: the pieces 2040..2047
+            s_base[ng + 2] = id + 8; // number of bins
+        }
     }
     __syncthreads();
     const uint32_t tot_bins = s_flag ? 0u : s_base[ng + 2];
@@ -425,32 +468,39 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
     uint32_t* blo = bin_lo + wr * (kMaxBins + 1);
     // entry i serves the cells (wlo - 1 + i) << cg ...; the first one everything below the window, the last one
     // everything above it
-    // (base, shift) of the region that holds a cell, as base << 5 | shift (base may be negative); the cells of a thread ascend
-    for (uint32_t i = threadIdx.x, a = 0; i < used; i += kBigThreads) {
-        const uint32_t cell = i + 1 == used ? 65535u : (i == 0 && wlo == 0 ? 0u : (wlo + i - 1u) << cg);
-        while (a < ng && cell > s_ct[ng - 1 - a]) ++a;
-        const uint32_t g = ng - 1 - a;
-        if (a < ng && cell >= s_cb[g]) {
-            const uint32_t cs = s_cs[g];
-            tab[i] = (uint32_t)(((int)s_base[kBaseWords + a] - (int)(s_cb[g] << (15 - cs))) * 32) | cs;
-        } else {
-            tab[i] = (uint32_t)(((int)s_base[a] - (int)(s_glo[a] >> 5)) * 32) | 20u;
-        }
+    // (base, shift) of a region, as base << 5 | shift (base may be negative)
+    auto group_entry = [&](uint32_t a) {
+        const uint32_t g = ng - 1 - a, cs = s_cs[g];
+        return (uint32_t)(((int)s_base[kBaseWords + a] - (int)(s_cb[g] << (15 - cs))) * 32) | cs;
+    };
+    auto gap_entry = [&](uint32_t a) { return (uint32_t)(((int)s_base[a] - (int)(s_glo[a] >> 5)) * 32) | 20u; };
+    // The tables are filled region by region (gap a, the group above it), the CTA's warps dealt out to the regions, several to each where
+    // there are few: a region's entries are all the same, its bins' keys equally spaced.
+    const uint32_t regions = 2u * ng + 2u, wid = threadIdx.x >> 5, sub = max(1u, (uint32_t)(kBigThreads / 32) / regions);
+    const uint32_t from = 32u * (wid % sub) + lane, step = 32u * sub;
+    if (threadIdx.x == 0) {
+        tab[0] = wlo == 0 && ng && s_cb[ng - 1] == 0u ? group_entry(0) : gap_entry(0);
+        tab[used - 1u] = gap_entry(ng);
+        if (ng == 0) tab[1] = gap_entry(0); // (no band: one gap)
     }
-    // lower key of every bin; the bins of a thread ascend, and with them the region they lie in
-    for (uint32_t x = threadIdx.x, a = 0; x < tot_bins; x += kBigThreads) {
-        while (a < ng && s_base[a + 1] <= x) ++a;
-        uint32_t key;
-        if (x >= s_base[ng + 1]) {
-            key = ((2040u + x - s_base[ng + 1]) << 20) | kGapBit;
-        } else if (a < ng && x >= s_base[kBaseWords + a]) {
-            const uint32_t g = ng - 1 - a;
-            key = (s_cb[g] << 15) + ((x - s_base[kBaseWords + a]) << s_cs[g]);
+    for (uint32_t r = wid / sub; r < regions; r += (uint32_t)(kBigThreads / 32) / sub) {
+        const uint32_t a = r >> 1;
+        if (r == regions - 1u) {
+            if (from < 8u) blo[s_base[ng + 1] + from] = ((2040u + from) << 20) | kGapBit;
+        } else if (r & 1u) {
+            const uint32_t g = ng - 1 - a, cs = s_cs[g], bins = (s_ct[g] - s_cb[g] + 1) << (15 - cs), key = s_cb[g] << 15, e = group_entry(a);
+            for (uint32_t i = (s_cb[g] >> cg) - wlo + 1u + from; i <= (s_ct[g] >> cg) - wlo + 1u; i += step) tab[i] = e;
+            uint32_t* to = blo + s_base[kBaseWords + a];
+#pragma unroll 4
+            for (uint32_t i = from; i < bins; i += step) to[i] = key + (i << cs);
         } else {
-            const uint32_t lo = s_glo[a];
-            key = (max(lo, ((lo >> 5) + x - s_base[a]) << 5) << 15) | kGapBit;
+            const uint32_t lo = s_glo[a], bins = s_base[a < ng ? kBaseWords + a : ng + 1] - s_base[a], e = gap_entry(a);
+            if (a != 0u && a < ng)
+                for (uint32_t i = (lo >> cg) - wlo + 1u + from; i < (s_cb[ng - 1 - a] >> cg) - wlo + 1u; i += step) tab[i] = e;
+            uint32_t* to = blo + s_base[a];
+#pragma unroll 4
+            for (uint32_t i = from; i < bins; i += step) to[i] = (max(lo, ((lo >> 5) + i) << 5) << 15) | kGapBit;
         }
-        blo[x] = key;
     }
     if (threadIdx.x == 0) {
         blo[tot_bins] = 0x80000000u;

@@ -231,7 +231,8 @@ __device__ __forceinline__ void choose_finish(const ChooseArgs& a, uint32_t w, u
 // ------------------------------------------------------------------------------------------------
 // k_dp: one CTA per worker; a thread owns CPT cells of a row (32 apart: a warp owns 32 CPT consecutive cells)
 // ------------------------------------------------------------------------------------------------
-template <int CPT>
+// (WINDOWS: contexts whose plan has them; apart, since the calls alone cost the others 4 us of 31)
+template <int CPT, bool WINDOWS>
 __global__ void __launch_bounds__(CPT <= 4 ? 512 : kDpMaxThreads, 1)
 k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double* __restrict__ cost /* [L][K], see kimad_common.h */,
      uint32_t* __restrict__ tab_all /* [W] at tab_stride words, [L][2][rw] each */, size_t tab_stride,
@@ -271,7 +272,7 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
     __syncthreads(); // (and the flags are read before the end of the choice resets them)
 
     // ---- windows of the rows first.  (Where the limit of the waits is set, the recursion whose warps wait for each other is what is asked for.)
-    if (status == KIMAD_OK && plan.window && plan.wait_clocks == kDpWaitClocks) {
+    if (WINDOWS && status == KIMAD_OK && plan.wait_clocks == kDpWaitClocks) {
         auto at = [&](const void* p) { return (uint32_t)(reinterpret_cast<const unsigned char*>(p) - smem_raw); };
         const WindowArgs wa{L, K, D, kr, rw, c, cost, a.err + (size_t)w * L * K, CL, 8u * CL * rw, plan.window, tab,
                             reinterpret_cast<unsigned char*>(hist), (hist_stride - (size_t)(hist - (hist_all + w * hist_stride))) * 4u, at(s_p), at(s_ex), at(s_j)};
