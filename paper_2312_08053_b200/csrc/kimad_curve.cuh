@@ -1222,20 +1222,29 @@ k_resolve_a(const LayerDesc* __restrict__ layers, const uint32_t* __restrict__ r
         // (1) entries and squares of every group; (2) exclusive prefixes over the groups; (3) a warp per candidate:
         // the group where the running count passes n - k_j by bisection over the prefixes, then the bin inside it
         bool nonfinite = false;
-        for (uint32_t g = wid; g < ngrp; g += kBigThreads / 32) {
-            const uint32_t bb = 32u * g + lane;
-            uint32_t c = 0;
-            double sv = 0.0;
-            if (bb < nb) {
-                c = gc[bb];
-                if (c) { sv = bin_sq(bb); nonfinite |= blo[bb] >= 0x7f800000u; }
+        constexpr uint32_t AHEAD = 4; // groups per warp whose bins are requested together
+        for (uint32_t g0 = wid; g0 < ngrp; g0 += AHEAD * (kBigThreads / 32)) {
+            uint32_t c[AHEAD], key[AHEAD];
+            unsigned long long sq[AHEAD];
+#pragma unroll
+            for (uint32_t q = 0; q < AHEAD; ++q) {
+                const uint32_t bb = 32u * (g0 + q * (kBigThreads / 32)) + lane;
+                c[q] = key[q] = 0;
+                sq[q] = 0ull;
+                if (bb < nb) { c[q] = gc[bb]; sq[q] = gs[bb]; key[q] = blo[bb]; }
             }
 #pragma unroll
-            for (int o = 16; o; o >>= 1) {
-                c += __shfl_xor_sync(0xffffffffu, c, o);
-                sv += __shfl_xor_sync(0xffffffffu, sv, o);
+            for (uint32_t q = 0; q < AHEAD; ++q) {
+                const uint32_t g = g0 + q * (kBigThreads / 32);
+                double sv = (double)sq[q] * (256.0 * sq_scale(key[q] >> 23)); // (as bin_sq; nothing where nothing was counted)
+                nonfinite |= c[q] && key[q] >= 0x7f800000u;
+#pragma unroll
+                for (int o = 16; o; o >>= 1) {
+                    c[q] += __shfl_xor_sync(0xffffffffu, c[q], o);
+                    sv += __shfl_xor_sync(0xffffffffu, sv, o);
+                }
+                if (lane == 0 && g < ngrp) { s_gc[g] = c[q]; s_gs[g] = sv; }
             }
-            if (lane == 0) { s_gc[g] = c; s_gs[g] = sv; }
         }
         if (nonfinite) atomicOr(&flags[w], 1u);
         __syncthreads();
@@ -1318,8 +1327,7 @@ k_resolve_a(const LayerDesc* __restrict__ layers, const uint32_t* __restrict__ r
     if (!mt.flagged) { // clean for the next step
         uint32_t* gc = bh_cnt + wr * kMaxBins;
         unsigned long long* gs = bh_sum + wr * kMaxBins;
-        for (uint32_t bb = threadIdx.x; bb < mt.n_bins; bb += kBigThreads)
-            if (gc[bb]) { gc[bb] = 0; gs[bb] = 0ull; }
+        for (uint32_t bb = threadIdx.x; bb < mt.n_bins; bb += kBigThreads) { gc[bb] = 0; gs[bb] = 0ull; } // (without a look at what is there)
     }
     __shared__ uint32_t s_at;
     if constexpr (!LISTS) {
