@@ -397,8 +397,9 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
     if (T) CUDA_TRY(cudaEventRecord(c->ev_fork, s)); // fork point of the tiny layers' kernel: the step's start
     // (a) + (b): sample -> bands, all workers
     if (R) {
-        CUDA_TRY(launch_pdl(k_sample, dim3(R, W), kBigThreads, c->sample_smem, s, grads, state, c->stride, layers, reg_layers, R,
-                            ktab, K, c->curve_mode == 1 ? 1u : 0u, cell_tab, cell_win, binlo, meta));
+        const uint32_t cz = sample_cluster((uint64_t)R * W);
+        CUDA_TRY(launch_clusters("k_sample", cz, k_sample, dim3(R, W, cz), kBigThreads, c->sample_smem, s, grads, state, c->stride, layers, reg_layers, R,
+                                 ktab, K, c->curve_mode == 1 ? 1u : 0u, cell_tab, cell_win, binlo, meta));
         c->launches += 1;
     }
     // Tiny layers: sorted in shared memory on the side stream, beside the sample kernel (its CTAs fill what that kernel leaves

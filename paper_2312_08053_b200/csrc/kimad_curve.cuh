@@ -43,6 +43,12 @@ constexpr int kSampleUnit = 32;                     // consecutive elements read
 constexpr int kSampleUnits = 2047;                  // units of a sample (<= 65504 elements: the u16 cell counters cannot overflow)
 constexpr int kWholeUnits = 1024;                   // layers of up to as many units are taken whole
 constexpr int kBigThreads = 1024;
+constexpr uint32_t kSampleClusterMost = 8, kSampleClusterCtas = 128;
+KIMAD_HD uint32_t sample_cluster(uint64_t ctas) {
+    uint32_t c = kSampleClusterMost;
+    while (c > 1u && ctas * c > kSampleClusterCtas) c >>= 1;
+    return c;
+}
 constexpr uint32_t kGapBit = 1u;                    // bin_lo entries carry this bit when the bin is a gap bin
 
 
@@ -62,8 +68,22 @@ __device__ __forceinline__ uint32_t hash_u32(uint32_t x) {
     return x;
 }
 
+// A cluster's CTAs meet; what one of them wrote before is seen by all of them after.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+// The word at `addr` (shared memory of this CTA) in the shared memory of the cluster's CTA `rank`.
+__device__ __forceinline__ uint32_t cluster_word(uint32_t addr, uint32_t rank) {
+    uint32_t at, x;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(addr), "r"(rank));
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(x) : "r"(at) : "memory");
+    return x;
+}
+
 // ------------------------------------------------------------------------------------------------
-// k_sample: one CTA per (regular layer, worker)
+// k_sample: one CTA per (regular layer, worker), or a cluster of up to kSampleClusterMost that read the layer's sample together.  A CTA's
+// 64 units per warp take 20 us of its 35 at the latency of DRAM, whatever the other SMs do: where the clusters of all layers are resident
+// at once (kSampleClusterCtas; a CTA fills an SM but for a CTA of the tiny layers' kernel), the others count their part of the units and the
+// first one adds the cells that hold anything to its own.
 // ------------------------------------------------------------------------------------------------
 // (48 registers: a CTA of the tiny layers' kernel, which runs beside this one, then fits on the same SM)
 __global__ void __maxnreg__(48)
@@ -89,8 +109,9 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
     const uint32_t l = reg_layers[r];
     const size_t wr = (size_t)w * R + r;
     BandMeta* mt = meta + wr;
+    const uint32_t rank = blockIdx.z, ranks = gridDim.z; // in the layer's cluster
     if (force_exact) {
-        if (threadIdx.x == 0) *mt = BandMeta{0, 0, 1, 0};
+        if (threadIdx.x == 0 && rank == 0) *mt = BandMeta{0, 0, 1, 0};
         return;
     }
     const LayerDesc ld = layers[l];
@@ -115,7 +136,8 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
     uint32_t top_key = 0;                                  // largest finite key
     // a warp reads one unit (128 bytes); eight units per thread are in flight before their keys are counted (this phase runs at
     // the DRAM's random-access rate on large layers; four and four, counted alternately, took a fifth longer)
-    for (uint32_t ib = threadIdx.x / kSampleUnit; ib < m_units; ib += 8 * (kBigThreads / kSampleUnit)) {
+    constexpr uint32_t kRound = 8 * (kBigThreads / kSampleUnit); // units of a round
+    for (uint32_t ib = rank * kRound + threadIdx.x / kSampleUnit; ib < m_units; ib += ranks * kRound) {
         float a[8], b[8];
         bool ok[8];
         // where the round's eight units start is the same for all lanes: lane u (mod 8) works out unit u's start
@@ -155,6 +177,45 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
     top_key = __reduce_max_sync(0xffffffffu, top_key);
     if ((threadIdx.x & 31) == 0) atomicMax(&s_top, top_key);
     __syncthreads();
+    if (ranks > 1u) {
+        const uint32_t ln = threadIdx.x & 31u, wd = threadIdx.x >> 5;
+        // segments of 64 cells (32 words) that hold anything, a bit each: bit w of word i stands for segment 32 i + w, so that the segments of a
+        // distribution, which lie side by side, fall to different warps below
+        if (rank) {
+            for (uint32_t i = 0; i < 32u; ++i) {
+                const uint32_t any = __reduce_or_sync(0xffffffffu, h32[32u * (32u * i + wd) + ln]);
+                if (ln == i) s_sq[32u * wd + i] = __uint_as_float(any ? 1u : 0u);
+            }
+            __syncthreads();
+            const uint32_t bits = __ballot_sync(0xffffffffu, __float_as_uint(s_sq[32u * ln + wd]) != 0u); // word wd: warp ln's segment
+            if (ln == 0) s_pre[wd] = bits;
+        }
+        cluster_arrive();
+        cluster_wait();
+        if (rank == 0) {
+            uint32_t all = 0; // lane i: the segments 32 i ... of the others
+            for (uint32_t r2 = 1; r2 < ranks; ++r2) all |= cluster_word(smem_u32(s_pre + ln), r2);
+            for (uint32_t todo = __ballot_sync(0xffffffffu, (all >> wd) & 1u); todo; todo &= todo - 1u) {
+                const uint32_t at = 32u * (32u * (__ffs(todo) - 1u) + wd) + ln;
+                uint32_t x[kSampleClusterMost];
+#pragma unroll
+                for (uint32_t r2 = 1; r2 < kSampleClusterMost; ++r2) x[r2] = r2 < ranks ? cluster_word(smem_u32(h32 + at), r2) : 0u;
+                uint32_t sum = h32[at];
+#pragma unroll
+                for (uint32_t r2 = 1; r2 < kSampleClusterMost; ++r2) sum += x[r2]; // (two counters a word: of 65504 entries at most in all)
+                h32[at] = sum;
+            }
+            if (threadIdx.x >= 1u && threadIdx.x < ranks) {
+                atomicMax(&s_top, cluster_word(smem_u32(&s_top), threadIdx.x));
+                atomicAdd(&s_z, cluster_word(smem_u32(&s_z), threadIdx.x));
+                const uint32_t lo = cluster_word(smem_u32(&s_zz), threadIdx.x), hi = cluster_word(smem_u32(&s_zz) + 4u, threadIdx.x);
+                atomicAdd(&s_zz, (unsigned long long)hi << 32 | lo);
+            }
+        }
+        cluster_arrive(); // the others' memory has been read
+        cluster_wait();
+        if (rank) return;
+    }
     auto cell_count = [&](uint32_t cell) { return (h32[cell >> 1] >> (16 * (cell & 1))) & 0xffffu; };
     // Square of the cell's middle value, in units that put the sample's largest value into [2^40, 2^41): sums of squares over the
     // layer stay finite, and squares of values down to 2^-113 of the largest one are there.  Only ratios of sums are used.
@@ -1046,10 +1107,6 @@ template <int LEVEL, int NT>
 __device__ __forceinline__ void fb23_resolve(const ListArgs& a, uint32_t l, uint32_t w, size_t wl, size_t wr) {
     fb_resolve23_layer<LEVEL, NT>(l, w, wl, wr, a.K, a.h23_cnt, a.h23_ss, a.cands, a.slots, a.err, a.tau, a.keep_eq, a.shift, a.codes);
 }
-
-// A cluster's CTAs meet; what one of them wrote before is seen by all of them after.
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 
 // All of it for one layer, by a cluster of n CTAs of kBigThreads threads: the chunks are dealt out to them, the steps that need all
 // chunks are the first one's.  exact: the exact path at once, else the refinement first.  word: the cluster's verdict, zero afterwards.

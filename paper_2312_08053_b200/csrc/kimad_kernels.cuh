@@ -39,6 +39,7 @@ constexpr int kThreads = 256;
 constexpr int kL1Bins = 2048;  // 8 exponent bits + 3 mantissa bits
 constexpr int kL23Bins = 1024; // 10 bits each
 
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ uint32_t key_of(float d) { return __float_as_uint(d) & 0x7fffffffu; }
 
 // Kernels launched with programmatic stream serialisation may be scheduled before their predecessor in the
