@@ -1420,85 +1420,93 @@ k_resolve_a(const LayerDesc* __restrict__ layers, const uint32_t* __restrict__ r
 }
 
 // ------------------------------------------------------------------------------------------------
-// Bitonic sort (descending) of np = 512 .. kTinyMax keys in shared memory with sixteen consecutive keys per thread
-// held in registers: compare-exchanges at distances below 16 stay inside a thread, distances 16 .. 256 are a
-// shuffle with the thread 1 .. 16 lanes away, and only distances of 512 and more (six of the 78 stages at 4096
-// keys) go through shared memory.  The first np / 16 threads hold keys (whole warps: np >= 512); all threads of
-// the CTA take part in the barriers.
+// Bitonic sort (descending) of np = 64 E .. kTinyMax keys in shared memory with E consecutive keys per thread
+// held in registers: compare-exchanges at distances below E stay inside a thread, those of E .. 16 E are a
+// shuffle with the thread 1 .. 16 lanes away, and only larger distances go through shared memory.  The first np / E threads hold
+// keys (whole warps: np >= 64 E); all threads of the CTA take part in the barriers.  E as small as the CTA's threads allow: the
+// stages are a chain of latencies (1024 keys with sixteen per thread 9000 cycles).  Which key of a pair is kept is written out as
+// selections.
 // ------------------------------------------------------------------------------------------------
-template <int STRIDE>
-__device__ __forceinline__ void tiny_ce_inside(uint32_t (&v)[16], bool desc) {
+template <int E, int STRIDE>
+__device__ __forceinline__ void tiny_ce_inside(uint32_t (&v)[E], uint32_t desc) {
+    if constexpr (STRIDE > 0) {
 #pragma unroll
-    for (int e = 0; e < 16; ++e)
-        if (!(e & STRIDE)) {
-            const uint32_t hi = max(v[e], v[e | STRIDE]), lo = min(v[e], v[e | STRIDE]);
-            v[e] = desc ? hi : lo;
-            v[e | STRIDE] = desc ? lo : hi;
-        }
-}
-// the stages of the sizes 2 .. 8: direction by the key's position inside the thread
-template <int SIZE>
-__device__ __forceinline__ void tiny_sort_inside(uint32_t (&v)[16]) {
-#pragma unroll
-    for (int str = SIZE / 2; str > 0; str >>= 1)
-#pragma unroll
-        for (int e = 0; e < 16; ++e)
-            if (!(e & str)) {
-                const uint32_t hi = max(v[e], v[e | str]), lo = min(v[e], v[e | str]);
-                const bool desc = (e & SIZE) == 0;
-                v[e] = desc ? hi : lo;
-                v[e | str] = desc ? lo : hi;
+        for (int e = 0; e < E; ++e)
+            if (!(e & STRIDE)) {
+                const uint32_t hi = max(v[e], v[e | STRIDE]), lo = min(v[e], v[e | STRIDE]);
+                v[e] = select(desc, hi, lo);
+                v[e | STRIDE] = select(desc, lo, hi);
             }
+        tiny_ce_inside<E, STRIDE / 2>(v, desc);
+    }
 }
+// the stages of the sizes 2 .. E / 2: direction by the key's position inside the thread
+template <int E, int SIZE>
+__device__ __forceinline__ void tiny_sort_inside(uint32_t (&v)[E]) {
+    if constexpr (SIZE < E) {
+#pragma unroll
+        for (int str = SIZE / 2; str > 0; str >>= 1)
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                if (!(e & str)) {
+                    const uint32_t hi = max(v[e], v[e | str]), lo = min(v[e], v[e | str]);
+                    const bool desc = (e & SIZE) == 0;
+                    v[e] = desc ? hi : lo;
+                    v[e | str] = desc ? lo : hi;
+                }
+        tiny_sort_inside<E, SIZE * 2>(v);
+    }
+}
+template <int E>
 __device__ __forceinline__ void tiny_sort_blocked(uint32_t* s_key, uint32_t np) {
-    const uint32_t t = threadIdx.x, nthr = np >> 4;
+    const uint32_t t = threadIdx.x, nthr = np / E;
     const bool holds = t < nthr;
-    uint32_t v[16];
+    uint32_t v[E];
     if (holds) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const uint4 x = reinterpret_cast<const uint4*>(s_key)[4 * t + q];
+        for (int q = 0; q < E / 4; ++q) {
+            const uint4 x = reinterpret_cast<const uint4*>(s_key)[E / 4 * t + q];
             v[4 * q] = x.x; v[4 * q + 1] = x.y; v[4 * q + 2] = x.z; v[4 * q + 3] = x.w;
         }
-        tiny_sort_inside<2>(v); tiny_sort_inside<4>(v); tiny_sort_inside<8>(v);
+        tiny_sort_inside<E, 2>(v);
     }
-    for (uint32_t size = 16; size <= np; size <<= 1) { // from here on the direction depends on the thread
-        const bool desc = ((16u * t) & size) == 0;
-        for (uint32_t str = size >> 1; str >= 16u; str >>= 1) {
-            const uint32_t dt = str >> 4;                  // the partner thread is t ^ dt
-            const bool keep_max = ((t & dt) == 0) == desc; // the lower position keeps the larger key when descending
+    for (uint32_t size = E; size <= np; size <<= 1) { // from here on the direction depends on the thread
+        const uint32_t desc = ((E * t) & size) == 0;
+        for (uint32_t str = size >> 1; str >= (uint32_t)E; str >>= 1) {
+            const uint32_t dt = str / E;                                    // the partner thread is t ^ dt
+            const uint32_t keep_max = (uint32_t)((t & dt) == 0) ^ desc ^ 1u; // the lower position keeps the larger key when descending
             if (dt >= 32u) { // another warp: through shared memory
                 __syncthreads(); // s_key is no longer read
                 if (holds) {
 #pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        reinterpret_cast<uint4*>(s_key)[4 * t + q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+                    for (int q = 0; q < E / 4; ++q)
+                        reinterpret_cast<uint4*>(s_key)[E / 4 * t + q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
                 }
                 __syncthreads();
                 if (holds) {
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const uint4 x = reinterpret_cast<const uint4*>(s_key)[4 * (t ^ dt) + q];
+                    for (int q = 0; q < E / 4; ++q) {
+                        const uint4 x = reinterpret_cast<const uint4*>(s_key)[E / 4 * (t ^ dt) + q];
                         const uint32_t pv[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) v[4 * q + i] = keep_max ? max(v[4 * q + i], pv[i]) : min(v[4 * q + i], pv[i]);
+                        for (int i = 0; i < 4; ++i) v[4 * q + i] = select(keep_max, max(v[4 * q + i], pv[i]), min(v[4 * q + i], pv[i]));
                     }
                 }
             } else if (holds) { // a lane of the same warp (the warps that hold keys are whole)
 #pragma unroll
-                for (int e = 0; e < 16; ++e) {
+                for (int e = 0; e < E; ++e) {
                     const uint32_t pv = __shfl_xor_sync(0xffffffffu, v[e], dt);
-                    v[e] = keep_max ? max(v[e], pv) : min(v[e], pv);
+                    v[e] = select(keep_max, max(v[e], pv), min(v[e], pv));
                 }
             }
         }
-        if (holds) { tiny_ce_inside<8>(v, desc); tiny_ce_inside<4>(v, desc); tiny_ce_inside<2>(v, desc); tiny_ce_inside<1>(v, desc); }
+        if (holds) tiny_ce_inside<E, E / 2>(v, desc);
     }
     __syncthreads();
     if (holds) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-            reinterpret_cast<uint4*>(s_key)[4 * t + q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        for (int q = 0; q < E / 4; ++q)
+            reinterpret_cast<uint4*>(s_key)[E / 4 * t + q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
     }
     __syncthreads();
 }
@@ -1534,18 +1542,29 @@ k_tiny_exact(const float* __restrict__ grads, const float* __restrict__ state, u
     }
     if (nonfinite) atomicOr(&flags[w], 1u);
     __syncthreads();
-    if (np >= 512u) tiny_sort_blocked(s_key, np);
-    else
-    for (uint32_t size = 2; size <= np; size <<= 1)       // bitonic sort, descending
-        for (uint32_t str = size >> 1; str > 0; str >>= 1) {
-            for (uint32_t i = threadIdx.x; i < np / 2; i += kThreads) {
-                const uint32_t a = 2 * i - (i & (str - 1)), b = a + str;
-                const bool desc = (a & size) == 0;
-                const uint32_t ka = s_key[a], kb = s_key[b];
-                if ((ka < kb) == desc) { s_key[a] = kb; s_key[b] = ka; }
-            }
-            __syncthreads();
+    // As many keys per thread as there are threads for; layers that a thread per key covers are ranked by counting (256 keys sorted with a
+    // barrier per stage: 12000 to 17000 cycles).
+    if (np > 2048u) tiny_sort_blocked<16>(s_key, np);
+    else if (np > 1024u) tiny_sort_blocked<8>(s_key, np);
+    else if (np > (uint32_t)kThreads) tiny_sort_blocked<4>(s_key, np);
+    else {
+        uint32_t rank = 0; // keys ahead of this thread's: larger ones, and equal ones with a lower index
+        const uint32_t mine = threadIdx.x < np ? s_key[threadIdx.x] : 0u;
+        uint32_t i = 0;
+        for (; i + 4u <= np; i += 4u) {
+            const uint4 x = *reinterpret_cast<const uint4*>(s_key + i);
+            rank += (uint32_t)(x.x > mine) + (uint32_t)(x.y > mine) + (uint32_t)(x.z > mine) + (uint32_t)(x.w > mine);
+            rank += (uint32_t)((x.x == mine) & (i < threadIdx.x)) + (uint32_t)((x.y == mine) & (i + 1u < threadIdx.x)) +
+                    (uint32_t)((x.z == mine) & (i + 2u < threadIdx.x)) + (uint32_t)((x.w == mine) & (i + 3u < threadIdx.x));
         }
+        for (; i < np; ++i) {
+            const uint32_t x = s_key[i];
+            rank += (uint32_t)(x > mine) + (uint32_t)((x == mine) & (i < threadIdx.x));
+        }
+        __syncthreads();
+        if (threadIdx.x < np) s_key[rank] = mine;
+        __syncthreads();
+    }
     // suffix sums of squares, smallest magnitudes first: position q = n-1-i runs over ascending magnitude
     constexpr int PER = kTinyMax / kThreads;
     double loc[PER];
@@ -1571,11 +1590,12 @@ k_tiny_exact(const float* __restrict__ grads, const float* __restrict__ state, u
         const uint32_t k = (uint32_t)ktab.at(w, (size_t)l * K + j);
         const size_t o = wl * K + j;
         const uint32_t t = s_key[k - 1];
-        int lo = 0, hi = (int)k - 1; // first rank whose key equals t
-        while (lo < hi) { const int mid = (lo + hi) >> 1; if (s_key[mid] == t) hi = mid; else lo = mid + 1; }
+        uint32_t lo = 0; // first rank whose key equals t: larger ones are counted
+#pragma unroll
+        for (uint32_t b = kTinyMax / 2; b; b >>= 1) lo += select((uint32_t)(lo + b < k) & (uint32_t)(s_key[min(lo + b, k) - 1u] > t), b, 0u);
         err_out[o] = k < n ? (float)s_suf[k] : 0.f;
         tau_out[o] = t;
-        rank_out[o] = k - (uint32_t)lo;
+        rank_out[o] = k - lo;
         shift_out[o] = code_of_key(t) << 8;
     }
 }
