@@ -689,8 +689,9 @@ int kimad_create(kimad_ctx** out, const uint64_t* layer_sizes, uint32_t n_layers
                 }
                 return n;
             };
-            uint64_t low = N / per_w, high = N + (uint64_t)c->reg_layers.size() * kSweepLayerElems; // too little (or just right), enough
-            while (high - low > 64) {
+            // too little (or just right); enough: all costs over the runs, and one chunk's on top
+            uint64_t low = N / per_w, high = (N + (c->reg_layers.size() + per_w) * kSweepLayerElems) / per_w + window + kSweepLayerElems + 1;
+            while (high - low > std::max<uint64_t>(64, low / 1024)) {
                 const uint64_t mid = low + (high - low) / 2;
                 if (cut(mid, nullptr) <= per_w) high = mid;
                 else low = mid;

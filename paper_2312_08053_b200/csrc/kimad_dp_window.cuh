@@ -33,6 +33,9 @@ constexpr uint32_t kWindowPiece = 32 * 1024;      // shared memory for the steps
 KIMAD_HD uint32_t window_layers(uint32_t cells) { return cells <= 1024u ? 100u : 40u; }
 constexpr uint32_t kWindowJump = 100;             // cells between two neighbouring prices' choices up to which 64 cells are tried first
 constexpr uint32_t kPrices = 8, kSearchRounds = 20, kSearchPrices = 24;
+// Many layers: what the price of a sample of them may be off (bits of a binary32: an eighth to a sixth), after which one round over all
+// layers finds it to 3 %.
+constexpr uint32_t kThinSpread = 3u << 19;
 constexpr uint32_t kPriceThreads = 64;            // threads that share a price's layers
 constexpr uint32_t kBackWarps = 16;
 constexpr uint32_t kWindowChunk = kDpMaxChunkLayers;
@@ -65,9 +68,9 @@ struct CellsOf {
 };
 
 struct WindowScratch { // shared memory
-    double run[2][kPrices], warp_sum[kPrices][2];
+    double run[2][kPrices], warp_sum[kPrices][kWindowChunk / kPriceThreads][2];
     float price[kPrices], all[kPrices];
-    int cells[2][2], warp_cells[2][2]; // of the two middle prices: so far (two turns), of the price's two warps
+    int cells[2][2], warp_cells[2][kWindowChunk / kPriceThreads][2]; // of the two middle prices: so far (two turns), of the price's two warps
     uint32_t mask[2 * kWindowChunk / 32], count[2 * kWindowChunk / 32]; // layers of a chunk that exchange their rows; operations per warp
     uint32_t listed[kWindowChunk]; // layers whose candidates take different numbers of cells
     uint32_t used[kSearchRounds][kSearchPrices];
@@ -109,6 +112,10 @@ __device__ __forceinline__ float pick_if(int c, float x, float y) { // c != 0 ? 
     float r;
     asm("{.reg .pred p; setp.ne.s32 p, %1, 0; selp.f32 %0, %2, %3, p;}" : "=f"(r) : "r"(c), "f"(x), "f"(y));
     return r;
+}
+
+__device__ __forceinline__ void store_if(int c, uint32_t at, uint32_t x) { // to shared memory
+    asm volatile("{.reg .pred p; setp.ne.s32 p, %0, 0; @p st.shared.u32 [%1], %2;}" ::"r"(c), "r"(at), "r"(x) : "memory");
 }
 
 __device__ __forceinline__ void window_sync(uint32_t warps) { // the warps that carry the recursion (all of them get here)
@@ -212,28 +219,26 @@ __device__ __noinline__ bool window_search(const WindowArgs& a, float* total) {
             const float2* in = raw + t * (K + 1u);
             uint32_t* rec = recs + t * rw;
             const float u0 = in[0].x, most = (float)D;
-            uint32_t nd = 0;
+            uint32_t at = 0; // the entry being made; stored when the next one is met
+            const uint32_t to = smem_u32(rec);
             float du = 0.f, e = in[0].y;
-            odd |= u0 > most; // not even the smallest candidate fits
-            top = __float_as_uint(e);
-            for (uint32_t j = 0; j < K; ++j) { // sizes ascend with j: the usable candidates come first
+            odd |= (uint32_t)(u0 > most) | (uint32_t)!(e >= 0.f && e < kInf); // (not even the smallest candidate fits)
+#pragma unroll 4
+            for (uint32_t j = 1; j < K; ++j) { // sizes ascend with j: the usable candidates come first
                 const float2 y = in[j];
-                if (y.x > most) break;
-                odd |= !(y.y >= 0.f && y.y < kInf);
+                const int ok = y.x <= most;
+                odd |= (uint32_t)ok & ((uint32_t)!(y.y >= 0.f) | (uint32_t)!(y.y < kInf));
                 const float d = fminf(y.x - u0, 8192.f);
-                if (d != du) {
-                    rec[nd] = __float_as_uint(du);
-                    rec[kr + nd] = __float_as_uint(e);
-                    ++nd;
-                    du = d;
-                    e = y.y;
-                } else {
-                    e = fminf(e, y.y);
-                }
+                const int fresh = ok & (int)(d != du);
+                store_if(fresh, to + 4u * at, __float_as_uint(du));
+                store_if(fresh, to + 4u * (kr + at), __float_as_uint(e));
+                at += fresh;
+                du = pick_if(fresh, d, du);
+                e = pick_if(fresh, y.y, pick_if(ok, fminf(e, y.y), e));
             }
-            rec[nd] = __float_as_uint(du);
-            rec[kr + nd] = __float_as_uint(e);
-            ++nd;
+            rec[at] = __float_as_uint(du);
+            rec[kr + at] = __float_as_uint(e);
+            const uint32_t nd = at + 1u;
             const uint32_t r0 = rec[0], r1 = rec[kr];
             for (uint32_t x = nd; x < ((nd + 7u) & ~7u); ++x) { rec[x] = r0; rec[kr + x] = r1; }
             rec[2u * kr] = nd;
@@ -327,14 +332,15 @@ __device__ __noinline__ bool window_search(const WindowArgs& a, float* total) {
     };
     if (!ONE) {
         rounds(true, (uint32_t)((uint64_t)C * n_thin / L), 1u << 18);
-        lo = lo > lowest + (1u << 21) ? lo - (1u << 21) : lowest;
-        hi = min(hi + (1u << 21), highest);
+        lo = lo > lowest + kThinSpread ? lo - kThinSpread : lowest;
+        hi = min(hi + kThinSpread, highest);
         __syncthreads(); // the staged records make room
     }
-    rounds(ONE, C, 1u << 15);
+    rounds(ONE, C, ONE ? 1u << 15 : 1u << 18);
     if (hi >= 0x7f000000u) return false; // (twice the price is finite)
 
-    // ---- 2. sums of the smallest priced errors; 64 threads share a price, each takes consecutive layers of the chunk
+    // ---- 2. sums of the smallest priced errors; 64 threads share a price, a layer each and up to four times (side by side:
+    // consecutive layers per thread lie on the same banks)
     // (prices at factors of 0.7 .. 1.4 or 0.3 .. 3.3 around the two middle ones leave up to three times as many cells open)
     const uint32_t pi = t / kPriceThreads, pg = t % kPriceThreads;
     const float x_hi = __uint_as_float(hi);
@@ -350,58 +356,58 @@ __device__ __noinline__ bool window_search(const WindowArgs& a, float* total) {
         const bool middle = pi == 3u || pi == 4u;
         uint32_t turn = 0;
         for_chunks([&](const uint32_t* recs, uint32_t l0, uint32_t nl) {
-            const uint32_t q = (nl + kPriceThreads - 1u) / kPriceThreads, from = min(pg * q, nl), upto = min(from + q, nl);
-            double sum = 0.0, off = 0.0;
-            int taken = 0, coff = 0;
-            float m[kWindowChunk / kPriceThreads], u[kWindowChunk / kPriceThreads]; // of the thread's layers
+            constexpr uint32_t Q = kWindowChunk / kPriceThreads;
+            double incl[Q];
+            int ic[Q];
 #pragma unroll
-            for (uint32_t i = 0; i < kWindowChunk / kPriceThreads; ++i) {
-                m[i] = u[i] = 0.f;
-                if (pi < kPrices && from + i < upto) { // (a product and a sum in binary32 per layer)
-                    m[i] = kInf;
-                    for_candidates(recs + (from + i) * rw, [&](float du, float e) { take_less(fmaf(x, du, e), m[i], du, u[i]); });
+            for (uint32_t i = 0; i < Q; ++i) {
+                const uint32_t l = i * kPriceThreads + pg;
+                float m = 0.f, u = 0.f;
+                if (pi < kPrices && l < nl) { // (a product and a sum in binary32 per layer)
+                    m = kInf;
+                    for_candidates(recs + l * rw, [&](float du, float e) { take_less(fmaf(x, du, e), m, du, u); });
                 }
-                sum += (double)m[i];
-                taken += (int)u[i];
+                incl[i] = (double)m;
+                ic[i] = (int)u;
             }
-            double incl = sum;
-            int ic = taken;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const double y = __shfl_up_sync(0xffffffffu, incl, o);
-                const int yc = __shfl_up_sync(0xffffffffu, ic, o);
-                if (lane >= (uint32_t)o) { incl += y; ic += yc; }
-            }
+            for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+                for (uint32_t i = 0; i < Q; ++i) {
+                    const double y = __shfl_up_sync(0xffffffffu, incl[i], o);
+                    const int yc = __shfl_up_sync(0xffffffffu, ic[i], o);
+                    if (lane >= (uint32_t)o) { incl[i] += y; ic[i] += yc; }
+                }
             if (lane == 31u && pi < kPrices) {
-                sc.warp_sum[pi][wid & 1u] = incl;
-                if (middle) sc.warp_cells[pi - 3u][wid & 1u] = ic;
+#pragma unroll
+                for (uint32_t i = 0; i < Q; ++i) {
+                    sc.warp_sum[pi][i][wid & 1u] = incl[i];
+                    if (middle) sc.warp_cells[pi - 3u][i][wid & 1u] = ic[i];
+                }
             }
             __syncthreads();
             if (pi < kPrices) {
-                const double base = sc.run[turn][pi], first = base + sc.warp_sum[pi][0];
-                off = (pg < 32u ? base : first) + (incl - sum);
-                int cfirst = 0;
-                if (middle) {
-                    const int cbase = sc.cells[turn][pi - 3u];
-                    cfirst = cbase + sc.warp_cells[pi - 3u][0];
-                    coff = (pg < 32u ? cbase : cfirst) + ic - taken;
-                }
+                double base = sc.run[turn][pi];
+                int cbase = middle ? sc.cells[turn][pi - 3u] : 0;
 #pragma unroll
-                for (uint32_t i = 0; i < kWindowChunk / kPriceThreads; ++i) {
-                    const size_t l = l0 + from + i;
-                    off += (double)m[i];
-                    coff += (int)u[i];
-                    if (from + i < upto) {
-                        sums[l * kPrices + pi] = (float)off;
-                        if (pi == 3u) cells[l].x = coff;
-                        if (pi == 4u) cells[l].y = coff;
+                for (uint32_t i = 0; i < Q; ++i) {
+                    const size_t l = l0 + i * kPriceThreads + pg;
+                    const double a0 = sc.warp_sum[pi][i][0], a1 = sc.warp_sum[pi][i][1];
+                    int c0 = 0, c1 = 0;
+                    if (middle) { c0 = sc.warp_cells[pi - 3u][i][0]; c1 = sc.warp_cells[pi - 3u][i][1]; }
+                    if (i * kPriceThreads + pg < nl) {
+                        sums[l * kPrices + pi] = (float)(base + (pg < 32u ? 0.0 : a0) + incl[i]);
+                        const int c = cbase + (pg < 32u ? 0 : c0) + ic[i];
+                        if (pi == 3u) cells[l].x = c;
+                        if (pi == 4u) cells[l].y = c;
                     }
+                    base += a0 + a1;
+                    cbase += c0 + c1;
                 }
                 if (pg == 0u) { // of all layers so far
-                    const double now = first + sc.warp_sum[pi][1];
-                    sc.run[turn ^ 1u][pi] = now;
-                    sc.all[pi] = (float)now;
-                    if (middle) sc.cells[turn ^ 1u][pi - 3u] = cfirst + sc.warp_cells[pi - 3u][1];
+                    sc.run[turn ^ 1u][pi] = base;
+                    sc.all[pi] = (float)base;
+                    if (middle) sc.cells[turn ^ 1u][pi - 3u] = cbase;
                 }
             }
             turn ^= 1u;
@@ -531,10 +537,11 @@ __device__ __noinline__ bool window_search(const WindowArgs& a, float* total) {
                     uint32_t c = half ? n_other : 0u;
                     if (exchanges)
                         my_candidates([&](float du, float e) {
-                            if (!leads(du, e)) return;
-                            ops[at + c / 4u].dist[c & 3u] = (int)du - move;
-                            ops[at + c / 4u].err[c & 3u] = e;
-                            ++c;
+                            const int yes = leads(du, e);
+                            const uint32_t to = smem_u32(&ops[at + c / 4u].dist[c & 3u]);
+                            store_if(yes, to, (uint32_t)((int)du - move));
+                            store_if(yes, to + 16u, __float_as_uint(e)); // (err lies behind dist)
+                            c += yes;
                         });
                     if (half) // the rest of the last operation
                         for (c = exchanges ? n : 1u; c < 4u * n_ops; ++c) { ops[at + c / 4u].dist[c & 3u] = (int)W; ops[at + c / 4u].err[c & 3u] = 0.f; }
