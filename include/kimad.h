@@ -301,8 +301,9 @@ int kimad_debug_stage_times(kimad_ctx* ctx, float* host_ms);
 int kimad_debug_set_schedule(kimad_ctx* ctx, int mode);
 
 /* Limit, in SM clocks, of the waits inside the knapsack kernel (its warps wait for one another; default and maximum 2^31,
- * about a second).  For tests: a wait that runs out makes the worker's result KIMAD_ERR_TIMEOUT, with nothing selected
- * and the estimator unchanged; the context stays usable.  Errors: INVALID_ARG. */
+ * about a second).  A lower limit also keeps the search to whole rows, which are what its warps hand on to one another.  For
+ * tests: a wait that runs out makes the worker's result KIMAD_ERR_TIMEOUT, with nothing selected and the estimator
+ * unchanged; the context stays usable.  Errors: INVALID_ARG. */
 int kimad_debug_set_wait_limit(kimad_ctx* ctx, uint64_t clocks);
 
 /* kimad_step with a pair of CUDA events around every kernel launch; synchronises the device before and after and

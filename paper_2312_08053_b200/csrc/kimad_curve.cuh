@@ -1424,18 +1424,17 @@ k_resolve_a(const LayerDesc* __restrict__ layers, const uint32_t* __restrict__ r
 // held in registers: compare-exchanges at distances below E stay inside a thread, those of E .. 16 E are a
 // shuffle with the thread 1 .. 16 lanes away, and only larger distances go through shared memory.  The first np / E threads hold
 // keys (whole warps: np >= 64 E); all threads of the CTA take part in the barriers.  E as small as the CTA's threads allow: the
-// stages are a chain of latencies (1024 keys with sixteen per thread 9000 cycles).  Which key of a pair is kept is written out as
-// selections.
+// stages are a chain of latencies (1024 keys with sixteen per thread 9000 cycles).
 // ------------------------------------------------------------------------------------------------
 template <int E, int STRIDE>
-__device__ __forceinline__ void tiny_ce_inside(uint32_t (&v)[E], uint32_t desc) {
+__device__ __forceinline__ void tiny_ce_inside(uint32_t (&v)[E], bool desc) {
     if constexpr (STRIDE > 0) {
 #pragma unroll
         for (int e = 0; e < E; ++e)
             if (!(e & STRIDE)) {
                 const uint32_t hi = max(v[e], v[e | STRIDE]), lo = min(v[e], v[e | STRIDE]);
-                v[e] = select(desc, hi, lo);
-                v[e | STRIDE] = select(desc, lo, hi);
+                v[e] = desc ? hi : lo;
+                v[e | STRIDE] = desc ? lo : hi;
             }
         tiny_ce_inside<E, STRIDE / 2>(v, desc);
     }
@@ -1471,10 +1470,10 @@ __device__ __forceinline__ void tiny_sort_blocked(uint32_t* s_key, uint32_t np) 
         tiny_sort_inside<E, 2>(v);
     }
     for (uint32_t size = E; size <= np; size <<= 1) { // from here on the direction depends on the thread
-        const uint32_t desc = ((E * t) & size) == 0;
+        const bool desc = ((E * t) & size) == 0;
         for (uint32_t str = size >> 1; str >= (uint32_t)E; str >>= 1) {
             const uint32_t dt = str / E;                                    // the partner thread is t ^ dt
-            const uint32_t keep_max = (uint32_t)((t & dt) == 0) ^ desc ^ 1u; // the lower position keeps the larger key when descending
+            const bool keep_max = ((t & dt) == 0) == desc;                  // the lower position keeps the larger key when descending
             if (dt >= 32u) { // another warp: through shared memory
                 __syncthreads(); // s_key is no longer read
                 if (holds) {
@@ -1489,14 +1488,14 @@ __device__ __forceinline__ void tiny_sort_blocked(uint32_t* s_key, uint32_t np) 
                         const uint4 x = reinterpret_cast<const uint4*>(s_key)[E / 4 * (t ^ dt) + q];
                         const uint32_t pv[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) v[4 * q + i] = select(keep_max, max(v[4 * q + i], pv[i]), min(v[4 * q + i], pv[i]));
+                        for (int i = 0; i < 4; ++i) v[4 * q + i] = keep_max ? max(v[4 * q + i], pv[i]) : min(v[4 * q + i], pv[i]);
                     }
                 }
             } else if (holds) { // a lane of the same warp (the warps that hold keys are whole)
 #pragma unroll
                 for (int e = 0; e < E; ++e) {
                     const uint32_t pv = __shfl_xor_sync(0xffffffffu, v[e], dt);
-                    v[e] = select(keep_max, max(v[e], pv), min(v[e], pv));
+                    v[e] = keep_max ? max(v[e], pv) : min(v[e], pv);
                 }
             }
         }
