@@ -1420,11 +1420,11 @@ k_resolve_a(const LayerDesc* __restrict__ layers, const uint32_t* __restrict__ r
 }
 
 // ------------------------------------------------------------------------------------------------
-// Bitonic sort (descending) of np = 64 E .. kTinyMax keys in shared memory with E consecutive keys per thread
+// Bitonic sort (descending) of kThreads E keys in shared memory with E consecutive keys per thread
 // held in registers: compare-exchanges at distances below E stay inside a thread, those of E .. 16 E are a
-// shuffle with the thread 1 .. 16 lanes away, and only larger distances go through shared memory.  The first np / E threads hold
-// keys (whole warps: np >= 64 E); all threads of the CTA take part in the barriers.  E as small as the CTA's threads allow: the
-// stages are a chain of latencies (1024 keys with sixteen per thread 9000 cycles).
+// shuffle with the thread 1 .. 16 lanes away, and only larger distances go through shared memory.  The stages are a chain of
+// latencies, so every thread of the CTA takes part (E = 2 .. 16) and all of them are written out: as loops they took 150 to 200
+// cycles each, most of it branches.
 // ------------------------------------------------------------------------------------------------
 template <int E, int STRIDE>
 __device__ __forceinline__ void tiny_ce_inside(uint32_t (&v)[E], bool desc) {
@@ -1457,56 +1457,57 @@ __device__ __forceinline__ void tiny_sort_inside(uint32_t (&v)[E]) {
     }
 }
 template <int E>
-__device__ __forceinline__ void tiny_sort_blocked(uint32_t* s_key, uint32_t np) {
-    const uint32_t t = threadIdx.x, nthr = np / E;
-    const bool holds = t < nthr;
-    uint32_t v[E];
-    if (holds) {
+__device__ __forceinline__ void tiny_store(uint32_t* at, const uint32_t (&v)[E]) {
+    if constexpr (E == 2) {
+        *reinterpret_cast<uint2*>(at) = make_uint2(v[0], v[1]);
+    } else {
+#pragma unroll
+        for (int q = 0; q < E / 4; ++q) reinterpret_cast<uint4*>(at)[q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    }
+}
+template <int E>
+__device__ __forceinline__ void tiny_load(uint32_t (&v)[E], const uint32_t* at) {
+    if constexpr (E == 2) {
+        const uint2 x = *reinterpret_cast<const uint2*>(at);
+        v[0] = x.x; v[1] = x.y;
+    } else {
 #pragma unroll
         for (int q = 0; q < E / 4; ++q) {
-            const uint4 x = reinterpret_cast<const uint4*>(s_key)[E / 4 * t + q];
+            const uint4 x = reinterpret_cast<const uint4*>(at)[q];
             v[4 * q] = x.x; v[4 * q + 1] = x.y; v[4 * q + 2] = x.z; v[4 * q + 3] = x.w;
         }
-        tiny_sort_inside<E, 2>(v);
     }
-    for (uint32_t size = E; size <= np; size <<= 1) { // from here on the direction depends on the thread
-        const bool desc = ((E * t) & size) == 0;
-        for (uint32_t str = size >> 1; str >= (uint32_t)E; str >>= 1) {
-            const uint32_t dt = str / E;                                    // the partner thread is t ^ dt
-            const bool keep_max = ((t & dt) == 0) == desc;                  // the lower position keeps the larger key when descending
-            if (dt >= 32u) { // another warp: through shared memory
+}
+template <int E>
+__device__ __forceinline__ void tiny_sort_blocked(uint32_t* s_key) {
+    const uint32_t t = threadIdx.x;
+    uint32_t v[E];
+    tiny_load<E>(v, s_key + E * t);
+    tiny_sort_inside<E, 2>(v);
+#pragma unroll
+    for (int size = E; size <= E * kThreads; size <<= 1) { // from here on the direction depends on the thread
+        const bool desc = ((E * t) & (uint32_t)size) == 0;
+#pragma unroll
+        for (int str = size >> 1; str >= E; str >>= 1) {
+            const int dt = str / E;                                  // the partner thread is t ^ dt
+            const bool keep_max = ((t & (uint32_t)dt) == 0) == desc; // the lower position keeps the larger key when descending
+            uint32_t pv[E];
+            if (dt >= 32) { // another warp: through shared memory
                 __syncthreads(); // s_key is no longer read
-                if (holds) {
-#pragma unroll
-                    for (int q = 0; q < E / 4; ++q)
-                        reinterpret_cast<uint4*>(s_key)[E / 4 * t + q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-                }
+                tiny_store<E>(s_key + E * t, v);
                 __syncthreads();
-                if (holds) {
+                tiny_load<E>(pv, s_key + E * (t ^ (uint32_t)dt));
+            } else { // a lane of the same warp
 #pragma unroll
-                    for (int q = 0; q < E / 4; ++q) {
-                        const uint4 x = reinterpret_cast<const uint4*>(s_key)[E / 4 * (t ^ dt) + q];
-                        const uint32_t pv[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) v[4 * q + i] = keep_max ? max(v[4 * q + i], pv[i]) : min(v[4 * q + i], pv[i]);
-                    }
-                }
-            } else if (holds) { // a lane of the same warp (the warps that hold keys are whole)
-#pragma unroll
-                for (int e = 0; e < E; ++e) {
-                    const uint32_t pv = __shfl_xor_sync(0xffffffffu, v[e], dt);
-                    v[e] = keep_max ? max(v[e], pv) : min(v[e], pv);
-                }
+                for (int e = 0; e < E; ++e) pv[e] = __shfl_xor_sync(0xffffffffu, v[e], dt);
             }
+#pragma unroll
+            for (int e = 0; e < E; ++e) v[e] = keep_max ? max(v[e], pv[e]) : min(v[e], pv[e]);
         }
-        if (holds) tiny_ce_inside<E, E / 2>(v, desc);
+        tiny_ce_inside<E, E / 2>(v, desc);
     }
     __syncthreads();
-    if (holds) {
-#pragma unroll
-        for (int q = 0; q < E / 4; ++q)
-            reinterpret_cast<uint4*>(s_key)[E / 4 * t + q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-    }
+    tiny_store<E>(s_key + E * t, v);
     __syncthreads();
 }
 
@@ -1541,11 +1542,12 @@ k_tiny_exact(const float* __restrict__ grads, const float* __restrict__ state, u
     }
     if (nonfinite) atomicOr(&flags[w], 1u);
     __syncthreads();
-    // As many keys per thread as there are threads for; layers that a thread per key covers are ranked by counting (256 keys sorted with a
+    // Keys per thread by the padded size; layers that a thread per key covers are ranked by counting (256 keys sorted with a
     // barrier per stage: 12000 to 17000 cycles).
-    if (np > 2048u) tiny_sort_blocked<16>(s_key, np);
-    else if (np > 1024u) tiny_sort_blocked<8>(s_key, np);
-    else if (np > (uint32_t)kThreads) tiny_sort_blocked<4>(s_key, np);
+    if (np > 2048u) tiny_sort_blocked<16>(s_key);
+    else if (np > 1024u) tiny_sort_blocked<8>(s_key);
+    else if (np > 512u) tiny_sort_blocked<4>(s_key);
+    else if (np > (uint32_t)kThreads) tiny_sort_blocked<2>(s_key);
     else {
         uint32_t rank = 0; // keys ahead of this thread's: larger ones, and equal ones with a lower index
         const uint32_t mine = threadIdx.x < np ? s_key[threadIdx.x] : 0u;

@@ -10,7 +10,7 @@
 //   1. The price at which the relaxed choice fills the axis: rounds of 8 to 24 prices at a time.
 //   2. Smallest priced errors summed up layer by layer (binary64) at eight prices around it, and the cells that the relaxed choice
 //      takes: two neighbouring prices, weighted so that the axis is filled.
-//   3. The recursion in windows of 64 cells around that line (256 where the two prices are far apart in cells), over the candidates
+//   3. The recursion in windows of 64 cells around that line (128 with hundreds of layers, 256 where the two prices are far apart in cells), over the candidates
 //      that cost little at this price, one warp per 64 cells: a total U, nearly always the smallest one already.
 //   4. Do the bounds at U rule out every cell outside the windows and every candidate left out?  Nearly always; else the
 //      recursion once more in windows around the cells they leave open (64, 128 or 256), with the candidates they leave.  More than
@@ -33,8 +33,8 @@ constexpr uint32_t kWindowPiece = 32 * 1024;      // shared memory for the steps
 KIMAD_HD uint32_t window_layers(uint32_t cells) { return cells <= 1024u ? 100u : 40u; }
 constexpr uint32_t kWindowJump = 100;             // cells between two neighbouring prices' choices up to which 64 cells are tried first
 constexpr uint32_t kPrices = 8, kSearchRounds = 20, kSearchPrices = 24;
-// Many layers: what the price of a sample of them may be off (bits of a binary32: an eighth to a sixth), after which one round over all
-// layers finds it to 3 %.
+// Many layers: what the price of a sample of them may be off (bits of a binary32: an eighth to a sixth), after which two rounds over all
+// layers find it.  (Stopped at 3 % after one round, 12 us less, the first windows are too narrow or off more often.)
 constexpr uint32_t kThinSpread = 3u << 19;
 constexpr uint32_t kPriceThreads = 64;            // threads that share a price's layers
 constexpr uint32_t kBackWarps = 16;
@@ -325,9 +325,12 @@ __device__ __noinline__ bool window_search(const WindowArgs& a, float* total) {
             if (over < n_try) hi = from + step * (over + 1u);
             ++round;
             if (!ONE && listed) continue;
-            if (over == 0u && !lo_sure) lo = lowest; // the sample of layers misled
-            if (over == n_try && !hi_sure) hi = highest;
-            lo_sure = hi_sure = true;
+            lo_sure |= over != 0u;
+            hi_sure |= over != n_try;
+            if (!lo_sure) lo = lo > lowest + (1u << 23) ? lo - (1u << 23) : lowest; // the sample of layers misled: a factor of two further
+            if (!hi_sure) hi = highest - hi > (1u << 23) ? hi + (1u << 23) : highest;
+            lo_sure |= lo == lowest;
+            hi_sure |= hi == highest;
         }
     };
     if (!ONE) {
@@ -336,7 +339,7 @@ __device__ __noinline__ bool window_search(const WindowArgs& a, float* total) {
         hi = min(hi + kThinSpread, highest);
         __syncthreads(); // the staged records make room
     }
-    rounds(ONE, C, ONE ? 1u << 15 : 1u << 18);
+    rounds(ONE, C, 1u << 15);
     if (hi >= 0x7f000000u) return false; // (twice the price is finite)
 
     // ---- 2. sums of the smallest priced errors; 64 threads share a price, a layer each and up to four times (side by side:
@@ -421,7 +424,9 @@ __device__ __noinline__ bool window_search(const WindowArgs& a, float* total) {
 
     // ---- 3. the recursion inside windows of W cells, over the candidates that cost at most `cost` at the higher middle price.  A
     // path that takes the relaxed choice at that price costs x_hi (C - above_all); the best one is nearly always far below.
-    uint32_t W = below_all - above_all <= (int)kWindowJump ? 64u : kWindowMost;
+    // (Many layers wander further from the line: 1995 blocks take 437 us where 64 cells are enough and 580 to 620 where they are not, which is
+    // the rule there, and 480 with 128 cells at once.)
+    uint32_t W = below_all - above_all <= (int)kWindowJump ? (ONE ? 64u : 128u) : kWindowMost;
     float most = 0.f;
     for (uint32_t i = 0; i < kPrices; ++i) most = fmaxf(most, sc.all[i] + sc.price[i] * (float)C);
     if (!(most < 1e37f)) return false;
