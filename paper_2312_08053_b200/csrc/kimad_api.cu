@@ -48,6 +48,8 @@ struct kimad_ctx {
     std::vector<unsigned char> static_image;                  // the static tables as they lie in the workspace, one block
     std::vector<size_t> guards;                               // checked build: offsets of the canary words between regions
     uint32_t most_chunks = 0; // of a layer
+    uint64_t most_elems = 0;
+    uint32_t sample_ctas = 1; // that read a layer's sample together (prepare_device)
     bool odd = false;         // workers may start at different distances from a 128-bit boundary
     uint32_t curve_mode = 0;
     uint32_t policy = 0, cost_model = 0;
@@ -285,10 +287,30 @@ static bool plan_choice(kimad_ctx* c) {
     return 8 * (size_t)c->L <= p.work_bytes;
 }
 
+// Clusters of n CTAs of the sample kernel that the current device holds at once.
+static cudaError_t sample_clusters(uint32_t n, size_t smem, uint32_t* resident) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(1, 1, n);
+    cfg.blockDim = kBigThreads;
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 1;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = n;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int m = 0;
+    const cudaError_t e = cudaOccupancyMaxActiveClusters(&m, k_sample, &cfg);
+    *resident = (uint32_t)std::max(m, 0);
+    return e;
+}
+
 // Once per device and process: shared-memory limits of the kernels (a property of the function, shared by all
-// contexts: the limits do not depend on the context) and the kernel preload.  Per context: its side stream.
+// contexts: the limits do not depend on the context), the sample kernel's clusters and the kernel preload.  Per context: its side stream.
 static int prepare_device(kimad_ctx* c) {
     static bool ready[KIMAD_BUILTIN_MAX_DEVICES] = {};
+    static uint32_t resident[KIMAD_BUILTIN_MAX_DEVICES][4] = {}; // clusters of 1, 2, 4, 8
     int dev = -1;
     CUDA_TRY(cudaGetDevice(&dev));
     if (dev < 0 || dev >= KIMAD_BUILTIN_MAX_DEVICES) return KIMAD_ERR_INVALID_ARG;
@@ -301,9 +323,11 @@ static int prepare_device(kimad_ctx* c) {
         CUDA_TRY(cudaFuncSetAttribute(k_pass_a<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->pass_a_smem));
         CUDA_TRY(cudaFuncSetAttribute(k_pass_a<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->pass_a_smem));
         CUDA_TRY(cudaFuncSetAttribute(k_tiny_exact, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->tiny_smem));
+        for (uint32_t i = 0; i < 4; ++i) CUDA_TRY(sample_clusters(1u << i, c->sample_smem, &resident[dev][i]));
         { const int rc_pre = preload_kernels(); if (rc_pre != KIMAD_OK) return rc_pre; }
         ready[dev] = true;
     }
+    c->sample_ctas = sample_cluster(c->most_elems, (uint64_t)c->W * c->reg_layers.size(), resident[dev]);
     return ensure_side_stream(c);
 }
 
@@ -397,7 +421,7 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
     if (T) CUDA_TRY(cudaEventRecord(c->ev_fork, s)); // fork point of the tiny layers' kernel: the step's start
     // (a) + (b): sample -> bands, all workers
     if (R) {
-        const uint32_t cz = sample_cluster((uint64_t)R * W);
+        const uint32_t cz = c->sample_ctas;
         CUDA_TRY(launch_clusters("k_sample", cz, k_sample, dim3(R, W, cz), kBigThreads, c->sample_smem, s, grads, state, c->stride, layers, reg_layers, R,
                                  ktab, K, c->curve_mode == 1 ? 1u : 0u, cell_tab, cell_win, binlo, meta));
         c->launches += 1;
@@ -644,6 +668,7 @@ int kimad_create(kimad_ctx** out, const uint64_t* layer_sizes, uint32_t n_layers
             ld.n_chunks = (uint32_t)c->chunks.size() - ld.first_chunk;
             c->layers.push_back(ld);
             c->most_chunks = std::max(c->most_chunks, ld.n_chunks);
+            c->most_elems = std::max(c->most_elems, n);
             if (n <= (uint64_t)kTinyMax) {
                 c->reg_index.push_back(0xffffffffu);
                 c->tiny_layers.push_back(l);

@@ -113,6 +113,33 @@ inline double candidate_cost(uint64_t n, uint64_t k, uint32_t bpe, uint32_t cost
     return dense ? -x : x;
 }
 
+// ---- The sample of a layer (k_sample) is read in units of consecutive elements, a warp each.  Half of the layer is enough: drawn without
+// replacement its ranks are as certain as those of kSampleUnits units of a large layer.  Up to kWholeUnits the layer is taken whole
+// (exact ranks, bands of one cell).
+constexpr int kSampleUnit = 32;    // elements (128 bytes)
+constexpr int kSampleUnits = 2047; // of a sample at most (65504 elements: the u16 cell counters cannot overflow)
+constexpr int kWholeUnits = 1024;
+constexpr uint32_t kSampleRound = 256; // units that a CTA has in flight together
+KIMAD_HD uint32_t sample_units(uint32_t units) {
+    const uint32_t half = units / 2u > (uint32_t)kWholeUnits ? units / 2u : (uint32_t)kWholeUnits;
+    return units <= (uint32_t)kWholeUnits ? units : (half < (uint32_t)kSampleUnits ? half : (uint32_t)kSampleUnits);
+}
+
+// CTAs that read a layer's sample together: `layers` of them (over all workers), the largest with `most` elements; resident[i]: clusters of
+// 2^i CTAs that the GPU holds at once (148, 74, 33 and 15 on a B200).  A second wave of clusters costs more than they save (16 layers of
+// 1 M elements: 37.4 us with one CTA each, 29.4 with four, 37.6 with eight), and so does every CTA of a cluster beyond the rounds of the largest
+// layer, for clearing its counters and meeting the others (stage in us with 1 / 2 / 4 / 8 CTAs, eight layers of 8 K elements:
+// 18.2 / 20.3 / 21.4 / 21.1, 16 K: 19.7 / 23.3 / 23.5 / 23.6, 32 K: 24.6 / 25.7 / 23.3 / 24.5, 70 K: 27.4 / 25.6 / 23.8 / 25.6,
+// 110 K: 31.8 / 27.7 / 25.2 / 25.5, 1 M: 36.0 / 31.5 / 27.9 / 25.7).
+constexpr uint32_t kSampleClusterMost = 8;
+KIMAD_HD uint32_t sample_cluster(uint64_t most, uint64_t layers, const uint32_t* resident) {
+    const uint32_t units = sample_units((uint32_t)((most + kSampleUnit - 1) / kSampleUnit)), rounds = (units + kSampleRound - 1) / kSampleRound;
+    if (rounds >= 7u && layers <= resident[3]) return 8u;
+    if (rounds >= 4u && layers <= resident[2]) return 4u;
+    if (rounds >= 5u && layers <= resident[1]) return 2u;
+    return 1u;
+}
+
 // ---- Planning of the sweep's bins from the sample (k_sample).  A fine bin is 2^shift keys wide, between kMinShift and a cell.
 constexpr uint32_t kMinShift = 5, kCellShift = 15;
 constexpr float kMostBins = 1024.f; // ... and a cell is cut into at most that many

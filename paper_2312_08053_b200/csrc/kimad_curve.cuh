@@ -39,16 +39,8 @@ constexpr int kBaseWords = kMaxGaps + 2;            // first bin of every gap an
 constexpr int kMaxBins = kFineBins + kL1Bins + 2 * kMaxGaps; // fine bins + gap regions cut at every 11-bit prefix
 static_assert(kBaseWords > KIMAD_MAX_RATIOS + 1 + 2, "a group of bands per candidate and one above them");
 constexpr int kMaxShift = 15;                       // a fine bin is 2^shift keys wide, at most a whole cell
-constexpr int kSampleUnit = 32;                     // consecutive elements read together (128 bytes, one warp)
-constexpr int kSampleUnits = 2047;                  // units of a sample (<= 65504 elements: the u16 cell counters cannot overflow)
-constexpr int kWholeUnits = 1024;                   // layers of up to as many units are taken whole
 constexpr int kBigThreads = 1024;
-constexpr uint32_t kSampleClusterMost = 8, kSampleClusterCtas = 128;
-KIMAD_HD uint32_t sample_cluster(uint64_t ctas) {
-    uint32_t c = kSampleClusterMost;
-    while (c > 1u && ctas * c > kSampleClusterCtas) c >>= 1;
-    return c;
-}
+static_assert(kSampleRound == 8 * (kBigThreads / kSampleUnit), "eight units per warp and round");
 constexpr uint32_t kGapBit = 1u;                    // bin_lo entries carry this bit when the bin is a gap bin
 
 
@@ -81,9 +73,9 @@ __device__ __forceinline__ uint32_t cluster_word(uint32_t addr, uint32_t rank) {
 
 // ------------------------------------------------------------------------------------------------
 // k_sample: one CTA per (regular layer, worker), or a cluster of up to kSampleClusterMost that read the layer's sample together.  A CTA's
-// 64 units per warp take 20 us of its 35 at the latency of DRAM, whatever the other SMs do: where the clusters of all layers are resident
-// at once (kSampleClusterCtas; a CTA fills an SM but for a CTA of the tiny layers' kernel), the others count their part of the units and the
-// first one adds the cells that hold anything to its own.
+// 64 units per warp take 20 us of its 35 at the latency of DRAM, whatever the other SMs do: where the layers are large enough and the
+// clusters of all of them resident at once (sample_cluster; a CTA fills an SM but for a CTA of the tiny layers' kernel), the others count
+// their part of the units and the first one adds the cells that hold anything to its own.
 // ------------------------------------------------------------------------------------------------
 // (48 registers: a CTA of the tiny layers' kernel, which runs beside this one, then fits on the same SM)
 __global__ void __maxnreg__(48)
@@ -127,17 +119,14 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
     const float* gr = grads + (size_t)w * stride + ld.begin;
     const float* st = state + (size_t)w * stride + ld.begin;
     const uint32_t n_units = n / kSampleUnit + ((n % kSampleUnit) != 0); // n may be as large as 2^32 - 1
-    // Half of the layer is enough of a sample: drawn without replacement its ranks are as certain as those of kSampleUnits units
-    // of a large layer.  Up to kWholeUnits the layer is taken whole (exact ranks, bands of one cell).
-    const uint32_t m_units = n_units <= (uint32_t)kWholeUnits ? n_units : min(max(n_units / 2u, (uint32_t)kWholeUnits), (uint32_t)kSampleUnits);
+    const uint32_t m_units = sample_units(n_units);
     const bool whole = m_units == n_units;
     const uint32_t sq_ = n / m_units, sr_ = n % m_units; // used when sampled
     const uint32_t m = whole ? n : kSampleUnit * m_units; // sample size (a stratum is no shorter than a unit), exact zeros included
     uint32_t top_key = 0;                                  // largest finite key
     // a warp reads one unit (128 bytes); eight units per thread are in flight before their keys are counted (this phase runs at
     // the DRAM's random-access rate on large layers; four and four, counted alternately, took a fifth longer)
-    constexpr uint32_t kRound = 8 * (kBigThreads / kSampleUnit); // units of a round
-    for (uint32_t ib = rank * kRound + threadIdx.x / kSampleUnit; ib < m_units; ib += ranks * kRound) {
+    for (uint32_t ib = rank * kSampleRound + threadIdx.x / kSampleUnit; ib < m_units; ib += ranks * kSampleRound) {
         float a[8], b[8];
         bool ok[8];
         // where the round's eight units start is the same for all lanes: lane u (mod 8) works out unit u's start

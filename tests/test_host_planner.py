@@ -17,6 +17,7 @@ extern "C" int coarsen(const uint32_t* bot, const uint32_t* top, uint32_t* shift
     for (uint32_t g = 0; g < n; ++g) fine += (top[g] - bot[g] + 1) << (kimad::kCellShift - shift[g]);
     return kimad::coarsen_groups(kimad::OneLane{}, bot, top, shift, need, n, fine, most, left);
 }
+extern "C" uint32_t cluster_of(uint64_t most, uint64_t layers, const uint32_t* resident) { return kimad::sample_cluster(most, layers, resident); }
 '''
 
 
@@ -73,3 +74,21 @@ def test_coarsening_ends(planner):
                 g = min((v * 2 ** x, g) for g, (v, x) in enumerate(zip(f32(*need), one)) if x < 15)[1]
                 one[g] += 1
             assert one == list(s)
+
+
+@pytest.mark.parametrize("resident", [(148, 74, 33, 15), (148, 74, 32, 12), (100, 44, 20, 0), (1, 0, 0, 0)])
+def test_clusters_are_resident_and_have_work(planner, resident):
+    """A layer's sample is read by a cluster only where all clusters run at once and none of their CTAs is without units."""
+    r = (ctypes.c_uint32 * 4)(*resident)
+    seen = set()
+    for most in (4097, 5000, 8192, 16384, 16385, 24577, 32768, 40000, 65536, 70000, 98304, 110000, 131072, 10 ** 6, 2 ** 32 - 1):
+        units = -(-most // 32)
+        units = units if units <= 1024 else min(max(units // 2, 1024), 2047)
+        for layers in (1, 2, 12, 13, 15, 16, 20, 21, 32, 33, 34, 44, 64, 65, 74, 75, 128, 149, 2000):
+            n = planner.cluster_of(ctypes.c_uint64(most), ctypes.c_uint64(layers), r)
+            seen.add(n)
+            assert n in (1, 2, 4, 8)
+            if n > 1:
+                assert layers <= resident[n.bit_length() - 1]
+                assert n * 256 < units + 2 * 256  # at most one CTA of a cluster idles
+    assert seen == {1 << i for i in range(4) if resident[i]}
