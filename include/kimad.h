@@ -300,6 +300,15 @@ int kimad_debug_stage_times(kimad_ctx* ctx, float* host_ms);
  * always run as one group. */
 int kimad_debug_set_schedule(kimad_ctx* ctx, int mode);
 
+/* How the knapsack is searched where there are enough layers for windows of its rows (their results do not differ).  mode 0
+ * (default): the windows and whole rows at the same time, and the first to have the answer gives it; 1: windows, then whole rows for the
+ * workers that these left undecided; 2: whole rows.  For tests and measurements.  Errors: INVALID_ARG. */
+int kimad_debug_set_search(kimad_ctx* ctx, int mode);
+/* Searches over windows since the workspace was attached, one per worker and step.  host_count: host, u64 [3]: those that did not decide
+ * (errors that are negative, infinite or all zero among them), that did with their first windows, with their second ones.  Under mode 0 a
+ * search that the whole rows made superfluous is in none of them.  Synchronises the device. */
+int kimad_debug_searches(kimad_ctx* ctx, uint64_t* host_count);
+
 /* Limit, in SM clocks, of the waits inside the knapsack kernel (its warps wait for one another; default and maximum 2^31,
  * about a second).  A lower limit also keeps the search to whole rows, which are what its warps hand on to one another.  For
  * tests: a wait that runs out makes the worker's result KIMAD_ERR_TIMEOUT, with nothing selected and the estimator

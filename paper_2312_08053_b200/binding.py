@@ -109,6 +109,10 @@ def load():
     L.kimad_debug_stage_times.argtypes = [vp, vp]
     L.kimad_debug_set_schedule.restype = C.c_int
     L.kimad_debug_set_schedule.argtypes = [vp, C.c_int]
+    L.kimad_debug_set_search.restype = C.c_int
+    L.kimad_debug_set_search.argtypes = [vp, C.c_int]
+    L.kimad_debug_searches.restype = C.c_int
+    L.kimad_debug_searches.argtypes = [vp, C.POINTER(u64)]
     L.kimad_debug_set_wait_limit.restype = C.c_int
     L.kimad_debug_set_wait_limit.argtypes = [vp, u64]
     L.kimad_debug_trace_step.restype = C.c_int
@@ -328,6 +332,11 @@ def kimad_debug_set_schedule(ctx: Ctx, mode: int) -> None:
     _check(load().kimad_debug_set_schedule(ctx.handle, int(mode)), "kimad_debug_set_schedule")
 
 
+def kimad_debug_set_search(ctx: Ctx, mode: int) -> None:
+    """0: windows of the knapsack's rows and whole rows at the same time, 1: one after the other, 2: whole rows (see kimad.h)."""
+    _check(load().kimad_debug_set_search(ctx.handle, int(mode)), "kimad_debug_set_search")
+
+
 def kimad_debug_set_wait_limit(ctx: Ctx, clocks: int) -> None:
     """Limit of the knapsack kernel's waits in SM clocks (see kimad.h); 2^31 by default."""
     _check(load().kimad_debug_set_wait_limit(ctx.handle, int(clocks)), "kimad_debug_set_wait_limit")
@@ -364,6 +373,13 @@ def kimad_debug_exact_path_layers(ctx: Ctx, detail: bool = False):
     n = (C.c_uint64 * (6 + ctx.K))()
     _check(load().kimad_debug_exact_path_layers(ctx.handle, n), "kimad_debug_exact_path_layers")
     return [int(x) for x in n] if detail else int(n[0])
+
+
+def kimad_debug_searches(ctx: Ctx) -> list:
+    """Searches over windows of the knapsack's rows so far: undecided, decided by their first windows, by their second ones."""
+    n = (C.c_uint64 * 3)()
+    _check(load().kimad_debug_searches(ctx.handle, n), "kimad_debug_searches")
+    return [int(x) for x in n]
 
 
 def kimad_debug_check(ctx: Ctx):

@@ -29,7 +29,7 @@ struct Layout {
     size_t zero_from, h1_cnt, h1_ss, h23_cnt, h23_ss, bh_cnt, bh_sum, in_n, fb, rc, flags;
     // scratch without initial-state requirements
     size_t cell_tab, cell_win, bin_lo, meta, cands, slots, err, tau, keep_eq, shift, sel, jobs, csel,
-        fb_chunks, rc_chunks, rf, rf_chunks, pd, rows, total;
+        fb_chunks, rc_chunks, rf, rf_chunks, pd, rows, windows, total;
 };
 
 } // namespace
@@ -57,9 +57,11 @@ struct kimad_ctx {
     Layout lay{};
     unsigned char* ws = nullptr;
     DpPlan dp_plan{};          // policy 0: the knapsack over the budget axis
-    uint32_t dp_cells = 0, dp_threads = 0; // most cells a row can have; threads of a CTA
+    uint32_t dp_cells = 0;     // most cells a row can have
     uint32_t hist_row = 0;     // words of a row of the knapsack kept for the backtracking ...
     bool rows_in_bins = false; // ... in the memory of the bin tables where those are large enough
+    bool windows_in_bins = false; // what the search over windows keeps in the workspace: behind the rows there
+    int search_mode = 0;          // kimad_debug_set_search
     PickPlan pick_plan{};      // the other policies, and given candidates
     size_t pick_smem = 0;
     uint32_t pd_stride = 0;    // policy 2: bytes of a row of back-pointers kept in the workspace (0: none are)
@@ -142,7 +144,14 @@ void plan_layout(kimad_ctx* c) {
     y.rf_chunks = take(kGroups * align_up((size_t)c->W * nch * sizeof(uint2)));
     y.pd = take((size_t)c->W * c->L * c->pd_stride);
     y.rows = take(c->policy == 0 && !c->rows_in_bins ? WL * c->hist_row * sizeof(float) + 16 : 0);
+    const size_t before = o;
+    y.windows = take(c->windows_in_bins ? 0 : (size_t)c->W * align_up(c->dp_plan.window_mem));
     y.total = o;
+    // Windows are no reason for a context to outgrow the built-in scratch.
+    if (y.total > KIMAD_BUILTIN_SCRATCH_BYTES && before <= KIMAD_BUILTIN_SCRATCH_BYTES) {
+        c->dp_plan.window = c->dp_plan.window_mem = 0;
+        plan_layout(c);
+    }
 }
 
 #define CUDA_TRY(x)                                  \
@@ -166,8 +175,9 @@ static int preload_kernels() {
 #define KIMAD_PRELOAD(f) CUDA_TRY(cudaFuncGetAttributes(&a, f))
     KIMAD_PRELOAD(k_sample); KIMAD_PRELOAD(k_pass_a<true>); KIMAD_PRELOAD(k_pass_a<false>); KIMAD_PRELOAD(k_resolve_a<true>); KIMAD_PRELOAD(k_resolve_a<false>);
     KIMAD_PRELOAD(k_refine); KIMAD_PRELOAD(k_tiny_exact); KIMAD_PRELOAD(k_fb1); KIMAD_PRELOAD(k_fb23<2>); KIMAD_PRELOAD(k_fb23<3>);
-    KIMAD_PRELOAD((k_dp<2, false>)); KIMAD_PRELOAD((k_dp<4, false>)); KIMAD_PRELOAD((k_dp<8, false>));
-    KIMAD_PRELOAD((k_dp<2, true>)); KIMAD_PRELOAD((k_dp<4, true>)); KIMAD_PRELOAD((k_dp<8, true>)); KIMAD_PRELOAD(k_pick); KIMAD_PRELOAD(k_fit_ratio); KIMAD_PRELOAD(k_sel_count);
+    KIMAD_PRELOAD((k_dp<2, kAlone>)); KIMAD_PRELOAD((k_dp<4, kAlone>)); KIMAD_PRELOAD((k_dp<8, kAlone>));
+    KIMAD_PRELOAD((k_dp<2, kWarpLooks>)); KIMAD_PRELOAD((k_dp<4, kWarpLooks>)); KIMAD_PRELOAD((k_dp<8, kWarpLooks>)); KIMAD_PRELOAD((k_dp<8, kFirstWarpLooks>));
+    KIMAD_PRELOAD(k_dp_windows<true>); KIMAD_PRELOAD(k_dp_windows<false>); KIMAD_PRELOAD(k_pick); KIMAD_PRELOAD(k_fit_ratio); KIMAD_PRELOAD(k_sel_count);
     KIMAD_PRELOAD((k_sel_offsets<128, true>)); KIMAD_PRELOAD((k_sel_offsets<128, false>)); KIMAD_PRELOAD((k_sel_offsets<512, false>)); KIMAD_PRELOAD(k_sel_recount);
     KIMAD_PRELOAD((k_sel_write<false, false>)); KIMAD_PRELOAD((k_sel_write<false, true>));
     KIMAD_PRELOAD((k_sel_write<true, false>)); KIMAD_PRELOAD((k_sel_write<true, true>));
@@ -240,7 +250,14 @@ static int ensure_side_stream(kimad_ctx* c) {
 // Cells of a row per thread of k_dp.  More cells per thread share the reads of a layer's record (a 1996-cell axis with 1995
 // layers: 2.57 ms with two, 1.87 with four, 1.94 with eight); with fewer, more warps overlap the latencies that bound short rows, and
 // with two all cells of a layer's candidates are requested together (707 cells, 148 layers: 69 us with two, 72 with four).
-static uint32_t dp_cells_per_thread(uint32_t cells) { return cells <= 1024 ? 2 : cells <= 2048 ? 4 : 8; }
+// Beside the search over windows there is a warp more, without cells, as far as there can be (rows_search); the form with two cells leaves
+// it one of its own.
+struct DpRows { uint32_t per, threads; };
+static DpRows dp_rows(uint32_t cells, bool beside) {
+    const uint32_t more = beside ? 32u : 0u;
+    const uint32_t per = cells <= 2 * (512 - more) ? 2 : (cells <= 2048 ? 4 : 8);
+    return DpRows{per, std::min<uint32_t>(kDpMaxThreads, std::max<uint32_t>(512, (((cells + per - 1) / per + 31) & ~31u) + more))};
+}
 
 // Shared-memory plans of the kernels that choose the candidates; false when the context's policy cannot be run.
 static bool plan_choice(kimad_ctx* c) {
@@ -264,8 +281,6 @@ static bool plan_choice(kimad_ctx* c) {
     // k_dp.  Every layer takes at least one cell, so a row has at most D - L + 1 cells.
     DpPlan& p = c->dp_plan;
     c->dp_cells = c->D - c->L + 1;
-    const uint32_t per = dp_cells_per_thread(c->dp_cells);
-    c->dp_threads = std::max<uint32_t>(512, ((c->dp_cells + per - 1) / per + 31) & ~31u);
     c->hist_row = (c->dp_cells + 3 + 4) & ~3u;
     c->rows_in_bins = c->reg_layers.size() * (size_t)(kMaxBins + 1) >= (size_t)c->L * c->hist_row + 4; // (rows start on a 16-byte boundary)
     p.kr = (c->K + 7) & ~7u;
@@ -280,6 +295,9 @@ static bool plan_choice(kimad_ctx* c) {
     const size_t fixed = sizeof(WindowScratch) + window_op_bytes(p.chunk_layers, p.kr) + sizeof(WindowOp) + 6 * (size_t)c->L + 32;
     const size_t want = tab + fixed + (one ? (size_t)c->L * (kWindowTables + kWindowMost) : kWindowPiece);
     const bool window = c->L >= window_layers(c->dp_cells) && want <= most;
+    p.window_mem = window ? (uint32_t)window_mem_bytes(c->L, p.rw, p.chunk_layers) : 0u;
+    const size_t bins = c->reg_layers.size() * (size_t)(kMaxBins + 1) * 4, rows = c->rows_in_bins ? (size_t)c->L * c->hist_row * 4 + 16 : 0;
+    c->windows_in_bins = bins >= rows + p.window_mem + 16;
     p.work_bytes = (uint32_t)std::min(most, (std::max<size_t>({tab + kDpMaxRing * slot, 96 * 1024, window ? want : 0}) + 15) & ~(size_t)15);
     p.window = window ? (uint32_t)(p.work_bytes - tab) : 0u;
     p.smem = (uint32_t)(p.work_bytes + tail + beyond);
@@ -316,8 +334,9 @@ static int prepare_device(kimad_ctx* c) {
     if (dev < 0 || dev >= KIMAD_BUILTIN_MAX_DEVICES) return KIMAD_ERR_INVALID_ARG;
     if (!ready[dev]) {
         auto dp_smem = [](auto kern) { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDpSmemMax); };
-        CUDA_TRY(dp_smem(k_dp<2, false>)); CUDA_TRY(dp_smem(k_dp<4, false>)); CUDA_TRY(dp_smem(k_dp<8, false>));
-        CUDA_TRY(dp_smem(k_dp<2, true>)); CUDA_TRY(dp_smem(k_dp<4, true>)); CUDA_TRY(dp_smem(k_dp<8, true>));
+        CUDA_TRY(dp_smem(k_dp<2, kAlone>)); CUDA_TRY(dp_smem(k_dp<4, kAlone>)); CUDA_TRY(dp_smem(k_dp<8, kAlone>));
+        CUDA_TRY(dp_smem(k_dp<2, kWarpLooks>)); CUDA_TRY(dp_smem(k_dp<4, kWarpLooks>)); CUDA_TRY(dp_smem(k_dp<8, kWarpLooks>)); CUDA_TRY(dp_smem(k_dp<8, kFirstWarpLooks>));
+        CUDA_TRY(dp_smem(k_dp_windows<true>)); CUDA_TRY(dp_smem(k_dp_windows<false>));
         CUDA_TRY(cudaFuncSetAttribute(k_pick, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDpSmemMax));
         CUDA_TRY(cudaFuncSetAttribute(k_sample, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->sample_smem));
         CUDA_TRY(cudaFuncSetAttribute(k_pass_a<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->pass_a_smem));
@@ -511,7 +530,7 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
                                     mode == kInjectErr ? err_dev : err, tau, keq, shf, flags, sel, out->k, out->j, out->offs,
                                     out->stats, out->dense, fb, when};
                 if (mode != kGivenJ && c->policy == 0) {
-                    const DpPlan& p = c->dp_plan;
+                    DpPlan p = c->dp_plan;
                     // A worker's candidate records lie where the exact path keeps its slots (for long grids its candidates): the
                     // DP only goes ahead when that path has nothing to do for the worker's group or is done.  The rows kept
                     // for the backtracking lie where the sample kernel left the bins' lower keys, which nobody reads after
@@ -521,13 +540,30 @@ int run_step(kimad_ctx* c, const float* grads, float* state, const double* bw, d
                     const size_t tab_stride = (in_slots ? L * sizeof(SlotTab) : (size_t)L * K * sizeof(Cand)) / 16 * 4;
                     float* rows = c->rows_in_bins ? reinterpret_cast<float*>(binlo) : c->at<float>(y.rows);
                     const size_t row_stride = c->rows_in_bins ? (size_t)R * (kMaxBins + 1) : (size_t)L * c->hist_row;
-                    auto launch = [&](auto kern) {
-                        return launch_named("k_dp", kern, nwa, c->dp_threads, p.smem, st, budgets_of(wa, nwa), wa, ca, p, c->at<double>(y.costs), tab, tab_stride,
-                                            rows, row_stride, c->hist_row);
+                    // What the search over windows keeps lies behind the rows where those are in the bins' memory.
+                    const size_t rows_bytes = c->rows_in_bins ? (size_t)L * c->hist_row * 4 + 16 : 0;
+                    unsigned char* windows = !p.window_mem ? nullptr : (c->windows_in_bins ? reinterpret_cast<unsigned char*>(binlo) + rows_bytes : c->at<unsigned char>(y.windows));
+                    const size_t window_stride = !p.window_mem ? 0 : (c->windows_in_bins ? (size_t)R * (kMaxBins + 1) * 4 : align_up(p.window_mem));
+                    const size_t window_room = c->windows_in_bins ? window_stride - rows_bytes : window_stride;
+                    // (a limit of the waits of its own asks for the recursion whose warps wait for each other)
+                    const bool race = p.window && p.wait_clocks == kDpWaitClocks && c->search_mode != 2;
+                    p.in_turn = c->search_mode == 1 ? 1u : 0u;
+                    if (race) {
+                        auto launch = [&](auto kern) {
+                            return launch_named("k_dp_windows", kern, nwa, kWindowThreads, p.smem, st, budgets_of(wa, nwa), wa, ca, p, c->at<double>(y.costs), windows, window_stride,
+                                                window_room);
+                        };
+                        CUDA_TRY(p.chunk_layers >= L ? launch(k_dp_windows<true>) : launch(k_dp_windows<false>));
+                        c->launches += 1;
+                    }
+                    auto launch = [&](auto kern, uint32_t threads) {
+                        return launch_named("k_dp", kern, nwa, threads, p.smem, st, budgets_of(wa, nwa), wa, ca, p, c->at<double>(y.costs), tab, tab_stride, rows,
+                                            row_stride, c->hist_row);
                     };
-                    const uint32_t per = dp_cells_per_thread(c->dp_cells);
-                    if (p.window) CUDA_TRY(per == 2 ? launch(k_dp<2, true>) : (per == 4 ? launch(k_dp<4, true>) : launch(k_dp<8, true>)));
-                    else CUDA_TRY(per == 2 ? launch(k_dp<2, false>) : (per == 4 ? launch(k_dp<4, false>) : launch(k_dp<8, false>)));
+                    const DpRows r = dp_rows(c->dp_cells, race);
+                    if (!race) CUDA_TRY(r.per == 2 ? launch(k_dp<2, kAlone>, r.threads) : (r.per == 4 ? launch(k_dp<4, kAlone>, r.threads) : launch(k_dp<8, kAlone>, r.threads)));
+                    else if (r.per < 8) CUDA_TRY(r.per == 2 ? launch(k_dp<2, kWarpLooks>, r.threads) : launch(k_dp<4, kWarpLooks>, r.threads));
+                    else CUDA_TRY((r.threads - 32) * 8 >= c->dp_cells ? launch(k_dp<8, kWarpLooks>, r.threads) : launch(k_dp<8, kFirstWarpLooks>, r.threads));
                 } else {
                     const int pick = mode == kGivenJ ? 1 : (c->policy == 1 ? 2 : (c->policy == 2 ? 3 : 4));
                     CUDA_TRY(launch_pdl(k_pick, nwa, kPickThreads, c->pick_smem, st, budgets_of(wa, nwa), wa, ca, pick, c->pick_plan, j_dev, pd));
@@ -837,6 +873,12 @@ int kimad_debug_set_wait_limit(kimad_ctx* c, uint64_t clocks) {
     return KIMAD_OK;
 }
 
+int kimad_debug_set_search(kimad_ctx* c, int mode) {
+    if (!c || mode < 0 || mode > 2) return KIMAD_ERR_INVALID_ARG;
+    c->search_mode = mode;
+    return KIMAD_OK;
+}
+
 int kimad_debug_stage_times(kimad_ctx* c, float* host_ms) {
     if (!c || !host_ms || !c->have_ev || !c->have_last) return KIMAD_ERR_INVALID_ARG;
     CUDA_TRY(cudaDeviceSynchronize());
@@ -999,6 +1041,19 @@ int kimad_debug_exact_path_layers(kimad_ctx* c, uint64_t* host_count) {
         for (int i = 0; i < 4; ++i) host_count[1 + i] += f.why[i];
         host_count[5] += f.refined;
         for (uint32_t j = 0; j < c->K; ++j) host_count[6 + j] += f.loose_j[j];
+    }
+    return KIMAD_OK;
+}
+
+int kimad_debug_searches(kimad_ctx* c, uint64_t* host_count) {
+    if (!c || !host_count) return KIMAD_ERR_INVALID_ARG;
+    if (!c->ws) return KIMAD_ERR_WORKSPACE;
+    CUDA_TRY(cudaDeviceSynchronize());
+    for (int i = 0; i < 3; ++i) host_count[i] = 0;
+    for (int g = 0; g < kGroups; ++g) {
+        FbList f{};
+        CUDA_TRY(cudaMemcpy(&f, c->ws + c->lay.fb + g * align_up(sizeof(FbList)), sizeof(FbList), cudaMemcpyDeviceToHost));
+        for (int i = 0; i < 3; ++i) host_count[i] += f.windows[i];
     }
     return KIMAD_OK;
 }

@@ -16,8 +16,12 @@
 //     exchanged rows go to the workspace, and the winning candidates -- the first that attains the minimum -- are found on
 //     the chosen path alone, last layer first, by repeating the one cell's sums.
 //
-// With many layers the few cells of every row that the chosen path can visit are worked out first (kimad_dp_window.cuh), and whole
-// rows are for what that does not decide.
+// With many layers a second kernel (k_dp_windows) looks at the few cells of every row that the chosen path can visit
+// (kimad_dp_window.cuh), at the same time: whole rows start as soon as the windows have, on another SM.  Both come to the same answer; the
+// first to have it gives it (a worker's flags), and the other one stops when it next looks there.  Windows are up to six times as fast where they
+// decide, but whether they will is known only at their end.  Where they do not, the whole rows now take 1 to 5 % longer than alone, and 4 us:
+// 148 layers, 16 candidates, D = 8191, errors of a few distinct values 516 us alone, 521 (one after the other: 569); 1000 such layers
+// 2780, 2865 (3480); 40 layers, 5 candidates, D = 2000 43, 46 (62).
 //
 // Whole rows: bound by instruction issue and shared-memory reads of one SM on wide axes (a record's uniform 128-bit reads cost about as
 // much as the cells they address), by the chain of latencies per exchange on short ones, and by the cold start of the
@@ -38,6 +42,8 @@ constexpr int kDpMaxThreads = 1024;
 constexpr int kDpMaxRing = 8;                  // rows in flight at most
 constexpr uint32_t kDpMaxChunkLayers = 256;    // layers whose records are staged at a time (two buffers)
 constexpr long long kDpWaitClocks = 1ll << 31; // limit of a wait unless set otherwise: about a second (an exchange takes about a microsecond)
+constexpr uint32_t kDpTimedOut = 1u, kDpStopped = 2u; // why a search over whole rows ends early: a wait ran out, the answer is there already
+constexpr uint32_t kDpMostLooks = 1u << 22; // of a thread that looks whether the answer is there: about a second
 constexpr uint32_t kDpSameBit = 0x10000u;      // head: all usable candidates of the layer take the same number of cells
 
 // Plan of a launch (host).  A layer has two records of rw = 2 kr + 4 words (kr = K rounded up to 8): {byte offsets of the
@@ -52,6 +58,8 @@ struct DpPlan {
     uint32_t work_bytes;
     uint32_t smem; // dynamic shared memory in all
     uint32_t window; // bytes of work_bytes behind the records for the search over windows (kimad_dp_window.cuh); 0: whole rows only
+    uint32_t window_mem; // ... and of the workspace, per worker
+    uint32_t in_turn;    // whole rows only after the windows
     long long wait_clocks; // limit of a wait
 };
 
@@ -73,16 +81,41 @@ __device__ __forceinline__ float min3(float a, float b, float c) { float m; asm(
 // with a fence before and after plain accesses the 1995 blocks took 1.87 instead of 1.76 ms.
 __device__ __forceinline__ void progress_set(uint32_t* counter, uint32_t x) { asm volatile("st.release.cta.shared.u32 [%0], %1;" ::"r"(smem_u32(counter)), "r"(x) : "memory"); }
 __device__ __forceinline__ int progress_get(uint32_t counter) { int x; asm volatile("ld.acquire.cta.shared.u32 %0, [%1];" : "=r"(x) : "r"(counter) : "memory"); return x; }
-__device__ __forceinline__ void progress_wait(const uint32_t* counter, int target, volatile uint32_t* failed, long long limit) {
+// A worker's flags: non-finite values were met; the search over windows runs, and what the kernels before it wrote can be read; one of the
+// searches has the answer; one of them is done (the other one clears the word for the next step).
+constexpr uint32_t kFlagNonfinite = 1u, kFlagReady = 2u, kFlagChosen = 4u, kFlagDone = 8u;
+// (acquire: what the one who set a flag has seen is seen; in a loop it would empty the SM's cache each time)
+__device__ __forceinline__ uint32_t flags_now(const uint32_t* flags) { uint32_t x; asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(x) : "l"(flags) : "memory"); return x; }
+__device__ __forceinline__ uint32_t flags_look(const uint32_t* flags) { uint32_t x; asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(x) : "l"(flags) : "memory"); return x; }
+
+// A look at a worker's flags that nobody waits for: the sixteen bytes they lie in are copied to shared memory now and then, and read
+// there.  (A load to a register makes its warp wait at the next branch: 10 to 35 % of the rows' time.)
+struct FlagsCopy {
+    const uint32_t* from;
+    uint32_t to, at; // in shared memory
+    __device__ __forceinline__ FlagsCopy(const uint32_t* flags, const uint32_t* copy /* [4], on a 16-byte boundary */)
+        : from(reinterpret_cast<const uint32_t*>(reinterpret_cast<uintptr_t>(flags) & ~(uintptr_t)15u)), to(smem_u32(copy)),
+          at(smem_u32(copy) + (uint32_t)(reinterpret_cast<uintptr_t>(flags) & 15u)) {}
+    __device__ __forceinline__ void ask() const { cp_async_16(to, from); }
+    __device__ __forceinline__ uint32_t chosen() const { uint32_t x; asm volatile("ld.volatile.shared.u32 %0, [%1];" : "=r"(x) : "r"(at) : "memory"); return x & kFlagChosen; }
+};
+
+// CAN_STOP: false when the warp has to wait and the search is over.  (The warps of a search that is timed out skip their waits.)
+template <bool CAN_STOP>
+__device__ __forceinline__ bool progress_wait(const uint32_t* counter, int target, volatile uint32_t* failed, long long limit) {
     const uint32_t at = smem_u32(counter);
     if (!__all_sync(0xffffffffu, progress_get(at) >= target)) {
         const long long start = clock64();
         while (!__all_sync(0xffffffffu, progress_get(at) >= target)) {
-            if (clock64() - start > limit) *failed = 1u;
-            if (__any_sync(0xffffffffu, *failed != 0u)) break;
+            if (clock64() - start > limit) *failed = kDpTimedOut;
+            if (__any_sync(0xffffffffu, *failed != 0u)) {
+                if (CAN_STOP) return false;
+                break;
+            }
         }
     }
     __syncwarp();
+    return true;
 }
 
 } // namespace kimad
@@ -108,7 +141,7 @@ struct ChooseArgs {
     uint64_t* out_offs;
     kimad_stats* out_stats;
     uint32_t* out_dense;       // may be null
-    const FbList* lists;
+    FbList* lists;
     uint32_t when; // 0: always; 1: only if no layer is listed for refinement or the exact path; 2: only if one is
 };
 
@@ -120,8 +153,9 @@ __device__ __forceinline__ bool choose_applies(const ChooseArgs& a) {
 
 // s_j[L]: the chosen candidates (read when status >= 0); s_k[L], s_e[L]: scratch.  `fitted`: the candidates come from the
 // ratio sized to the budget, feasibility is decided here.  The total error is added left to right in binary32, over the
-// layers in order, unless the caller already has that sum (`total`: the knapsack's own value of the chosen cell).
-template <typename J>
+// layers in order, unless the caller already has that sum (`total`: the knapsack's own value of the chosen cell).  CLEAR: the worker's
+// flags have served.
+template <bool CLEAR = true, typename J>
 __device__ __forceinline__ void choose_finish(const ChooseArgs& a, uint32_t w, uint64_t c, int status, bool fitted,
                                               const float* total, const J* s_j, uint32_t* s_k, float* s_e) {
     __shared__ unsigned long long s_nsel, s_used, s_part[kDpMaxThreads / 32];
@@ -183,7 +217,7 @@ __device__ __forceinline__ void choose_finish(const ChooseArgs& a, uint32_t w, u
         s.status = status;
         a.out_stats[w] = s;
         s_final = status;
-        a.flags[w] = 0; // consumed
+        if (CLEAR) a.flags[w] = 0;
     }
     __syncthreads();
     status = s_final;
@@ -228,62 +262,64 @@ __device__ __forceinline__ void choose_finish(const ChooseArgs& a, uint32_t w, u
 }
 
 // ------------------------------------------------------------------------------------------------
-// k_dp: one CTA per worker; a thread owns CPT cells of a row (32 apart: a warp owns 32 CPT consecutive cells)
+// The search over whole rows; a thread owns CPT cells of a row (32 apart: a warp owns 32 CPT consecutive cells).  Returns the
+// status, or kRowsStopped.  The chosen candidates are left in shared memory, the total in *total where there was a search.
 // ------------------------------------------------------------------------------------------------
-// (WINDOWS: contexts whose plan has them; apart, since the calls alone cost the others 4 us of 31)
-template <int CPT, bool WINDOWS>
-__global__ void __launch_bounds__(CPT <= 4 ? 512 : kDpMaxThreads, 1)
-k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double* __restrict__ cost /* [L][K], see kimad_common.h */,
-     uint32_t* __restrict__ tab_all /* [W] at tab_stride words, [L][2][rw] each */, size_t tab_stride,
-     float* __restrict__ hist_all /* [W] at hist_stride words, [exchanges][hist_row] each */, size_t hist_stride, uint32_t hist_row) {
-    pdl_wait();
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ uint32_t s_prog[32], s_failed, s_reach, s_cell, s_left, s_signed;
-    __shared__ unsigned long long s_sum;
-    __shared__ float s_redv[kDpMaxThreads / 32], s_total;
-    __shared__ uint32_t s_redb[kDpMaxThreads / 32];
+constexpr int kRowsStopped = 1 << 30;
+struct RowsArgs {
+    uint32_t L, K, D;
+    uint64_t c;            // budget in bytes
+    const double* cost;    // [L][K] and the worker's errors
+    const float* err;
+    uint32_t* tab;         // [L][2][rw]
+    float* hist;           // [exchanges][hist_row], on a 16-byte boundary
+    uint32_t hist_row;
+    const uint32_t* flags; // of the worker
+};
 
-    const uint32_t w = w_base + blockIdx.x;
-    if (!choose_applies(a)) return;
-    const uint32_t L = a.L, K = a.K, D = a.D, T = blockDim.x;
+// RACE: beside the search over windows, until that has the answer.
+enum Race { kAlone, kWarpLooks, kFirstWarpLooks }; // no other search; a warp without cells looks for its answer; all have cells, the first looks
+template <int CPT, Race RACE>
+__device__ __forceinline__ int rows_search(const RowsArgs& a, const DpPlan& plan, int status, float* total) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ uint32_t s_prog[32], s_failed, s_reach, s_cell, s_left, s_signed, s_rows;
+    __shared__ unsigned long long s_sum;
+    __shared__ float s_redv[kDpMaxThreads / 32];
+    __shared__ uint32_t s_redb[kDpMaxThreads / 32];
+    __shared__ __align__(16) uint32_t s_seen[4];
+    __shared__ const uint32_t* s_w_flags;
+
+    const uint32_t L = a.L, K = a.K, D = a.D, T = blockDim.x, hist_row = a.hist_row;
     const uint32_t t = threadIdx.x, lane = t & 31, wid = t >> 5;
-    const uint64_t c = budgets.c[blockIdx.x];
+    const uint64_t c = a.c;
+    const double* __restrict__ cost = a.cost;
+    const float* __restrict__ err = a.err;
     const float kInf = __int_as_float(0x7f800000);
-    const uint32_t kr = plan.kr, rw = plan.rw, rec16 = rw / 4u, CL = plan.chunk_layers;
+    const uint32_t kr = plan.kr, rw = plan.rw, rec16 = rw / 4u, CL = plan.chunk_layers, work_bytes = plan.work_bytes;
+    const long long wait_clocks = plan.wait_clocks;
     uint32_t* s_tab = reinterpret_cast<uint32_t*>(smem_raw);           // [2][CL * rw]
     float* ring = reinterpret_cast<float*>(s_tab + 2u * CL * rw);
-    float* s_p = reinterpret_cast<float*>(smem_raw + plan.work_bytes); // [L] smallest error, later the value before the layer
+    float* s_p = reinterpret_cast<float*>(smem_raw + work_bytes);      // [L] smallest error, later the value before the layer
     uint16_t* s_ex = reinterpret_cast<uint16_t*>(s_p + L);             // [L] layer of every exchange
     uint8_t* s_j = reinterpret_cast<uint8_t*>(s_ex + L);               // [L]
-    uint32_t* s_k = reinterpret_cast<uint32_t*>(smem_raw);             // [L], [L]: scratch of the end (work_bytes >= 8 L)
-    float* s_e = reinterpret_cast<float*>(s_k + L);
-    uint32_t* tab = tab_all + w * tab_stride;
-    float* hist = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(hist_all + w * hist_stride) + 15u) & ~(uintptr_t)15u);
-
-    // the records and the rows fit where they are put
-    if (t == 0) (void)KIMAD_CHECK((size_t)L * 2u * rw <= tab_stride && (size_t)L * hist_row + (hist - (hist_all + w * hist_stride)) <= hist_stride &&
-                                  D - L + 1u <= hist_row, 4);
-    int status = KIMAD_OK;
-    if (a.check_finite && (a.flags[w] & 1u)) status = KIMAD_ERR_NONFINITE;
-    else if (c >= a.full_bytes) status = KIMAD_STATUS_PLATEAU;
-    else if (c == 0) status = KIMAD_STATUS_INFEASIBLE;
+    uint32_t* tab = a.tab;
+    float* hist = a.hist;
     if (t == 0) { s_failed = 0; s_sum = 0; s_reach = 0; s_signed = 0; }
-    __syncthreads(); // (and the flags are read before the end of the choice resets them)
-
-    // ---- windows of the rows first.  (Where the limit of the waits is set, the recursion whose warps wait for each other is what is asked for.)
-    if (WINDOWS && status == KIMAD_OK && plan.wait_clocks == kDpWaitClocks) {
-        auto at = [&](const void* p) { return (uint32_t)(reinterpret_cast<const unsigned char*>(p) - smem_raw); };
-        const WindowArgs wa{L, K, D, kr, rw, c, cost, a.err + (size_t)w * L * K, CL, 8u * CL * rw, plan.window, tab,
-                            reinterpret_cast<unsigned char*>(hist), (hist_stride - (size_t)(hist - (hist_all + w * hist_stride))) * 4u, at(s_p), at(s_ex), at(s_j)};
-        float value;
-        if (CL >= L ? window_search<true>(wa, &value) : window_search<false>(wa, &value)) {
-            if (t == 0) s_total = value;
-            __syncthreads();
-            choose_finish(a, w, c, status, false, &s_total, s_j, s_k, s_e);
-            return;
+    if (RACE && t < 4u) s_seen[t] = 0;
+    if (RACE && t == 0) { s_rows = 0; s_w_flags = a.flags; }
+    const uint32_t* const volatile* w_flags = &s_w_flags; // (in shared memory: the recursion has no registers to spare)
+    volatile uint32_t* failed = &s_failed;
+    auto look_while = [&](auto busy) -> bool {
+        for (uint32_t n = 0; n < kDpMostLooks && busy(); ++n) {
+            if (flags_look(*w_flags) & kFlagChosen) {
+                *failed = kDpStopped;
+                return true;
+            }
+            __nanosleep(200);
         }
-        __syncthreads();
-    }
+        return false;
+    };
+    __syncthreads();
 
     // ---- the layers' records; 8, 16 or 32 lanes per layer, the loads of the next layers ahead of the current ones' work
     const uint32_t G = kr <= 8u ? 8u : (kr <= 16u ? 16u : 32u), per = 32u / G; // lanes per layer, layers per warp
@@ -301,7 +337,7 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
             float e_[AHEAD];
             auto fetch = [&](uint32_t l, uint32_t j, double& x, float& e) {
                 x = 0.0; e = 0.f;
-                if (l < L && j < K) { x = cost[(size_t)l * K + j]; e = a.err[((size_t)w * L + l) * K + j]; }
+                if (l < L && j < K) { x = cost[(size_t)l * K + j]; e = err[(size_t)l * K + j]; }
             };
 #pragma unroll
             for (int i = 0; i < AHEAD; ++i) fetch(l4 + i * stride + sub, jj, x_[i], e_[i]);
@@ -368,15 +404,14 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
     if (status != KIMAD_OK) { // nothing to search
         for (uint32_t l = t; l < L; l += T) s_j[l] = (uint8_t)(status == KIMAD_STATUS_PLATEAU ? K - 1 : 0u);
         __syncthreads();
-        choose_finish(a, w, c, status, false, nullptr, s_j, s_k, s_e);
-        return;
+        return status;
     }
     const uint32_t width = D - (uint32_t)least + 1u; // cells 0 .. width - 1 above the smallest total
     const uint32_t reach = s_reach;                  // cells that a candidate reads below its own at most
     // a row has +inf in front of it, for the cells below its start
     const uint32_t margin = (reach + 3u) & ~3u, slot_words = margin + ((width + 3u) & ~3u);
-    const uint32_t n_ring = min((uint32_t)kDpMaxRing, (plan.work_bytes - 8u * CL * rw) / (4u * slot_words)); // (at least 2)
-    if (t == 0) (void)KIMAD_CHECK(n_ring >= 2u && 8u * CL * rw + 4u * n_ring * slot_words <= plan.work_bytes, 4);
+    const uint32_t n_ring = min((uint32_t)kDpMaxRing, (work_bytes - 8u * CL * rw) / (4u * slot_words)); // (at least 2)
+    if (t == 0) (void)KIMAD_CHECK(n_ring >= 2u && 8u * CL * rw + 4u * n_ring * slot_words <= work_bytes, 4);
     for (uint32_t i = t; i < n_ring * margin; i += T) ring[(i / margin) * slot_words + i % margin] = kInf;
 
 
@@ -386,7 +421,6 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
     // Progress: a warp publishes s + 1 when its part of row s is written; it is then done with reading row s - 1.
     if (t < 32u) s_prog[t] = t < T / 32u && t * (32u * CPT) < width ? 0u : 0x7fffffffu; // no work: never holds anybody up
     uint32_t* prog = s_prog;
-    volatile uint32_t* failed = &s_failed;
     const uint32_t n_chunks = (L + CL - 1) / CL;
     auto stage_tab = [&](uint32_t ch) { // the first records of a chunk of layers
         const uint32_t l0 = ch * CL, n16 = min(CL, L - l0) * rec16;
@@ -401,11 +435,24 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
     stage_tab(0);
     uint32_t seq = 0, slot = 0; // exchanges so far; slot of the next one
     float* hist_at = hist + cell0;
+    // A thread of a warp without cells looks whether the other search has the answer, until the first warp is through with the chunk, and
+    // then holds up the others by the counter of a warp without cells: those that work never look.  (A look at shared memory by every
+    // warp and row took 3 to 5 % of the rows' time.)  Where all warps have cells the first one looks, every four
+    // rows where these are short (at every row: 10 %).
+    volatile uint32_t* rows_of = &s_rows;
     for (uint32_t ch = 0; ch < n_chunks; ++ch) {
         cp_async_wait();
-        __syncthreads(); // this chunk's records are there, nobody reads the other buffer any more
+        // this chunk's records are there, nobody reads the other buffer any more
+        if (RACE) {
+            if (__syncthreads_or(*failed == kDpStopped)) break; // (for all threads or none)
+        } else {
+            __syncthreads();
+        }
         if (ch + 1 < n_chunks) stage_tab(ch + 1);
-        if (!busy) continue;
+        if (!busy) {
+            if (RACE == kWarpLooks && t == T - 32u && look_while([&]() { return *rows_of <= ch; })) progress_set(prog + 31, 0x80000000u); // everybody has to wait
+            continue;
+        }
         const uint32_t* rec = s_tab + (ch & 1u) * CL * rw;
         const uint32_t l0 = ch * CL, nl = min(CL, L - l0);
         uint2 head = *reinterpret_cast<const uint2*>(rec + 2u * kr);
@@ -446,7 +493,15 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
                 }
             }
             // the warps below have written their part of this row; the others are done with the slot of the next one
-            progress_wait(prog + lane, lane < wid ? (int)seq + 1 : (lane == wid ? 0 : (int)seq + 3 - (int)n_ring), failed, plan.wait_clocks);
+            if (RACE == kFirstWarpLooks && wid == 0) { // asks at one row, looks at the next
+                const FlagsCopy copy(*w_flags, s_seen);
+                if ((kr > 16u || (seq & 3u) == 1u) && __any_sync(0xffffffffu, copy.chosen())) {
+                    *failed = kDpStopped;
+                    break;
+                }
+                if ((kr > 16u || (seq & 3u) == 0u) && lane == 0) copy.ask();
+            }
+            if (!progress_wait<RACE != kAlone>(prog + lane, lane < wid ? (int)seq + 1 : (lane == wid ? 0 : (int)seq + 3 - (int)n_ring), failed, wait_clocks)) break;
             const uint32_t addr = smem_u32(row + cell0);
             // a candidate's cells: no further below the row's start than its margin (the last warp's, past the row's end, stay in the CTA's memory)
             auto at = [&](uint32_t off) {
@@ -496,6 +551,7 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
             ++seq;
             if (++slot == n_ring) slot = 0;
         }
+        if (RACE && t == 0) *rows_of = ch + 1u;
     }
 
     // ---- lowest cell attaining the minimum: lexicographic (value, cell)
@@ -516,6 +572,7 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
     if (lane == 0) { s_redv[wid] = bv; s_redb[wid] = bb; }
     if (t == 0) s_left = seq; // (warp 0 owns the lowest cells: always busy)
     __syncthreads();          // the recursion is over for all warps, its rows are in the workspace
+    if (RACE && *failed == kDpStopped) return kRowsStopped;
     const uint32_t n_ex = s_left;
     bv = s_redv[0]; bb = s_redb[0];
     for (uint32_t i = 1; i < T / 32; ++i)
@@ -531,6 +588,7 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
         // the first candidate that attains the minimum, and the cell it came from.
         __syncthreads(); // everybody has read the number of exchanges
         if (t == 0) s_cell = bb;
+        const volatile uint32_t* walked = &s_left; // exchanges left: less once the first warp is through with the staged ones
         // Errors that the curve stage computes are not negative, and neither are their sums: they order as their bits do.
         const bool any_sign = s_signed != 0u;
         auto warp_min = [](float x, auto any) {
@@ -546,7 +604,7 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
         for (uint32_t left = n_ex; left;) {
             const uint32_t b0 = s_cell, lo = (b0 - min(b0, reach + 256u)) & ~3u;
             const uint32_t row16 = (b0 - lo) / 4u + 1u, per16 = rec16 + row16;
-            const uint32_t nx = min(left, plan.work_bytes / (16u * per16));
+            const uint32_t nx = min(left, work_bytes / (16u * per16));
             uint4* buf = reinterpret_cast<uint4*>(smem_raw);
             for (uint32_t i = wid; i < nx; i += T / 32) { // a warp per exchange
                 const uint4* r16 = reinterpret_cast<const uint4*>(tab + (size_t)s_ex[left - 1u - i] * 2u * rw + rw);
@@ -556,6 +614,8 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
             }
             cp_async_wait();
             __syncthreads();
+            // (while the first warp walks, which does not look: a test per exchange took 7 % of the search's time with 50 candidates)
+            if (RACE && t == 32u) (void)look_while([&]() { return *walked == left; });
             if (wid == 0) {
                 uint32_t b = b0, i = 0;
                 const uint32_t* rec = reinterpret_cast<const uint32_t*>(buf);
@@ -628,6 +688,7 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
                 if (lane == 0) { s_cell = b; s_left = left - i; }
             }
             __syncthreads();
+            if (RACE && *failed) return kRowsStopped;
             left = s_left;
         }
         // The layers in between: the value before each of them (a thread per run of such layers), then the first candidate
@@ -659,9 +720,118 @@ k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double
             s_j[l] = (uint8_t)j;
         }
     }
-    if (t == 0) s_total = bv;
+    *total = bv;
     __syncthreads();
-    choose_finish(a, w, c, status, false, status == KIMAD_OK ? &s_total : nullptr, s_j, s_k, s_e);
+    return status;
+}
+
+// ------------------------------------------------------------------------------------------------
+// k_dp, k_dp_windows: a CTA per worker
+// ------------------------------------------------------------------------------------------------
+__device__ __forceinline__ int choose_status(const ChooseArgs& a, uint64_t c, uint32_t flags) {
+    if (a.check_finite && (flags & kFlagNonfinite)) return KIMAD_ERR_NONFINITE;
+    return c >= a.full_bytes ? KIMAD_STATUS_PLATEAU : (c == 0 ? KIMAD_STATUS_INFEASIBLE : KIMAD_OK);
+}
+// Of two searches: gives the answer left in shared memory, unless the other one has given it.
+__device__ __forceinline__ void choose_first(const ChooseArgs& a, const DpPlan& plan, uint32_t w, uint64_t c, int status, float total) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ uint32_t s_flags;
+    __shared__ float s_total;
+    if (threadIdx.x == 0) {
+        s_flags = atomicOr(&a.flags[w], kFlagChosen);
+        s_total = total;
+    }
+    __syncthreads();
+    if (s_flags & kFlagChosen) return;
+    uint32_t* s_k = reinterpret_cast<uint32_t*>(smem_raw); // [L], [L]: scratch (work_bytes >= 8 L)
+    choose_finish<false>(a, w, c, status, false, status == KIMAD_OK ? &s_total : nullptr, smem_raw + plan.work_bytes + 6u * a.L, s_k, reinterpret_cast<float*>(s_k + a.L));
+}
+__device__ __forceinline__ void choose_done(const ChooseArgs& a, uint32_t w) { // (both searches get here, once)
+    if (threadIdx.x == 0 && (atomicOr(&a.flags[w], kFlagDone) & kFlagDone)) a.flags[w] = 0;
+}
+
+// RACE: beside k_dp_windows, which precedes it on the stream.
+template <int CPT, Race RACE>
+__global__ void __launch_bounds__(CPT == 2 ? 512 : (CPT == 4 ? (RACE ? 544 : 512) : kDpMaxThreads), 1)
+k_dp(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double* __restrict__ cost /* [L][K], see kimad_common.h */,
+     uint32_t* __restrict__ tab_all /* [W] at tab_stride words, [L][2][rw] each */, size_t tab_stride,
+     float* __restrict__ hist_all /* [W] at hist_stride words, [exchanges][hist_row] each */, size_t hist_stride, uint32_t hist_row) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ uint32_t s_flags;
+    __shared__ float s_total;
+    const uint32_t w = w_base + blockIdx.x, L = a.L, K = a.K, D = a.D, t = threadIdx.x;
+    const float* err = a.err + (size_t)w * L * K;
+    uint32_t flags = 0;
+    if (RACE) {
+        // Started while the windows' kernel runs, once that has started: it says when what the kernels before it wrote can be read (or it
+        // has ended, if it does not).  Its end is waited for at the end here: the kernels that follow wait for this one.
+        if (t == 0) s_flags = flags_now(a.flags + w);
+        __syncthreads();
+        if (plan.in_turn || !(s_flags & kFlagReady)) {
+            __syncthreads();
+            pdl_wait();
+            if (t == 0) s_flags = flags_now(a.flags + w);
+            __syncthreads();
+        } else {
+            pdl_launch();
+        }
+        flags = s_flags;
+        if (!choose_applies(a)) return;
+    } else {
+        pdl_wait();
+        if (!choose_applies(a)) return;
+        if (a.check_finite) flags = a.flags[w];
+    }
+    const uint64_t c = budgets.c[blockIdx.x];
+    const int known = choose_status(a, c, flags);
+    if (!RACE || !(flags & kFlagChosen)) {
+        float* hist = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(hist_all + w * hist_stride) + 15u) & ~(uintptr_t)15u);
+        // the records and the rows fit where they are put
+        if (t == 0) (void)KIMAD_CHECK((size_t)L * 2u * plan.rw <= tab_stride && (size_t)L * hist_row + (hist - (hist_all + w * hist_stride)) <= hist_stride &&
+                                      D - L + 1u <= hist_row, 4);
+        const RowsArgs ra{L, K, D, c, cost, err, tab_all + w * tab_stride, hist, hist_row, a.flags + w};
+        float value = 0.f;
+        const int status = rows_search<CPT, RACE>(ra, plan, known, &value); // (the flags are read before the end of the choice resets them)
+        if constexpr (RACE) {
+            if (status != kRowsStopped) choose_first(a, plan, w, c, status, value);
+        } else {
+            if (t == 0) s_total = value;
+            __syncthreads();
+            uint32_t* s_k = reinterpret_cast<uint32_t*>(smem_raw); // [L], [L]: scratch (work_bytes >= 8 L)
+            choose_finish(a, w, c, status, false, status == KIMAD_OK ? &s_total : nullptr, smem_raw + plan.work_bytes + 6u * L, s_k, reinterpret_cast<float*>(s_k + L));
+        }
+    }
+    if (RACE) {
+        choose_done(a, w);
+        pdl_wait();
+    }
+}
+
+// ONE: all layers' records are staged at once.
+template <bool ONE>
+__global__ void __launch_bounds__(kWindowThreads, 1)
+k_dp_windows(DpBudgets budgets, uint32_t w_base, ChooseArgs a, DpPlan plan, const double* __restrict__ cost,
+             unsigned char* __restrict__ mem_all /* [W] at mem_stride bytes, mem_room each */, size_t mem_stride, size_t mem_room) {
+    pdl_wait_only();
+    const uint32_t w = w_base + blockIdx.x, L = a.L, t = threadIdx.x;
+    if (!choose_applies(a)) return;
+    if (t == 0) { // (release: what this kernel waited for is there for those who see it)
+        asm volatile("red.release.gpu.global.or.b32 [%0], %1;" ::"l"(a.flags + w), "r"(kFlagReady) : "memory");
+        pdl_launch();
+    }
+    const uint64_t c = budgets.c[blockIdx.x];
+    const int status = choose_status(a, c, a.check_finite ? flags_now(a.flags + w) : 0u); // (the word is cleared when both searches are done)
+    if (status == KIMAD_OK) { // (else whole rows have nothing to search either)
+        unsigned char* mem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(mem_all + w * mem_stride) + 15u) & ~(uintptr_t)15u);
+        const uint32_t at_p = plan.work_bytes, at_x = at_p + 4u * L, at_j = at_x + 2u * L; // the tail of the shared memory
+        const WindowArgs wa{L, a.K, a.D, plan.kr, plan.rw, c, cost, a.err + (size_t)w * L * a.K, plan.chunk_layers, 8u * plan.chunk_layers * plan.rw, plan.window,
+                            mem, mem_all ? mem_room - (size_t)(mem - (mem_all + w * mem_stride)) : 0u, a.flags + w, at_p, at_x, at_j};
+        float value;
+        const uint32_t how = window_search<ONE>(wa, &value);
+        if (t == 0 && how != kWindowStopped) atomicAdd(&a.lists->windows[how], 1u);
+        if (how == kWindowFirst || how == kWindowSecond) choose_first(a, plan, w, c, KIMAD_OK, value);
+    }
+    choose_done(a, w);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -698,7 +868,7 @@ k_pick(DpBudgets budgets, uint32_t w_base, ChooseArgs a, int mode, PickPlan plan
     const KTab ktab = a.ktab;
 
     int status = KIMAD_OK;
-    if (a.check_finite && (a.flags[w] & 1u)) status = KIMAD_ERR_NONFINITE;
+    if (a.check_finite && (a.flags[w] & kFlagNonfinite)) status = KIMAD_ERR_NONFINITE;
     __syncthreads(); // the flags are read before the end of the choice resets them
     if (status == KIMAD_OK) {
         if (mode == 1) {

@@ -17,10 +17,12 @@
 //      256 cells: whole rows.
 //   5. The way back along one byte per cell of the window (the cell it came from), a piece of the layers per warp.
 //
-// Bound by chains of latencies: 170 cycles per four candidates of a layer in the recursion (row to shared memory, cells back, sums,
+// Bound by chains of latencies: about 130 cycles per four candidates of a layer in the recursion (row to shared memory, cells back, sums,
 // minimum), a few thousand for each of the steps around it, whose instructions are fetched anew in every step.  GPT-2 small's 148 layers
 // leave at most 35 cells of 852 open, 1995 blocks of it 33 of 1996, ResNet-50's 161 layers 127 of 835.  Against whole rows: 148 layers, 16
-// candidates 67 -> 58 us, 161 layers 71 -> 57, 201 layers 149 -> 69, 1995 blocks 1733 -> 545.
+// candidates 68 -> 46 us, 161 layers, 7 candidates 70 -> 52, 201 layers 150 -> 56, 1995 blocks 1732 -> 465 to 480, and 790 where the
+// bounds leave the first windows.  (A kernel of 512 threads of its own: inside the whole rows' kernel the search took 57 us on the 148 layers, and
+// spilled where that has 1024 threads.)
 #pragma once
 #include "kimad_kernels.cuh"
 
@@ -28,14 +30,15 @@ namespace kimad {
 
 constexpr uint32_t kWindowMost = 256;             // cells of a window at most (a byte names one of them)
 constexpr uint32_t kWindowPiece = 32 * 1024;      // shared memory for the steps back where not all of them fit
-// Windows are tried from so many layers on: against whole rows they take 30 us and 0.17 us per layer instead of 10 us and
-// 0.4 us (up to 1024 cells) or 0.85 us (more).  62 layers, 747 cells: 39 us instead of 31; 148 layers, 707 cells: 58 instead of 67.
+// Windows are tried from so many layers on.  They take about 20 us and 0.2 us per layer (16 candidates), whole rows 10 us and 0.5 us (up to 1024
+// cells, and 0.7 us where all of them are there) or 0.85 us and more.  62 layers of 747 cells: 39 us with windows, 31 with whole rows.
 KIMAD_HD uint32_t window_layers(uint32_t cells) { return cells <= 1024u ? 100u : 40u; }
 constexpr uint32_t kWindowJump = 100;             // cells between two neighbouring prices' choices up to which 64 cells are tried first
 constexpr uint32_t kPrices = 8, kSearchRounds = 20, kSearchPrices = 24;
 // Many layers: what the price of a sample of them may be off (bits of a binary32: an eighth to a sixth), after which two rounds over all
 // layers find it.  (Stopped at 3 % after one round, 12 us less, the first windows are too narrow or off more often.)
 constexpr uint32_t kThinSpread = 3u << 19;
+constexpr int kWindowThreads = 512;
 constexpr uint32_t kPriceThreads = 64;            // threads that share a price's layers
 constexpr uint32_t kBackWarps = 16;
 constexpr uint32_t kWindowChunk = kDpMaxChunkLayers;
@@ -83,8 +86,8 @@ constexpr uint32_t kWindowTables = 40; // bytes per layer: sums at the eight pri
 // candidate's cells}: of the usable candidates that take the same cells the smallest error; the last eight are filled up with entry 0.
 // Shared memory (offsets): records at 0, those of all layers or [2][chunk_layers]; mem: scratch | operations of a chunk (before them
 // what its records are made of) | word per layer | windows' ends [L + 1] | tables and steps back, where all records are there at once
-// (else these and the records, 2 rw words apart, are in the workspace, and pieces of the steps are staged here).
-// Workspace: [tables | steps back].
+// (else these are in the workspace, and pieces of the steps are staged here).
+// Workspace (window_mem_bytes): [records | tables | steps back], nothing where all records are staged at once.
 struct WindowArgs {
     uint32_t L, K, D, kr, rw;
     uint64_t c;            // budget in bytes
@@ -92,12 +95,19 @@ struct WindowArgs {
     const float* err;
     uint32_t chunk_layers;
     uint32_t mem, mem_bytes;
-    uint32_t* tab;
-    unsigned char* g_mem;
+    unsigned char* g_mem;  // on a 16-byte boundary
     size_t g_bytes;
+    const uint32_t* flags; // of the worker: kFlagChosen once the whole rows have the answer
     uint32_t p, x, j;      // offsets of: float [L] scratch; uint16_t [L] scratch; uint8_t [L] out: the chosen candidates
 };
 KIMAD_HD uint32_t window_op_bytes(uint32_t chunk_layers, uint32_t kr) { return chunk_layers * (kr / 4u) * (uint32_t)sizeof(WindowOp); }
+KIMAD_HD size_t window_table_bytes(uint32_t L, uint32_t rw) { return ((size_t)L * (rw * 4u + kWindowTables) + 15u) & ~(size_t)15u; }
+KIMAD_HD size_t window_mem_bytes(uint32_t L, uint32_t rw, uint32_t chunk_layers) {
+    return chunk_layers >= L ? 0u : window_table_bytes(L, rw) + (size_t)L * kWindowMost;
+}
+// What a search came to: nothing, the answer in the first or the second windows, or nothing since it was no longer needed.
+enum : uint32_t { kWindowNone = 0, kWindowFirst = 1, kWindowSecond = 2, kWindowStopped = 3 };
+constexpr uint32_t kWindowPoll = 64; // operations of the recursion between two looks at the worker's flags
 
 // Selections, written out: as conditional expressions they become branches, which cost the recursion's loop 130 cycles of 285 per operation.
 __device__ __forceinline__ void take_less(float v, float& least, float x, float& with) { // the smaller value and what came with it
@@ -122,25 +132,27 @@ __device__ __forceinline__ void window_sync(uint32_t warps) { // the warps that 
     if (warps == 1u) __syncwarp();
     else asm volatile("bar.sync 1, %0;" ::"r"(32u * warps) : "memory");
 }
+__device__ __forceinline__ bool window_any(uint32_t warps, uint32_t x) { // x != 0 in any of these warps' threads
+    if (warps == 1u) return __any_sync(0xffffffffu, x);
+    uint32_t r;
+    asm volatile("{.reg .pred p, q; setp.ne.u32 q, %1, 0; barrier.cta.red.or.pred p, 1, %2, q; selp.u32 %0, 1, 0, p;}" : "=r"(r) : "r"(x), "r"(32u * warps) : "memory");
+    return r != 0u;
+}
 
-// True: the candidates and *total are the knapsack's.  False: not found this way (nothing but scratch was written).  By the whole
-// CTA (512 threads or more).  ONE: the records of all layers are staged at once.
-// (Not inlined: its registers are its own.  Loops are not unrolled over candidates or layers: in a step, every instruction is fetched
-// anew.)
+// kWindowFirst, kWindowSecond: the candidates and *total are the knapsack's.  Else nothing but scratch was written.  By the whole
+// CTA (kWindowThreads).  ONE: the records of all layers are staged at once.  (Loops are not unrolled over candidates or layers: in a
+// step, every instruction is fetched anew.)
 template <bool ONE>
-__device__ __noinline__ bool window_search(const WindowArgs& a, float* total) {
+__device__ __forceinline__ uint32_t window_search(const WindowArgs& a, float* total) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ uint32_t s_top, s_bad, s_most, s_at;
+    __shared__ uint32_t s_top, s_bad, s_most, s_at, s_stop;
+    __shared__ __align__(16) uint32_t s_seen[4];
     __shared__ unsigned long long s_least;
     __shared__ float s_bestv[kWindowMost / 64];
     __shared__ uint32_t s_bestb[kWindowMost / 64];
     const uint32_t t = threadIdx.x, T = blockDim.x, lane = t & 31u, wid = t >> 5;
     const uint32_t L = a.L, K = a.K, D = a.D, kr = a.kr, rw = a.rw, rec16 = rw / 4u, CL = a.chunk_layers;
     const float kInf = __int_as_float(0x7f800000);
-    const size_t g_tables = ONE ? 0 : ((size_t)kWindowTables * L + 15u) & ~(size_t)15u;
-    // workspace for windows of W cells (rows shorter than a few hundred cells leave too little)
-    auto fits = [&](uint32_t W) { return ONE || g_tables + (size_t)L * W <= a.g_bytes; };
-    if (!fits(64u)) return false;
     WindowScratch& sc = *reinterpret_cast<WindowScratch*>(smem_raw + a.mem);
     float* s_p = reinterpret_cast<float*>(smem_raw + a.p);
     uint16_t* s_x = reinterpret_cast<uint16_t*>(smem_raw + a.x);
@@ -150,19 +162,22 @@ __device__ __noinline__ bool window_search(const WindowArgs& a, float* total) {
     WindowOp* ops = reinterpret_cast<WindowOp*>(smem_raw + at_ops);
     uint32_t* meta = reinterpret_cast<uint32_t*>(smem_raw + at_meta);
     int16_t* s_lo = reinterpret_cast<int16_t*>(smem_raw + at_lo); // lowest cell of the window before layer 0, after layer 0, ...
-    float* sums = ONE ? reinterpret_cast<float*>(smem_raw + at_tables) : reinterpret_cast<float*>(a.g_mem); // [L][kPrices]
-    int2* cells = reinterpret_cast<int2*>(sums + (size_t)L * kPrices);                                      // [L]
-    uint8_t* back = ONE ? smem_raw + at_back : a.g_mem + g_tables; // [exchanges][W]; in the workspace staged in units of 16 bytes
+    uint32_t* tab = reinterpret_cast<uint32_t*>(a.g_mem); // [L][rw]
+    float* sums = reinterpret_cast<float*>(ONE ? smem_raw + at_tables : a.g_mem + (size_t)L * rw * 4u); // [L][kPrices]
+    int2* cells = reinterpret_cast<int2*>(sums + (size_t)L * kPrices);                                  // [L]
+    uint8_t* back = ONE ? smem_raw + at_back : a.g_mem + window_table_bytes(L, rw); // [exchanges][W]; in the workspace staged in units of 16 bytes
     const uint32_t n_chunks = ONE ? 1u : (L + CL - 1u) / CL;
-    if (t == 0) (void)KIMAD_CHECK(at_back + (ONE ? L * kWindowMost : kWindowPiece) <= a.mem + a.mem_bytes && T >= kPrices * kPriceThreads && CL <= kWindowChunk, 4);
+    if (t == 0)
+        (void)KIMAD_CHECK(at_back + (ONE ? L * kWindowMost : kWindowPiece) <= a.mem + a.mem_bytes && T >= kPrices * kPriceThreads && CL <= kWindowChunk &&
+                          window_mem_bytes(L, rw, CL) <= a.g_bytes, 4);
     auto stage = [&](uint32_t buf, uint32_t first, uint32_t step, uint32_t n) { // records first, first + step, ...
         const uint32_t dst = smem_u32(smem_raw) + buf * CL * rw * 4u;
         for (uint32_t i = t; i < n * rec16; i += T) {
             const uint32_t r = i / rec16;
-            cp_async_16(dst + 16u * i, reinterpret_cast<const uint4*>(a.tab + (size_t)(first + r * step) * 2u * rw) + (i - r * rec16));
+            cp_async_16(dst + 16u * i, reinterpret_cast<const uint4*>(tab + (size_t)(first + r * step) * rw) + (i - r * rec16));
         }
     };
-    // f(records, first layer, layers) for the layers in order, chunk by chunk, by the whole CTA
+    // f(records, first layer, layers) for the layers in order, chunk by chunk, by the whole CTA (up to the chunk in which it is stopped)
     auto for_chunks = [&](auto f) {
         if (ONE) {
             f(reinterpret_cast<const uint32_t*>(smem_raw), 0u, L);
@@ -174,7 +189,9 @@ __device__ __noinline__ bool window_search(const WindowArgs& a, float* total) {
             __syncthreads(); // this chunk's records are there, nobody reads the other buffer any more
             if (ch + 1u < n_chunks) stage((ch + 1u) & 1u, (ch + 1u) * CL, 1, min(CL, L - (ch + 1u) * CL));
             f(reinterpret_cast<const uint32_t*>(smem_raw) + (ch & 1u) * CL * rw, ch * CL, min(CL, L - ch * CL));
+            if (s_stop) break;
         }
+        cp_async_wait(); // (the next chunk's, where it was stopped)
         __syncthreads();
     };
     // f(cells above the smallest candidate's, error) for a record's candidates, eight at a time (the last ones repeat candidate 0)
@@ -192,7 +209,9 @@ __device__ __noinline__ bool window_search(const WindowArgs& a, float* total) {
     // ---- 0. the records: cells and errors of a chunk's candidates, a thread each, then a thread per layer
     const CellsOf cells_of(a.c, D);
     auto error_of = [](double cost, float e) { return cost < 0.0 ? 0.f : e; }; // a layer sent densely (negative cost) loses nothing
-    if (t == 0) { s_top = 0; s_bad = 0; s_most = 0; s_least = 0ull; }
+    if (t == 0) { s_top = 0; s_bad = 0; s_most = 0; s_least = 0ull; s_stop = 0; }
+    if (t < 4u) s_seen[t] = 0;
+    const FlagsCopy copy(a.flags, s_seen);
     for (uint32_t i = t; i < kSearchRounds * kSearchPrices; i += T) (&sc.used[0][0])[i] = 0;
     float2* raw = reinterpret_cast<float2*>(ops); // [chunk_layers][K + 1]
     for (uint32_t ch = 0; ch < n_chunks; ++ch) {
@@ -252,14 +271,11 @@ __device__ __noinline__ bool window_search(const WindowArgs& a, float* total) {
         if (odd) s_bad = 1u;
         __syncthreads();
         if (!ONE) {
-            for (uint32_t i = t; i < nl * rec16; i += T) {
-                const uint32_t r = i / rec16;
-                reinterpret_cast<uint4*>(a.tab + (size_t)(l0 + r) * 2u * rw)[i - r * rec16] = reinterpret_cast<const uint4*>(recs)[i];
-            }
+            for (uint32_t i = t; i < nl * rec16; i += T) reinterpret_cast<uint4*>(tab + (size_t)l0 * rw)[i] = reinterpret_cast<const uint4*>(recs)[i];
             __syncthreads();
         }
     }
-    if (s_bad || s_top == 0u || s_least > D) return false; // (errors of any sign, infinite ones, no room: whole rows)
+    if (s_bad || s_top == 0u || s_least > D) return kWindowNone; // (errors of any sign, infinite ones, no room: whole rows)
     const uint32_t C = D - (uint32_t)s_least;              // cells of the row are 0 .. C
     __syncthreads();
     const uint32_t thin = ONE ? 1u : (L + CL - 1u) / CL, n_thin = (L + thin - 1u) / thin; // every thin-th layer
@@ -340,7 +356,7 @@ __device__ __noinline__ bool window_search(const WindowArgs& a, float* total) {
         __syncthreads(); // the staged records make room
     }
     rounds(ONE, C, 1u << 15);
-    if (hi >= 0x7f000000u) return false; // (twice the price is finite)
+    if (hi >= 0x7f000000u) return kWindowNone; // (twice the price is finite)
 
     // ---- 2. sums of the smallest priced errors; 64 threads share a price, a layer each and up to four times (side by side:
     // consecutive layers per thread lie on the same banks)
@@ -429,7 +445,7 @@ __device__ __noinline__ bool window_search(const WindowArgs& a, float* total) {
     uint32_t W = below_all - above_all <= (int)kWindowJump ? (ONE ? 64u : 128u) : kWindowMost;
     float most = 0.f;
     for (uint32_t i = 0; i < kPrices; ++i) most = fmaxf(most, sc.all[i] + sc.price[i] * (float)C);
-    if (!(most < 1e37f)) return false;
+    if (!(most < 1e37f)) return kWindowNone;
     const float binary32 = (float)(L + 16u) * 0x1p-24f; // relative error of a path's sum at most
     const float rounded = most * 0x1p-19f;              // of what is computed here from the sums: 32 roundings
     float cost = x_hi * (3.f + 0.4f * (float)max((int)C - above_all, 0)) + 2.f * binary32 * fmaxf(sc.all[4] - x_hi * (float)C, 0.f) + 4.f * rounded;
@@ -442,8 +458,7 @@ __device__ __noinline__ bool window_search(const WindowArgs& a, float* total) {
         }
         if (t == 0) s_lo[0] = (int16_t)(-(int)(W / 2u));
     };
-    auto recursion = [&]() -> bool { // false: the workspace has no room for the steps back
-        if (!fits(W)) return false;
+    auto recursion = [&]() -> bool { // false: stopped
         const uint32_t warps = W / 64u;
         for (uint32_t i = t; i < 6u * W; i += T) sc.rows[i] = kInf;
         float v0 = kInf, v1 = kInf;
@@ -564,40 +579,48 @@ __device__ __noinline__ bool window_search(const WindowArgs& a, float* total) {
                 int other = buf ? -3 * (int)W : 3 * (int)W; // from row to row
                 float p0 = v0, p1 = v1; // the row before the layer
                 int y0 = 0, y1 = 0;     // distances to the cells that the values come from
+                bool stop = false;
 #pragma unroll 1
-                for (uint32_t left = total & 0xffffu; left; --left) {
-                    const bool first = h.x != 0u;
-                    const float own0 = __uint_as_float(h.y), own1 = __uint_as_float(h.z);
-                    uint8_t* at = to + h.w * W;
-                    p0 = first ? __fadd_rn(__fadd_rn(v0, own0), own1) : p0;
-                    p1 = first ? __fadd_rn(__fadd_rn(v1, own0), own1) : p1;
-                    v0 = first ? kInf : v0;
-                    v1 = first ? kInf : v1;
-                    row[0] = p0;
-                    row[32] = p1;
-                    if (decltype(one_warp)::value) __syncwarp();
-                    else window_sync(warps);
-                    const float *r0 = row - d.x, *r1 = row - d.y, *r2 = row - d.z, *r3 = row - d.w;
-                    float a0 = r0[0], a1 = r1[0], a2 = r2[0], a3 = r3[0], b0 = r0[32], b1 = r1[32], b2 = r2[32], b3 = r3[32];
-                    const int4 dc = d;
-                    const float4 ec = e;
-                    op += 3; // (the last one read lies behind the operations, in the same memory)
-                    h = op[0];
-                    d = *reinterpret_cast<const int4*>(op + 1);
-                    e = *reinterpret_cast<const float4*>(op + 2);
-                    a0 = __fadd_rn(a0, ec.x); a1 = __fadd_rn(a1, ec.y); a2 = __fadd_rn(a2, ec.z); a3 = __fadd_rn(a3, ec.w);
-                    b0 = __fadd_rn(b0, ec.x); b1 = __fadd_rn(b1, ec.y); b2 = __fadd_rn(b2, ec.z); b3 = __fadd_rn(b3, ec.w);
-                    const float m0 = min3(min3(a0, a1, a2), a3, v0), m1 = min3(min3(b0, b1, b2), b3, v1);
-                    // the first candidate that attains the minimum (beside the chain of the values)
-                    y0 = pick_equal(v0, m0, y0, pick_equal(a0, m0, dc.x, pick_equal(a1, m0, dc.y, pick_equal(a2, m0, dc.z, dc.w))));
-                    y1 = pick_equal(v1, m1, y1, pick_equal(b0, m1, dc.x, pick_equal(b1, m1, dc.y, pick_equal(b2, m1, dc.z, dc.w))));
-                    v0 = m0;
-                    v1 = m1;
-                    at[0] = (uint8_t)(x0 - (uint32_t)y0);
-                    at[32] = (uint8_t)(x1 - (uint32_t)y1);
-                    row += other;
-                    other = -other;
+                for (uint32_t left = total & 0xffffu; left && !stop;) {
+                    const uint32_t until = left > kWindowPoll ? left - kWindowPoll : 0u;
+                    if (t == 0) copy.ask();
+#pragma unroll 1
+                    for (; left > until; --left) {
+                        const bool first = h.x != 0u;
+                        const float own0 = __uint_as_float(h.y), own1 = __uint_as_float(h.z);
+                        uint8_t* at = to + h.w * W;
+                        p0 = first ? __fadd_rn(__fadd_rn(v0, own0), own1) : p0;
+                        p1 = first ? __fadd_rn(__fadd_rn(v1, own0), own1) : p1;
+                        v0 = first ? kInf : v0;
+                        v1 = first ? kInf : v1;
+                        row[0] = p0;
+                        row[32] = p1;
+                        if (decltype(one_warp)::value) __syncwarp();
+                        else window_sync(warps);
+                        const float *r0 = row - d.x, *r1 = row - d.y, *r2 = row - d.z, *r3 = row - d.w;
+                        float a0 = r0[0], a1 = r1[0], a2 = r2[0], a3 = r3[0], b0 = r0[32], b1 = r1[32], b2 = r2[32], b3 = r3[32];
+                        const int4 dc = d;
+                        const float4 ec = e;
+                        op += 3; // (the last one read lies behind the operations, in the same memory)
+                        h = op[0];
+                        d = *reinterpret_cast<const int4*>(op + 1);
+                        e = *reinterpret_cast<const float4*>(op + 2);
+                        a0 = __fadd_rn(a0, ec.x); a1 = __fadd_rn(a1, ec.y); a2 = __fadd_rn(a2, ec.z); a3 = __fadd_rn(a3, ec.w);
+                        b0 = __fadd_rn(b0, ec.x); b1 = __fadd_rn(b1, ec.y); b2 = __fadd_rn(b2, ec.z); b3 = __fadd_rn(b3, ec.w);
+                        const float m0 = min3(min3(a0, a1, a2), a3, v0), m1 = min3(min3(b0, b1, b2), b3, v1);
+                        // the first candidate that attains the minimum (beside the chain of the values)
+                        y0 = pick_equal(v0, m0, y0, pick_equal(a0, m0, dc.x, pick_equal(a1, m0, dc.y, pick_equal(a2, m0, dc.z, dc.w))));
+                        y1 = pick_equal(v1, m1, y1, pick_equal(b0, m1, dc.x, pick_equal(b1, m1, dc.y, pick_equal(b2, m1, dc.z, dc.w))));
+                        v0 = m0;
+                        v1 = m1;
+                        at[0] = (uint8_t)(x0 - (uint32_t)y0);
+                        at[32] = (uint8_t)(x1 - (uint32_t)y1);
+                        row += other;
+                        other = -other;
+                    }
+                    stop = window_any(decltype(one_warp)::value ? 1u : warps, copy.chosen()); // (the same for all of these warps)
                 }
+                if (stop && t == 0) s_stop = 1u;
                 buf ^= total & 1u;
             };
             if (wid < warps) {
@@ -607,6 +630,7 @@ __device__ __noinline__ bool window_search(const WindowArgs& a, float* total) {
             n_ex += total >> 16;
             __syncthreads();
         });
+        if (s_stop) return false;
         // lowest cell attaining the minimum
         if (wid < warps) {
             const int end = (int)s_lo[L];
@@ -628,15 +652,16 @@ __device__ __noinline__ bool window_search(const WindowArgs& a, float* total) {
             if (s_bestv[i] < best) { best = s_bestv[i]; best_b = s_bestb[i]; } // (cells ascend with the warp)
         return true;
     };
+    uint32_t found = kWindowFirst;
     windows_on_line();
-    if (!recursion()) return false;
+    if (!recursion()) return kWindowStopped;
     if (!(best < kInf) && W < kWindowMost) {
         __syncthreads();
         W = kWindowMost;
         windows_on_line();
-        if (!recursion()) return false;
+        if (!recursion()) return kWindowStopped;
     }
-    if (!(best < kInf)) return false;
+    if (!(best < kInf)) return kWindowNone;
 
     // ---- 4. the bounds at a total of `best`
     const float limit = best + best * binary32 + rounded;
@@ -686,7 +711,7 @@ __device__ __noinline__ bool window_search(const WindowArgs& a, float* total) {
         widest = __reduce_max_sync(0xffffffffu, widest);
         if (lane == 0) atomicMax(&s_most, widest);
         __syncthreads();
-        if (s_most > kWindowMost) return false;
+        if (s_most > kWindowMost) return kWindowNone;
         W = s_most <= 64u ? 64u : (s_most <= 128u ? 128u : kWindowMost);
         for (uint32_t l = t; l < L; l += T) {
             const int c_lo = (int)(meta[l] & 0xffffu), c_hi = (int)(meta[l] >> 16);
@@ -695,7 +720,9 @@ __device__ __noinline__ bool window_search(const WindowArgs& a, float* total) {
         if (t == 0) s_lo[0] = (int16_t)(-(int)(W / 2u));
         cost = dear;
         __syncthreads();
-        if (!recursion() || !(best < kInf)) return false;
+        if (!recursion()) return kWindowStopped;
+        if (!(best < kInf)) return kWindowNone;
+        found = kWindowSecond;
     }
 
     // ---- 5. the way back over the exchanges.  Every warp takes a piece of them: first from all cells of its last window, then, once the
@@ -795,7 +822,7 @@ __device__ __noinline__ bool window_search(const WindowArgs& a, float* total) {
     }
     *total = best;
     __syncthreads();
-    return true;
+    return found;
 }
 
 } // namespace kimad

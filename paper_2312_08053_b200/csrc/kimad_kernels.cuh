@@ -46,9 +46,11 @@ __device__ __forceinline__ uint32_t key_of(float d) { return __float_as_uint(d) 
 // stream has finished (which hides their launch latency); they wait here, before touching anything it wrote.
 // A no-op for an ordinary launch.  From then on the next kernel in the stream may be scheduled as SMs come free: its CTAs
 // start and wait here in their turn, which takes most of a launch off every link of the chain.
+__device__ __forceinline__ void pdl_wait_only() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    pdl_wait_only();
+    pdl_launch();
 }
 
 // Aligned view of a chunk for 128-bit loads of the inputs (quads of elements) and of the code plane (sixteen
@@ -226,6 +228,7 @@ struct FbList { // layers handed to the exact radix path in this step, and their
     uint32_t rf_chunks;
     uint32_t rf_layers;
     uint32_t refined; // never reset: layers that took the refinement
+    uint32_t windows[3]; // never reset: searches over windows that did not decide, that did in the first windows, in the second
 };
 // A candidate of a refined layer: its threshold lies in the bin [klo, klo + 2^shift), which holds cb entries of which
 // the `drop` smallest are not kept; `below` = the squares of everything below the bin.  shift = kNoRefine: this
