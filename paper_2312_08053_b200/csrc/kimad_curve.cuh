@@ -108,8 +108,6 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
     }
     const LayerDesc ld = layers[l];
     const uint32_t n = (uint32_t)ld.n;
-    // the candidate of the thread's warp, asked for ahead of its use (the first one, where a warp takes several)
-    const uint64_t k_first = (threadIdx.x >> 5) < K ? ktab.at(w, (size_t)l * K + (threadIdx.x >> 5)) : 0ull;
     for (int i = threadIdx.x; i < 32768 / 4; i += kBigThreads) reinterpret_cast<uint4*>(h32)[i] = make_uint4(0u, 0u, 0u, 0u);
     if (threadIdx.x == 0) { s_flag = 0; s_ng = 0; s_cg = 0; s_z = 0; s_zz = 0ull; s_clip = 0; s_top = 0; s_fine = 0; }
     __syncthreads();
@@ -288,7 +286,7 @@ k_sample(const float* __restrict__ grads, const float* __restrict__ state, uint6
 
     // ---- bands: the cells that can hold the k_j-th largest key, and how finely to cut them (one warp per candidate)
     for (uint32_t j = threadIdx.x >> 5; j < K; j += kBigThreads / 32) {
-        const uint64_t k = j < kBigThreads / 32 ? k_first : ktab.at(w, (size_t)l * K + j);
+        const uint64_t k = ktab.at(w, (size_t)l * K + j);
         uint32_t o_cb = 1, o_ct = 0, o_cs = 15; // k == n keeps everything: no threshold, no band
         float o_nd = 1.f;                        // bins per cell it needs
         if (k < n) {
