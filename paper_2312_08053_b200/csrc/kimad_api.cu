@@ -731,22 +731,22 @@ int kimad_create(kimad_ctx** out, const uint64_t* layer_sizes, uint32_t n_layers
             const uint32_t gw = (c->W + 1) / 2; // workers in the larger group (1 for a single worker)
             const uint64_t waves = std::min<uint64_t>(4, std::max<uint64_t>(1, (N * gw + 148ull * kSweepRunElems - 1) / (148ull * kSweepRunElems)));
             const uint32_t per_w = std::max<uint32_t>(1u, std::min<uint32_t>(nch, (uint32_t)((waves * 148u + gw - 1) / gw)));
+            // elements and layers entered before a chunk, and what both cost; a run ends at the last chunk that it can pay for
+            std::vector<uint64_t> swept(nch + 1, 0), entered(nch + 1, 0), cost(nch + 1, 0);
+            auto regular = [&](uint32_t f) { return c->reg_index[c->chunks[f].layer] != 0xffffffffu; };
+            for (uint32_t f = 0; f < nch; ++f) {
+                const bool enters = regular(f) && (f == 0 || c->chunks[f].layer != c->chunks[f - 1].layer);
+                swept[f + 1] = swept[f] + c->chunks[f].end - c->chunks[f].begin;
+                entered[f + 1] = entered[f] + (enters ? kSweepLayerElems : 0);
+                cost[f + 1] = swept[f + 1] + entered[f + 1];
+            }
             // runs of a worker when none may cost more than `most`
             auto cut = [&](uint64_t most, std::vector<uint32_t>* starts) {
-                uint64_t cost = 0;
-                uint32_t n = 0, layer = 0;
-                for (uint32_t f = 0; f < nch; ++f) {
-                    const Chunk& ch = c->chunks[f];
-                    const uint64_t swept = ch.end - ch.begin, entry = c->reg_index[ch.layer] != 0xffffffffu ? kSweepLayerElems : 0;
-                    const uint64_t more = swept + (f && ch.layer == layer ? 0 : entry);
-                    if (f == 0 || cost + more > most) {
-                        cost = swept + entry;
-                        if (starts) starts->push_back(f);
-                        ++n;
-                    } else {
-                        cost += more;
-                    }
-                    layer = ch.layer;
+                uint32_t n = 0;
+                for (uint32_t f = 0; f < nch; ++n) {
+                    if (starts) starts->push_back(f);
+                    const uint64_t before = swept[f] + entered[f + 1] - (regular(f) ? kSweepLayerElems : 0); // (the first chunk's layer is entered in any case)
+                    f = std::max(f + 1, (uint32_t)(std::upper_bound(cost.begin() + f + 1, cost.end(), before + most) - cost.begin()) - 1);
                 }
                 return n;
             };
