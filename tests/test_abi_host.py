@@ -94,3 +94,15 @@ def test_schedule_modes_are_validated():
             kb.kimad_debug_set_schedule(ctx, mode)
         assert e.value.code == kb.KIMAD_ERR_INVALID_ARG
     kb.kimad_destroy(ctx)
+
+
+@pytest.mark.parametrize("L,D", [(500, 1000), (800, 2000)])
+def test_windows_do_not_outgrow_the_built_in_scratch(L, D):
+    """What the knapsack's search over windows keeps in the workspace is left out where a context would pass the built-in scratch with it only."""
+    record = 2 * 16 + 4  # words, 16 candidates
+    windows = -(-(-(-(L * (4 * record + 40)) // 16) * 16 + 256 * L) // 256) * 256  # per worker
+    sizes = [kb.kimad_workspace_bytes(kb.kimad_create([20] * L, W, list(np.geomspace(0.01, 1.0, 16)), D=D)) for W in range(1, 20)]
+    limit = 32 << 20
+    assert all(b - W * windows > limit for W, b in enumerate(sizes, 1) if b > limit)
+    without = [W for W in range(2, 20) if sizes[W - 1] <= limit and sizes[W - 1] - sizes[W - 2] < sizes[1] - sizes[0] - windows]
+    assert without and all(sizes[W - 1] + W * windows > limit for W in without)

@@ -35,8 +35,8 @@ def test_parity_selection_under_the_checked_build():
 
 
 def test_edges_and_slow_paths_under_the_checked_build():
-    """The knapsack's, the selection's and the planner's edges: where rows, lists and tables end."""
-    files = ["alignment", "knapsack", "planning", "repeated_values", "slow_paths", "write_groups"]
+    """The knapsack's, the selection's, the sample's and the planner's edges: where rows, windows, clusters, lists and tables end."""
+    files = ["alignment", "knapsack", "knapsack_windows", "planning", "repeated_values", "slow_paths", "small_contexts", "write_groups"]
     res = _run_checked([f"tests/test_gpu_{f}.py" for f in files], is_code=False)
     assert res.returncode == 0, res.stdout[-3000:] + res.stderr[-2000:]
     assert " passed" in res.stdout and "failed" not in res.stdout

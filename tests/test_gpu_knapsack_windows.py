@@ -71,13 +71,14 @@ def test_windows_decide_as_whole_rows(L, K, D, big):
 
 @pytest.mark.parametrize("L,K,D,big", [
     (148, 16, 148, 0), (148, 16, 149, 0), (148, 16, 1000, 40000),  # no spare cell, one, most of a thousand
+    (301, 17, 301, 0), (301, 127, 302, 0),                         # ... records in pieces
     (45, 8, 8191, 0), (100, 50, 8191, 3000),                       # 1024 threads; records in one piece and in pieces
     (400, 16, 1200, 0), (1995, 16, 3990, 0),                       # in pieces; the steps back as well
 ])
 @pytest.mark.parametrize("schedule", [0, 1])
 def test_every_way_of_searching(L, K, D, big, schedule):
     """Windows and whole rows at the same time, one after the other, and whole rows alone: the same choice.  One after the other, convex
-    curves are decided by windows (but for the widest axes) and errors of any sign by whole rows."""
+    curves are decided by windows (but for some on the widest axis) and errors of any sign by whole rows."""
     rng = np.random.default_rng(11 * L + D)
     sizes = [int(v) for v in np.exp(rng.uniform(0, np.log(200), L)).astype(int) + 1]
     sizes[L // 3] += big
@@ -101,8 +102,8 @@ def test_every_way_of_searching(L, K, D, big, schedule):
             none, first, second = (b - a for a, b in zip(before, kb.kimad_debug_searches(r.ctx)))
             if mode == 2:
                 assert none + first + second == 0
-            if mode == 1 and kind == "convex" and D < 8191:
-                assert first + second == (W if D - L > 1 else first + second) and none + first + second == W, (none, first, second)
+            if mode == 1 and kind == "convex":
+                assert none + first + second == W and (none == 0 or D == 8191), (none, first, second)
             if mode == 1 and kind in ("odd", "nothing"):
                 assert none == W and first + second == 0
         for other in got[1:]:

@@ -36,3 +36,31 @@ def test_tiny_layers_of_every_size_class(distinct):
     if distinct:  # ties: a few magnitudes of both signs, zeros among them
         x = np.round(x * distinct / 3).astype(np.float32)
     step(sizes, 2, x, 0.2, [0.01, 0.05, 0.1, 0.3, 0.7, 1.0])
+
+
+@pytest.mark.parametrize("R,W,n,ctas", [(2, 1, 1 << 20, 8), (5, 3, 114700, 8), (16, 1, 131072, 4), (11, 3, 40000, 4), (17, 2, 98310, 2), (60, 1, 70001, 2),
+                                        (15, 1, 16384, 1)])
+def test_a_cluster_counts_the_sample_that_one_CTA_counts(R, W, n, ctas):
+    """The bands planned from a sample that all CTAs of a cluster have read (sizes of a full round of units each) are those of the same layers
+    in a context of so many layers that one CTA reads each; without zeros, no layer is left to the exact path."""
+    sizes, more = [n + 3 * i for i in range(R)], [4097] * 160
+    grid = [0.01, 0.02, 0.05, 0.1, 0.2, 0.5, 1.0]
+    rounds = -(-min(max(n // 64, 1024), 2047, -(-n // 32)) // 256)
+    resident = {8: 15, 4: 33, 2: 74, 1: 148}[ctas]
+    assert R * W <= resident and ctas <= max(1, rounds + 1)  # (the size that the dispatch takes on a B200)
+    rng = np.random.default_rng(n)
+    x = (rng.standard_t(3, (W, sum(sizes))) * np.repeat(np.exp(rng.uniform(-4, 4, R)), sizes)).astype(np.float32)
+    rest = rng.standard_normal((W, sum(more))).astype(np.float32)
+    for zeros in (False, True):
+        if zeros:  # in a run: their spread over the units is counted as well
+            x[W - 1, : n // 2] = 0.0
+        metas = []
+        for layers, values in ((sizes, x), (sizes + more, np.concatenate([x, rest], axis=1))):
+            N = sum(layers)
+            ctx = kb.new_context(layers, W, grid)
+            state = torch.zeros((W, N), dtype=torch.float32, device="cuda")
+            kb.kimad_step(ctx, torch.from_numpy(np.ascontiguousarray(values)).cuda(), state, [0.1 * 4 * N] * W, 1.0, kb.Packed(ctx))
+            assert zeros or kb.kimad_debug_exact_path_layers(ctx) == 0
+            metas.append(kb.kimad_debug_get_band_meta(ctx, len(layers))[:, :R])
+        assert (metas[0][..., 0] > 0).any() and (zeros or (metas[0][..., 2] == 0).all())
+        assert np.array_equal(metas[0], metas[1])
