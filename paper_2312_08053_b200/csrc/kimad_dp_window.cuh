@@ -10,8 +10,9 @@
 //   1. The price at which the relaxed choice fills the axis: rounds of 8 to 24 prices at a time.
 //   2. Smallest priced errors summed up layer by layer (binary64) at eight prices around it, and the cells that the relaxed choice
 //      takes: two neighbouring prices, weighted so that the axis is filled.
-//   3. The recursion in windows of 64 cells around that line (128 with hundreds of layers, 256 where the two prices are far apart in cells), over the candidates
-//      that cost little at this price, one warp per 64 cells: a total U, nearly always the smallest one already.
+//   3. The recursion in windows of 64 cells around that line (128 where the records of all layers are not staged at once, 256 where the
+//      two prices are far apart in cells), over the candidates that cost little at this price, one warp per 64 cells: a total U, nearly
+//      always the smallest one already.
 //   4. Do the bounds at U rule out every cell outside the windows and every candidate left out?  Nearly always; else the
 //      recursion once more in windows around the cells they leave open (64, 128 or 256), with the candidates they leave.  More than
 //      256 cells: whole rows.
@@ -30,13 +31,16 @@ namespace kimad {
 
 constexpr uint32_t kWindowMost = 256;             // cells of a window at most (a byte names one of them)
 constexpr uint32_t kWindowPiece = 32 * 1024;      // shared memory for the steps back where not all of them fit
-// Windows are tried from so many layers on.  They take about 20 us and 0.2 us per layer (16 candidates), whole rows 10 us and 0.5 us (up to 1024
-// cells, and 0.7 us where all of them are there) or 0.85 us and more.  62 layers of 747 cells: 39 us with windows, 31 with whole rows.
+// Windows are tried from so many layers on.  They take about 20 us and 0.2 us per layer (16 candidates), whole rows 10 us and 0.4 to 0.7 us (up
+// to 1024 cells) or 0.85 us and more.  With fewer layers the cells of one candidate are many and windows seldom decide: ResNet-18's 62
+// layers, 7 candidates, 939 cells leave too much open in every step, and whole rows take 31 us alone, 38 beside windows; 40 to 64
+// layers on 2000 cells and more are decided on half of the curves tried, 2 to 5 times as fast.
 KIMAD_HD uint32_t window_layers(uint32_t cells) { return cells <= 1024u ? 100u : 40u; }
 constexpr uint32_t kWindowJump = 100;             // cells between two neighbouring prices' choices up to which 64 cells are tried first
 constexpr uint32_t kPrices = 8, kSearchRounds = 20, kSearchPrices = 24;
-// Many layers: what the price of a sample of them may be off (bits of a binary32: an eighth to a sixth), after which two rounds over all
-// layers find it.  (Stopped at 3 % after one round, 12 us less, the first windows are too narrow or off more often.)
+// Where the records are not staged at once, a sample of the layers tells the price first: what it may be off (bits of a binary32: 3/32 to 3/16
+// of the price), after which two rounds over all layers find it.  (Stopped at 3 % after one round, 12 us less, the first windows are too narrow
+// or off more often.)
 constexpr uint32_t kThinSpread = 3u << 19;
 constexpr int kWindowThreads = 512;
 constexpr uint32_t kPriceThreads = 64;            // threads that share a price's layers
@@ -285,7 +289,7 @@ __device__ __forceinline__ uint32_t window_search(const WindowArgs& a, float* to
     }
 
     // ---- 1. the price: bits of a binary32 number, cut into equal pieces (about equal ratios).  Above the largest error nothing
-    // but the smallest candidates is taken.  Many layers: every thin-th of them first.
+    // but the smallest candidates is taken.  Records that are not staged at once: those of every thin-th layer first.
     const uint32_t highest = s_top + 1u, lowest = highest > (40u << 23) ? highest - (40u << 23) : 1u;
     uint32_t lo = lowest, hi = highest, round = 0;
     bool lo_sure = ONE, hi_sure = ONE; // the answer is known to lie on this side
@@ -440,8 +444,8 @@ __device__ __forceinline__ uint32_t window_search(const WindowArgs& a, float* to
 
     // ---- 3. the recursion inside windows of W cells, over the candidates that cost at most `cost` at the higher middle price.  A
     // path that takes the relaxed choice at that price costs x_hi (C - above_all); the best one is nearly always far below.
-    // (Many layers wander further from the line: 1995 blocks take 437 us where 64 cells are enough and 580 to 620 where they are not, which is
-    // the rule there, and 480 with 128 cells at once.)
+    // (Many layers wander further from the line: of 1995 blocks most steps need more than 64 cells, and starting with 64 the search is a
+    // tenth faster where they are enough and a quarter slower where they are not.)
     uint32_t W = below_all - above_all <= (int)kWindowJump ? (ONE ? 64u : 128u) : kWindowMost;
     float most = 0.f;
     for (uint32_t i = 0; i < kPrices; ++i) most = fmaxf(most, sc.all[i] + sc.price[i] * (float)C);
